@@ -140,30 +140,58 @@ int get_rule4(bem_ctx *ctx, int cas, int rule, int q, Rule4D &out)
     r.xi = xi ? 1 : 0;
     r.q = q;
     r.n = (int)(soa.size() / kRuleCols);
-    cudaError_t e = cudaMalloc((void **)&r.d, soa.size() * sizeof(double));
+    // one allocation and one copy: the doubles, their float roundings, and the
+    // rounding remainders ((f, fl) is the rule as double-float pairs)
+    const size_t n = soa.size();
+    std::vector<double> buf(2 * n);
+    std::memcpy(buf.data(), soa.data(), n * sizeof(double));
+    float *sf = reinterpret_cast<float *>(buf.data() + n);
+    for (size_t k = 0; k < n; ++k) {
+        sf[k] = (float)soa[k];
+        sf[n + k] = (float)(soa[k] - (double)sf[k]);
+    }
+    cudaError_t e = cudaMalloc((void **)&r.d, buf.size() * sizeof(double));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
-    e = cudaMemcpy(r.d, soa.data(), soa.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpy(rule)");
-    std::vector<float> sf(soa.begin(), soa.end());
-    e = cudaMalloc((void **)&r.f, sf.size() * sizeof(float));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
-    e = cudaMemcpy(r.f, sf.data(), sf.size() * sizeof(float), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpy(rule)");
-    // the rounding remainders: (f, fl) is the rule as double-float pairs
-    std::vector<float> sl(soa.size());
-    for (size_t k = 0; k < soa.size(); ++k) sl[k] = (float)(soa[k] - (double)sf[k]);
-    e = cudaMalloc((void **)&r.fl, sl.size() * sizeof(float));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
-    e = cudaMemcpy(r.fl, sl.data(), sl.size() * sizeof(float), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpy(rule)");
+    r.f = reinterpret_cast<float *>(r.d + n);
+    r.fl = r.f + n;
+    e = cudaMemcpy(r.d, buf.data(), buf.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaFree(r.d);
+        return cuda_fail(ctx, e, "cudaMemcpy(rule)");
+    }
     ctx->rules4[key] = r;
+    out = r;
+    return BEM_OK;
+}
+
+// The FP64 form's fixed-point table of a touching rule with xi integrated out,
+// built on first use per basis.
+int touch_table(bem_ctx *ctx, int cas, int q, int basis, Rule4D &out)
+{
+    Rule4D &r = ctx->rules4[std::make_tuple(cas, kRuleXiOut, q)];
+    int2 *&tab = basis == BEM_P0 ? r.fx0 : r.fx1;
+    if (!tab) {
+        std::vector<int32_t> words;
+        if (!make_touch_fixed(cas, q, basis, words)) return fail(ctx, BEM_ERR_INVALID_ARG, "bad rule");
+        int2 *d = nullptr;
+        cudaError_t e = cudaMalloc((void **)&d, words.size() * sizeof(int32_t));
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
+        e = cudaMemcpy(d, words.data(), words.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFree(d);
+            return cuda_fail(ctx, e, "cudaMemcpy(rule)");
+        }
+        tab = d;
+    }
     out = r;
     return BEM_OK;
 }
 
 int touch_rule(bem_ctx *ctx, int cas, int q, int kind, int basis, bool f32, Rule4D &out)
 {
-    return get_rule4(ctx, cas, touch_xi_out(kind, basis, q, f32) ? kRuleXiOut : 0, q, out);
+    const bool xi = touch_xi_out(kind, basis, q, f32);
+    const int rc = get_rule4(ctx, cas, xi ? kRuleXiOut : 0, q, out);
+    return rc || !xi || f32 ? rc : touch_table(ctx, cas, q, basis, out);
 }
 
 // Evaluates every touching pair of the mesh into its touching table.
@@ -223,6 +251,7 @@ int run_guard(bem_ctx *ctx, Mesh *m, const BlockLaunch &L, const bem_quad_desc &
         if (ctx->guard_buf) {
             cudaStreamSynchronize(ctx->stream);
             cudaFree(ctx->guard_buf);
+    cudaFree(ctx->scratch);
             ctx->guard_buf = nullptr;
             ctx->guard_cap = 0;
         }
@@ -343,6 +372,18 @@ namespace bem {
 
 int api_fail(bem_ctx *ctx, int code, const char *msg) { return fail(ctx, code, msg); }
 int api_ensure_prefix(bem_ctx *ctx, int64_t n) { return ensure_prefix(ctx, n); }
+int api_ensure_scratch(bem_ctx *ctx, size_t bytes)
+{
+    if (bytes <= ctx->scratch_cap) return BEM_OK;
+    cudaStreamSynchronize(ctx->stream);   // earlier calls may still read the old one
+    cudaFree(ctx->scratch);
+    ctx->scratch = nullptr;
+    ctx->scratch_cap = 0;
+    cudaError_t e = cudaMalloc(&ctx->scratch, bytes);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(scratch)");
+    ctx->scratch_cap = bytes;
+    return BEM_OK;
+}
 int api_cuda_fail(bem_ctx *ctx, cudaError_t e, const char *where) { return cuda_fail(ctx, e, where); }
 int api_touch_rule(bem_ctx *ctx, int cas, int q, int kind, int basis, bool f32, Rule4D &out)
 {
@@ -420,9 +461,9 @@ int bem_destroy(bem_ctx *ctx)
     plan_forget(ctx);
     for (auto &kv : ctx->meshes) free_mesh(kv.second);
     for (auto &kv : ctx->rules4) {
-        cudaFree(kv.second.d);
-        cudaFree(kv.second.f);
-        cudaFree(kv.second.fl);
+        cudaFree(kv.second.d);      // holds f and fl too
+        cudaFree(kv.second.fx0);
+        cudaFree(kv.second.fx1);
     }
     for (auto &r : ctx->prof_pending) {
         cudaEventDestroy(r.a);
@@ -432,6 +473,7 @@ int bem_destroy(bem_ctx *ctx)
     cudaFree(ctx->status);
     cudaFree(ctx->tile_prefix);
     cudaFree(ctx->guard_buf);
+    cudaFree(ctx->scratch);
     learned_free(ctx->learned);
     delete ctx;
     return BEM_OK;

@@ -121,10 +121,12 @@ __global__ void __launch_bounds__(1024) k_job_scan(const int64_t *job_total, int
     for (int k = lo; k < hi; ++k) job_end[k] += base;
 }
 
-// The float form is capped at 64 registers (four CTAs, 32 warps per SM): the
-// tiles' dependent loads (block, cluster, index, geometry) want the warps.
+// Capped at 64 registers (four CTAs, 32 warps per SM): the float form's
+// dependent loads (block, cluster, index, geometry) and the FP64 form's integer
+// chains (bem_fixed_pair.cuh) want the warps.
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(256, MIXED ? 4 : 1) k_block_p0(MeshView m, BlockLaunch L, Rule2D R,
+__global__ void __launch_bounds__(256, 4) k_block_p0(MeshView m, BlockLaunch L,
+                                                  const __grid_constant__ Rule2D R,
                                                   const int64_t *__restrict__ prefix,
                                                   int *status)
 {
@@ -147,9 +149,9 @@ __global__ void __launch_bounds__(256, MIXED ? 4 : 1) k_block_p0(MeshView m, Blo
 // same tile body as the single-list kernels, so the results are identical.
 // ---------------------------------------------------------------------------
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(256, MIXED ? 4 : 1) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
-                                                  const int64_t *__restrict__ job_end, Rule2D R,
-                                                  int *status)
+__global__ void __launch_bounds__(256, 4) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
+                                                  const int64_t *__restrict__ job_end,
+                                                  const __grid_constant__ Rule2D R, int *status)
 {
     // contiguous runs of tiles per CTA (see k_block_p0); the block hint is
     // kept while the run stays in one job

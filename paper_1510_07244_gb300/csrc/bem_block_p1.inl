@@ -12,8 +12,8 @@
 namespace bem {
 
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(p1_threads(MIXED), p1_min_blocks(MIXED))
-k_block_p1(MeshView m, BlockLaunch L, Rule2D R, const int64_t *__restrict__ prefix, int *status)
+__global__ void __launch_bounds__(p1_threads(MIXED), p1_min_blocks(MIXED, KIND))
+k_block_p1(MeshView m, BlockLaunch L, const __grid_constant__ Rule2D R, const int64_t *__restrict__ prefix, int *status)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t total = L.n_blocks > 0 ? prefix[L.n_blocks - 1] : 0;
@@ -22,9 +22,9 @@ k_block_p1(MeshView m, BlockLaunch L, Rule2D R, const int64_t *__restrict__ pref
 }
 
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(p1_threads(MIXED), p1_min_blocks(MIXED))
+__global__ void __launch_bounds__(p1_threads(MIXED), p1_min_blocks(MIXED, KIND))
 k_batch_p1(const BatchJob *__restrict__ jobs, int n_jobs, const int64_t *__restrict__ job_end,
-           Rule2D R, int *status)
+           const __grid_constant__ Rule2D R, int *status)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int64_t next_tile;

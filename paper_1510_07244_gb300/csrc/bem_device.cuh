@@ -766,12 +766,13 @@ __device__ __forceinline__ FF operator-(FF a, FF b)
     return r;
 }
 
-// xi = 1: the rule has xi integrated out (Laplace kernels only, see
-// touch_xi_out); the moments take their xi_moment factors at the end.
+// xi = 1: the rule has xi integrated out (see touch_xi_out): the Laplace moments
+// take their xi_moment factors at the end; the complex kinds run over the Gauss
+// nodes of xi (X) at each point.
 template <int KIND, int BASIS, int CAS>
 __device__ __forceinline__ void touch_pair(const MeshView &m, int idx, const double *__restrict__ rule,
-                                           int np, double kappa, int lane, double eta = 0.0,
-                                           int xi = 0)
+                                           int np, double kappa, int lane, double eta, int xi,
+                                           const XiFixed &X)
 {
     const int a = __ldg(m.nb_src + idx), b = __ldg(m.nb_tri + idx);
     const int pc = __ldg(m.nb_perm + idx);
@@ -832,33 +833,44 @@ __device__ __forceinline__ void touch_pair(const MeshView &m, int idx, const dou
                 dy = x1 * e1a[1] + x2 * e2a[1] - y1 * e1b[1] - y2 * e2b[1];
                 dz = x1 * e1a[2] + x2 * e2a[2] - y1 * e1b[2] - y2 * e2b[2];
             }
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double ri = rsqrt(r2);
-            double kr, ki = 0.0;
-            if (KIND == BEM_LAPLACE_SLP) {
-                kr = ri;
-            } else if (KIND == BEM_LAPLACE_DLP) {
-                const double dn = CAS == kEdge ? x2 * H : dx * nb[0] + dy * nb[1] + dz * nb[2];
-                kr = dn * ri * ri * ri;
-            } else if (KIND == BEM_HELMHOLTZ_SLP) {
-                double sn, cs;
-                sincos(kappa * (r2 * ri), &sn, &cs);
-                kr = cs * ri;
-                ki = sn * ri;
+            double kr = 0.0, ki = 0.0;
+            if (CPLX) {
+                // one node (1, 1) without the sum over xi; a node scales the point by g
+                // and the weight by its own weight times g^3
+                const int nk = xi ? X.q : 1;
+#pragma unroll 1
+                for (int k = 0; k < nk; ++k) {
+                    const double g = xi ? X.g[k] : 1.0, wg = xi ? X.w[k] * g * g * g : 1.0;
+                    const double ex = g * dx, ey = g * dy, ez = g * dz;
+                    const double r2 = ex * ex + ey * ey + ez * ez;
+                    const double ri = rsqrt(r2);
+                    const double kd = kappa * (r2 * ri);
+                    double sn, cs;
+                    sincos(kd, &sn, &cs);
+                    if (KIND == BEM_HELMHOLTZ_SLP) {
+                        kr += wg * cs * ri;
+                        ki += wg * sn * ri;
+                        continue;
+                    }
+                    // Helmholtz double layer (and Brakhage-Werner): the height is
+                    // zero on an identical flat pair, x2 H on a common edge
+                    const double dn = CAS == kIdentical ? 0.0
+                                      : (CAS == kEdge ? g * x2 * H : ex * nb[0] + ey * nb[1] + ez * nb[2]);
+                    const double f = dn * ri * ri * ri;
+                    double vr = f * (cs + kd * sn), vi = f * (sn - kd * cs);
+                    if (KIND == BEM_HELMHOLTZ_BW) {
+                        vr += eta * sn * ri;
+                        vi -= eta * cs * ri;
+                    }
+                    kr += wg * vr;
+                    ki += wg * vi;
+                }
             } else {
-                // Helmholtz double layer (and Brakhage-Werner): the height is
-                // zero on an identical flat pair, x2 H on a common edge
-                const double dn = CAS == kIdentical ? 0.0
-                                  : (CAS == kEdge ? x2 * H : dx * nb[0] + dy * nb[1] + dz * nb[2]);
-                const double kd = kappa * (r2 * ri);
-                double sn, cs;
-                sincos(kd, &sn, &cs);
-                const double f = dn * ri * ri * ri;
-                kr = f * (cs + kd * sn);
-                ki = f * (sn - kd * cs);
-                if (KIND == BEM_HELMHOLTZ_BW) {
-                    kr += eta * sn * ri;
-                    ki -= eta * cs * ri;
+                const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+                kr = ri;
+                if (KIND == BEM_LAPLACE_DLP) {
+                    const double dn = CAS == kEdge ? x2 * H : dx * nb[0] + dy * nb[1] + dz * nb[2];
+                    kr = dn * ri * ri * ri;
                 }
             }
             const double wr = w * kr, wi = w * ki;
@@ -1239,43 +1251,44 @@ __device__ __forceinline__ void touch_f32(const MeshView &m, int idx, const floa
 }
 
 // ---------------------------------------------------------------------------
-// Regular pair integrals in one thread (product of a 2D rule with itself).
+// Regular pair integrals in FP64 arithmetic (product of a 2D rule with itself):
+// the few pairs whose distances span more than the fixed-point range of
+// bem_fixed_pair.cuh.  Not inlined, loops rolled: one small copy per kernel.
 // ---------------------------------------------------------------------------
-template <int KIND, int NP>
-__device__ __forceinline__ void regular_p0(const Tri &A, const Tri &B, const Rule2D &R,
-                                           double kappa, double &out_re, double &out_im,
-                                           double eta = 0.0)
-{
-    double e1a[3], e2a[3], d0[3], yx[NP], yy[NP], yz[NP];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        e1a[c] = A.v[1][c] - A.v[0][c];
-        e2a[c] = A.v[2][c] - A.v[1][c];
-        d0[c] = A.v[0][c] - B.v[0][c];
-    }
+// Trial points relative to B's vertex 0, test points relative to them
+struct PairFrame {
+    double d0[3], e1a[3], e2a[3], e1b[3], e2b[3];
+    __device__ __forceinline__ PairFrame(const Tri &A, const Tri &B)
     {
-        const double e1b0 = B.v[1][0] - B.v[0][0], e1b1 = B.v[1][1] - B.v[0][1],
-                     e1b2 = B.v[1][2] - B.v[0][2];
-        const double e2b0 = B.v[2][0] - B.v[1][0], e2b1 = B.v[2][1] - B.v[1][1],
-                     e2b2 = B.v[2][2] - B.v[1][2];
 #pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            yx[j] = R.s[j] * e1b0 + R.t[j] * e2b0;
-            yy[j] = R.s[j] * e1b1 + R.t[j] * e2b1;
-            yz[j] = R.s[j] * e1b2 + R.t[j] * e2b2;
+        for (int c = 0; c < 3; ++c) {
+            d0[c] = A.v[0][c] - B.v[0][c];
+            e1a[c] = A.v[1][c] - A.v[0][c];
+            e2a[c] = A.v[2][c] - A.v[1][c];
+            e1b[c] = B.v[1][c] - B.v[0][c];
+            e2b[c] = B.v[2][c] - B.v[1][c];
         }
     }
+    __device__ __forceinline__ double diff(int c, double s, double t, double u, double v) const
+    {
+        return (d0[c] + s * e1a[c] + t * e2a[c]) - (u * e1b[c] + v * e2b[c]);
+    }
+};
+
+template <int KIND>
+__device__ __noinline__ void double_p0(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
+                                       double &out_re, double &out_im, double eta)
+{
+    const PairFrame F(A, B);
     double sr = 0.0, si = 0.0;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        const double xx = d0[0] + R.s[i] * e1a[0] + R.t[i] * e2a[0];
-        const double xy = d0[1] + R.s[i] * e1a[1] + R.t[i] * e2a[1];
-        const double xz = d0[2] + R.s[i] * e1a[2] + R.t[i] * e2a[2];
+#pragma unroll 1
+    for (int i = 0; i < R.np; ++i) {
         double ir = 0.0, ii = 0.0;
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
+#pragma unroll 1
+        for (int j = 0; j < R.np; ++j) {
             double kr, ki;
-            kval<KIND>(xx - yx[j], xy - yy[j], xz - yz[j], B.n, kappa, kr, ki, eta);
+            kval<KIND>(F.diff(0, R.s[i], R.t[i], R.s[j], R.t[j]), F.diff(1, R.s[i], R.t[i], R.s[j], R.t[j]),
+                       F.diff(2, R.s[i], R.t[i], R.s[j], R.t[j]), B.n, kappa, kr, ki, eta);
             ir += R.w[j] * kr;
             if (kind_complex(KIND)) ii += R.w[j] * ki;
         }
@@ -1287,68 +1300,62 @@ __device__ __forceinline__ void regular_p0(const Tri &A, const Tri &B, const Rul
     out_im = si * scale;
 }
 
-template <int KIND, int NP>
-__device__ __forceinline__ void regular_p1(const Tri &A, const Tri &B, const Rule2D &R,
-                                           double kappa, double *accr, double *acci,
-                                           double eta = 0.0)
+template <int KIND>
+__device__ __noinline__ void double_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
+                                       double *accr, double *acci, double eta)
 {
-    double e1a[3], e2a[3], d0[3], yx[NP], yy[NP], yz[NP];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        e1a[c] = A.v[1][c] - A.v[0][c];
-        e2a[c] = A.v[2][c] - A.v[1][c];
-        d0[c] = A.v[0][c] - B.v[0][c];
-    }
-    {
-        const double e1b0 = B.v[1][0] - B.v[0][0], e1b1 = B.v[1][1] - B.v[0][1],
-                     e1b2 = B.v[1][2] - B.v[0][2];
-        const double e2b0 = B.v[2][0] - B.v[1][0], e2b1 = B.v[2][1] - B.v[1][1],
-                     e2b2 = B.v[2][2] - B.v[1][2];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            yx[j] = R.s[j] * e1b0 + R.t[j] * e2b0;
-            yy[j] = R.s[j] * e1b1 + R.t[j] * e2b1;
-            yz[j] = R.s[j] * e1b2 + R.t[j] * e2b2;
-        }
-    }
-#pragma unroll
+    const PairFrame F(A, B);
+#pragma unroll 1
     for (int k = 0; k < 9; ++k) accr[k] = acci[k] = 0.0;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        const double xx = d0[0] + R.s[i] * e1a[0] + R.t[i] * e2a[0];
-        const double xy = d0[1] + R.s[i] * e1a[1] + R.t[i] * e2a[1];
-        const double xz = d0[2] + R.s[i] * e1a[2] + R.t[i] * e2a[2];
+    const double scale = A.sg * B.sg * kInv4Pi;
+#pragma unroll 1
+    for (int i = 0; i < R.np; ++i) {
         double ir[3] = {0.0, 0.0, 0.0}, ii[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
+#pragma unroll 1
+        for (int j = 0; j < R.np; ++j) {
             double kr, ki;
-            kval<KIND>(xx - yx[j], xy - yy[j], xz - yz[j], B.n, kappa, kr, ki, eta);
+            kval<KIND>(F.diff(0, R.s[i], R.t[i], R.s[j], R.t[j]), F.diff(1, R.s[i], R.t[i], R.s[j], R.t[j]),
+                       F.diff(2, R.s[i], R.t[i], R.s[j], R.t[j]), B.n, kappa, kr, ki, eta);
             const double lb[3] = {1.0 - R.s[j], R.s[j] - R.t[j], R.t[j]};
-            const double wr = R.w[j] * kr;
-            const double wi = R.w[j] * ki;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                ir[q] += wr * lb[q];
-                if (kind_complex(KIND)) ii[q] += wi * lb[q];
+                ir[q] += R.w[j] * kr * lb[q];
+                ii[q] += R.w[j] * ki * lb[q];
             }
         }
         const double la[3] = {1.0 - R.s[i], R.s[i] - R.t[i], R.t[i]};
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            const double f = R.w[i] * la[p];
+        for (int p = 0; p < 3; ++p)
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                accr[p * 3 + q] += f * ir[q];
-                if (kind_complex(KIND)) acci[p * 3 + q] += f * ii[q];
+                accr[p * 3 + q] += R.w[i] * la[p] * ir[q] * scale;
+                if (kind_complex(KIND)) acci[p * 3 + q] += R.w[i] * la[p] * ii[q] * scale;
             }
-        }
     }
-    const double scale = A.sg * B.sg * kInv4Pi;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        accr[k] *= scale;
-        acci[k] *= scale;
-    }
+}
+
+}  // namespace bem
+
+#include "bem_fixed_pair.cuh"
+
+namespace bem {
+
+// The FP64 form's regular pairs: fixed point, or FP64 arithmetic where a pair's
+// distances span more than the fixed-point range (S / r above 16).
+template <int KIND, int NP>
+__device__ __forceinline__ void regular_p0(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
+                                           double &out_re, double &out_im, double eta)
+{
+    if (!fixed_p0<KIND, NP>(A, B, R, kappa, out_re, out_im, eta))
+        double_p0<KIND>(A, B, R, kappa, out_re, out_im, eta);
+}
+
+template <int KIND, int NP>
+__device__ __forceinline__ void regular_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
+                                           double *accr, double *acci, double eta)
+{
+    if (!fixed_p1<KIND, NP>(A, B, R, kappa, accr, acci, eta))
+        double_p1<KIND>(A, B, R, kappa, accr, acci, eta);
 }
 
 // ---------------------------------------------------------------------------
@@ -1692,11 +1699,11 @@ __device__ __forceinline__ int p1_load_support(const int32_t *__restrict__ rec, 
     return nt;
 }
 
-// Threads per CTA of the P1 block engine: the FP64 form saturates the FP64
-// pipe with one 256-thread CTA per SM; the float form runs 128-thread CTAs,
-// several per SM, so that one CTA's barrier waits overlap another's math.
+// Threads per CTA of the P1 block engine: 128 in the float form, several CTAs per
+// SM, so that one CTA's barrier waits overlap another's math; 256 in the FP64
+// form, two CTAs per SM (one for the complex kinds, whose sums need the registers).
 __host__ __device__ constexpr int p1_threads(bool mixed) { return mixed ? 128 : 256; }
-__host__ __device__ constexpr int p1_min_blocks(bool mixed) { return mixed ? 4 : 1; }
+__host__ __device__ constexpr int p1_min_blocks(bool mixed, int kind) { return mixed ? 4 : (kind_complex(kind) ? 1 : 2); }
 
 // One 32 x 32 tile of one block list (called by every thread of the CTA).
 template <int KIND, int NP, bool MIXED>

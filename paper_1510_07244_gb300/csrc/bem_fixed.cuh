@@ -1,0 +1,204 @@
+// 64-bit fixed-point arithmetic for the FP64 form's quadrature points.
+//
+// The FP64 pipe of sm_103a retires 2 lanes per SM and cycle (measured: 1.6
+// DFMA), the integer pipe 64 widening 32 x 32 + 64 multiply-adds (60 measured)
+// and 128 additions, so one FP64 operation costs as much as 30 to 70 integer
+// ones.  A quadrature point needs a difference of points, a squared distance,
+// a reciprocal square root and a weighted sum: 13 FP64 operations for the single
+// layer, about 60 with a sine and cosine.  Here the points of a pair are
+// integers scaled to the pair (62 bits), and a point costs about 75 integer
+// issue slots instead of the FP64 form's 13 x 70.
+//
+// Precision: a coordinate carries an absolute error of a few 2^-59 S, S = the
+// power of two above the largest coordinate difference of the pair; FP64
+// arithmetic on the same differences carries 2^-53 S.  The squared distance is
+// held to 2^-60 S^2, the reciprocal distance to about 2^-57 of itself.  The
+// distances of a pair must stay above S / 16 (fx_rinv flags smaller ones, and
+// the caller evaluates that pair in FP64); disjoint pairs of shape-regular
+// meshes keep S / r below 8 or so.
+//
+// Host compilable (tests of the arithmetic on the CPU).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include <string.h>
+
+#include <cmath>
+
+namespace bem {
+
+#define BEM_HD __host__ __device__ __forceinline__
+
+typedef long long s64;
+typedef unsigned long long u64;
+
+// h 2^32 + l with l signed: products of two such numbers need signed 32 x 32
+// multiplications only.
+struct Fx2 {
+    int h, l;
+};
+
+BEM_HD Fx2 fx_split(s64 a)
+{
+    Fx2 r;
+    r.l = (int)(unsigned)(u64)a;
+    r.h = (int)(a >> 32) + (int)((unsigned)(u64)a >> 31);
+    return r;
+}
+
+BEM_HD s64 fx_mad(int a, int b, s64 c) { return (s64)a * (s64)b + c; }
+
+// a b / 2^64 rounded, the product of the low words dropped (at most a quarter
+// unit); |a.h|, |b.h| <= 2^30 keep the middle sum within 64 bits
+BEM_HD s64 fx_mul(Fx2 a, Fx2 b)
+{
+    const s64 mid = fx_mad(a.h, b.l, fx_mad(a.l, b.h, (s64)1 << 31));
+    return fx_mad(a.h, b.h, mid >> 32);
+}
+
+// a b / 2^(64 - K): K more bits of the same product (which must fit)
+template <int K>
+BEM_HD s64 fx_mul_up(Fx2 a, Fx2 b)
+{
+    const s64 mid = fx_mad(a.h, b.l, fx_mad(a.l, b.h, (s64)1 << (31 - K)));
+    return (s64)((u64)((s64)a.h * b.h) << K) + (mid >> (32 - K));
+}
+
+BEM_HD int fx_float_bits(float f)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_int(f);
+#else
+    int i;
+    memcpy(&i, &f, 4);
+    return i;
+#endif
+}
+
+BEM_HD float fx_rsqrt_estimate(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / sqrtf(x);
+#endif
+}
+
+BEM_HD int fx_round(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float2int_rn(x);
+#else
+    return (int)lrintf(x);
+#endif
+}
+
+// Squared length of (x, y, z), |x|, |y|, |z| <= 2^62: the sum of squares / 2^64
+// (the squares of the low words dropped: below one unit), at most 3 2^60.
+BEM_HD s64 fx_norm2(s64 x, s64 y, s64 z)
+{
+    const Fx2 a = fx_split(x), b = fx_split(y), c = fx_split(z);
+    const s64 hh = fx_mad(a.h, a.h, fx_mad(b.h, b.h, (s64)c.h * c.h));
+    const s64 hl = fx_mad(a.h, a.l, fx_mad(b.h, b.l, fx_mad(c.h, c.l, (s64)1 << 30)));
+    return hh + (hl >> 31);
+}
+
+// Reciprocal square root: r2 = 2^60 (r / S)^2 -> 2^(62 - kb) S / r, given
+// S / r <= 2^kb, 0 <= kb <= 4.  A 20-bit estimate m of 2^16 S / r (hardware
+// reciprocal square root, rounded by adding 12, whose ulp is 2^-20) has the
+// residual E = 1 - r2 m^2 / 2^92 with |E| < 2^-15, formed exactly to 2^-60;
+// (1 - E)^(-1/2) = 1 + E/2 + 3/8 E^2 + 5/16 E^3 + ... corrects it, the second
+// and third terms in float (they are below 2^-31, so 24 bits leave 2^-56).
+// flag collects the estimates: any bit from 2^20 on means a distance below
+// S / 16 (or a zero one), where the result is meaningless.
+BEM_HD s64 fx_rinv(s64 r2, int kb, int &flag)
+{
+    const unsigned rl = (unsigned)(u64)r2, rh = (unsigned)((u64)r2 >> 32);
+    const float y = fx_rsqrt_estimate((float)(int)rh);
+    const float g = y * 1024.0f + 12.0f;
+    const unsigned m = (unsigned)(fx_float_bits(g) - 0x41400000);
+    flag |= (int)m;
+    const u64 q = (u64)m * m;
+    const unsigned ql = (unsigned)q, qh = (unsigned)(q >> 32);
+    // r2 q / 2^32 modulo 2^64 (it is 2^60 (1 - E))
+    u64 b = (u64)rh * ql + (((u64)rl * ql) >> 32);
+    b += (u64)rl * qh;
+    b += (u64)(rh * qh) << 32;
+    const s64 E = (s64)(((u64)1 << 60) - b);
+    const float e = (float)(int)(E >> 15);          // E 2^45
+    // 2 c = E + 3/4 E^2 + 5/8 E^3 in units of 2^-60
+    const float k2 = e * (float)(0.625 / 1073741824.0 / 35184372088832.0) + (float)(0.75 / 1073741824.0);
+    const s64 C = E + (s64)fx_round((e * e) * k2);
+    // m (1 + c) 2^(46 - kb)
+    const s64 mc = (s64)((u64)m * (unsigned)(u64)C + ((u64)(m * (unsigned)((u64)C >> 32)) << 32));
+    return ((s64)m << (46 - kb)) + (mc >> (15 + kb));
+}
+
+// Cosine and sine of `turn` (2^64 = one turn), scaled by 2^61.  The argument is
+// reduced to an eighth of a turn on either side of a multiple of a quarter;
+// Taylor polynomials in the squared remainder (quarter turns), the terms from the
+// fifth power of the square on in 32 bits (below 2^-28 of the result's unit
+// sum).  Truncation below 2^-58.
+// (pi/2)^n / n! in units of 2^-61 (n <= 9), 2^-45 (even n from 10 on) and 2^-48 (odd n from 11 on)
+constexpr s64 kFxT1 = 3622009729038561421ll;
+constexpr s64 kFxT2 = 2844719788994575541ll;
+constexpr s64 kFxT3 = 1489491798437810879ll;
+constexpr s64 kFxT4 = 584922061444309466ll;
+constexpr s64 kFxT5 = 183758685115604026ll;
+constexpr s64 kFxT6 = 48107911266041808ll;
+constexpr s64 kFxT7 = 10795390043781899ll;
+constexpr s64 kFxT8 = 2119669878386351ll;
+constexpr s64 kFxT9 = 369952184331896ll;
+constexpr int kFxT10 = 886718036;
+constexpr int kFxT11 = 1012984316;
+constexpr int kFxT12 = 16574917;
+constexpr int kFxT13 = 16022042;
+constexpr int kFxT14 = 224709;
+constexpr int kFxT15 = 188251;
+constexpr int kFxT16 = 2310;
+constexpr int kFxT17 = 1708;
+BEM_HD int fx_mulhi(int a, int b)
+{
+#ifdef __CUDA_ARCH__
+    return __mulhi(a, b);
+#else
+    return (int)(((s64)a * b) >> 32);
+#endif
+}
+
+BEM_HD void fx_sincos(u64 turn, s64 &c, s64 &s)
+{
+    const unsigned quad = (unsigned)((turn + ((u64)1 << 61)) >> 62);
+    // remainder, 2^63 = a quarter turn (at 2^64 a value next to half of one has no split)
+    const Fx2 xs = fx_split((s64)(turn << 2) >> 1);
+    const s64 z = fx_mul_up<2>(xs, xs);           // x^2 2^64 <= 2^62
+    const Fx2 zs = fx_split(z);
+    const int z32 = (int)(z >> 32);
+    // cosine: coefficients (-1)^k (pi/2)^(2k) / (2k)!; the tail k = 5..8 scaled by 2^45
+    int q = fx_mulhi(kFxT16, z32) - kFxT14;
+    q = fx_mulhi(q, z32) + kFxT12;
+    q = fx_mulhi(q, z32) - kFxT10;
+    s64 p = kFxT8 + (fx_mad(q, z32, 0) >> 16);
+    p = fx_mul(fx_split(p), zs) - kFxT6;
+    p = fx_mul(fx_split(p), zs) + kFxT4;
+    p = fx_mul(fx_split(p), zs) - kFxT2;
+    const s64 cv = fx_mul(fx_split(p), zs) + ((s64)1 << 61);
+    // sine: x times coefficients (-1)^k (pi/2)^(2k + 1) / (2k + 1)!; the tail scaled by 2^48
+    q = fx_mulhi(kFxT17, z32) - kFxT15;
+    q = fx_mulhi(q, z32) + kFxT13;
+    q = fx_mulhi(q, z32) - kFxT11;
+    p = kFxT9 + (fx_mad(q, z32, 0) >> 19);
+    p = fx_mul(fx_split(p), zs) - kFxT7;
+    p = fx_mul(fx_split(p), zs) + kFxT5;
+    p = fx_mul(fx_split(p), zs) - kFxT3;
+    p = fx_mul(fx_split(p), zs) + kFxT1;
+    const s64 sv = fx_mul_up<1>(fx_split(p), xs);
+    const s64 a = (quad & 1) ? sv : cv, b = (quad & 1) ? cv : sv;
+    c = ((quad + 1) & 2) ? -a : a;                // quadrants 1 and 2
+    s = (quad & 2) ? -b : b;
+}
+
+}  // namespace bem

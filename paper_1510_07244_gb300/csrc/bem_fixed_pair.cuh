@@ -1,0 +1,494 @@
+// Regular (disjoint) pairs of the FP64 form in the fixed-point arithmetic of
+// bem_fixed.cuh: the product of a 2D rule with itself, one thread per pair.
+// Included by bem_device.cuh (needs Tri, Rule2D and the FP64 pair integrals,
+// which take over pairs outside the fixed-point range).
+#pragma once
+
+#include "bem_fixed.cuh"
+
+namespace bem {
+
+__device__ __forceinline__ double fx_pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
+
+// Upper bound of |a|: the high word of a double, its lowest bit raised
+__device__ __forceinline__ int fx_mag(double a) { return (__double2hiint(a) & 0x7fffffff) + 1; }
+
+// kappa S / (2 pi) = kn 2^(kexp - 62), S = 2^E, |kn| <= 2^62: the factor that takes a
+// length in units of S to a phase in turns.  1 / (2 pi) and the product as sums of two
+// doubles: a relative error of kn is one of every phase of the pair.  kexp >= low.
+__device__ __forceinline__ bool fx_wave(double kappa, int E, int low, Fx2 &kn, int &kexp)
+{
+    const double hi = kappa * 0.15915494309189535;
+    const double lo = fma(kappa, 0.15915494309189535, -hi) + kappa * -9.839338337591243e-18;
+    kexp = max(((__double2hiint(hi) >> 20) & 2047) - 1022 + E, low);
+    if (kexp > 20) return false;
+    const double up = fx_pow2(62 + E - kexp);
+    kn = fx_split(__double2ll_rn(hi * up) + __double2ll_rn(lo * up));
+    return true;
+}
+
+// Weighted sum of 64-bit values T with weights w = 2^63 times a rule's:
+// value() = sum w T / 2 (the products of the low words dropped).  |T| <= 2^59
+// keeps the middle sum within 64 bits for every rule (at most 25 points).
+struct FxSum {
+    s64 hi, mid;
+    __device__ __forceinline__ void clear()
+    {
+        hi = 0;
+        mid = (s64)1 << 31;   // rounds sum()
+    }
+    __device__ __forceinline__ void add(const int32_t *w, Fx2 T)
+    {
+        hi = fx_mad(w[0], T.h, hi);
+        mid = fx_mad(w[0], T.l, fx_mad(w[1], T.h, mid));
+    }
+    __device__ __forceinline__ s64 sum() const { return hi + (mid >> 32); }
+    __device__ __forceinline__ double value() const { return (double)sum(); }
+};
+
+// Vertices of a pair relative to the trial triangle's vertex 0, scaled to
+// 2^61 / S with S = 2^E above every coordinate difference of the two triangles.
+struct FxPair {
+    s64 x0[3];                 // test triangle's vertex 0 / 4
+    Fx2 a1[3], a2[3];          // test triangle's edges v1 - v0, v2 - v1
+    Fx2 b1[3], b2[3];          // trial triangle's
+    int E;
+    int kb;                    // S / r <= 2^kb for every point of the pair (4: no bound known)
+};
+
+// kb of a lower bound r of the distances (S = 2^29)
+__device__ __forceinline__ int fx_kb(float r)
+{
+    return r >= 33554432.0f ? max(0, 29 - ((__float_as_int(r) >> 23) - 127)) : 4;
+}
+
+__device__ __forceinline__ float fx_hi(s64 v) { return (float)(int)(v >> 32); }
+
+// kb of a pair from a lower bound of its distances, the centroids' minus both
+// circumradii about them; 8 covers the truncations (X, Y: vertices at 2^61 / S)
+__device__ __forceinline__ int fx_centroid_kb(const s64 X[3][3], const s64 Y[3][3])
+{
+    float xf[3][3], yf[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            xf[k][c] = fx_hi(X[k][c]);   // S = 2^29
+            yf[k][c] = fx_hi(Y[k][c]);
+        }
+    float d2 = 0.0f, ra = 0.0f, rb = 0.0f, ca[3], cb[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        ca[c] = (xf[0][c] + xf[1][c] + xf[2][c]) * (1.0f / 3.0f);
+        cb[c] = (yf[0][c] + yf[1][c] + yf[2][c]) * (1.0f / 3.0f);
+        d2 = fmaf(ca[c] - cb[c], ca[c] - cb[c], d2);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        float u = 0.0f, v = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            u = fmaf(xf[k][c] - ca[c], xf[k][c] - ca[c], u);
+            v = fmaf(yf[k][c] - cb[c], yf[k][c] - cb[c], v);
+        }
+        ra = fmaxf(ra, u);
+        rb = fmaxf(rb, v);
+    }
+    return fx_kb((sqrtf(d2) - sqrtf(ra) - sqrtf(rb)) * 0.99999f - 8.0f);
+}
+
+// false: out of range (the caller takes the FP64 path).  BOUND: also kb (the
+// single layer's sums of 1/r do without: 2^-55 of the largest possible term).
+template <bool BOUND>
+__device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P)
+{
+    double x[3][3], y[3][3];
+    int top = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        int mx = 0, my = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k][c] = A.v[k][c] - B.v[0][c];
+            y[k][c] = B.v[k][c] - B.v[0][c];
+            mx = max(mx, fx_mag(x[k][c]));
+            my = max(my, fx_mag(y[k][c]));
+        }
+        top = max(top, fx_mag(__hiloint2double(mx, 0) + __hiloint2double(my, 0)));
+    }
+    const int e = top >> 20;               // the sum is below 2^(e - 1022)
+    if (e < 823 || e > 1223) return false;
+    P.E = e - 1022;
+    const double sc = fx_pow2(61 - P.E);
+    s64 X[3][3], Y[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            X[k][c] = __double2ll_rn(x[k][c] * sc);
+            Y[k][c] = k == 0 ? 0 : __double2ll_rn(y[k][c] * sc);
+        }
+    P.kb = 4;
+    if (BOUND) P.kb = fx_centroid_kb(X, Y);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        P.x0[c] = X[0][c] >> 2;
+        P.a1[c] = fx_split(X[1][c] - X[0][c]);
+        P.a2[c] = fx_split(X[2][c] - X[1][c]);
+        P.b1[c] = fx_split(Y[1][c]);
+        P.b2[c] = fx_split(Y[2][c] - Y[1][c]);
+    }
+    return true;
+}
+
+// v0 + s e1 + t e2 at scale 2^62 / S (v0 comes divided by 4; s, t scaled by
+// 2^62): a few units of 2^-59 S
+__device__ __forceinline__ s64 fx_point(s64 v0, Fx2 e1, Fx2 e2, const int32_t *s, const int32_t *t)
+{
+    const s64 mid = fx_mad(e1.h, s[1], fx_mad(e1.l, s[0], fx_mad(e2.h, t[1], (s64)e2.l * t[0])));
+    return fx_mad(e1.h, s[0], fx_mad(e2.h, t[0], v0 + (mid >> 32))) << 3;
+}
+
+// kb of near pairs from their points: the powers of 1/r of the double layers
+// lose 2 or 3 bits per unit of an overestimated kb.  The centroid bound is within
+// a factor 2 for pairs apart; for the others (kb >= 3) the smallest distance of
+// the rule's points in float, 7 FP32 operations per point.
+template <int NP>
+__device__ __forceinline__ int fx_near_kb(const FxPair &P, const Rule2D &R)
+{
+    float a0[3], a1[3], a2[3], b1[3], b2[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        a0[c] = 4.0f * fx_hi(P.x0[c]);
+        a1[c] = (float)P.a1[c].h;
+        a2[c] = (float)P.a2[c].h;
+        b1[c] = (float)P.b1[c].h;
+        b2[c] = (float)P.b2[c].h;
+    }
+    float lo = 3.0e38f;
+#pragma unroll 1
+    for (int j = 0; j < NP; ++j) {
+        float y[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) y[c] = fmaf(R.sf[j], b1[c], R.tf[j] * b2[c]) - a0[c];
+#pragma unroll 3
+        for (int i = 0; i < NP; ++i) {
+            float d2 = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float d = fmaf(R.sf[i], a1[c], fmaf(R.tf[i], a2[c], -y[c]));
+                d2 = fmaf(d, d, d2);
+            }
+            lo = fminf(lo, d2);
+        }
+    }
+    return fx_kb(sqrtf(lo) * 0.9999f - 32.0f);   // roundings: a few units of 2^-24 S
+}
+
+// Heights of the test triangle above the trial plane: h(s, t) = h[0] + s h[1] +
+// t h[2], in units of S / 2^58
+__device__ __forceinline__ void fx_heights(const FxPair &P, const Tri &B, s64 h[3])
+{
+    h[0] = h[1] = h[2] = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const Fx2 n = fx_split(__double2ll_rn(B.n[c] * 2305843009213693952.0));   // 2^61
+        h[0] += fx_mul(fx_split(P.x0[c] << 2), n);
+        h[1] += fx_mul(P.a1[c], n);
+        h[2] += fx_mul(P.a2[c], n);
+    }
+}
+
+// Trial-side sums of one test point: NM weights per trial point (the rule's
+// weights, or those times the three hat functions), kernel KIND.  The sums'
+// units: power 1 of 1/r 2^-(59 - kb), power 2 2^-(59 - 2 kb) and power 3
+// 2^-(57 - 3 kb) (complex kinds; 2^-(59 - 3 kb) for the Laplace double layer).
+template <int KIND, int NM>
+struct FxInner {
+    static constexpr bool HELM = kind_complex(KIND);
+    static constexpr bool P1 = KIND == BEM_LAPLACE_SLP || KIND == BEM_HELMHOLTZ_SLP ||
+                               KIND == BEM_HELMHOLTZ_BW;
+    static constexpr bool P3 = KIND == BEM_LAPLACE_DLP || KIND == BEM_HELMHOLTZ_DLP ||
+                               KIND == BEM_HELMHOLTZ_BW;
+    FxSum c1[NM], s1[NM], c2[NM], s2[NM], c3[NM], s3[NM];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int q = 0; q < NM; ++q) {
+            c1[q].clear(); s1[q].clear(); c2[q].clear();
+            s2[q].clear(); c3[q].clear(); s3[q].clear();
+        }
+    }
+    __device__ __forceinline__ void point(s64 dx, s64 dy, s64 dz, int kb, Fx2 kn, int shl,
+                                          const int32_t *const *w, int &flag)
+    {
+        const s64 r2 = fx_norm2(dx, dy, dz);
+        if (KIND == BEM_LAPLACE_SLP) {
+            const Fx2 T = fx_split(fx_rinv(r2, 7, flag));      // 2^55 S / r
+#pragma unroll
+            for (int q = 0; q < NM; ++q) c1[q].add(w[q], T);
+            return;
+        }
+        const Fx2 T = fx_split(fx_rinv(r2, kb, flag));     // 2^(62 - kb) S / r
+        Fx2 t2, t3;
+        if (P3) {
+            const s64 a = fx_mul(T, T) << (HELM ? 2 : 1);  // 2^(62 - 2 kb) (S / r)^2, Laplace 2^(61 - 2 kb)
+            t2 = fx_split(a);
+            t3 = fx_split(fx_mul(t2, T));                  // 2^(60 - 3 kb) (S / r)^3, Laplace 2^(59 - 3 kb)
+        }
+        if (!HELM) {
+#pragma unroll
+            for (int q = 0; q < NM; ++q) c3[q].add(w[q], t3);
+            return;
+        }
+        // kappa r / (2 pi) modulo 1
+        const s64 rho = fx_mul_up<4>(fx_split(r2), T);          // 2^(62 - kb) r / S
+        const u64 turn = (u64)fx_mul(fx_split(rho), kn) << shl;
+        s64 cs, sn;
+        fx_sincos(turn, cs, sn);
+        const Fx2 c = fx_split(cs), s = fx_split(sn);
+        if (P1) {
+            const Fx2 vc = fx_split(fx_mul(c, T)), vs = fx_split(fx_mul(s, T));
+#pragma unroll
+            for (int q = 0; q < NM; ++q) {
+                c1[q].add(w[q], vc);
+                s1[q].add(w[q], vs);
+            }
+        }
+        if (P3) {
+            const Fx2 vc2 = fx_split(fx_mul(c, t2)), vs2 = fx_split(fx_mul(s, t2));
+            const Fx2 vc3 = fx_split(fx_mul(c, t3)), vs3 = fx_split(fx_mul(s, t3));
+#pragma unroll
+            for (int q = 0; q < NM; ++q) {
+                c2[q].add(w[q], vc2);
+                s2[q].add(w[q], vs2);
+                c3[q].add(w[q], vc3);
+                s3[q].add(w[q], vs3);
+            }
+        }
+    }
+};
+
+// The factors that take FxInner's sums to the kernel's value (without 1/(4 pi))
+struct FxUnits {
+    double f1, f2, f3;      // 1/r, kappa / r^2, 1/r^3 (with S for the height's unit)
+    Fx2 kn;                 // kappa S / (2 pi) = kn 2^(kexp - 62)
+    int shl;
+};
+
+template <int KIND>
+__device__ __forceinline__ bool fx_units(const FxPair &P, double kappa, double eta, FxUnits &U)
+{
+    const int kb = P.kb;
+    U.f1 = fx_pow2(1 - (59 - kb) - P.E);
+    if (KIND == BEM_HELMHOLTZ_BW) U.f1 *= eta;
+    U.f2 = U.f3 = 0.0;
+    U.kn = Fx2{0, 0};
+    U.shl = 0;
+    if (KIND == BEM_LAPLACE_DLP) U.f3 = fx_pow2(1 - (59 - 3 * kb) - 2 * P.E);
+    if (kind_complex(KIND)) {
+        int kexp;
+        if (!fx_wave(kappa, P.E, -4 - kb, U.kn, kexp)) return false;   // shl >= 0
+        U.shl = 4 + kb + kexp;
+        U.f2 = kappa * fx_pow2(1 - (59 - 2 * kb) - P.E);
+        U.f3 = fx_pow2(1 - (57 - 3 * kb) - 2 * P.E);
+    }
+    return true;
+}
+
+// FxInner's sums q -> kernel sums (re, im); h: height / S
+template <int KIND, int NM>
+__device__ __forceinline__ void fx_combine(const FxInner<KIND, NM> &I, int q, const FxUnits &U, double h,
+                                           double &re, double &im)
+{
+    im = 0.0;
+    if (KIND == BEM_LAPLACE_SLP) {
+        re = I.c1[q].value();          // factor f1 at the end
+    } else if (KIND == BEM_LAPLACE_DLP) {
+        re = h * I.c3[q].value();      // factor f3 at the end
+    } else if (KIND == BEM_HELMHOLTZ_SLP) {
+        re = I.c1[q].value();
+        im = I.s1[q].value();
+    } else {
+        re = h * fma(U.f3, I.c3[q].value(), U.f2 * I.s2[q].value());
+        im = h * fma(U.f3, I.s3[q].value(), -U.f2 * I.c2[q].value());
+        if (KIND == BEM_HELMHOLTZ_BW) {
+            re = fma(U.f1, I.s1[q].value(), re);
+            im = fma(-U.f1, I.c1[q].value(), im);
+        }
+    }
+}
+
+template <int KIND>
+__device__ __forceinline__ double fx_final(const FxUnits &U)
+{
+    return KIND == BEM_LAPLACE_SLP || KIND == BEM_HELMHOLTZ_SLP ? U.f1
+                                                                : (KIND == BEM_LAPLACE_DLP ? U.f3 : 1.0);
+}
+
+// Trial points at a time: a Laplace point is about 110 instructions, a complex
+// one 400 to 580.  Three Laplace points overlap their dependent chains with 64
+// registers and 32 warps per SM (2048-triangle dense matrix, Duffy q = 3: single
+// layer 1.62 ms; all nine points unrolled at 128 registers 1.72 ms, one at a
+// time 1.80 ms); the complex chains overlap by themselves.  The trial points are
+// indexed in local memory (L1).
+template <int KIND>
+__device__ __forceinline__ constexpr int fx_unroll()
+{
+    return kind_complex(KIND) ? 1 : 3;
+}
+
+// Regular pair, piecewise constant: regular_p0's integral.
+template <int KIND, int NP>
+__device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
+                                         double &out_re, double &out_im, double eta)
+{
+    FxPair P;
+    FxUnits U;
+    if (!fx_pair<KIND != BEM_LAPLACE_SLP>(A, B, P)) return false;
+    if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
+    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
+    double h[3] = {0.0, 0.0, 0.0};
+    if (kind_has_height(KIND)) {
+        s64 hs[3];
+        fx_heights(P, B, hs);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-58);
+    }
+    s64 yx[NP], yy[NP], yz[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        yx[j] = fx_point(0, P.b1[0], P.b2[0], R.sx[j], R.tx[j]);
+        yy[j] = fx_point(0, P.b1[1], P.b2[1], R.sx[j], R.tx[j]);
+        yz[j] = fx_point(0, P.b1[2], P.b2[2], R.sx[j], R.tx[j]);
+    }
+    int flag = 0;
+    double sr = 0.0, si = 0.0;
+#pragma unroll 1
+    for (int i = 0; i < NP; ++i) {
+        const s64 xx = fx_point(P.x0[0], P.a1[0], P.a2[0], R.sx[i], R.tx[i]);
+        const s64 xy = fx_point(P.x0[1], P.a1[1], P.a2[1], R.sx[i], R.tx[i]);
+        const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
+        FxInner<KIND, 1> I;
+        I.clear();
+        constexpr int UN = fx_unroll<KIND>();
+#pragma unroll UN
+        for (int j = 0; j < NP; ++j) {
+            const int32_t *w[1] = {R.wx[3][j]};
+            I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
+        }
+        double re, im;
+        fx_combine<KIND, 1>(I, 0, U, fma(R.t[i], h[2], fma(R.s[i], h[1], h[0])), re, im);
+        sr = fma(R.w[i], re, sr);
+        if (kind_complex(KIND)) si = fma(R.w[i], im, si);
+    }
+    const double scale = A.sg * B.sg * kInv4Pi * fx_final<KIND>(U);
+    out_re = sr * scale;
+    out_im = si * scale;
+    return (flag >> (16 + P.kb)) == 0;
+}
+
+// Regular pair, piecewise linear (3 x 3 local matrix): regular_p1's integrals.
+// The nine outer sums of the Laplace kernels stay in fixed point too (27
+// widening multiply-adds per test point; in FP64 three conversions and nine
+// products would take ten times the integer work of a whole point).  The double
+// layer's heights are scaled to the largest of their three coefficients.
+template <int KIND, int NP>
+__device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
+                                         double *accr, double *acci, double eta)
+{
+    constexpr bool HELM = kind_complex(KIND);
+    FxPair P;
+    FxUnits U;
+    if (!fx_pair<KIND != BEM_LAPLACE_SLP>(A, B, P)) return false;
+    if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
+    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
+    double h[3] = {0.0, 0.0, 0.0};
+    s64 hs[3];
+    int up = 0;
+    Fx2 h1, h2;
+    if (kind_has_height(KIND)) {
+        fx_heights(P, B, hs);
+        if (HELM) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-58);
+        } else {
+            // below 2^59 each: a height, a sum of up to three, stays below 2^61
+            const s64 top = (hs[0] ^ (hs[0] >> 63)) | (hs[1] ^ (hs[1] >> 63)) | (hs[2] ^ (hs[2] >> 63));
+            up = max(__clzll(top) - 5, 0);
+            h1 = fx_split(hs[1] << up);
+            h2 = fx_split(hs[2] << up);
+        }
+    }
+    s64 yx[NP], yy[NP], yz[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        yx[j] = fx_point(0, P.b1[0], P.b2[0], R.sx[j], R.tx[j]);
+        yy[j] = fx_point(0, P.b1[1], P.b2[1], R.sx[j], R.tx[j]);
+        yz[j] = fx_point(0, P.b1[2], P.b2[2], R.sx[j], R.tx[j]);
+    }
+    int flag = 0;
+    FxSum acc[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        accr[k] = acci[k] = 0.0;
+        acc[k].clear();
+    }
+#pragma unroll 1
+    for (int i = 0; i < NP; ++i) {
+        const s64 xx = fx_point(P.x0[0], P.a1[0], P.a2[0], R.sx[i], R.tx[i]);
+        const s64 xy = fx_point(P.x0[1], P.a1[1], P.a2[1], R.sx[i], R.tx[i]);
+        const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
+        FxInner<KIND, 3> I;
+        I.clear();
+        constexpr int UN = fx_unroll<KIND>();
+#pragma unroll UN
+        for (int j = 0; j < NP; ++j) {
+            const int32_t *w[3] = {R.wx[0][j], R.wx[1][j], R.wx[2][j]};
+            I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
+        }
+        if (!HELM) {
+            Fx2 hi;   // height in units of S / 2^(58 + up)
+            if (KIND == BEM_LAPLACE_DLP)
+                hi = fx_split(fx_point((hs[0] << up) >> 2, h1, h2, R.sx[i], R.tx[i]) >> 1);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                s64 v = KIND == BEM_LAPLACE_SLP ? I.c1[q].sum() : I.c3[q].sum();
+                if (KIND == BEM_LAPLACE_DLP) v = fx_mul(fx_split(v << 5), hi);   // v below 2^57
+                const Fx2 V = fx_split(v);
+#pragma unroll
+                for (int p = 0; p < 3; ++p) acc[p * 3 + q].add(R.wx[p][i], V);
+            }
+        } else {
+            const double hi = fma(R.t[i], h[2], fma(R.s[i], h[1], h[0]));
+            double re[3], im[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) fx_combine<KIND, 3>(I, q, U, hi, re[q], im[q]);
+            const double la[3] = {R.w[i] * (1.0 - R.s[i]), R.w[i] * (R.s[i] - R.t[i]), R.w[i] * R.t[i]};
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    accr[p * 3 + q] = fma(la[p], re[q], accr[p * 3 + q]);
+                    acci[p * 3 + q] = fma(la[p], im[q], acci[p * 3 + q]);
+                }
+        }
+    }
+    double scale = A.sg * B.sg * kInv4Pi * fx_final<KIND>(U);
+    if (!HELM) {
+        // the outer sum's factor 2; the double layer: also the product's 2^64 / 2^5 and
+        // the heights' 2^(58 + up)
+        scale *= KIND == BEM_LAPLACE_SLP ? 2.0 : fx_pow2(1 + 64 - 5 - (58 + up));
+#pragma unroll
+        for (int k = 0; k < 9; ++k) accr[k] = acc[k].value() * scale;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            accr[k] *= scale;
+            acci[k] *= scale;
+        }
+    }
+    return (flag >> (16 + P.kb)) == 0;
+}
+
+}  // namespace bem

@@ -39,6 +39,9 @@ struct Rule2D {
     // w_k lambda_q(s_k, t_k) in float: the weights times the three linear
     // basis functions of the reference triangle, lambda = (1 - s, s - t, t)
     float wl[3][kMaxNp];
+    // the rule in fixed point (bem_fixed.cuh), high and signed low words: s, t
+    // times 2^62; w lambda_q (q < 3) and w (q = 3) times 2^63
+    int32_t sx[kMaxNp][2], tx[kMaxNp][2], wx[4][kMaxNp][2];
 };
 
 // 4D rule on D x D, device SoA with kRuleCols columns of n values:
@@ -52,7 +55,28 @@ struct Rule4D {
     float *f = nullptr;    // device, kRuleCols n floats (mixed form), may be null
     float *fl = nullptr;   // device, kRuleCols n floats: d - f (double-float form), may be null
     int xi = 0;            // 1: a touching rule with xi integrated out (at xi = 1)
+    // device, fixed-point tables of the FP64 form (rules with xi integrated out): the
+    // columns of the piecewise-constant and of the piecewise-linear basis
+    int2 *fx0 = nullptr, *fx1 = nullptr;
 };
+// Columns of a touching rule in fixed point (bem_touch_fixed.cuh): high and
+// signed low words, the coordinates times 2^61, g times 2^62, the weights times 2^63.
+// g: the factor common to the coordinates and differences of a common-edge or
+// identical rule (eta_1), 1 for a common vertex; w: the weight at xi = 1.
+enum FxTouchCol {
+    kFxX = 0,     // vertex: x1, x2, y1, y2; edge: d1, x2, y2; identical: d1, d2; each / g
+    // piecewise constant
+    kFxG = 4,     // g
+    kFxA = 5,     // w / g (terms in 1/r)
+    kFxB = 6,     // w h_k / g^3 (1/r^3): h_k = x1, x2, the coefficients of the heights
+    kFxC = 8,     // w h_k / g^2 (1/r^2)
+    kFxCols0 = 10,
+    // piecewise linear (Laplace kernels)
+    kFxMS = 4,    // (w / g) x^i y^j, i, j = 0..2 (single layer)
+    kFxMD = 13,   // vertex: w x^i y^j; edge: (w x2 / g^3) x^i y^j (double layer)
+    kFxCols1 = 22
+};
+bool make_touch_fixed(int cas, int q, int basis, std::vector<int32_t> &words);
 // Rule id of the touching rules with xi integrated out (the rule cache's key).
 constexpr int kRuleXiOut = 1;
 
@@ -69,6 +93,19 @@ struct XiRule {
     float cmid[3] = {0.0f, 0.0f, 0.0f};
 };
 bool make_xi_rule(int q, XiRule &out);
+
+// The same sums for the FP64 form in fixed point (bem_touch_fixed.cuh), powers xi^n
+// with n = 1, 2 (piecewise constant: the double layers' two powers of r): t, cp, cm
+// times 2^62, cmid times 2^59; and the Gauss nodes and weights themselves.
+constexpr int kMaxXiFixedPairs = 4;
+struct XiFixed {
+    int npair = 0, q = 0;
+    int32_t t[kMaxXiFixedPairs][2];
+    int32_t cp[kMaxXiFixedPairs][2][2], cm[kMaxXiFixedPairs][2][2];
+    int64_t cmid[2] = {0, 0};
+    double g[2 * kMaxXiFixedPairs + 1], w[2 * kMaxXiFixedPairs + 1];
+};
+bool make_xi_fixed(int q, XiFixed &out);
 
 // Device view of an uploaded mesh.
 struct MeshView {
@@ -145,6 +182,8 @@ struct bem_ctx {
     int64_t tile_prefix_cap = 0;
     void *guard_buf = nullptr;             // scratch: cancellation guard of one call
     size_t guard_cap = 0;
+    void *scratch = nullptr;               // scratch of one solver or potential call, grown to the largest
+    size_t scratch_cap = 0;
     int num_sms = 0;
     std::map<int, bem::Mesh *> meshes;
     int next_mesh = 1;
@@ -178,6 +217,7 @@ namespace bem {
 // bem_api.cpp helpers shared with the plan driver
 int api_fail(bem_ctx *ctx, int code, const char *msg);
 int api_ensure_prefix(bem_ctx *ctx, int64_t n);   // grows the tile-prefix scratch
+int api_ensure_scratch(bem_ctx *ctx, size_t bytes);   // grows ctx->scratch
 int api_cuda_fail(bem_ctx *ctx, cudaError_t e, const char *where);
 int api_check_job(bem_ctx *ctx, const bem_block_job &J, Rule2D &r2, Mesh **mesh);
 int api_get_rule4(bem_ctx *ctx, int cas, int rule, int q, Rule4D &out);
@@ -289,9 +329,11 @@ __host__ __device__ constexpr bool kind_has_height(int kind)
 __host__ __device__ constexpr int xi_base(int kind) { return kind == BEM_LAPLACE_SLP ? 2 : 1; }
 inline bool touch_xi_out(int kind, int basis, int q, bool f32)
 {
-    // the float Helmholtz single layer sums over xi at each point (XiRule)
-    if (kind == BEM_HELMHOLTZ_SLP) return f32 && q <= 2 * kMaxXiPairs;
-    if (kind != BEM_LAPLACE_SLP && kind != BEM_LAPLACE_DLP) return false;
+    // the Helmholtz kernels sum over xi at each point: the float single layer
+    // (XiRule), the FP64 form of the piecewise-constant basis (XiFixed)
+    if (kind_complex(kind))
+        return f32 ? kind == BEM_HELMHOLTZ_SLP && q <= 2 * kMaxXiPairs
+                   : basis == BEM_P0 && q <= 2 * kMaxXiFixedPairs + 1;
     const int deg = xi_base(kind) + (basis == BEM_P1 ? 2 : 0);
     return 2 * q - 1 >= deg;
 }

@@ -90,9 +90,23 @@ bool gauss_legendre_unit(int q, std::vector<double> &x, std::vector<double> &w)
     return true;
 }
 
+// v 2^bits as high and signed low words
+static void fixed_words(double v, int bits, int32_t out[2])
+{
+    const int64_t f = std::llround(v * (double)((uint64_t)1 << bits));
+    out[1] = (int32_t)(uint32_t)(uint64_t)f;
+    out[0] = (int32_t)((f - out[1]) / ((int64_t)1 << 32));
+}
+
 static void round_rule(Rule2D &r)
 {
     for (int k = 0; k < r.np; ++k) {
+        fixed_words(r.s[k], 62, r.sx[k]);
+        fixed_words(r.t[k], 62, r.tx[k]);
+        fixed_words(r.w[k] * (1.0 - r.s[k]), 63, r.wx[0][k]);
+        fixed_words(r.w[k] * (r.s[k] - r.t[k]), 63, r.wx[1][k]);
+        fixed_words(r.w[k] * r.t[k], 63, r.wx[2][k]);
+        fixed_words(r.w[k], 63, r.wx[3][k]);
         r.sf[k] = (float)r.s[k];
         r.tf[k] = (float)r.t[k];
         r.wf[k] = (float)r.w[k];
@@ -159,6 +173,33 @@ bool make_xi_rule(int q, XiRule &out)
     return true;
 }
 
+bool make_xi_fixed(int q, XiFixed &out)
+{
+    std::vector<double> g, gw;
+    if (q < 1 || q > 2 * kMaxXiFixedPairs + 1 || !gauss_legendre_unit(q, g, gw)) return false;
+    out = XiFixed();
+    out.q = q;
+    out.npair = q / 2;
+    for (int k = 0; k < q; ++k) {
+        out.g[k] = g[k];
+        out.w[k] = gw[k];
+    }
+    for (int k = 0; k < q / 2; ++k) {
+        const double a = g[q - 1 - k], b = g[k];
+        const double w = 0.5 * (gw[k] + gw[q - 1 - k]);
+        fixed_words(a - 0.5, 62, out.t[k]);
+        for (int n = 0; n < 2; ++n) {
+            const double pa = std::pow(a, 1 + n), pb = std::pow(b, 1 + n);
+            fixed_words(w * (pa + pb), 62, out.cp[k][n]);
+            fixed_words(w * (pa - pb), 62, out.cm[k][n]);
+        }
+    }
+    if (q % 2)
+        for (int n = 0; n < 2; ++n)
+            out.cmid[n] = std::llround(std::ldexp(gw[q / 2] * std::pow(0.5, 1 + n), 59));
+    return true;
+}
+
 namespace {
 
 struct Pt {
@@ -207,6 +248,54 @@ std::vector<Piece> pieces(int cas)
 }
 
 }  // namespace
+
+bool make_touch_fixed(int cas, int q, int basis, std::vector<int32_t> &words)
+{
+    std::vector<double> gl, gw;
+    if (cas < kVertex || cas > kIdentical || !gauss_legendre_unit(q, gl, gw)) return false;
+    const std::vector<Piece> P = pieces(cas);
+    const size_t n = P.size() * 2 * q * q * q;
+    words.assign(2 * (basis == BEM_P0 ? kFxCols0 : kFxCols1) * n, 0);
+    size_t p = 0;
+    auto put = [&](int col, double v, int bits) { fixed_words(v, bits, &words[2 * (col * n + p)]); };
+    // the order of make_rule4d_host with xi integrated out
+    for (const Piece &f : P)
+        for (int swap = 0; swap < 2; ++swap)
+            for (int j = 0; j < q; ++j)
+                for (int k = 0; k < q; ++k)
+                    for (int l = 0; l < q; ++l, ++p) {
+                        Pt t = f(1.0, gl[j], gl[k], gl[l]);
+                        const double w = t.w * gw[j] * gw[k] * gw[l];
+                        if (swap) {
+                            std::swap(t.x1, t.y1);
+                            std::swap(t.x2, t.y2);
+                            t.d1 = -t.d1;
+                            t.d2 = -t.d2;
+                        }
+                        const double g = cas == kVertex ? 1.0 : gl[j];
+                        const double vert[4] = {t.x1, t.x2, t.y1, t.y2};
+                        const double edge[4] = {t.d1 / g, t.x2 / g, t.y2 / g, 0.0};
+                        const double same[4] = {t.d1 / g, t.d2 / g, 0.0, 0.0};
+                        for (int c = 0; c < 4; ++c)
+                            put(kFxX + c, cas == kVertex ? vert[c] : (cas == kEdge ? edge[c] : same[c]), 61);
+                        const double x[3] = {1.0, t.x1, t.x2}, y[3] = {1.0, t.y1, t.y2};
+                        const double wd = cas == kVertex ? w : w * t.x2 / (g * g * g);
+                        if (basis == BEM_P0) {
+                            put(kFxG, g, 62);
+                            put(kFxA, w / g, 63);
+                            for (int h = cas == kVertex ? 0 : 1; h < 2 && cas != kIdentical; ++h) {
+                                put(kFxB + h, w * x[1 + h] / (g * g * g), 63);
+                                put(kFxC + h, w * x[1 + h] / (g * g), 63);
+                            }
+                        } else {
+                            for (int i = 0; i < 9; ++i) {
+                                put(kFxMS + i, w / g * x[i / 3] * y[i % 3], 63);
+                                if (cas != kIdentical) put(kFxMD + i, wd * x[i / 3] * y[i % 3], 63);
+                            }
+                        }
+                    }
+    return true;
+}
 
 bool make_rule4d_host(int cas, int regular_rule, int q, std::vector<double> &soa, bool xi_out)
 {

@@ -1,35 +1,67 @@
-// Touching-pair kernels (Sauter-Schwab rules, Section 2.2): one warp per pair,
-// single-mesh and batched forms, FP64 and the float kernels of the mixed forms.
+// Touching-pair kernels (Sauter-Schwab rules, Section 2.2): one warp per pair in
+// the FP64 form (fixed point, bem_touch_fixed.cuh), single-mesh and batched forms,
+// and the float kernels of the mixed forms.
 // Rules with xi integrated out (Rule4D::xi, the Laplace kernels, and the
 // float Helmholtz single layer with its xi sums) come from the host's choice.
 #include <cuda_runtime.h>
 
 #include "bem_device.cuh"
+#include "bem_touch_fixed.cuh"
 
 namespace bem {
 
+struct TouchRuleDev {
+    const double *d;
+    const int2 *fx;
+    int n, xi;
+};
+
+static TouchRuleDev rule_dev(const Rule4D &r, int basis)
+{
+    return TouchRuleDev{r.d, basis == BEM_P0 ? r.fx0 : r.fx1, r.n, r.xi};
+}
+
+// FP64 form of one pair: fixed point where the rule has its table (fx), FP64
+// arithmetic for the other rules and for pairs outside the fixed-point range.
 template <int KIND, int BASIS, int CAS>
-__global__ void __launch_bounds__(256) k_touching(MeshView m, const int *__restrict__ list,
-                                                  int64_t n, const double *__restrict__ rule,
-                                                  int np, double kappa, double eta, int xi)
+__device__ __noinline__ void touch_double(const MeshView &m, int idx, const double *rule, int np,
+                                          double kappa, int lane, double eta, int xi, const XiFixed &X)
+{
+    touch_pair<KIND, BASIS, CAS>(m, idx, rule, np, kappa, lane, eta, xi, X);
+}
+
+template <int KIND, int BASIS, int CAS>
+__device__ __forceinline__ void touch_fp64(const MeshView &m, int idx, const TouchRuleDev &R,
+                                           double kappa, int lane, double eta, const XiFixed &X)
+{
+    bool done = false;
+    if constexpr (!kind_complex(KIND) || BASIS == BEM_P0)
+        done = R.fx && touch_fixed<KIND, BASIS, CAS>(m, idx, R.fx, R.n, kappa, eta, lane, X);
+    if (!done) touch_double<KIND, BASIS, CAS>(m, idx, R.d, R.n, kappa, lane, eta, R.xi, X);
+}
+
+template <int KIND, int BASIS, int CAS>
+__global__ void __launch_bounds__(256) k_touching(const __grid_constant__ MeshView m, const int *__restrict__ list,
+                                                  int64_t n, TouchRuleDev R, double kappa,
+                                                  double eta, const __grid_constant__ XiFixed X)
 {
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= n) return;
-    touch_pair<KIND, BASIS, CAS>(m, __ldg(list + wid), rule, np, kappa, threadIdx.x & 31, eta, xi);
+    touch_fp64<KIND, BASIS, CAS>(m, __ldg(list + wid), R, kappa, threadIdx.x & 31, eta, X);
 }
 
 // Batched: items[k] = (job, touching index) over many meshes / kernels.
 template <int KIND, int BASIS, int CAS>
 __global__ void __launch_bounds__(256) k_touching_batch(const TouchJob *__restrict__ jobs,
                                                         const int2 *__restrict__ items, int64_t n,
-                                                        const double *__restrict__ rule, int np,
-                                                        int xi)
+                                                        TouchRuleDev R,
+                                                        const __grid_constant__ XiFixed X)
 {
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= n) return;
     const int2 it = items[wid];
-    touch_pair<KIND, BASIS, CAS>(jobs[it.x].m, it.y, rule, np, jobs[it.x].kappa, threadIdx.x & 31,
-                                 jobs[it.x].eta, xi);
+    touch_fp64<KIND, BASIS, CAS>(jobs[it.x].m, it.y, R, jobs[it.x].kappa, threadIdx.x & 31,
+                                 jobs[it.x].eta, X);
 }
 
 // Float kernels: a pair per group of LPP lanes (touch_f32).  The first group
@@ -108,7 +140,9 @@ cudaError_t launch_touching(const MeshView &m, int cas, const int *list, int64_t
 #undef BEM_TVL
         return cudaGetLastError();
     }
-#define BEM_TOUCH(K, B, C) k_touching<K, B, C><<<blocks, 256, 0, st>>>(m, list, n, rule.d, rule.n, kappa, eta, rule.xi)
+    XiFixed xf;
+    if (rule.xi && kind_complex(kind) && !make_xi_fixed(rule.q, xf)) return cudaErrorInvalidValue;
+#define BEM_TOUCH(K, B, C) k_touching<K, B, C><<<blocks, 256, 0, st>>>(m, list, n, rule_dev(rule, B), kappa, eta, xf)
 #define BEM_TOUCH_CASE(K, B)                                   \
     do {                                                       \
         if (cas == kIdentical) BEM_TOUCH(K, B, kIdentical);    \
@@ -158,7 +192,9 @@ cudaError_t launch_touching_batch(const TouchJob *jobs, int basis, int kind, int
 #undef BEM_TVBL
         return cudaGetLastError();
     }
-#define BEM_TB(K, B, C) k_touching_batch<K, B, C><<<blocks, 256, 0, st>>>(jobs, items, n, rule.d, rule.n, rule.xi)
+    XiFixed xf;
+    if (rule.xi && kind_complex(kind) && !make_xi_fixed(rule.q, xf)) return cudaErrorInvalidValue;
+#define BEM_TB(K, B, C) k_touching_batch<K, B, C><<<blocks, 256, 0, st>>>(jobs, items, n, rule_dev(rule, B), xf)
 #define BEM_TB_CASE(K, B)                                  \
     do {                                                   \
         if (cas == kIdentical) BEM_TB(K, B, kIdentical);   \

@@ -1,0 +1,321 @@
+// Touching pairs of the FP64 form in the fixed-point arithmetic of bem_fixed.cuh:
+// the Sauter-Schwab rules with xi integrated out (q^3 points per subdomain at
+// xi = 1; for the complex kinds the sum over xi at each point in node pairs), one
+// warp per pair.
+//
+// At xi = 1 every coordinate and difference of a common-edge or identical rule
+// is e1 = eta_1 times a function of (eta_2, eta_3), so the table holds the
+// columns divided by g = e1 (g = 1 for a common vertex): the direction v = (x - y)
+// / g keeps a length of the order of the edges, within the fixed-point range,
+// and r = g |v|.  The factors of g go into the weights.  A pair with a direction
+// shorter than S / 16 (slivers) returns false and is evaluated in FP64.
+#pragma once
+
+#include "bem_device.cuh"
+
+namespace bem {
+
+// Sums over xi at one direction point: G_n = sum_k w_k xi_k^n exp(i theta xi_k), n = 1, 2.
+// G_n = exp(i theta / 2) (A + i B)
+__device__ __forceinline__ void fx_xi_sum(const XiFixed &X, int n, const s64 *c, const s64 *s, Fx2 c0,
+                                          Fx2 s0, Fx2 &gr, Fx2 &gi)
+{
+    FxSum a, b;
+    a.clear();
+    b.clear();
+#pragma unroll
+    for (int j = 0; j < kMaxXiFixedPairs; ++j) {
+        if (j >= X.npair) break;
+        a.add(X.cp[j][n], fx_split(c[j]));
+        b.add(X.cm[j][n], fx_split(s[j]));
+    }
+    // A, B at 2^59, the rotation's result at 2^58; returned at 2^61
+    const Fx2 A = fx_split((a.sum() + X.cmid[n]) << 2), B = fx_split(b.sum() << 2);
+    gr = fx_split((fx_mul(A, c0) - fx_mul(B, s0)) << 3);
+    gi = fx_split((fx_mul(A, s0) + fx_mul(B, c0)) << 3);
+}
+
+template <int KIND, int BASIS, int CAS>
+__device__ __forceinline__ bool touch_fixed(const MeshView &m, int idx, const int2 *__restrict__ fx,
+                                            int np, double kappa, double eta, int lane,
+                                            const XiFixed &X)
+{
+    constexpr bool HELM = kind_complex(KIND);
+    static_assert(!HELM || BASIS == BEM_P0, "complex kinds: piecewise constant");
+    constexpr bool HEIGHT = kind_has_height(KIND) && CAS != kIdentical;
+    constexpr bool ONE = KIND == BEM_LAPLACE_SLP || KIND == BEM_HELMHOLTZ_SLP || KIND == BEM_HELMHOLTZ_BW;
+    constexpr int NH = CAS == kVertex ? 2 : 1;             // heights' coefficients
+    constexpr int H0 = CAS == kVertex ? 0 : 1;             // first of them
+    // sums: [ONE: re, im] [per height: 1/r^3 re, im, 1/r^2 re, im]; Laplace: one per height, or nine moments
+    constexpr int NS = BASIS == BEM_P1 ? 9
+                       : !HELM ? (ONE ? 1 : NH)
+                               : (ONE ? 2 : 0) + (HEIGHT ? 4 * NH : 0);
+    constexpr bool ZERO = NS == 0 || (KIND == BEM_LAPLACE_DLP && CAS == kIdentical);
+    const int a = __ldg(m.nb_src + idx), b = __ldg(m.nb_tri + idx);
+    const int pc = __ldg(m.nb_perm + idx);
+    const int *pa = c_perm[pc / 6], *pb = c_perm[pc % 6];
+    const double *ga = m.geom + (int64_t)a * kGeomStride, *gb = m.geom + (int64_t)b * kGeomStride;
+    s64 tot[NS > 0 ? NS : 1];
+#pragma unroll
+    for (int k = 0; k < (NS > 0 ? NS : 1); ++k) tot[k] = 0;
+    double h1 = 0.0, h21 = 0.0;
+    int E = 0, flag = 0, kbs = 0;
+    if (!ZERO) {
+        // lane 3 e + c: component c of edge e (a: v1 - v0, v2 - v1; b: the same)
+        double val = 0.0;
+        if (lane < 12) {
+            const int e = lane / 3, c = lane - 3 * e, hi = (e & 1) + 1;
+            const double *g = e < 2 ? ga : gb;
+            const int *p = e < 2 ? pa : pb;
+            val = __ldg(g + 3 * p[hi] + c) - __ldg(g + 3 * p[hi - 1] + c);
+        }
+        // S = 2^E above the sum of the four edges' components
+        const float f = __double2float_ru(fabs(val));
+        float sum = f + __shfl_sync(0xffffffffu, f, (lane + 3) & 31) +
+                    __shfl_sync(0xffffffffu, f, (lane + 6) & 31) +
+                    __shfl_sync(0xffffffffu, f, (lane + 9) & 31);
+        sum = fmaxf(fmaxf(__shfl_sync(0xffffffffu, sum, 0), __shfl_sync(0xffffffffu, sum, 1)),
+                    __shfl_sync(0xffffffffu, sum, 2)) * 1.000001f;
+        const int ex = __float_as_int(sum) >> 23;
+        if (ex < 7 || ex > 246) return false;   // uniform across the warp
+        E = ex - 126;
+        const Fx2 mine = fx_split(__double2ll_rn(val * fx_pow2(61 - E)));
+        Fx2 ed[4][3];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                ed[e][c].h = __shfl_sync(0xffffffffu, mine.h, 3 * e + c);
+                ed[e][c].l = __shfl_sync(0xffffffffu, mine.l, 3 * e + c);
+            }
+        // heights of a's vertices 1, 2 above b's plane (vertex 0 lies in it):
+        // x1 h1 + x2 h21, for a common edge h1 = 0
+        Fx2 n1 = {0, 0}, n2 = {0, 0};
+        int eh = 0;
+        if (HEIGHT) {
+            double t = 0.0;
+            if (lane < 6) {
+                const int k = lane / 3, c = lane - 3 * k;
+                t = (__ldg(ga + 3 * pa[k + 1] + c) - __ldg(gb + 3 * pb[0] + c)) * __ldg(gb + 9 + c);
+            }
+            t += __shfl_sync(0xffffffffu, t, (lane + 1) & 31) + __shfl_sync(0xffffffffu, t, (lane + 2) & 31);
+            const double d1 = __shfl_sync(0xffffffffu, t, 0), d2 = __shfl_sync(0xffffffffu, t, 3);
+            h1 = CAS == kVertex ? d1 : 0.0;
+            h21 = CAS == kVertex ? d2 - d1 : d2;
+            if (BASIS == BEM_P1 && CAS == kVertex) {
+                // both below 2^59 in units of 2^(eh - 59)
+                eh = (max(fx_mag(h1), fx_mag(h21)) >> 20) - 1022;
+                eh = max(eh, -900);
+                n1 = fx_split(__double2ll_rn(h1 * fx_pow2(59 - eh)));
+                n2 = fx_split(__double2ll_rn(h21 * fx_pow2(59 - eh)));
+            }
+        }
+        Fx2 kn = {0, 0};
+        int kexp = -2;
+        if (HELM && !fx_wave(kappa, E, -2, kn, kexp)) return false;   // uniform across the warp
+        auto col = [&](int c, int p) {
+            const int2 v = __ldg(fx + (int64_t)c * np + p);
+            Fx2 r;
+            r.h = v.x;
+            r.l = v.y;
+            return r;
+        };
+        // kb: S / |v| <= 2^kb, from the shortest direction of all points in float (a
+        // tenth of a point's work; the powers of 1/r gain up to 3 bits per unit)
+        float lo = 3.0e38f;
+#pragma unroll 2
+        for (int p = lane; p < np; p += 32) {
+            const float w0 = (float)__ldg(&fx[p].x), w1 = (float)__ldg(&fx[np + p].x);
+            const float w2 = CAS != kIdentical ? (float)__ldg(&fx[2 * np + p].x) : 0.0f;
+            const float w3 = CAS == kVertex ? (float)__ldg(&fx[3 * np + p].x) : 0.0f;
+            float d2 = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float d = fmaf(w0, (float)ed[0][c].h, w1 * (float)ed[1][c].h);
+                if (CAS == kVertex) d = fmaf(-w2, (float)ed[2][c].h, fmaf(-w3, (float)ed[3][c].h, d));
+                if (CAS == kEdge) d = fmaf(-w2, (float)ed[3][c].h, d);
+                d2 = fmaf(d, d, d2);
+            }
+            lo = fminf(lo, d2);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        const int kb = fx_kb(sqrtf(lo) * (float)(0.9999 / 536870912.0) - 64.0f);   // 2^58 -> 2^29
+        // a lane's points in runs of 4: values up to 2^61 keep the sums' middle parts
+        // within 64 bits
+        constexpr int RUN = 32 * 4;
+        for (int p0 = lane; p0 < np; p0 += RUN) {
+            FxSum acc[NS > 0 ? NS : 1];
+#pragma unroll
+            for (int k = 0; k < NS; ++k) acc[k].clear();
+#pragma unroll 1
+            for (int p = p0; p < min(np, p0 + RUN); p += 32) {
+                // direction at 2^62 / S
+                s64 v[3];
+                const Fx2 u0 = col(kFxX, p), u1 = col(kFxX + 1, p);
+                Fx2 u2 = {0, 0}, u3 = {0, 0};
+                if (CAS != kIdentical) u2 = col(kFxX + 2, p);
+                if (CAS == kVertex) u3 = col(kFxX + 3, p);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    // identical: d1 e1 + d2 e2; edge: d1 e1 + x2 e2 - y2 e2b;
+                    // vertex: x1 e1 + x2 e2 - y1 e1b - y2 e2b
+                    const Fx2 e1 = ed[0][c], e2 = ed[1][c];
+                    s64 mid = fx_mad(e1.h, u0.l, fx_mad(e1.l, u0.h, fx_mad(e2.h, u1.l, (s64)e2.l * u1.h)));
+                    s64 hi = fx_mad(e1.h, u0.h, (s64)e2.h * u1.h);
+                    if (CAS != kIdentical) {
+                        const Fx2 e3 = CAS == kEdge ? ed[3][c] : ed[2][c];
+                        mid -= fx_mad(e3.h, u2.l, (s64)e3.l * u2.h);
+                        hi -= (s64)e3.h * u2.h;
+                    }
+                    if (CAS == kVertex) {
+                        const Fx2 e4 = ed[3][c];
+                        mid -= fx_mad(e4.h, u3.l, (s64)e4.l * u3.h);
+                        hi -= (s64)e4.h * u3.h;
+                    }
+                    v[c] = (hi + (mid >> 32)) << 4;
+                }
+                const s64 r2 = fx_norm2(v[0], v[1], v[2]);
+                auto add = [&](int k, int c, Fx2 value) {
+                    const Fx2 w = col(c, p);
+                    const int32_t ww[2] = {w.h, w.l};
+                    acc[k].add(ww, value);
+                };
+                if (!HELM && ONE) {
+                    const Fx2 T = fx_split(fx_rinv(r2, kb + 1, flag));        // 2^(61 - kb) S / |v|
+                    if (BASIS == BEM_P0) {
+                        add(0, kFxA, T);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 9; ++k) add(k, kFxMS + k, T);
+                    }
+                    continue;
+                }
+                const Fx2 T = fx_split(fx_rinv(r2, kb, flag));                // 2^(62 - kb) S / |v|
+                Fx2 t2, t3;
+                if (HEIGHT) {
+                    // (S/|v|)^2 at 2^(62 - 2 kb), (S/|v|)^3 at 2^(62 - 3 kb) (2^61 where it is summed)
+                    t2 = fx_split(fx_mul_up<2>(T, T));
+                    constexpr int K3 = !HELM && (BASIS == BEM_P0 || CAS == kEdge) ? 1 : 2;
+                    t3 = fx_split(fx_mul_up<K3>(t2, T));
+                }
+                if (!HELM) {
+                    if (BASIS == BEM_P0) {
+#pragma unroll
+                        for (int k = 0; k < NH; ++k) add(k, kFxB + H0 + k, t3);
+                    } else {
+                        if (CAS == kVertex) {
+                            // height at 2^60 in units of 2^eh
+                            const s64 mid = fx_mad(n1.h, u0.l, fx_mad(n1.l, u0.h, fx_mad(n2.h, u1.l, (s64)n2.l * u1.h)));
+                            const s64 dn = (fx_mad(n1.h, u0.h, fx_mad(n2.h, u1.h, mid >> 32))) << 4;
+                            t3 = fx_split(fx_mul_up<3>(t3, fx_split(dn)));    // 2^(61 - 3 kb) (S/|v|)^3 dn
+                        }
+#pragma unroll
+                        for (int k = 0; k < 9; ++k) add(k, kFxMD + k, t3);
+                    }
+                    continue;
+                }
+                // theta = kappa g |v|: |v| at 2^58 / S, times g, times kappa S / (2 pi)
+                const s64 rho = fx_mul_up<4>(fx_split(r2), T) >> (4 - kb);
+                const s64 rg = CAS == kVertex ? rho : fx_mul(fx_split(rho << 2), col(kFxG, p));   // g at 2^62
+                const s64 turns = fx_mul_up<4>(fx_split(rg), kn);                  // theta / (2 pi) 2^(60 - kexp)
+                const Fx2 th = fx_split(turns);
+                s64 cs[kMaxXiFixedPairs], sn[kMaxXiFixedPairs];
+#pragma unroll
+                for (int j = 0; j < kMaxXiFixedPairs; ++j) {
+                    if (j >= X.npair) break;
+                    Fx2 tj;
+                    tj.h = X.t[j][0];
+                    tj.l = X.t[j][1];
+                    fx_sincos((u64)fx_mul_up<4>(th, tj) << (kexp + 2), cs[j], sn[j]);   // t_j at 2^62
+                }
+                s64 c0, s0;
+                fx_sincos((u64)turns << (kexp + 3), c0, s0);                  // half of theta
+                const Fx2 C0 = fx_split(c0), S0 = fx_split(s0);
+                Fx2 g2r, g2i;
+                fx_xi_sum(X, 1, cs, sn, C0, S0, g2r, g2i);
+                if (ONE) {
+                    add(0, kFxA, fx_split(fx_mul_up<2>(g2r, T)));             // 2^(61 - kb) S / |v|
+                    add(1, kFxA, fx_split(fx_mul_up<2>(g2i, T)));
+                }
+                if (HEIGHT) {
+                    Fx2 g1r, g1i;
+                    fx_xi_sum(X, 0, cs, sn, C0, S0, g1r, g1i);
+                    const Fx2 xr = fx_split(fx_mul_up<2>(g1r, t3)), xi = fx_split(fx_mul_up<2>(g1i, t3));   // 2^(61 - 3 kb) (S/|v|)^3
+                    const Fx2 yr = fx_split(fx_mul_up<2>(g2r, t2)), yi = fx_split(fx_mul_up<2>(g2i, t2));   // 2^(61 - 2 kb) (S/|v|)^2
+#pragma unroll
+                    for (int k = 0; k < NH; ++k) {
+                        const int o = (ONE ? 2 : 0) + 4 * k;
+                        add(o, kFxB + H0 + k, xr);
+                        add(o + 1, kFxB + H0 + k, xi);
+                        add(o + 2, kFxC + H0 + k, yr);
+                        add(o + 3, kFxC + H0 + k, yi);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < NS; ++k) tot[k] += acc[k].sum();
+        }
+        flag = __reduce_or_sync(0xffffffffu, (unsigned)flag);
+        if (flag >> (16 + kb)) return false;
+        kbs = kb;
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], o);
+        if (BASIS == BEM_P1 && KIND == BEM_LAPLACE_DLP) {
+            // heights: in units of 2^eh (vertex), or the edge's single one
+            h1 = CAS == kVertex ? fx_pow2(min(max(eh, -1000), 1000)) : h21;
+        }
+    }
+    if (lane == 0) {
+        const double scale = __ldg(ga + 12) * __ldg(gb + 12) * kInv4Pi;
+        if (BASIS == BEM_P0) {
+            double re = 0.0, im = 0.0;
+            if (!ZERO && !HELM) {
+                // weights at 2^63: sums / 2
+                if (ONE) re = (double)tot[0] * fx_pow2(1 - 61 + kbs - E);
+                else if (CAS == kVertex) re = fma(h1, (double)tot[0], h21 * (double)tot[NH - 1]) * fx_pow2(1 - 61 + 3 * kbs - 3 * E);
+                else re = h21 * (double)tot[0] * fx_pow2(1 - 61 + 3 * kbs - 3 * E);
+                re *= xi_moment(KIND, 0, 0);
+            } else if (!ZERO) {
+                if (ONE) {
+                    const double f1 = fx_pow2(1 - 61 + kbs - E), zr = (double)tot[0] * f1, zi = (double)tot[1] * f1;
+                    re = KIND == BEM_HELMHOLTZ_BW ? eta * zi : zr;
+                    im = KIND == BEM_HELMHOLTZ_BW ? -eta * zr : zi;
+                }
+                if (HEIGHT) {
+                    const double f3 = fx_pow2(1 - 61 + 3 * kbs - 3 * E), f2 = kappa * fx_pow2(1 - 61 + 2 * kbs - 2 * E);
+#pragma unroll
+                    for (int k = 0; k < NH; ++k) {
+                        const int o = (ONE ? 2 : 0) + 4 * k;
+                        const double h = CAS == kVertex && k == 0 ? h1 : h21;
+                        re += h * fma(f3, (double)tot[o], f2 * (double)tot[o + 3]);
+                        im += h * fma(f3, (double)tot[o + 1], -f2 * (double)tot[o + 2]);
+                    }
+                }
+            }
+            m.table[idx] = make_double2(re * scale, im * scale);
+        } else {
+            double M[9], hr[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                M[k] = 0.0;
+                if (!ZERO) {
+                    M[k] = (double)tot[k] * xi_moment(KIND, k / 3, k % 3);
+                    if (KIND == BEM_LAPLACE_SLP) M[k] *= fx_pow2(1 - 61 + kbs - E);
+                    else M[k] *= h1 * fx_pow2(1 - 61 + 3 * kbs - 3 * E);
+                }
+            }
+            moments_to_hats(M, hr);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    m.table[(int64_t)idx * 9 + pa[i] * 3 + pb[j]] = make_double2(hr[i * 3 + j] * scale, 0.0);
+        }
+    }
+    return true;
+}
+
+}  // namespace bem
