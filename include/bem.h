@@ -575,7 +575,9 @@ int64_t bem_rule_points(int32_t cas, int32_t regular_rule, int32_t q, double *ou
  * the q-point Gauss rule in xi is exact for degree n, the q^4-point sum equals
  * 1/(n+1) times the sum over these points.  The library evaluates Laplace
  * touching pairs this way wherever that holds (2q - 1 >= n); the Helmholtz
- * kernels keep the q^4 rule.  Returns n, or a negative BEM_ERR_* for another
+ * kernels take the Gauss sum over xi at each of these points (the float single
+ * layer, and the FP64 form of the piecewise-constant basis for q <= 9) or keep
+ * the q^4 rule.  Returns n, or a negative BEM_ERR_* for another
  * case or order.  Needs no device and no context. */
 int64_t bem_rule_points_xi(int32_t cas, int32_t q, double *out, int64_t cap);
 
@@ -683,9 +685,9 @@ int bem_h2_destroy(bem_ctx *ctx, bem_h2 *h2);
  *   DEVICE complex vector or NULL, b and x DEVICE complex vectors (x is
  *   overwritten, starting from 0); classical Gram-Schmidt applied twice,
  *   `restart` Krylov vectors per cycle (<= 500), at most maxit iterations,
- *   until |b - (A + D) x| <= tol |b|.  Allocates (restart + 1) n complex
- *   values of scratch per call and waits for the stream at every Arnoldi
- *   step.  Returns the iterations and the relative residual. */
+ *   until |b - (A + D) x| <= tol |b|.  Keeps its (restart + 2 + ranges) n complex
+ *   values of scratch in the context (grown to the largest call, freed by
+ *   bem_destroy) and waits for the stream at every Arnoldi step.  Returns the iterations and the relative residual. */
 int bem_potentials(bem_ctx *ctx, int32_t mesh_id, const bem_kernel_desc *kernel, int32_t q,
                    const double *points, int64_t n_points, const double *density, double *out);
 int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag,

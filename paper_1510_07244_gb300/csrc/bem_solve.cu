@@ -3,15 +3,17 @@
 //
 //   bem_potentials     u(z_k) = sum_j w_j int_{T_j} k(z_k, y) dy for points z_k
 //                      off the surface (piecewise-constant density w), with the
-//                      library's kernels; one warp per point, the lanes over the
-//                      triangles, a Duffy q x q rule per triangle (FP64).
+//                      library's kernels; one thread per (point, triangle) in the
+//                      FP64 form's fixed-point arithmetic, a Duffy q x q rule per
+//                      triangle, partial sums per CTA added in order.
 //   bem_dense_gmres    restarted GMRES (Saad and Schultz) for a dense complex
 //                      system (A + diag(d)) x = b: Arnoldi with classical
 //                      Gram-Schmidt applied twice, Givens rotations on the host.
-//                      The matrix-vector product (memory-bound, one thread per
-//                      row, column-major A) and the Gram-Schmidt projections
-//                      run in kernels; each Arnoldi step reads its projection
-//                      coefficients back (a few hundred bytes).
+//                      The matrix-vector product (column-major A, 32-row tiles
+//                      times column ranges) and both projections run in kernels
+//                      one after the other; each Arnoldi step reads its projection
+//                      coefficients and the new vector's norm back once (a few
+//                      hundred bytes).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,41 +27,114 @@ namespace bem {
 
 namespace {
 
-struct PotRule {
-    int np;
-    double s[kMaxNp], t[kMaxNp], w[kMaxNp];
-};
+// FP64 arithmetic for a triangle too close to the point for the fixed-point range
+template <int KIND>
+__device__ __noinline__ void potential_double(const double *z, const Tri &B, const Rule2D &R,
+                                              double kappa, double eta, double &sr, double &si)
+{
+    sr = si = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < R.np; ++k) {
+        double d[3], kr, ki;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            d[c] = z[c] - (B.v[0][c] + R.s[k] * (B.v[1][c] - B.v[0][c]) + R.t[k] * (B.v[2][c] - B.v[1][c]));
+        kval<KIND>(d[0], d[1], d[2], B.n, kappa, kr, ki, eta);
+        sr += R.w[k] * kr;
+        si += R.w[k] * ki;
+    }
+}
+
+// int_T k(z, y) dy without sqrt(g) / (4 pi): the trial side of a regular pair
+// (bem_fixed_pair.cuh) for one test point
+template <int KIND>
+__device__ __forceinline__ bool potential_fixed(const double *z, const Tri &B, const Rule2D &R,
+                                                double kappa, double eta, double &sr, double &si)
+{
+    double x[3], y[2][3], h = 0.0;
+    int top = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        x[c] = z[c] - B.v[0][c];
+        y[0][c] = B.v[1][c] - B.v[0][c];
+        y[1][c] = B.v[2][c] - B.v[0][c];
+        h = fma(x[c], B.n[c], h);
+        const int my = max(fx_mag(y[0][c]), fx_mag(y[1][c]));
+        top = max(top, fx_mag(__hiloint2double(fx_mag(x[c]), 0) + __hiloint2double(my, 0)));
+    }
+    const int e = top >> 20;
+    if (e < 823 || e > 1223) return false;
+    FxPair P;
+    P.E = e - 1022;
+    const double sc = fx_pow2(61 - P.E);
+    s64 X[3];
+    float d2 = 0.0f, rb = 0.0f, cb[3], yf[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        X[c] = __double2ll_rn(x[c] * sc);
+        const s64 y1 = __double2ll_rn(y[0][c] * sc), y2 = __double2ll_rn(y[1][c] * sc);
+        P.b1[c] = fx_split(y1);
+        P.b2[c] = fx_split(y2 - y1);
+        yf[0][c] = 0.0f;
+        yf[1][c] = fx_hi(y1);
+        yf[2][c] = fx_hi(y2);
+        cb[c] = (yf[1][c] + yf[2][c]) * (1.0f / 3.0f);
+        const float d = fx_hi(X[c]) - cb[c];
+        d2 = fmaf(d, d, d2);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        float v = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v = fmaf(yf[k][c] - cb[c], yf[k][c] - cb[c], v);
+        rb = fmaxf(rb, v);
+    }
+    P.kb = KIND == BEM_LAPLACE_SLP ? 4 : fx_kb((sqrtf(d2) - sqrtf(rb)) * 0.99999f - 8.0f);
+    FxUnits U;
+    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
+    FxInner<KIND, 1> I;
+    I.clear();
+    int flag = 0;
+#pragma unroll 1
+    for (int k = 0; k < R.np; ++k) {
+        s64 d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = (X[c] << 1) - fx_point(0, P.b1[c], P.b2[c], R.sx[k], R.tx[k]);
+        const int32_t *w[1] = {R.wx[3][k]};
+        I.point(d[0], d[1], d[2], P.kb, U.kn, U.shl, w, flag);
+    }
+    fx_combine<KIND, 1>(I, 0, U, h * fx_pow2(-P.E), sr, si);
+    const double f = fx_final<KIND>(U);
+    sr *= f;
+    si *= f;
+    return (flag >> (16 + P.kb)) == 0;
+}
+
+// CTA (s, p): point p0 + p, the triangles [s per, (s + 1) per); its sum goes to
+// part[p * gridDim.x + s] (the output itself when gridDim.x is 1).  A point's
+// triangles spread over several CTAs where the points alone would not fill the
+// GPU (256 points, 2048 triangles, Duffy q = 4, Brakhage-Werner kernel: one warp
+// per point in FP64 arithmetic took 9.4 ms).
+constexpr int kPotTri = 128;
 
 template <int KIND>
-__global__ void __launch_bounds__(256) k_potentials(MeshView m, const double *__restrict__ z,
-                                                    int64_t n_pts, const double2 *__restrict__ w,
-                                                    PotRule R, double kappa, double eta,
-                                                    double2 *out)
+__global__ void __launch_bounds__(kPotTri) k_potentials(MeshView m, const double *__restrict__ z,
+                                                        int64_t p0, int64_t per,
+                                                        const double2 *__restrict__ w,
+                                                        const __grid_constant__ Rule2D R, double kappa,
+                                                        double eta, double2 *part)
 {
-    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (p >= n_pts) return;
-    const double zx = z[3 * p], zy = z[3 * p + 1], zz = z[3 * p + 2];
+    __shared__ double2 ws[kPotTri / 32];
+    const int64_t p = p0 + blockIdx.y;
+    const int64_t j0 = (int64_t)blockIdx.x * per, j1 = min(m.nt, j0 + per);
+    const double zp[3] = {z[3 * p], z[3 * p + 1], z[3 * p + 2]};
     double ar = 0.0, ai = 0.0;
-    for (int64_t j = lane; j < m.nt; j += 32) {
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += kPotTri) {
         Tri B;
         load_tri(m.geom, j, B);
-        double e1[3], e2[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            e1[c] = B.v[1][c] - B.v[0][c];
-            e2[c] = B.v[2][c] - B.v[1][c];
-        }
-        double sr = 0.0, si = 0.0;
-        for (int k = 0; k < R.np; ++k) {
-            const double dx = zx - (B.v[0][0] + R.s[k] * e1[0] + R.t[k] * e2[0]);
-            const double dy = zy - (B.v[0][1] + R.s[k] * e1[1] + R.t[k] * e2[1]);
-            const double dz = zz - (B.v[0][2] + R.s[k] * e1[2] + R.t[k] * e2[2]);
-            double kr, ki;
-            kval<KIND>(dx, dy, dz, B.n, kappa, kr, ki, eta);
-            sr += R.w[k] * kr;
-            si += R.w[k] * ki;
-        }
+        double sr, si;
+        if (!potential_fixed<KIND>(zp, B, R, kappa, eta, sr, si))
+            potential_double<KIND>(zp, B, R, kappa, eta, sr, si);
         const double2 wj = w[j];
         const double sc = B.sg * kInv4Pi;
         sr *= sc;
@@ -69,21 +144,84 @@ __global__ void __launch_bounds__(256) k_potentials(MeshView m, const double *__
     }
     ar = warp_sum(ar);
     ai = warp_sum(ai);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = make_double2(ar, ai);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double2 s = ws[0];
+        for (int k = 1; k < kPotTri / 32; ++k) {
+            s.x += ws[k].x;
+            s.y += ws[k].y;
+        }
+        part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// one warp per point: its partial sums in a fixed order
+__global__ void __launch_bounds__(256) k_potential_sum(const double2 *__restrict__ part, int ns,
+                                                       int64_t n, double2 *out)
+{
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (p >= n) return;
+    double ar = 0.0, ai = 0.0;
+    for (int s = lane; s < ns; s += 32) {
+        const double2 v = part[p * ns + s];
+        ar += v.x;
+        ai += v.y;
+    }
+    ar = warp_sum(ar);
+    ai = warp_sum(ai);
     if (lane == 0) out[p] = make_double2(ar, ai);
 }
 
-// y = (A + diag(d)) x, A column-major n x n complex; one thread per row
-__global__ void __launch_bounds__(256) k_zgemv(int64_t n, const double2 *__restrict__ A,
-                                               const double2 *__restrict__ d,
-                                               const double2 *__restrict__ x, double2 *y)
+// Partial products of y = A x, A column-major n x n complex: CTA (r, s) takes the
+// 32 rows of tile r and the columns [s per, (s + 1) per), one row per lane, every
+// 8th column per warp; the warps' sums are added in order into part[s n + row].
+// FP64-bound (four FMAs per 16-byte entry, 2 lanes per SM and cycle: 29 us for
+// n = 2048); one thread per row and all columns kept 8 CTAs busy there.
+__global__ void __launch_bounds__(256) k_zgemv_part(int64_t n, int64_t per,
+                                                    const double2 *__restrict__ A,
+                                                    const double2 *__restrict__ x, double2 *part)
+{
+    __shared__ double2 ws[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    const int64_t j0 = (int64_t)blockIdx.y * per, j1 = min(n, j0 + per);
+    double ar = 0.0, ai = 0.0;
+    if (i < n) {
+#pragma unroll 8
+        for (int64_t j = j0 + warp; j < j1; j += 8) {
+            const double2 a = __ldg(A + i + j * n), v = __ldg(x + j);
+            ar = fma(a.x, v.x, fma(-a.y, v.y, ar));
+            ai = fma(a.x, v.y, fma(a.y, v.x, ai));
+        }
+    }
+    ws[warp][lane] = make_double2(ar, ai);
+    __syncthreads();
+    if (warp == 0 && i < n) {
+        double2 s = ws[0][lane];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) {
+            s.x += ws[k][lane].x;
+            s.y += ws[k][lane].y;
+        }
+        part[(int64_t)blockIdx.y * n + i] = s;
+    }
+}
+
+// y = sum of the ns partial products + diag(d) x
+__global__ void __launch_bounds__(128) k_zgemv_sum(int64_t n, int ns, const double2 *__restrict__ part,
+                                                   const double2 *__restrict__ d,
+                                                   const double2 *__restrict__ x, double2 *y)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double ar = 0.0, ai = 0.0;
-    for (int64_t j = 0; j < n; ++j) {
-        const double2 a = A[i + j * n], v = x[j];
-        ar = fma(a.x, v.x, fma(-a.y, v.y, ar));
-        ai = fma(a.x, v.y, fma(a.y, v.x, ai));
+#pragma unroll 4
+    for (int s = 0; s < ns; ++s) {
+        const double2 v = part[(int64_t)s * n + i];
+        ar += v.x;
+        ai += v.y;
     }
     if (d) {
         const double2 a = d[i], v = x[i];
@@ -121,12 +259,13 @@ __global__ void __launch_bounds__(256) k_project(int64_t n, const double2 *__res
 }
 
 // w -= V h (the first kk columns)
-__global__ void __launch_bounds__(256) k_subtract(int64_t n, int kk, const double2 *__restrict__ V,
-                                                  const double2 *__restrict__ h, double2 *w)
+__global__ void __launch_bounds__(64) k_subtract(int64_t n, int kk, const double2 *__restrict__ V,
+                                                 const double2 *__restrict__ h, double2 *w)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double ar = w[i].x, ai = w[i].y;
+#pragma unroll 8
     for (int k = 0; k < kk; ++k) {
         const double2 a = V[i + (int64_t)k * n], b = h[k];
         ar -= a.x * b.x - a.y * b.y;
@@ -143,7 +282,7 @@ __global__ void __launch_bounds__(256) k_residual(int64_t n, const double2 *__re
     w[i] = make_double2(b[i].x - w[i].x, b[i].y - w[i].y);
 }
 
-// v = s w (complex scale), and x += V y (the first kk columns)
+// v = s w (complex scale)
 __global__ void __launch_bounds__(256) k_scale(int64_t n, double sr, double si,
                                                const double2 *__restrict__ w, double2 *v)
 {
@@ -153,6 +292,19 @@ __global__ void __launch_bounds__(256) k_scale(int64_t n, double sr, double si,
     v[i] = make_double2(sr * a.x - si * a.y, sr * a.y + si * a.x);
 }
 
+// v = w / |w| with |w|^2 = norm2[0] (real part); nothing for a zero vector
+__global__ void __launch_bounds__(256) k_normalise(int64_t n, const double2 *__restrict__ norm2,
+                                                   const double2 *__restrict__ w, double2 *v)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const double s = sqrt(fmax(norm2->x, 0.0));
+    if (i >= n || !(s > 0.0)) return;
+    const double f = 1.0 / s;
+    const double2 a = w[i];
+    v[i] = make_double2(f * a.x, f * a.y);
+}
+
+// x += V y (the first kk columns)
 __global__ void __launch_bounds__(256) k_update(int64_t n, int kk, const double2 *__restrict__ V,
                                                 const double2 *__restrict__ y, double2 *x)
 {
@@ -196,25 +348,35 @@ int bem_potentials(bem_ctx *ctx, int32_t mesh_id, const bem_kernel_desc *kernel,
                         "bem_potentials: null or misaligned pointer (complex arrays: 16 bytes)");
     Rule2D r2;
     if (!make_rule2d(BEM_RULE_DUFFY, q, r2)) return api_fail(ctx, BEM_ERR_INVALID_ARG, "bad order");
-    PotRule R;
-    R.np = r2.np;
-    for (int k = 0; k < r2.np; ++k) {
-        R.s[k] = r2.s[k];
-        R.t[k] = r2.t[k];
-        R.w[k] = r2.w[k];
-    }
-    const unsigned grid = (unsigned)((n_points * 32 + 255) / 256);
     const double2 *w = reinterpret_cast<const double2 *>(density);
     double2 *o = reinterpret_cast<double2 *>(out);
     const double ka = kernel->kappa, et = kernel->eta;
     cudaStream_t st = ctx->stream;
-    switch (kernel->kind) {
-    case BEM_LAPLACE_SLP: k_potentials<BEM_LAPLACE_SLP><<<grid, 256, 0, st>>>(m, points, n_points, w, R, ka, et, o); break;
-    case BEM_LAPLACE_DLP: k_potentials<BEM_LAPLACE_DLP><<<grid, 256, 0, st>>>(m, points, n_points, w, R, ka, et, o); break;
-    case BEM_HELMHOLTZ_SLP: k_potentials<BEM_HELMHOLTZ_SLP><<<grid, 256, 0, st>>>(m, points, n_points, w, R, ka, et, o); break;
-    case BEM_HELMHOLTZ_DLP: k_potentials<BEM_HELMHOLTZ_DLP><<<grid, 256, 0, st>>>(m, points, n_points, w, R, ka, et, o); break;
-    default: k_potentials<BEM_HELMHOLTZ_BW><<<grid, 256, 0, st>>>(m, points, n_points, w, R, ka, et, o); break;
+    // CTAs per point: about eight per SM in all; one CTA writes its point's result
+    // itself, several need scratch for their sums (not grown while capturing)
+    const int64_t chunks = (m.nt + kPotTri - 1) / kPotTri;
+    int64_t ns = std::min(chunks, std::max<int64_t>(1, (8 * ctx->num_sms + n_points - 1) / n_points));
+    const size_t bytes = sizeof(double2) * (size_t)(n_points * ns);
+    if (ns > 1 && bytes > ctx->scratch_cap) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) ns = 1;
+        else if (int rc = api_ensure_scratch(ctx, bytes)) return rc;
     }
+    const int64_t per = (chunks + ns - 1) / ns * kPotTri;
+    double2 *part = ns > 1 ? reinterpret_cast<double2 *>(ctx->scratch) : o;
+    constexpr int64_t kRows = 65535;   // grid limit
+    for (int64_t p0 = 0; p0 < n_points; p0 += kRows) {
+        const dim3 grid((unsigned)ns, (unsigned)std::min(kRows, n_points - p0));
+        double2 *to = part + p0 * ns;
+        switch (kernel->kind) {
+        case BEM_LAPLACE_SLP: k_potentials<BEM_LAPLACE_SLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
+        case BEM_LAPLACE_DLP: k_potentials<BEM_LAPLACE_DLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
+        case BEM_HELMHOLTZ_SLP: k_potentials<BEM_HELMHOLTZ_SLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
+        case BEM_HELMHOLTZ_DLP: k_potentials<BEM_HELMHOLTZ_DLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
+        default: k_potentials<BEM_HELMHOLTZ_BW><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
+        }
+    }
+    if (ns > 1) k_potential_sum<<<(unsigned)((n_points + 7) / 8), 256, 0, st>>>(part, (int)ns, n_points, o);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return api_cuda_fail(ctx, e, "bem_potentials");
     return BEM_OK;
@@ -239,24 +401,33 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
     const double2 *db = reinterpret_cast<const double2 *>(b);
     double2 *dx = reinterpret_cast<double2 *>(x);
     const int m = restart;
-    double2 *V = nullptr, *w = nullptr, *h = nullptr;
-    cudaError_t e = cudaMalloc((void **)&V, sizeof(double2) * (size_t)n * (m + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&w, sizeof(double2) * (size_t)n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h, sizeof(double2) * (size_t)(m + 2));
-    auto done = [&](int rc) {
+    // column ranges of the product: enough CTAs for two per SM, at least 64 columns each
+    const unsigned tiles = (unsigned)((n + 31) / 32);
+    int64_t ns = std::max<int64_t>(1, std::min<int64_t>((2 * ctx->num_sms + tiles - 1) / tiles, n / 64));
+    const int64_t per = (n + ns - 1) / ns;
+    ns = (n + per - 1) / per;
+    // scratch: V (restart + 1 vectors), w, the partial products, and the projection
+    // coefficients of one step (both passes, then the squared norm)
+    const size_t nh = 2 * (size_t)(m + 1) + 1;
+    int rc = api_ensure_scratch(ctx, sizeof(double2) * ((size_t)n * (m + 2 + ns) + nh));
+    if (rc) return rc;
+    double2 *V = reinterpret_cast<double2 *>(ctx->scratch), *w = V + (size_t)n * (m + 1);
+    double2 *part = w + n, *h = part + (size_t)n * ns;
+    cudaError_t e = cudaSuccess;
+    auto done = [&](int code) {
         cudaStreamSynchronize(st);
-        cudaFree(V);
-        cudaFree(w);
-        cudaFree(h);
-        return rc;
+        return code;
     };
-    if (e != cudaSuccess) return done(api_cuda_fail(ctx, e, "cudaMalloc(gmres)"));
-    const unsigned g = grid_of(n);
+    const unsigned g = grid_of(n), gs = (unsigned)((n + 63) / 64);
+    auto product = [&](const double2 *v, double2 *y) {
+        k_zgemv_part<<<dim3(tiles, (unsigned)ns), 256, 0, st>>>(n, per, dA, v, part);
+        k_zgemv_sum<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(n, (int)ns, part, dd, v, y);
+    };
     // |b|
     auto norm = [&](const double2 *v, double &out) -> cudaError_t {
-        k_project<<<1, 256, 0, st>>>(n, v, v, h + m + 1);
+        k_project<<<1, 256, 0, st>>>(n, v, v, h);
         double2 r;
-        cudaError_t ee = cudaMemcpyAsync(&r, h + m + 1, sizeof(r), cudaMemcpyDeviceToHost, st);
+        cudaError_t ee = cudaMemcpyAsync(&r, h, sizeof(r), cudaMemcpyDeviceToHost, st);
         if (ee == cudaSuccess) ee = cudaStreamSynchronize(st);
         out = std::sqrt(std::max(r.x, 0.0));
         return ee;
@@ -267,10 +438,11 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
     if (e != cudaSuccess) return done(api_cuda_fail(ctx, e, "bem_dense_gmres"));
     int it = 0;
     double res = bn > 0.0 ? 1.0 : 0.0;
-    std::vector<cplx> H((size_t)(m + 1) * m), cs(m), sn(m), gvec(m + 1), hk(m + 1);
+    std::vector<cplx> H((size_t)(m + 1) * m), cs(m), sn(m), gvec(m + 1), hk(m + 2);
+    std::vector<double2> hh(nh);
     while (it < maxit && res > tol && bn > 0.0) {
         // r = b - (A + D) x (into w), beta = |r|, V_0 = r / beta
-        k_zgemv<<<g, 256, 0, st>>>(n, dA, dd, dx, w);
+        product(dx, w);
         k_residual<<<g, 256, 0, st>>>(n, db, w);
         double beta = 0.0;
         e = norm(w, beta);
@@ -282,23 +454,25 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
         gvec[0] = beta;
         int k = 0;
         for (; k < m && it < maxit; ++k, ++it) {
-            k_zgemv<<<g, 256, 0, st>>>(n, dA, dd, V + (size_t)k * n, w);
-            // classical Gram-Schmidt, twice
-            std::fill(hk.begin(), hk.end(), cplx(0.0));
+            product(V + (size_t)k * n, w);
+            // classical Gram-Schmidt, twice, the norm of what is left and the next
+            // vector; the coefficients and the norm come back in one copy
             for (int pass = 0; pass < 2; ++pass) {
-                k_project<<<k + 1, 256, 0, st>>>(n, V, w, h);
-                k_subtract<<<g, 256, 0, st>>>(n, k + 1, V, h, w);
-                std::vector<double2> hh(k + 1);
-                e = cudaMemcpyAsync(hh.data(), h, sizeof(double2) * (size_t)(k + 1),
-                                    cudaMemcpyDeviceToHost, st);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-                if (e != cudaSuccess) return done(api_cuda_fail(ctx, e, "bem_dense_gmres"));
-                for (int i = 0; i <= k; ++i) hk[i] += cplx(hh[i].x, hh[i].y);
+                k_project<<<k + 1, 256, 0, st>>>(n, V, w, h + pass * (k + 1));
+                k_subtract<<<gs, 64, 0, st>>>(n, k + 1, V, h + pass * (k + 1), w);
             }
-            double hn = 0.0;
-            if ((e = norm(w, hn)) != cudaSuccess) return done(api_cuda_fail(ctx, e, "bem_dense_gmres"));
+            k_project<<<1, 256, 0, st>>>(n, w, w, h + 2 * (k + 1));
+            k_normalise<<<g, 256, 0, st>>>(n, h + 2 * (k + 1), w, V + (size_t)(k + 1) * n);
+            e = cudaMemcpyAsync(hh.data(), h, sizeof(double2) * (size_t)(2 * (k + 1) + 1),
+                                cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return done(api_cuda_fail(ctx, e, "bem_dense_gmres"));
+            for (int i = 0; i <= k; ++i) {
+                hk[i] = cplx(hh[i].x, hh[i].y);
+                hk[i] += cplx(hh[k + 1 + i].x, hh[k + 1 + i].y);
+            }
+            const double hn = std::sqrt(std::max(hh[2 * (k + 1)].x, 0.0));
             hk[k + 1] = hn;
-            if (hn > 0.0) k_scale<<<g, 256, 0, st>>>(n, 1.0 / hn, 0.0, w, V + (size_t)(k + 1) * n);
             // apply the previous rotations, then a new one that zeroes hk[k + 1]
             for (int i = 0; i < k; ++i) {
                 const cplx t = std::conj(cs[i]) * hk[i] + std::conj(sn[i]) * hk[i + 1];
