@@ -18,14 +18,20 @@
 // D = {0 <= t <= s <= 1} with the affine map Phi(s,t) = v0 + s (v1 - v0) +
 // t (v2 - v1) and Gram factor sqrt(g) (Section 2.2), in FP64.
 //
-// Work split: one CTA per cluster, one warp per row (basis function) and the
-// cluster's points across the lanes, 32 at a time.  The lanes of a warp walk
-// the same support triangles and rule points, so geometry loads are warp-
-// uniform broadcasts and the support loop of the piecewise-linear basis does
-// not diverge; the lanes differ only in z_nu.  The plus and minus entries
-// share the distance and its reciprocal square root.
+// Work split: a few CTAs per cluster; their warps take units of one row (basis
+// function) and 32 of the cluster's points, one per lane.  The lanes of a warp
+// walk the same support triangles and rule points, so the support loop of the
+// piecewise-linear basis does not diverge and a triangle's rule points are
+// computed by the lanes together; the lanes differ only in z_nu.  The plus and
+// minus entries share the distance and its reciprocal square root.
+//
+// Arithmetic: the fixed point of bem_fixed.cuh in one frame per cluster (origin
+// at the middle of its rows' and points' box, S = 2^E above every coordinate
+// difference).  In FP64 a point took 25 operations on a pipe of 2 lanes per SM and
+// cycle (62% of its peak); triangles nearer than S / 16 to a point still do.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -34,7 +40,7 @@
 namespace bem {
 namespace {
 
-constexpr int kGreenThreads = 256;
+constexpr int kGreenThreads = 128;
 
 struct GreenArgs {
     const int32_t *row_ptr, *row_idx, *pt_ptr;
@@ -46,34 +52,28 @@ struct GreenArgs {
 };
 
 // Sums over one support triangle T of the rule points' contributions for the
-// point z with normal n (Section 2.3), without sqrt(g) and 1/(4 pi):
+// point z with normal n (Section 2.3), without sqrt(g) and 1/(4 pi), FP64:
 //   plus  += w_q phi(s_q, t_q) exp(i kappa r) / r
 //   minus += w_q phi(s_q, t_q) (x - z).n (1 - i kappa r) exp(i kappa r) / r^3
 // with x = Phi_T(s_q, t_q), r = |x - z|.  loc < 0: constant basis; otherwise
 // the local vertex (original order) whose hat function phi is.
-template <bool HELM, int NP>
-__device__ __forceinline__ void green_triangle(const Tri &T, int loc, const double *z,
-                                               const double *n, const Rule2D &R, double kappa,
-                                               double &pr, double &pi, double &mr, double &mi)
+template <bool HELM>
+__device__ __noinline__ void green_double(const Tri &T, int loc, const double *z, const double *n,
+                                          const Rule2D &R, double kappa, double out[4])
 {
-    double e1[3], e2[3], d0[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        e1[c] = T.v[1][c] - T.v[0][c];
-        e2[c] = T.v[2][c] - T.v[1][c];
-        d0[c] = T.v[0][c] - z[c];
-    }
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
+    double pr = 0.0, pi = 0.0, mr = 0.0, mi = 0.0;
+#pragma unroll 1
+    for (int q = 0; q < R.np; ++q) {
         const double s = R.s[q], t = R.t[q];
         const double phi = loc < 0 ? 1.0 : (loc == 0 ? 1.0 - s : (loc == 1 ? s - t : t));
         const double wq = R.w[q] * phi;
-        const double dx = d0[0] + s * e1[0] + t * e2[0];
-        const double dy = d0[1] + s * e1[1] + t * e2[1];
-        const double dz = d0[2] + s * e1[2] + t * e2[2];
-        const double r2 = dx * dx + dy * dy + dz * dz;
+        double d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            d[c] = (T.v[0][c] - z[c]) + s * (T.v[1][c] - T.v[0][c]) + t * (T.v[2][c] - T.v[1][c]);
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
         const double ri = rsqrt(r2);
-        const double dn = dx * n[0] + dy * n[1] + dz * n[2];
+        const double dn = d[0] * n[0] + d[1] * n[1] + d[2] * n[2];
         const double h = wq * dn * (ri * ri * ri);
         if (!HELM) {
             pr += wq * ri;
@@ -88,15 +88,212 @@ __device__ __forceinline__ void green_triangle(const Tri &T, int loc, const doub
             mi += h * (sn - kr * cs);
         }
     }
+    out[0] = pr;
+    out[1] = pi;
+    out[2] = mr;
+    out[3] = mi;
+}
+
+// The cluster's frame: origin, S = 2^E, and for the Helmholtz kernel the phase
+// factor (fx_wave).
+struct GreenFrame {
+    double c0[3];
+    int E, ok, kexp;
+    Fx2 kn;
+};
+
+// Scale of the frame: the box of the points and of the rows' support triangles
+// relative to the first point, in float (min, max: [x/z][min/max][3]).  Called by
+// every thread of the CTA.
+__device__ __forceinline__ void green_frame(const MeshView &m, const GreenArgs &a, int rb, int nr, int pb,
+                                            int mp, int64_t lim, bool helm, float (*box)[12],
+                                            GreenFrame &F)
+{
+    float lo[2][3], hi[2][3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            lo[k][c] = 3.0e38f;
+            hi[k][c] = -3.0e38f;
+        }
+    double ref[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ref[c] = __ldg(a.z + 3 * (int64_t)pb + c);
+    for (int k = threadIdx.x; k < mp; k += blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float d = (float)(__ldg(a.z + 3 * (int64_t)(pb + k) + c) - ref[c]);
+            lo[1][c] = fminf(lo[1][c], d);
+            hi[1][c] = fmaxf(hi[1][c], d);
+        }
+    for (int k = threadIdx.x; k < nr; k += blockDim.x) {
+        const int i = __ldg(a.row_idx + rb + k);
+        if (i < 0 || i >= lim) continue;
+        const int klo = m.basis == BEM_P0 ? 0 : __ldg(m.vt_ptr + i);
+        const int khi = m.basis == BEM_P0 ? 1 : __ldg(m.vt_ptr + i + 1);
+        for (int t = klo; t < khi; ++t) {
+            const double *g = m.geom + (int64_t)(m.basis == BEM_P0 ? i : __ldg(m.vt_tri + t)) * kGeomStride;
+#pragma unroll
+            for (int v = 0; v < 9; ++v) {
+                const float d = (float)(__ldg(g + v) - ref[v % 3]);
+                lo[0][v % 3] = fminf(lo[0][v % 3], d);
+                hi[0][v % 3] = fmaxf(hi[0][v % 3], d);
+            }
+        }
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                lo[k][c] = fminf(lo[k][c], __shfl_xor_sync(0xffffffffu, lo[k][c], o));
+                hi[k][c] = fmaxf(hi[k][c], __shfl_xor_sync(0xffffffffu, hi[k][c], o));
+            }
+            if (lane == 0) {
+                box[warp][6 * k + c] = lo[k][c];
+                box[warp][6 * k + 3 + c] = hi[k][c];
+            }
+        }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float top = 0.0f;
+        for (int c = 0; c < 3; ++c) {
+            float b[4] = {3.0e38f, -3.0e38f, 3.0e38f, -3.0e38f};
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+                for (int k = 0; k < 2; ++k) {
+                    b[2 * k] = fminf(b[2 * k], box[w][6 * k + c]);
+                    b[2 * k + 1] = fmaxf(b[2 * k + 1], box[w][6 * k + 3 + c]);
+                }
+            const float mid = 0.5f * (fminf(b[0], b[2]) + fmaxf(b[1], b[3]));
+            F.c0[c] = ref[c] + (double)mid;
+            const float x = fmaxf(b[1] - mid, mid - b[0]), z = fmaxf(b[3] - mid, mid - b[2]);
+            top = fmaxf(top, x + z);
+        }
+        top *= 1.00001f;
+        const int ex = __float_as_int(top) >> 23;
+        F.ok = ex > 27 && ex < 227;          // also false for boxes without rows or beyond float
+        F.E = ex - 126;
+        if (F.ok && helm) F.ok = fx_wave(a.kappa, F.E, -4, F.kn, F.kexp);   // the phase's shift stays >= 0
+    }
+    __syncthreads();
+}
+
+// green_double's sums in fixed point; Z and N: the lane's point (2^62 / S) and normal
+// (2^61).  The lanes compute the triangle's rule points together (lane 3 q + c:
+// component c of point q, eight points at a time): every lane of the warp calls
+// this with the same triangle.
+template <bool HELM, int NP>
+__device__ __forceinline__ bool green_fixed(const GreenFrame &F, const Tri &T, int loc, const s64 *Z,
+                                            const Fx2 *N, const Rule2D &R, double kappa, int lane,
+                                            double out[4])
+{
+    const double sc = fx_pow2(61 - F.E);
+    // this lane's rule point components, 2^62 / S
+    constexpr int NR = (NP + 7) / 8;
+    s64 mine[NR];
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+        const int q = 8 * u + lane / 3, c = lane % 3;
+        mine[u] = 0;
+        if (lane < 24 && q < NP) {
+            const double v0 = c == 0 ? T.v[0][0] : (c == 1 ? T.v[0][1] : T.v[0][2]);
+            const double v1 = c == 0 ? T.v[1][0] : (c == 1 ? T.v[1][1] : T.v[1][2]);
+            const double v2 = c == 0 ? T.v[2][0] : (c == 1 ? T.v[2][1] : T.v[2][2]);
+            const double x = (v0 - F.c0[c]) + R.s[q] * (v1 - v0) + R.t[q] * (v2 - v1);
+            mine[u] = __double2ll_rn(x * sc) << 1;
+        }
+    }
+    auto component = [&](int q, int c) {
+        s64 part = mine[0];
+#pragma unroll
+        for (int u = 1; u < NR; ++u)
+            if (q >= 8 * u) part = mine[u];
+        return __shfl_sync(0xffffffffu, part, 3 * (q & 7) + c);
+    };
+    // kb from the smallest distance of the rule's points, in float
+    float lo = 3.0e38f;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        float d2 = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float d = __shfl_sync(0xffffffffu, fx_hi(mine[q / 8]), 3 * (q & 7) + c) - fx_hi(Z[c]);
+            d2 = fmaf(d, d, d2);
+        }
+        lo = fminf(lo, d2);
+    }
+    const int kb = fx_kb(sqrtf(lo) * 0.49995f - 64.0f);   // S = 2^30 here
+    FxSum pr, pi, m3r, m3i, m2r, m2i;
+    pr.clear();
+    pi.clear();
+    m3r.clear();
+    m3i.clear();
+    m2r.clear();
+    m2i.clear();
+    int flag = 0;
+    const int wl = loc < 0 ? 3 : loc;
+#pragma unroll 1
+    for (int q = 0; q < NP; ++q) {
+        s64 d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = component(q, c) - Z[c];
+        const s64 r2 = fx_norm2(d[0], d[1], d[2]);
+        const s64 y = fx_rinv(r2, kb, flag);                     // 2^(62 - kb) S / r
+        const Fx2 t1 = fx_split(y);
+        const Fx2 t2 = fx_split(fx_mul_up<2>(t1, t1));           // 2^(62 - 2 kb) (S / r)^2
+        const Fx2 t3 = fx_split(fx_mul_up<2>(t2, t1));           // 2^(62 - 3 kb) (S / r)^3
+        // (x - z).n at 2^60 / S (at most sqrt(3)), times (S / r)^3
+        const Fx2 a = fx_split(d[0]), b = fx_split(d[1]), e = fx_split(d[2]);
+        const s64 mid = fx_mad(a.h, N[0].l, fx_mad(a.l, N[0].h, fx_mad(b.h, N[1].l, (s64)b.l * N[1].h))) +
+                        fx_mad(e.h, N[2].l, (s64)e.l * N[2].h);
+        const Fx2 dn = fx_split((fx_mad(a.h, N[0].h, fx_mad(b.h, N[1].h, fx_mad(e.h, N[2].h, mid >> 32)))) << 1);
+        const Fx2 h3 = fx_split(fx_mul(t3, dn));                 // 2^(58 - 3 kb) (S / r)^3 dn / S
+        const int32_t *w = R.wx[wl][q];
+        if (!HELM) {
+            pr.add(w, fx_split(y >> 3));                         // 2^(59 - kb)
+            m3r.add(w, h3);
+            continue;
+        }
+        const Fx2 h2 = fx_split(fx_mul(t2, dn));                 // 2^(58 - 2 kb) (S / r)^2 dn / S
+        const Fx2 rho = fx_split(fx_mul_up<4>(fx_split(r2), t1));   // 2^(62 - kb) r / S
+        s64 cs, sn;
+        fx_sincos((u64)fx_mul(rho, F.kn) << (4 + kb + F.kexp), cs, sn);
+        const Fx2 c = fx_split(cs), s = fx_split(sn);
+        pr.add(w, fx_split(fx_mul(c, t1)));                      // 2^(59 - kb)
+        pi.add(w, fx_split(fx_mul(s, t1)));
+        // (c + kappa r s) / r^3 and (s - kappa r c) / r^3, the two powers apart
+        m3r.add(w, fx_split(fx_mul_up<4>(c, h3)));               // 2^(59 - 3 kb)
+        m3i.add(w, fx_split(fx_mul_up<4>(s, h3)));
+        m2r.add(w, fx_split(fx_mul_up<3>(s, h2)));               // 2^(58 - 2 kb)
+        m2i.add(w, fx_split(fx_mul_up<3>(c, h2)));
+    }
+    // the sums hold half of their values
+    const double fp = fx_pow2(1 - (59 - kb) - F.E);
+    out[0] = pr.value() * fp;
+    if (!HELM) {
+        out[2] = m3r.value() * fx_pow2(1 - (58 - 3 * kb) - 2 * F.E);
+    } else {
+        const double f3 = fx_pow2(1 - (59 - 3 * kb) - 2 * F.E);
+        const double f2 = kappa * fx_pow2(1 - (58 - 2 * kb) - F.E);
+        out[1] = pi.value() * fp;
+        out[2] = fma(f3, m3r.value(), f2 * m2r.value());
+        out[3] = fma(f3, m3i.value(), -f2 * m2i.value());
+    }
+    return (flag >> (16 + kb)) == 0;
 }
 
 template <bool HELM, int NP>
-__global__ void __launch_bounds__(kGreenThreads) k_green(MeshView m, GreenArgs a, Rule2D R,
-                                                         int *status)
+__global__ void __launch_bounds__(kGreenThreads) k_green(MeshView m, GreenArgs a,
+                                                         const __grid_constant__ Rule2D R, int *status)
 {
     __shared__ int s_ok;
     __shared__ int s_rb, s_nr, s_pb, s_mp;
     __shared__ long long s_off;
+    __shared__ float box[kGreenThreads / 32][12];
+    __shared__ GreenFrame F;
     const int c = blockIdx.x;
     if (threadIdx.x == 0) {
         const int32_t rb = a.row_ptr[c], re = a.row_ptr[c + 1];
@@ -125,7 +322,11 @@ __global__ void __launch_bounds__(kGreenThreads) k_green(MeshView m, GreenArgs a
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int64_t lim = m.basis == BEM_P0 ? m.nt : m.nv;
-    for (int r = warp; r < nr; r += nwarps) {
+    green_frame(m, a, rb, nr, pb, mp, lim, HELM, box, F);
+    const int chunks = (mp + 31) / 32;
+    const int64_t units = (int64_t)nr * chunks;
+    for (int64_t u = (int64_t)blockIdx.y * nwarps + warp; u < units; u += (int64_t)gridDim.y * nwarps) {
+        const int r = (int)(u / chunks), base = (int)(u - (int64_t)r * chunks) * 32;
         const int i = __ldg(a.row_idx + rb + r);
         if (i < 0 || i >= lim) {
             if (lane == 0) set_status(status, BEM_ERR_INVALID_ARG);
@@ -133,60 +334,73 @@ __global__ void __launch_bounds__(kGreenThreads) k_green(MeshView m, GreenArgs a
         }
         const int klo = m.basis == BEM_P0 ? 0 : __ldg(m.vt_ptr + i);
         const int khi = m.basis == BEM_P0 ? 1 : __ldg(m.vt_ptr + i + 1);
-        for (int base = 0; base < mp; base += 32) {
-            const int nu = base + lane;
-            const bool act = nu < mp;
-            // idle lanes of the last chunk repeat the cluster's last point and write nothing
-            const int64_t p = pb + (act ? nu : mp - 1);
-            double z[3], n[3];
+        const int nu = base + lane;
+        const bool act = nu < mp;
+        // idle lanes of the last chunk repeat the cluster's last point and write nothing
+        const int64_t p = pb + (act ? nu : mp - 1);
+        double z[3], n[3];
+        s64 Z[3];
+        Fx2 N[3];
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                z[d] = __ldg(a.z + 3 * p + d);
-                n[d] = __ldg(a.nz + 3 * p + d);
+        for (int d = 0; d < 3; ++d) {
+            z[d] = __ldg(a.z + 3 * p + d);
+            n[d] = __ldg(a.nz + 3 * p + d);
+            Z[d] = F.ok ? __double2ll_rn((z[d] - F.c0[d]) * fx_pow2(61 - F.E)) << 1 : 0;
+            N[d] = fx_split(__double2ll_rn(n[d] * 2305843009213693952.0));
+        }
+        // normals are unit vectors; anything longer leaves the fixed-point range
+        const bool unit = fmax(fmax(fabs(n[0]), fabs(n[1])), fabs(n[2])) <= 1.0;
+        const bool fixed = F.ok && __all_sync(0xffffffffu, unit);
+        double pr = 0.0, pi = 0.0, mr = 0.0, mi = 0.0;
+        for (int k = klo; k < khi; ++k) {
+            const int tr = m.basis == BEM_P0 ? i : __ldg(m.vt_tri + k);
+            Tri T;
+            load_tri(m.geom, tr, T);
+            int loc = -1;
+            if (m.basis == BEM_P1) {
+                const int4 tv = __ldg(m.tvid + tr);
+                loc = tv.x == i ? 0 : (tv.y == i ? 1 : 2);
             }
-            double pr = 0.0, pi = 0.0, mr = 0.0, mi = 0.0;
-            for (int k = klo; k < khi; ++k) {
-                const int tr = m.basis == BEM_P0 ? i : __ldg(m.vt_tri + k);
-                Tri T;
-                load_tri(m.geom, tr, T);
-                int loc = -1;
-                if (m.basis == BEM_P1) {
-                    const int4 tv = __ldg(m.tvid + tr);
-                    loc = tv.x == i ? 0 : (tv.y == i ? 1 : 2);
-                }
-                double tpr = 0.0, tpi = 0.0, tmr = 0.0, tmi = 0.0;
-                green_triangle<HELM, NP>(T, loc, z, n, R, a.kappa, tpr, tpi, tmr, tmi);
-                pr += T.sg * tpr;
-                mr += T.sg * tmr;
-                if (HELM) {
-                    pi += T.sg * tpi;
-                    mi += T.sg * tmi;
-                }
+            double v[4];
+            if (!fixed || !green_fixed<HELM, NP>(F, T, loc, Z, N, R, a.kappa, lane, v))
+                green_double<HELM>(T, loc, z, n, R, a.kappa, v);
+            pr += T.sg * v[0];
+            mr += T.sg * v[2];
+            if (HELM) {
+                pi += T.sg * v[1];
+                mi += T.sg * v[3];
             }
-            if (act) {
-                const double fp = (a.sp ? __ldg(a.sp + p) : 1.0) * kInv4Pi;
-                const double fm = (a.sm ? __ldg(a.sm + p) : 1.0) * kInv4Pi;
-                const int64_t ep = off + r + (int64_t)nu * nr;          // A+ column nu
-                const int64_t em = off + r + (int64_t)(mp + nu) * nr;   // A- column nu
-                if (HELM) {
-                    double2 *o = reinterpret_cast<double2 *>(a.out);
-                    o[ep] = make_double2(fp * pr, fp * pi);
-                    o[em] = make_double2(fm * mr, fm * mi);
-                } else {
-                    double *o = reinterpret_cast<double *>(a.out);
-                    o[ep] = fp * pr;
-                    o[em] = fm * mr;
-                }
+        }
+        if (act) {
+            const double fp = (a.sp ? __ldg(a.sp + p) : 1.0) * kInv4Pi;
+            const double fm = (a.sm ? __ldg(a.sm + p) : 1.0) * kInv4Pi;
+            const int64_t ep = off + r + (int64_t)nu * nr;          // A+ column nu
+            const int64_t em = off + r + (int64_t)(mp + nu) * nr;   // A- column nu
+            if (HELM) {
+                double2 *o = reinterpret_cast<double2 *>(a.out);
+                o[ep] = make_double2(fp * pr, fp * pi);
+                o[em] = make_double2(fm * mr, fm * mi);
+            } else {
+                double *o = reinterpret_cast<double *>(a.out);
+                o[ep] = fp * pr;
+                o[em] = fm * mr;
             }
         }
     }
 }
 
+// CTAs (cluster, part): the parts of a cluster share its units, so that a tree of a
+// few hundred clusters of about 30 rows still fills the GPU several times over
+// (four CTAs per SM are resident; one CTA of eight warps per cluster left the
+// last of 3 waves nearly empty).  More than eight parts would repeat the frame's
+// set-up for less than two units a warp.
 template <bool HELM>
 cudaError_t launch_green(const MeshView &m, const GreenArgs &a, int n_clusters, const Rule2D &R,
-                         int *status, cudaStream_t st)
+                         int *status, int num_sms, cudaStream_t st)
 {
-#define BEM_GREEN(NP) k_green<HELM, NP><<<n_clusters, kGreenThreads, 0, st>>>(m, a, R, status)
+    const int parts = std::min(8, (24 * num_sms + n_clusters - 1) / n_clusters);
+    const dim3 grid((unsigned)n_clusters, (unsigned)parts);
+#define BEM_GREEN(NP) k_green<HELM, NP><<<grid, kGreenThreads, 0, st>>>(m, a, R, status)
     switch (R.np) {
     case 1: BEM_GREEN(1); break;
     case 4: BEM_GREEN(4); break;
@@ -247,8 +461,8 @@ extern "C" int bem_green_matrices(bem_ctx *ctx, const bem_green_job *job)
     cudaError_t e;
     {
         ProfScope ps(ctx, "green");
-        e = helm ? launch_green<true>(mesh->v, a, J.n_clusters, R, ctx->status, ctx->stream)
-                 : launch_green<false>(mesh->v, a, J.n_clusters, R, ctx->status, ctx->stream);
+        e = helm ? launch_green<true>(mesh->v, a, J.n_clusters, R, ctx->status, ctx->num_sms, ctx->stream)
+                 : launch_green<false>(mesh->v, a, J.n_clusters, R, ctx->status, ctx->num_sms, ctx->stream);
     }
     if (e != cudaSuccess) return api_cuda_fail(ctx, e, "green kernel");
     return BEM_OK;
@@ -327,8 +541,8 @@ extern "C" int bem_gca_pivots_device(bem_ctx *ctx, int32_t mesh_id, const double
         a.kappa = cplx_out ? kappa : 0.0;
         {
             ProfScope ps(ctx, "green");
-            e = cplx_out ? launch_green<true>(mesh->v, a, (int)n_cl, R, ctx->status, ctx->stream)
-                         : launch_green<false>(mesh->v, a, (int)n_cl, R, ctx->status, ctx->stream);
+            e = cplx_out ? launch_green<true>(mesh->v, a, (int)n_cl, R, ctx->status, ctx->num_sms, ctx->stream)
+                         : launch_green<false>(mesh->v, a, (int)n_cl, R, ctx->status, ctx->num_sms, ctx->stream);
         }
         if (e != cudaSuccess) return api_cuda_fail(ctx, e, "green kernel");
         e = cudaMemcpyAsync(out.data(), S.p + at[8], parts[8], cudaMemcpyDeviceToHost, ctx->stream);

@@ -80,3 +80,64 @@ def test_rules(pkg, ctx, kernel, rule, q, singular):
     quad = dict(q_regular=q, regular_rule=rule, q_identical=singular, q_edge=singular,
                 q_vertex=singular)
     _check(pkg, ctx, mesh, "p0", kernel, 40.0, quad)
+
+
+def _duffy(q):
+    x, w = np.polynomial.legendre.leggauss(q)
+    x, w = 0.5 + 0.5 * x, 0.5 * w
+    return np.repeat(x, q), np.outer(x, x).ravel(), np.outer(w * x, w).ravel()
+
+
+@pytest.mark.parametrize("away", [3.0, 0.3, 0.01])
+@pytest.mark.parametrize("kernel", ["laplace_slp", "helmholtz_slp", "helmholtz_bw"])
+def test_points_towards_the_surface(pkg, ctx, kernel, away):
+    """Green matrices and potentials for points at a distance down to a hundredth of the edge
+    length (below S / 16, the FP64 path), against numpy with the same rule; normals longer than 1
+    leave the fixed-point range too.  Tolerance 1e-12 of the sum of the terms' magnitudes."""
+    import torch
+    kappa = 0.0 if kernel == "laplace_slp" else 3.0
+    mesh = synth.jitter(synth.torus(7, 5), 0.05, 5)
+    v = mesh.verts[mesh.tris]
+    n = np.cross(v[:, 1] - v[:, 0], v[:, 2] - v[:, 1])
+    gram = np.linalg.norm(n, axis=1)
+    n /= gram[:, None]
+    h = np.sqrt(gram.mean())
+    z = v.mean(1) + away * h * n
+    s, t, w = _duffy(3)
+    y = (v[:, None, 0] + s[None, :, None] * (v[:, 1] - v[:, 0])[:, None]
+         + t[None, :, None] * (v[:, 2] - v[:, 1])[:, None])
+    d = z[:, None, None] - y[None]
+    r = np.linalg.norm(d, axis=3)
+    wave = np.exp(1j * kappa * r) / r
+    wt = w[None, None] * gram[None, :, None] / (4 * np.pi)
+    double = (d * n[None, :, None]).sum(3) / r ** 2 * (1 - 1j * kappa * r) * wave
+    mid = ctx.bem_mesh_upload(mesh.verts, mesh.tris, "p0")
+    dens = np.exp(1j * np.arange(mesh.nt))
+    val = double - 1j * kappa * wave if kernel == "helmholtz_bw" else wave
+    out = torch.zeros(mesh.nt, dtype=torch.complex128, device="cuda")
+    ctx.bem_potentials(mid, pkg.kernel_desc(kernel, kappa, kappa), torch.as_tensor(z).cuda(),
+                       torch.as_tensor(dens).cuda(), out, q=3)
+    ctx.bem_sync()
+    ref = (val * wt).sum(2) @ dens
+    A = (np.abs(val) * wt).sum((1, 2))
+    assert (np.abs(out.cpu().numpy() - ref) / A).max() < 1e-12
+    if kernel != "helmholtz_bw":
+        # every triangle a row of one cluster, normals of length 1 and of length 7
+        nz = n * np.where(np.arange(mesh.nt) % 40 < 35, 1.0, 7.0)[:, None]
+        cols = 2 * mesh.nt
+        cplx = kernel == "helmholtz_slp"
+        o = torch.zeros(mesh.nt * cols, dtype=torch.complex128 if cplx else torch.float64, device="cuda")
+        i32 = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.int32).cuda()
+        ctx.bem_green_matrices(pkg.GreenJob(mid, i32([0, mesh.nt]), i32(np.arange(mesh.nt)),
+                                            i32([0, mesh.nt]), torch.as_tensor(z).cuda(),
+                                            torch.as_tensor(nz).cuda(),
+                                            torch.zeros(1, dtype=torch.int64, device="cuda"), o,
+                                            kernel=pkg.kernel_desc(kernel, kappa), rule="duffy", q=3))
+        ctx.bem_sync()
+        got = o.cpu().numpy().reshape(cols, mesh.nt).T
+        minus = -(d * nz[:, None, None]).sum(3) / r ** 2 * (1 - 1j * kappa * r) * wave
+        for k, f in ((0, wave), (1, minus)):
+            ref, A = (f * wt).sum(2).T, (np.abs(f) * wt).sum(2).T
+            err = np.abs(got[:, k * mesh.nt:(k + 1) * mesh.nt] - (ref if cplx else ref.real))
+            assert (err / A.max(1, keepdims=True)).max() < 1e-12
+    ctx.bem_mesh_free(mid)
