@@ -5,15 +5,28 @@
 // V_t S_ts V_s^T with nested cluster bases: V_t of a leaf is its
 // interpolation matrix, V_t of a cluster with sons is diag(V_t1, V_t2) V^_t
 // (transfer matrix V^_t, rows = the sons' pivots).  y = G x runs as
-//   near     y|t = sum_s N_ts x|s                 one CTA per leaf, row per lane
-//   forward  x^_s = V_s^T x|s (leaf) or V^_s^T (x^_s1; x^_s2), deepest level first
-//   coupling y^_t = sum_s S_ts x^_s               one CTA per cluster
-//   backward (y^_t1; y^_t2) += V^_t y^_t, y|t += V_t y^_t (leaf), top level first
-// Every output element is written by one lane in a fixed order (no atomics),
-// so products are bitwise reproducible.  The near field runs on a second
-// stream beside the forward and coupling passes.  All arithmetic is FP64.  The matrix
-// is memory- and latency-bound: per product it reads every near-field and
-// coupling entry once (8 bytes each) and does 2 flops per entry.
+//   near     p_b = N_ts x|s for every near block b            one warp per block
+//   forward  x^_s = V_s^T x|s (all leaves), then V^_s^T (x^_s1; x^_s2), deepest level first
+//   coupling p_b = S_ts x^_s for every admissible block b     one warp per block
+//   backward y^_t = sum_b p_b + the father's part, (parts of y^_t1; y^_t2) = V^_t y^_t,
+//            top level first; then y|t = sum_b p_b (near) + V_t y^_t (all leaves)
+// Every sum has a fixed order (no atomics), so products are bitwise reproducible.
+// The near field runs beside the levels and the coupling, which have a stream of
+// their own.
+// Clusters above the first admissible block take part in neither transformation.
+// All arithmetic is FP64.  The matrix is memory- and latency-bound: per product it
+// reads every near-field and coupling entry once (8 bytes each) and does 2 flops
+// per entry; the levels are a chain of small launches.
+//   - A warp per block, all its column loads in flight at once, keeps the two
+//     block passes at the memory system's rate whatever the blocks per cluster
+//     (one CTA per cluster with a warp per eighth block: 2.6 TB/s, 2 waves).
+//   - The level launches overlap (programmatic dependent launch): each reads its
+//     own matrices into registers before it waits for the level before it.
+// 32768-triangle sphere, 14.2 M near and 30.7 M coupling entries, 13 levels:
+// 336 us per product with a CTA per cluster everywhere and plain launches, 208 us
+// so: near field 17 us beside the rest, coupling about 108 us (its multiplications
+// alone keep the FP64 pipe busy for 63 us, its entries take 36 us of bandwidth), the
+// chain of 19 level launches and the leaves 83 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -22,40 +35,53 @@
 
 #include "bem_internal.h"
 
+namespace bem {
+
+struct alignas(16) H2Node {
+    int64_t v_off;             // its matrix in vals / valsT
+    int64_t src_off;           // its row sources in src
+    int64_t near_off, far_off; // its blocks' products in near_part / far_part
+    int32_t rows, rank;        // R_c, K_c
+    int32_t hat;               // x^_c, y^_c in the hat vectors
+    int32_t n_near, n_far;     // its near / admissible blocks
+    int32_t idx;               // its index set in cl_idx
+    int32_t leaf;
+    int32_t up;                // 1: the father's part of y^_c is in yhat; bit 1: y^_c is needed at all
+};
+
+struct alignas(16) H2Block {
+    int64_t val;               // first entry of the block's values
+    int64_t out;               // its product in near_part / far_part
+    int32_t nr, nc;            // rows, columns
+    int32_t src, pad;          // near: column indices in cl_idx; far: x^ of the column cluster
+};
+
+}  // namespace bem
+
 struct bem_h2 {
     int64_t n = 0;
     int32_t nc = 0, max_rank = 0;
     std::vector<void *> allocs;
-    // per cluster (device): rows of its basis matrix, pivots, offsets
-    int32_t *rows = nullptr;       // basis rows R_c
-    int32_t *rank = nullptr;       // K_c
-    int64_t *v_off = nullptr;      // offset of the R_c x K_c row-major matrix in vals
-    int64_t *src_off = nullptr;    // offset of the R_c row sources in src
-    int64_t *hat_off = nullptr;    // offset of x^_c / y^_c in the hat vectors
-    int32_t *leaf = nullptr;       // 1 for leaves
+    bem::H2Node *nodes = nullptr;  // per cluster (device)
     int32_t *src = nullptr;        // row sources: vector index (leaf) or hat index (else)
-    double *vals = nullptr;        // basis matrices
-    double *valsT = nullptr;       // the same, each transposed (K_c x R_c row-major)
-    // near blocks by leaf row cluster (CSR over nc), far blocks by row cluster
-    int32_t *near_ptr = nullptr, *near_col = nullptr;
-    int64_t *near_off = nullptr;
-    int32_t *far_ptr = nullptr, *far_col = nullptr;
-    int64_t *far_off = nullptr;
+    double *vals = nullptr;        // basis matrices (rows x K_c row-major)
+    double *valsT = nullptr;       // the same, each transposed (K_c x rows row-major)
+    // near and admissible blocks, ordered by row cluster
+    bem::H2Block *near_blk = nullptr, *far_blk = nullptr;
+    int64_t n_near = 0, n_far = 0;
     const double *near_vals = nullptr, *far_vals = nullptr;
-    int32_t *cl_ptr = nullptr, *cl_idx = nullptr;   // cluster index sets
-    // levels (host lists of device cluster arrays), deepest last
-    std::vector<int32_t *> level;
-    std::vector<int32_t> level_n;
-    std::vector<int32_t> leaves_h;
-    int32_t *leaves = nullptr;
-    int32_t n_leaves = 0;
+    double *near_part = nullptr, *far_part = nullptr;   // the blocks' products
+    int32_t *cl_idx = nullptr;     // cluster index sets
+    // device cluster lists: forward passes (all leaves, then by level, deepest
+    // first), backward passes (by level from the top, then all leaves)
+    std::vector<int32_t *> fwd, bwd;
+    std::vector<int32_t> fwd_n, bwd_n;
     double *xhat = nullptr, *yhat = nullptr;
     int64_t n_hat = 0;
     double *diag = nullptr;        // added to the diagonal (null: none)
     // conjugate gradients: vectors and scalars
     double *r = nullptr, *p = nullptr, *q = nullptr, *part = nullptr, *scal = nullptr;
-    // the near field runs on a second stream beside the forward and coupling
-    // passes (it writes y, the backward pass then adds to it)
+    // the levels and the coupling run on a stream of their own beside the near field
     cudaStream_t side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
 };
@@ -73,74 +99,101 @@ __device__ __forceinline__ double warp_sum_d(double v)
     return v;
 }
 
-struct H2View {
-    const int32_t *rows, *rank, *leaf, *src;
-    const int64_t *v_off, *src_off, *hat_off;
-    const double *vals, *valsT;
-    const int32_t *near_ptr, *near_col, *far_ptr, *far_col, *cl_ptr, *cl_idx;
-    const int64_t *near_off, *far_off;
-    const double *near_vals, *far_vals;
-    const double *diag;
-};
+// Programmatic dependent launch: wait for the launch before this one in the
+// stream to finish (all of its writes visible); let the next one start.  Both are
+// no-ops in a plain launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 
-// near field: one CTA per leaf row cluster; its 8 warps take every 8th near
-// block, lane i = row i (rows in passes of 32), and the warps' partial sums
-// are added in warp order (fixed, so the result is reproducible)
 constexpr int kH2Warps = 8;
 
-__global__ void __launch_bounds__(256) k_h2_near(H2View H, const int32_t *leaves, int n_leaves,
-                                                 const double *__restrict__ x, double *y)
+// Product of one block by one warp: lane i = row i (rows in passes of 32), all
+// 32 column loads of a pass in flight; x: the column values, gathered through idx
+// if GATHER.
+template <bool GATHER>
+__global__ void __launch_bounds__(256) k_h2_blocks(const H2Block *__restrict__ blk, int64_t n,
+                                                   const double *__restrict__ vals,
+                                                   const int32_t *__restrict__ idx,
+                                                   const double *__restrict__ x, double *part)
 {
-    __shared__ double part[kH2Warps][32];
-    const int t = leaves[blockIdx.x];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r0 = H.cl_ptr[t], nr = H.cl_ptr[t + 1] - r0;
-    for (int i0 = 0; i0 < nr; i0 += 32) {
-        const int i = i0 + lane;
-        double acc = 0.0;
-        if (i < nr)
-            for (int b = H.near_ptr[t] + warp; b < H.near_ptr[t + 1]; b += kH2Warps) {
-                const int s = H.near_col[b];
-                const int c0 = H.cl_ptr[s], ncl = H.cl_ptr[s + 1] - c0;
-                const double *N = H.near_vals + H.near_off[b] + i;
-#pragma unroll 4
-                for (int j = 0; j < ncl; ++j) acc = fma(N[(int64_t)j * nr], x[H.cl_idx[c0 + j]], acc);
-            }
-        part[warp][lane] = acc;
-        __syncthreads();
-        if (warp == 0 && i < nr) {
-            double sum = 0.0;
+    const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    H2Block B = {};
+    if (b < n) B = blk[b];
+    // entries of the first pass before the wait
+    double a[32];
+    const double *v = vals + B.val;
+    auto load = [&](int i0, int c0) {
+        const double *w = v + min(i0 + lane, B.nr - 1) + (int64_t)c0 * B.nr;
 #pragma unroll
-            for (int k = 0; k < kH2Warps; ++k) sum += part[k][lane];
-            const int gi = H.cl_idx[r0 + i];
-            if (H.diag) sum = fma(H.diag[gi], x[gi], sum);
-            y[gi] = sum;
+        for (int j = 0; j < 32; ++j) a[j] = c0 + j < B.nc ? __ldg(w + (int64_t)j * B.nr) : 0.0;
+    };
+    if (B.nr > 0) load(0, 0);
+    if (!GATHER) {
+        pdl_wait();
+        pdl_launch();
+    }
+    for (int i0 = 0; i0 < B.nr; i0 += 32) {
+        double acc = 0.0;
+        for (int c0 = 0; c0 < B.nc; c0 += 32) {
+            if (i0 + c0 > 0) load(i0, c0);
+            const int nc = min(32, B.nc - c0);
+            double xc = 0.0;
+            if (lane < nc) xc = x[GATHER ? __ldg(idx + B.src + c0 + lane) : B.src + c0 + lane];
+            double odd = 0.0;
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+                if (j >= nc) break;                    // uniform across the warp
+                acc = fma(a[j], __shfl_sync(0xffffffffu, xc, j), acc);
+                odd = fma(a[j + 1], __shfl_sync(0xffffffffu, xc, j + 1), odd);
+            }
+            acc += odd;
         }
-        __syncthreads();
+        if (i0 + lane < B.nr) part[B.out + i0 + lane] = acc;
     }
 }
 
-// forward transformation of one level: x^_c = V_c^T v, v = x at the leaf's
-// indices or the sons' x^ entries.  One CTA per cluster: lane k = column k
-// (K_c <= 32), the 8 warps take every 8th row, and their partial sums are
-// added in warp order (fixed, so the result is reproducible).  A level is
-// latency-bound (a few rows per warp), so the rows are spread over warps.
-__global__ void __launch_bounds__(256) k_h2_forward(H2View H, const int32_t *level, int n,
+// Forward transformation of a list of clusters: x^_c = V_c^T v, v = x at the
+// leaf's indices or the sons' x^ entries.  One CTA per cluster: lane k = column k
+// (K_c <= 32), the 8 warps take every 8th row, and their partial sums are added in
+// warp order.  Up to 64 rows (every cluster with sons) the matrix and the row
+// sources are in registers before the wait.
+__global__ void __launch_bounds__(256) k_h2_forward(const H2Node *__restrict__ nodes,
+                                                    const int32_t *__restrict__ list,
+                                                    const double *__restrict__ vals,
+                                                    const int32_t *__restrict__ sources,
                                                     const double *__restrict__ x, double *xhat)
 {
     __shared__ double part[kH2Warps][32];
-    const int c = level[blockIdx.x];
+    const H2Node N = nodes[list[blockIdx.x]];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int R = H.rows[c], K = H.rank[c];
-    if (K == 0) return;                 // uniform across the CTA
-    const double *V = H.vals + H.v_off[c];
-    const int32_t *src = H.src + H.src_off[c];
-    const double *v = H.leaf[c] ? x : xhat;
+    const int R = N.rows, K = N.rank;
+    const double *V = vals + N.v_off;
+    const int32_t *src = sources + N.src_off;
+    const double *v = N.leaf ? x : xhat;
     double acc = 0.0;
-    if (lane < K) {
+    if (R <= 8 * kH2Warps) {
+        double a[8];
+        int32_t at[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = warp + kH2Warps * u;
+            at[u] = i < R ? __ldg(src + i) : 0;
+            a[u] = i < R && lane < K ? __ldg(V + (int64_t)i * K + lane) : 0.0;
+        }
+        pdl_wait();
+        pdl_launch();
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (warp + kH2Warps * u < R) acc = fma(a[u], v[at[u]], acc);
+    } else {
+        pdl_wait();
+        pdl_launch();
+        if (lane < K) {
 #pragma unroll 4
-        for (int i = warp; i < R; i += kH2Warps)
-            acc = fma(V[(int64_t)i * K + lane], __ldg(v + __ldg(src + i)), acc);
+            for (int i = warp; i < R; i += kH2Warps)
+                acc = fma(V[(int64_t)i * K + lane], v[__ldg(src + i)], acc);
+        }
     }
     part[warp][lane] = acc;
     __syncthreads();
@@ -148,73 +201,89 @@ __global__ void __launch_bounds__(256) k_h2_forward(H2View H, const int32_t *lev
         double sum = 0.0;
 #pragma unroll
         for (int k = 0; k < kH2Warps; ++k) sum += part[k][lane];
-        xhat[H.hat_off[c] + lane] = sum;
+        xhat[N.hat + lane] = sum;
     }
 }
 
-// coupling: y^_t = sum over t's admissible blocks of S_ts x^_s (column-major
-// K_t x K_s); one CTA per cluster, its 8 warps over every 8th block, lane =
-// row, partial sums added in warp order; every cluster's y^ is written here,
-// zero without blocks
-__global__ void __launch_bounds__(256) k_h2_coupling(H2View H, int nc, const double *__restrict__ xhat,
-                                                     double *yhat)
+// Backward transformation of a list of clusters: y^_c = the father's part + the
+// sum of its blocks' products; every row i of V_c then gives (V_c y^_c)_i, the
+// father's part of a son's y^ entry, or for a leaf (LEAF), added to its near
+// blocks' products and diag x, the result at the leaf's index.  One CTA per
+// cluster; four threads per row (columns k = part mod 4, combined by two fixed
+// shuffles; the transposed basis makes consecutive rows consecutive words).
+template <bool LEAF>
+__global__ void __launch_bounds__(256) k_h2_backward(const H2Node *__restrict__ nodes,
+                                                     const int32_t *__restrict__ list,
+                                                     const double *__restrict__ valsT,
+                                                     const int32_t *__restrict__ sources,
+                                                     const double *__restrict__ far_part,
+                                                     const double *__restrict__ near_part,
+                                                     const double *__restrict__ diag,
+                                                     const double *__restrict__ x, double *yhat,
+                                                     double *y)
 {
     __shared__ double part[kH2Warps][32];
-    const int t = blockIdx.x;
+    __shared__ double yc[32];
+    const H2Node N = nodes[list[blockIdx.x]];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int K = H.rank[t];
-    if (K == 0) return;                 // uniform across the CTA
-    double acc = 0.0;
-    if (lane < K)
-        for (int b = H.far_ptr[t] + warp; b < H.far_ptr[t + 1]; b += kH2Warps) {
-            const int s = H.far_col[b], Ks = H.rank[s];
-            const double *S = H.far_vals + H.far_off[b] + lane;
-            const double *xs = xhat + H.hat_off[s];
-#pragma unroll 4
-            for (int l = 0; l < Ks; ++l) acc = fma(S[(int64_t)l * K], xs[l], acc);
+    const int R = N.rows, K = (N.up & 2) ? N.rank : 0;
+    const double *VT = valsT + N.v_off;
+    const int32_t *src = sources + N.src_off;
+    const int row = threadIdx.x >> 2, quarter = threadIdx.x & 3;
+    // first 64 rows: matrix (eight columns per thread) and target before the wait
+    double a[8];
+    int32_t to = 0;
+    if (row < R) {
+        to = __ldg(src + row);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int k = quarter + 4 * u;
+            a[u] = k < K ? __ldg(VT + (int64_t)k * R + row) : 0.0;
         }
+    }
+    pdl_wait();
+    pdl_launch();
+    double acc = 0.0;
+    if (lane < K) {
+        if (warp == 0 && (N.up & 1)) acc = yhat[N.hat + lane];
+#pragma unroll 4
+        for (int b = warp; b < N.n_far; b += kH2Warps) acc += far_part[N.far_off + (int64_t)b * K + lane];
+    }
     part[warp][lane] = acc;
     __syncthreads();
-    if (warp == 0 && lane < K) {
+    if (warp == 0) {
         double sum = 0.0;
 #pragma unroll
         for (int k = 0; k < kH2Warps; ++k) sum += part[k][lane];
-        yhat[H.hat_off[t] + lane] = sum;
+        yc[lane] = lane < K ? sum : 0.0;
     }
-}
-
-// backward transformation of one level: every row i of V_c adds (V_c y^_c)_i
-// to its target, the vector y at a leaf's index, the son's y^ entry otherwise.
-// One CTA per cluster; rows of at most 64 take four threads each (columns
-// k = part mod 4, combined by two fixed shuffles), longer ones one thread per
-// row.  The transposed basis makes consecutive rows consecutive words.
-__global__ void __launch_bounds__(256) k_h2_backward(H2View H, const int32_t *level, int n,
-                                                     double *yhat, double *y)
-{
-    const int c = level[blockIdx.x];
-    const int R = H.rows[c], K = H.rank[c];
-    if (K == 0) return;                 // uniform across the CTA
-    const double *VT = H.valsT + H.v_off[c];
-    const int32_t *src = H.src + H.src_off[c];
-    const double *yc = yhat + H.hat_off[c];
-    double *dst = H.leaf[c] ? y : yhat;
-    if (R <= 64) {
-        const int i = threadIdx.x >> 2, part = threadIdx.x & 3;
-        double acc = 0.0;
+    __syncthreads();
+    for (int i0 = 0; i0 < R; i0 += 64) {
+        const int i = i0 + row;
+        double s = 0.0;
         if (i < R) {
+            if (LEAF) {
 #pragma unroll 4
-            for (int k = part; k < K; k += 4) acc = fma(VT[(int64_t)k * R + i], yc[k], acc);
+                for (int b = quarter; b < N.n_near; b += 4) s += near_part[N.near_off + (int64_t)b * R + i];
+            }
+            if (i0 == 0) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) s = fma(a[u], yc[quarter + 4 * u], s);
+            } else {
+                to = __ldg(src + i);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int k = quarter + 4 * u;
+                    if (k < K) s = fma(__ldg(VT + (int64_t)k * R + i), yc[k], s);
+                }
+            }
         }
         // the four parts of a row sit in four consecutive lanes
-        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-        if (i < R && part == 0) dst[src[i]] += acc;
-    } else {
-        for (int i = threadIdx.x; i < R; i += blockDim.x) {
-            double acc = 0.0;
-#pragma unroll 8
-            for (int k = 0; k < K; ++k) acc = fma(VT[(int64_t)k * R + i], yc[k], acc);
-            dst[src[i]] += acc;
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (i < R && quarter == 0) {
+            if (LEAF) y[to] = diag ? fma(diag[to], x[to], s) : s;
+            else yhat[to] = s;
         }
     }
 }
@@ -277,51 +346,60 @@ __global__ void __launch_bounds__(256) k_cg_dir(int64_t n, double *scal, const d
 
 __global__ void k_cg_roll(double *scal) { scal[0] = scal[2]; }
 
-H2View view(const bem_h2 *h)
+// Launch in the stream; PDL: it may start while the launch before it still runs
+// (its kernel waits by itself).
+template <class... P, class... A>
+cudaError_t h2_launch(bool pdl, unsigned grid, cudaStream_t st, void (*k)(P...), A... args)
 {
-    H2View v;
-    v.rows = h->rows;
-    v.rank = h->rank;
-    v.leaf = h->leaf;
-    v.src = h->src;
-    v.v_off = h->v_off;
-    v.src_off = h->src_off;
-    v.hat_off = h->hat_off;
-    v.vals = h->vals;
-    v.valsT = h->valsT;
-    v.near_ptr = h->near_ptr;
-    v.near_col = h->near_col;
-    v.near_off = h->near_off;
-    v.far_ptr = h->far_ptr;
-    v.far_col = h->far_col;
-    v.far_off = h->far_off;
-    v.near_vals = h->near_vals;
-    v.far_vals = h->far_vals;
-    v.cl_ptr = h->cl_ptr;
-    v.cl_idx = h->cl_idx;
-    v.diag = h->diag;
-    return v;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(256);
+    c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
 }
-
 
 cudaError_t matvec(const bem_h2 *h, const double *x, double *y, cudaStream_t st)
 {
-    const H2View H = view(h);
-    // fork: the near field on the side stream, joined before the backward pass
+    const double *no = nullptr;
+    const int32_t *noi = nullptr;
+    auto warps = [](int64_t n) { return (unsigned)((n + kH2Warps - 1) / kH2Warps); };
+    // fork: the chain of levels on the side stream of highest priority, the near
+    // field on the caller's stream beside it (its CTAs fill the SMs that the chain's
+    // small launches leave idle), joined before the leaves' pass
     cudaError_t e = cudaEventRecord(h->fork, st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->fork, 0);
-    if (e != cudaSuccess) return e;
-    if (h->n_leaves > 0) k_h2_near<<<h->n_leaves, 256, 0, h->side>>>(H, h->leaves, h->n_leaves, x, y);
-    if ((e = cudaEventRecord(h->join, h->side)) != cudaSuccess) return e;
-    for (int d = (int)h->level.size() - 1; d >= 0; --d)
-        if (h->level_n[d] > 0)
-            k_h2_forward<<<h->level_n[d], 256, 0, st>>>(H, h->level[d], h->level_n[d], x, h->xhat);
-    k_h2_coupling<<<h->nc, 256, 0, st>>>(H, h->nc, h->xhat, h->yhat);
-    if ((e = cudaStreamWaitEvent(st, h->join, 0)) != cudaSuccess) return e;
-    for (size_t d = 0; d < h->level.size(); ++d)
-        if (h->level_n[d] > 0)
-            k_h2_backward<<<h->level_n[d], 256, 0, st>>>(H, h->level[d], h->level_n[d], h->yhat, y);
-    return cudaGetLastError();
+    bool pdl = false;   // the first launch of the chain waits for all earlier work
+    for (size_t k = 0; k < h->fwd.size() && e == cudaSuccess; ++k)
+        if (h->fwd_n[k] > 0) {
+            e = h2_launch(pdl, (unsigned)h->fwd_n[k], h->side, k_h2_forward, h->nodes, h->fwd[k], h->vals,
+                          h->src, x, h->xhat);
+            pdl = true;
+        }
+    if (e == cudaSuccess && h->n_near > 0)
+        e = h2_launch(false, warps(h->n_near), st, k_h2_blocks<true>, h->near_blk, h->n_near,
+                      h->near_vals, h->cl_idx, x, h->near_part);
+    if (e == cudaSuccess && h->n_far > 0) {
+        e = h2_launch(pdl, warps(h->n_far), h->side, k_h2_blocks<false>, h->far_blk, h->n_far, h->far_vals,
+                      noi, h->xhat, h->far_part);
+        pdl = true;
+    }
+    for (size_t k = 0; k + 1 < h->bwd.size() && e == cudaSuccess; ++k)
+        if (h->bwd_n[k] > 0) {
+            e = h2_launch(pdl, (unsigned)h->bwd_n[k], h->side, k_h2_backward<false>, h->nodes, h->bwd[k],
+                          h->valsT, h->src, h->far_part, no, no, no, h->yhat, y);
+            pdl = true;
+        }
+    if (e == cudaSuccess) e = cudaEventRecord(h->join, h->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->join, 0);
+    if (e == cudaSuccess && h->bwd_n.back() > 0)
+        e = h2_launch(false, (unsigned)h->bwd_n.back(), st, k_h2_backward<true>, h->nodes, h->bwd.back(),
+                      h->valsT, h->src, h->far_part, h->near_part, h->diag, x, h->yhat, y);
+    return e;
 }
 
 cudaError_t dot(const bem_h2 *h, const double *a, const double *b, double *out, cudaStream_t st)
@@ -474,32 +552,62 @@ int bem_h2_create(bem_ctx *ctx, int64_t n, int32_t n_clusters, const int32_t *cl
             h2_free(h);
             return api_fail(ctx, BEM_ERR_INVALID_ARG, "bem_h2_create: near block on a non-leaf row cluster");
         }
-    std::vector<std::vector<int32_t>> lev(max_depth + 1);
+    // clusters that take part: x^_c is used by an admissible block of c's column or of
+    // an ancestor's, y^_c gets one of c's row or of an ancestor's
+    std::vector<char> has_col(nc, 0), need_f(nc, 0), need_b(nc, 0);
+    for (int32_t s : fcol) has_col[s] = 1;
+    std::vector<int32_t> order(nc);
+    for (int c = 0; c < nc; ++c) order[c] = c;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return depth[a] < depth[b]; });
+    for (int c : order) {
+        need_f[c] = has_col[c] || (parent[c] >= 0 && need_f[parent[c]]);
+        need_b[c] = fptr[c + 1] > fptr[c] || (parent[c] >= 0 && need_b[parent[c]]);
+    }
+    std::vector<std::vector<int32_t>> fl(max_depth + 2), bl(max_depth + 2);
+    std::vector<H2Node> nodes(nc);
+    std::vector<H2Block> nblk(n_near), fblk(n_far);
+    int64_t np = 0, fp = 0;
     for (int c = 0; c < nc; ++c) {
-        lev[depth[c]].push_back(c);
-        if (leaf[c]) h->leaves_h.push_back(c);
+        H2Node &N = nodes[c];
+        N.v_off = voff[c];
+        N.src_off = soff[c];
+        N.near_off = np;
+        N.far_off = fp;
+        N.rows = rows[c];
+        N.rank = rank[c];
+        N.hat = (int32_t)hoff[c];
+        N.n_near = nptr[c + 1] - nptr[c];
+        N.n_far = fptr[c + 1] - fptr[c];
+        N.idx = cl_ptr[c];
+        N.leaf = leaf[c];
+        N.up = (parent[c] >= 0 && need_b[parent[c]] && rank[parent[c]] > 0 ? 1 : 0) | (need_b[c] ? 2 : 0);
+        const int nr = cl_ptr[c + 1] - cl_ptr[c];
+        for (int32_t b = nptr[c]; b < nptr[c + 1]; ++b, np += nr)
+            nblk[b] = H2Block{noff[b], np, nr, cl_ptr[ncol[b] + 1] - cl_ptr[ncol[b]], cl_ptr[ncol[b]], 0};
+        for (int32_t b = fptr[c]; b < fptr[c + 1]; ++b, fp += rank[c])
+            fblk[b] = H2Block{foff[b], fp, rank[c], rank[fcol[b]], (int32_t)hoff[fcol[b]], 0};
+        if (need_f[c] && rank[c] > 0) fl[leaf[c] ? 0 : 1 + max_depth - depth[c]].push_back(c);
+        if (leaf[c]) bl[max_depth + 1].push_back(c);
+        else if (need_b[c] && rank[c] > 0) bl[depth[c]].push_back(c);
     }
     cudaSetDevice(ctx->device);
     cudaError_t e = cudaSuccess;
-    std::vector<int32_t> cp(cl_ptr, cl_ptr + nc + 1), ci(cl_idx, cl_idx + cl_ptr[nc]);
+    std::vector<int32_t> ci(cl_idx, cl_idx + cl_ptr[nc]);
     std::vector<double> vals(V, V + v_off[nc]), valsT(vals.size());
     for (int c = 0; c < nc; ++c)
         for (int i = 0; i < rows[c]; ++i)
             for (int k = 0; k < rank[c]; ++k)
                 valsT[voff[c] + (int64_t)k * rows[c] + i] = vals[voff[c] + (int64_t)i * rank[c] + k];
-    if ((e = h2_upload(h, &h->rows, rows)) || (e = h2_upload(h, &h->rank, rank)) ||
-        (e = h2_upload(h, &h->leaf, leaf)) || (e = h2_upload(h, &h->src, src)) ||
-        (e = h2_upload(h, &h->v_off, voff)) || (e = h2_upload(h, &h->src_off, soff)) ||
-        (e = h2_upload(h, &h->hat_off, hoff)) || (e = h2_upload(h, &h->vals, vals)) ||
-        (e = h2_upload(h, &h->valsT, valsT)) ||
-        (e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking)) ||
+    int low = 0, high = 0;
+    if ((e = h2_upload(h, &h->nodes, nodes)) || (e = h2_upload(h, &h->src, src)) ||
+        (e = h2_upload(h, &h->vals, vals)) || (e = h2_upload(h, &h->valsT, valsT)) ||
+        (e = cudaDeviceGetStreamPriorityRange(&low, &high)) ||
+        (e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, high)) ||
         (e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming)) ||
         (e = cudaEventCreateWithFlags(&h->join, cudaEventDisableTiming)) ||
-        (e = h2_upload(h, &h->near_ptr, nptr)) || (e = h2_upload(h, &h->near_col, ncol)) ||
-        (e = h2_upload(h, &h->near_off, noff)) || (e = h2_upload(h, &h->far_ptr, fptr)) ||
-        (e = h2_upload(h, &h->far_col, fcol)) || (e = h2_upload(h, &h->far_off, foff)) ||
-        (e = h2_upload(h, &h->cl_ptr, cp)) || (e = h2_upload(h, &h->cl_idx, ci)) ||
-        (e = h2_upload(h, &h->leaves, h->leaves_h)) || (e = h2_alloc(h, &h->xhat, hat)) ||
+        (e = h2_upload(h, &h->near_blk, nblk)) || (e = h2_upload(h, &h->far_blk, fblk)) ||
+        (e = h2_upload(h, &h->cl_idx, ci)) || (e = h2_alloc(h, &h->near_part, np)) ||
+        (e = h2_alloc(h, &h->far_part, fp)) || (e = h2_alloc(h, &h->xhat, hat)) ||
         (e = h2_alloc(h, &h->yhat, hat)) || (e = h2_alloc(h, &h->r, n)) ||
         (e = h2_alloc(h, &h->p, n)) || (e = h2_alloc(h, &h->q, n)) ||
         (e = h2_alloc(h, &h->part, kDotBlocks)) || (e = h2_alloc(h, &h->scal, 4))) {
@@ -513,16 +621,18 @@ int bem_h2_create(bem_ctx *ctx, int64_t n, int32_t n_clusters, const int32_t *cl
             return api_cuda_fail(ctx, e, "bem_h2_create");
         }
     }
-    for (auto &l : lev) {
-        int32_t *d = nullptr;
-        if ((e = h2_upload(h, &d, l)) != cudaSuccess) {
-            h2_free(h);
-            return api_cuda_fail(ctx, e, "bem_h2_create");
+    for (int pass = 0; pass < 2; ++pass)
+        for (auto &l : pass ? bl : fl) {
+            int32_t *d = nullptr;
+            if ((e = h2_upload(h, &d, l)) != cudaSuccess) {
+                h2_free(h);
+                return api_cuda_fail(ctx, e, "bem_h2_create");
+            }
+            (pass ? h->bwd : h->fwd).push_back(d);
+            (pass ? h->bwd_n : h->fwd_n).push_back((int32_t)l.size());
         }
-        h->level.push_back(d);
-        h->level_n.push_back((int32_t)l.size());
-    }
-    h->n_leaves = (int32_t)h->leaves_h.size();
+    h->n_near = n_near;
+    h->n_far = n_far;
     h->n_hat = hat;
     h->near_vals = near_vals;
     h->far_vals = far_vals;
