@@ -123,9 +123,12 @@ __global__ void __launch_bounds__(1024) k_job_scan(const int64_t *job_total, int
 
 // Capped at 64 registers (four CTAs, 32 warps per SM): the float form's
 // dependent loads (block, cluster, index, geometry) and the FP64 form's integer
-// chains (bem_fixed_pair.cuh) want the warps.
+// chains (bem_fixed_pair.cuh) want the warps.  The float Helmholtz pair holds ten
+// packed constants and spills at 64, so it takes three CTAs (2% over four).
+constexpr int p0_ctas(int kind, bool mixed) { return mixed && kind == BEM_HELMHOLTZ_SLP ? 3 : 4; }
+
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(256, 4) k_block_p0(MeshView m, BlockLaunch L,
+__global__ void __launch_bounds__(256, p0_ctas(KIND, MIXED)) k_block_p0(MeshView m, BlockLaunch L,
                                                   const __grid_constant__ Rule2D R,
                                                   const int64_t *__restrict__ prefix,
                                                   int *status)
@@ -149,7 +152,7 @@ __global__ void __launch_bounds__(256, 4) k_block_p0(MeshView m, BlockLaunch L,
 // same tile body as the single-list kernels, so the results are identical.
 // ---------------------------------------------------------------------------
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(256, 4) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
+__global__ void __launch_bounds__(256, p0_ctas(KIND, MIXED)) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
                                                   const int64_t *__restrict__ job_end,
                                                   const __grid_constant__ Rule2D R, int *status)
 {

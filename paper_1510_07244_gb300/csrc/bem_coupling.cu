@@ -26,11 +26,11 @@ namespace {
 constexpr int kCouplingThreads = 256;
 
 // Sum over the product rule of one disjoint pair for the basis functions at
-// local vertices la (test) and the precomputed trial side (yx, yy, yz, wy).
+// local vertices la (test) and the precomputed trial side (T, wy).
 template <int KIND, int NP>
 __device__ __forceinline__ float coupling_pair(const TriF &A, const TriF &B, int la,
-                                               const Rule2D &R, const float *yx, const float *yy,
-                                               const float *yz, const float *wy)
+                                               const Rule2D &R, const TrialX2<NP> &T,
+                                               const float *wy)
 {
     float d0[3];
 #pragma unroll
@@ -48,9 +48,9 @@ __device__ __forceinline__ float coupling_pair(const TriF &A, const TriF &B, int
         const float xz = fmaf(s, A.e1[2], fmaf(t, A.e2[2], d0[2]));
         const float dn = KIND == BEM_LAPLACE_DLP ? height_at_far(H, s, t) : 0.0f;
         float inner = 0.0f;
-#pragma unroll
-        for (int j = 0; j < NP; ++j)
-            inner = fmaf(wy[j], kvalf_r<KIND>(xx - yx[j], xy - yy[j], xz - yz[j]), inner);
+        for_trial<NP>(T, xx, xy, xz, [&](int j, float ri, float r3) {
+            inner = fmaf(wy[j], KIND == BEM_LAPLACE_SLP ? ri : r3, inner);
+        });
         if (KIND == BEM_LAPLACE_DLP) inner *= dn;
         const float wx = la == 0 ? R.wl[0][i] : (la == 1 ? R.wl[1][i] : R.wl[2][i]);
         sum = fmaf(wx, inner, sum);
@@ -63,8 +63,8 @@ __device__ __forceinline__ float coupling_pair(const TriF &A, const TriF &B, int
 // does, sharing the points, the distances and the reciprocal square roots.
 template <int NP>
 __device__ __forceinline__ void coupling_pair2(const TriF &A, const TriF &B, int la, const Rule2D &R,
-                                               const float *yx, const float *yy, const float *yz,
-                                               const float *wy, float &out_s, float &out_d)
+                                               const TrialX2<NP> &T, const float *wy,
+                                               float &out_s, float &out_d)
 {
     float d0[3];
 #pragma unroll
@@ -80,14 +80,10 @@ __device__ __forceinline__ void coupling_pair2(const TriF &A, const TriF &B, int
         const float xz = fmaf(s, A.e1[2], fmaf(t, A.e2[2], d0[2]));
         const float dn = height_at_far(H, s, t);
         float in_s = 0.0f, in_d = 0.0f;
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const float dx = xx - yx[j], dy = xy - yy[j], dz = xz - yz[j];
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float ri = rsqrt_fast(r2);
+        for_trial<NP>(T, xx, xy, xz, [&](int j, float ri, float r3) {
             in_s = fmaf(wy[j], ri, in_s);
-            in_d = fmaf(wy[j], ri * ri * ri, in_d);
-        }
+            in_d = fmaf(wy[j], r3, in_d);
+        });
         in_d *= dn;
         const float wx = la == 0 ? R.wl[0][i] : (la == 1 ? R.wl[1][i] : R.wl[2][i]);
         sum_s = fmaf(wx, in_s, sum_s);
@@ -129,15 +125,11 @@ __device__ __forceinline__ void coupling_tile(const MeshView &m, const BlockLaun
         TriF B;
         load_trif(m.geomf, b, B);
         // trial side of the product rule, relative to B's vertex 0
-        float yx[NP], yy[NP], yz[NP], wy[NP];
+        const TrialX2<NP> T = trial_x2<NP>(B, R);
+        float wy[NP];
 #pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            const float s = R.sf[q], t = R.tf[q];
-            yx[q] = fmaf(s, B.e1[0], t * B.e2[0]);
-            yy[q] = fmaf(s, B.e1[1], t * B.e2[1]);
-            yz[q] = fmaf(s, B.e1[2], t * B.e2[2]);
+        for (int q = 0; q < NP; ++q)
             wy[q] = lb == 0 ? R.wl[0][q] : (lb == 1 ? R.wl[1][q] : R.wl[2][q]);
-        }
         for (int ka = alo; ka < ahi; ++ka) {
             const int a = __ldg(m.vt_tri + ka);
             const int4 va = __ldg(m.tvid + a);
@@ -147,7 +139,7 @@ __device__ __forceinline__ void coupling_tile(const MeshView &m, const BlockLaun
             }
             TriF A;
             load_trif(m.geomf, a, A);
-            const float p = coupling_pair<KIND, NP>(A, B, local_of(va, i), R, yx, yy, yz, wy) *
+            const float p = coupling_pair<KIND, NP>(A, B, local_of(va, i), R, T, wy) *
                             (A.sg * B.sg);
             const float y = p - cmp;
             const float t = acc + y;
@@ -195,15 +187,11 @@ __device__ __forceinline__ void coupling_tile_fused(const MeshView &m, const Blo
         const int lb = local_of(vb, j);
         TriF B;
         load_trif(m.geomf, b, B);
-        float yx[NP], yy[NP], yz[NP], wy[NP];
+        const TrialX2<NP> T = trial_x2<NP>(B, R);
+        float wy[NP];
 #pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            const float s = R.sf[q], t = R.tf[q];
-            yx[q] = fmaf(s, B.e1[0], t * B.e2[0]);
-            yy[q] = fmaf(s, B.e1[1], t * B.e2[1]);
-            yz[q] = fmaf(s, B.e1[2], t * B.e2[2]);
+        for (int q = 0; q < NP; ++q)
             wy[q] = lb == 0 ? R.wl[0][q] : (lb == 1 ? R.wl[1][q] : R.wl[2][q]);
-        }
         for (int ka = alo; ka < ahi; ++ka) {
             const int a = __ldg(m.vt_tri + ka);
             const int4 va = __ldg(m.tvid + a);
@@ -214,7 +202,7 @@ __device__ __forceinline__ void coupling_tile_fused(const MeshView &m, const Blo
             TriF A;
             load_trif(m.geomf, a, A);
             float ps, pd;
-            coupling_pair2<NP>(A, B, local_of(va, i), R, yx, yy, yz, wy, ps, pd);
+            coupling_pair2<NP>(A, B, local_of(va, i), R, T, wy, ps, pd);
             const float sg = A.sg * B.sg;
             float y = ps * sg - cmp_s, t = acc_s + y;
             cmp_s = (t - acc_s) - y;

@@ -118,6 +118,47 @@ __device__ __forceinline__ float rsqrt_fast(float x)
     return y;
 }
 
+// Packed FP32 pairs (sm_100 and later): sub/add/mul/fma .f32x2 apply the scalar
+// operation, with its rounding, to both halves of a 64-bit register pair in
+// one instruction.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_dup(float v) { return f2_pack(v, v); }
+__device__ __forceinline__ void f2_unpack(f32x2 v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 // ---------------------------------------------------------------------------
 // Mixed form: float arithmetic with double-float set-up.  Every vertex is held
 // as hi + lo floats; differences of vertices and the heights of one
@@ -130,6 +171,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     s = a + b;
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
+}
+
+// The same error-free steps on both halves of a packed pair.
+__device__ __forceinline__ void two_sum_x2(f32x2 a, f32x2 b, f32x2 &s, f32x2 &e)
+{
+    s = f2_add(a, b);
+    const f32x2 bb = f2_sub(s, a);
+    e = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
 }
 
 // (ah + al) - (bh + bl) as an unevaluated hi + lo pair
@@ -154,13 +203,18 @@ __device__ __forceinline__ void dd_height(const float *ah, const float *al, cons
                                           const float *bl, const float *nh, const float *nl,
                                           float &hh, float &hl)
 {
-    float S = 0.0f, E = 0.0f;
+    float S, E;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         float dh, dl;
         dd_sub(ah[c], al[c], bh[c], bl[c], dh, dl);
         const float p = dh * nh[c];
         const float pe = fmaf(dh, nh[c], -p) + fmaf(dh, nl[c], dl * nh[c]);
+        if (c == 0) {   // 0 + p is exact
+            S = p;
+            E = pe;
+            continue;
+        }
         float s2, e2;
         two_sum(S, p, s2, e2);
         S = s2;
@@ -186,6 +240,20 @@ __device__ __forceinline__ float height_at(const Height &H, float s, float t)
     two_sum(a, H.h0, b, eb);
     const float lo = ea + eb + e1 + e2 + H.h0l + fmaf(s, H.h10l, t * H.h21l);
     return b + lo;
+}
+
+// The heights at two points: height_at on packed pairs, each half rounded as there.
+__device__ __forceinline__ f32x2 height_at_x2(const Height &H, f32x2 s, f32x2 t)
+{
+    const f32x2 h10 = f2_dup(H.h10), h21 = f2_dup(H.h21);
+    const f32x2 p1 = f2_mul(s, h10), p2 = f2_mul(t, h21);
+    const f32x2 m1 = f2_fma(s, f2_dup(-H.h10), p1), m2 = f2_fma(t, f2_dup(-H.h21), p2);   // -e1, -e2
+    f32x2 a, ea, b, eb;
+    two_sum_x2(p1, p2, a, ea);
+    two_sum_x2(a, f2_dup(H.h0), b, eb);
+    const f32x2 lo = f2_add(f2_add(f2_sub(f2_sub(f2_add(ea, eb), m1), m2), f2_dup(H.h0l)),
+                            f2_fma(s, f2_dup(H.h10l), f2_mul(t, f2_dup(H.h21l))));
+    return f2_add(b, lo);
 }
 
 // The same height in plain float from the rounded coefficients, for pairs of
@@ -344,6 +412,16 @@ __device__ __forceinline__ void dd_mul(float ah, float al, float bh, float bl, f
     l = e - (h - p);
 }
 
+// kappa as hi + lo floats (split once per thread: two conversions and a
+// subtraction on the slow FP64 pipe)
+struct KappaF {
+    float h, l;
+    __device__ __forceinline__ explicit KappaF(double kappa)
+        : h((float)kappa), l((float)(kappa - (double)(float)kappa))
+    {
+    }
+};
+
 // phase data of a pair: cos/sin of kappa r0 and the float quantities per point
 struct HelmPhase {
     float dcx, dcy, dcz;   // centroid difference d_c (float)
@@ -354,7 +432,7 @@ struct HelmPhase {
     float kap;
 };
 
-__device__ __forceinline__ HelmPhase helm_phase(const TriF &A, const TriF &B, double kappa)
+__device__ __forceinline__ HelmPhase helm_phase(const TriF &A, const TriF &B, KappaF kappa)
 {
     // centroid difference in double-float: (sum of vertices of A - of B) / 3
     float dh[3], dl[3];
@@ -388,9 +466,8 @@ __device__ __forceinline__ HelmPhase helm_phase(const TriF &A, const TriF &B, do
     float r0h, r0l;
     two_sum(rh0, corr, r0h, r0l);
     // kappa r0 in double-float, reduced modulo 2 pi
-    const float kh = (float)kappa, kl = (float)(kappa - (double)kh);
     float ph, pl;
-    dd_mul(kh, kl, r0h, r0l, ph, pl);
+    dd_mul(kappa.h, kappa.l, r0h, r0l, ph, pl);
     const float n = rintf(ph * 0.159154943092f);
     const float two_pi_h = 6.28318548202514648f, two_pi_l = -1.74845553e-07f;
     float t = fmaf(-n, two_pi_h, ph);
@@ -405,7 +482,7 @@ __device__ __forceinline__ HelmPhase helm_phase(const TriF &A, const TriF &B, do
     P.m2r0l = -2.0f * r0l;
     P.r0sqh = sh;
     P.r0sql = sl;
-    P.kap = kh;
+    P.kap = kappa.h;
     return P;
 }
 
@@ -442,107 +519,93 @@ __device__ __forceinline__ void helm_rotate(const HelmPhase &P, float sr, float 
     im = P.s0 * sr + P.c0 * si;
 }
 
-// Packed FP32 pairs (sm_100 and later): sub/add/mul/fma .f32x2 apply the scalar
-// operation, with its rounding, to both halves of a 64-bit register pair in
-// one instruction.
-typedef unsigned long long f32x2;
+// helm_offset at two packed offsets: the same operations per point, each rounded
+// as there; the reciprocal square roots, sines and cosines stay scalar.
+struct HelmX2 {
+    f32x2 tdx, tdy, tdz, r0sqh, nr0sqh, r0sql, r0h, m2r0l, kap, half;
+    __device__ __forceinline__ explicit HelmX2(const HelmPhase &P)
+        : tdx(f2_dup(2.0f * P.dcx)), tdy(f2_dup(2.0f * P.dcy)), tdz(f2_dup(2.0f * P.dcz)),
+          r0sqh(f2_dup(P.r0sqh)), nr0sqh(f2_dup(-P.r0sqh)), r0sql(f2_dup(P.r0sql)),
+          r0h(f2_dup(P.r0h)), m2r0l(f2_dup(P.m2r0l)), kap(f2_dup(P.kap)), half(f2_dup(0.5f))
+    {
+    }
+    __device__ __forceinline__ void at(f32x2 ex, f32x2 ey, f32x2 ez, f32x2 &ri, float &ca, float &cb,
+                                       float &sa, float &sb) const
+    {
+        // q = (2 d_c + e) . e, r^2 = r0^2 + q
+        const f32x2 qq = f2_fma(f2_add(tdx, ex), ex,
+                                f2_fma(f2_add(tdy, ey), ey, f2_mul(f2_add(tdz, ez), ez)));
+        const f32x2 r2 = f2_add(r0sqh, qq);
+        float r2a, r2b;
+        f2_unpack(r2, r2a, r2b);
+        ri = f2_pack(rsqrt_fast(r2a), rsqrt_fast(r2b));
+        const f32x2 ra = f2_mul(r2, ri);
+        // (r0sq_hi - ra^2) + (q + r0sq_lo), with ra^2 - r0sq_hi from one FMA
+        const f32x2 res = f2_sub(f2_add(qq, r0sql), f2_fma(ra, ra, nr0sqh));
+        const f32x2 delta = f2_fma(half, f2_fma(res, ri, m2r0l), f2_sub(ra, r0h));
+        float ta, tb;
+        f2_unpack(f2_mul(kap, delta), ta, tb);
+        __sincosf(ta, &sa, &ca);
+        __sincosf(tb, &sb, &cb);
+    }
+};
 
-__device__ __forceinline__ f32x2 f2_pack(float lo, float hi)
+// centroid-relative offset of a rule point: (s - 2/3) e1 + (t - 1/3) e2
+__device__ __forceinline__ float helm_point(float s, float t, const TriF &A, int c)
 {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f32x2 v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
+    return fmaf(s - 0.666666687f, A.e1[c], (t - 0.333333343f) * A.e2[c]);
 }
 
-// The float Helmholtz pair of regular_p0_f32_helm with two trial points per
-// packed instruction: the same operations per point (helm_offset), each rounded
-// as there; the reciprocal square roots, sines and cosines stay scalar.  The
-// inner sums run as two partial sums (even and odd trial points) added per
-// test point; an odd rule's last pair repeats its last point with weight 0.
+// The float Helmholtz pair with two points per packed instruction.  Bound by the
+// special functions (three per point, 16 lanes per SM and cycle) and the FP32 pipe
+// alike.  The inner sums run as two partial sums (even and odd trial points) added
+// per test point.  An odd rule's last trial point is packed over two test points
+// (41 evaluations instead of 45 at nine points); the last test point takes it alone.
 template <int NP>
 __device__ __forceinline__ void regular_p0_f32_helm_x2(const TriF &A, const TriF &B,
-                                                       const Rule2D &R, double kappa,
+                                                       const Rule2D &R, KappaF kappa,
                                                        float &out_re, float &out_im)
 {
-    constexpr int NQ = (NP + 1) / 2;
+    constexpr int NQ = NP / 2;
+    constexpr bool ODD = NP % 2 != 0;
     const HelmPhase P = helm_phase(A, B, kappa);
     f32x2 yx[NQ], yy[NQ], yz[NQ], w2[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const int j0 = 2 * q, j1 = 2 * q + 1 < NP ? 2 * q + 1 : NP - 1;
-        const float a0 = R.sf[j0] - 0.666666687f, b0 = R.tf[j0] - 0.333333343f;
-        const float a1 = R.sf[j1] - 0.666666687f, b1 = R.tf[j1] - 0.333333343f;
-        yx[q] = f2_pack(fmaf(a0, B.e1[0], b0 * B.e2[0]), fmaf(a1, B.e1[0], b1 * B.e2[0]));
-        yy[q] = f2_pack(fmaf(a0, B.e1[1], b0 * B.e2[1]), fmaf(a1, B.e1[1], b1 * B.e2[1]));
-        yz[q] = f2_pack(fmaf(a0, B.e1[2], b0 * B.e2[2]), fmaf(a1, B.e1[2], b1 * B.e2[2]));
-        w2[q] = f2_pack(R.wf[j0], 2 * q + 1 < NP ? R.wf[j1] : 0.0f);
+        const int j0 = 2 * q, j1 = 2 * q + 1;
+        yx[q] = f2_pack(helm_point(R.sf[j0], R.tf[j0], B, 0), helm_point(R.sf[j1], R.tf[j1], B, 0));
+        yy[q] = f2_pack(helm_point(R.sf[j0], R.tf[j0], B, 1), helm_point(R.sf[j1], R.tf[j1], B, 1));
+        yz[q] = f2_pack(helm_point(R.sf[j0], R.tf[j0], B, 2), helm_point(R.sf[j1], R.tf[j1], B, 2));
+        w2[q] = f2_pack(R.wf[j0], R.wf[j1]);
     }
-    const f32x2 tdx = f2_pack(2.0f * P.dcx, 2.0f * P.dcx), tdy = f2_pack(2.0f * P.dcy, 2.0f * P.dcy),
-                tdz = f2_pack(2.0f * P.dcz, 2.0f * P.dcz);
-    const f32x2 r0sqh = f2_pack(P.r0sqh, P.r0sqh), nr0sqh = f2_pack(-P.r0sqh, -P.r0sqh),
-                r0sql = f2_pack(P.r0sql, P.r0sql), r0h = f2_pack(P.r0h, P.r0h),
-                m2r0l = f2_pack(P.m2r0l, P.m2r0l), kap = f2_pack(P.kap, P.kap),
-                half = f2_pack(0.5f, 0.5f);
+    float ox = 0.0f, oy = 0.0f, oz = 0.0f;
+    if (ODD) {
+        ox = helm_point(R.sf[NP - 1], R.tf[NP - 1], B, 0);
+        oy = helm_point(R.sf[NP - 1], R.tf[NP - 1], B, 1);
+        oz = helm_point(R.sf[NP - 1], R.tf[NP - 1], B, 2);
+    }
+    const HelmX2 H(P);
     float sr = 0.0f, si = 0.0f, cr = 0.0f, ci = 0.0f;
-#pragma unroll 1
-    for (int i = 0; i < NP; ++i) {
-        const float a = R.sf[i] - 0.666666687f, b = R.tf[i] - 0.333333343f;
-        const float xx = fmaf(a, A.e1[0], b * A.e2[0]);
-        const float xy = fmaf(a, A.e1[1], b * A.e2[1]);
-        const float xz = fmaf(a, A.e1[2], b * A.e2[2]);
-        const f32x2 X = f2_pack(xx, xx), Y = f2_pack(xy, xy), Z = f2_pack(xz, xz);
-        f32x2 ir = f2_pack(0.0f, 0.0f), ii = ir;
+    // even and odd partial sums of the paired trial points at test point x
+    auto inner = [&](float xx, float xy, float xz, f32x2 &ir, f32x2 &ii) {
+        const f32x2 X = f2_dup(xx), Y = f2_dup(xy), Z = f2_dup(xz);
+        ir = ii = f2_dup(0.0f);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            const f32x2 ex = f2_sub(X, yx[q]), ey = f2_sub(Y, yy[q]), ez = f2_sub(Z, yz[q]);
-            // q = (2 d_c + e) . e, r^2 = r0^2 + q (helm_offset)
-            const f32x2 qq = f2_fma(f2_add(tdx, ex), ex,
-                                    f2_fma(f2_add(tdy, ey), ey, f2_mul(f2_add(tdz, ez), ez)));
-            const f32x2 r2 = f2_add(r0sqh, qq);
-            float r2a, r2b;
-            f2_unpack(r2, r2a, r2b);
-            const f32x2 ri = f2_pack(rsqrt_fast(r2a), rsqrt_fast(r2b));
-            const f32x2 ra = f2_mul(r2, ri);
-            // (r0sq_hi - ra^2) + (q + r0sq_lo), with ra^2 - r0sq_hi from one FMA
-            const f32x2 res = f2_sub(f2_add(qq, r0sql), f2_fma(ra, ra, nr0sqh));
-            const f32x2 delta = f2_fma(half, f2_fma(res, ri, m2r0l), f2_sub(ra, r0h));
-            float ta, tb;
-            f2_unpack(f2_mul(kap, delta), ta, tb);
-            float sa, ca, sb, cb;
-            __sincosf(ta, &sa, &ca);
-            __sincosf(tb, &sb, &cb);
+            f32x2 ri;
+            float ca, cb, sa, sb;
+            H.at(f2_sub(X, yx[q]), f2_sub(Y, yy[q]), f2_sub(Z, yz[q]), ri, ca, cb, sa, sb);
             const f32x2 wr = f2_mul(w2[q], ri);
             ir = f2_fma(f2_pack(ca, cb), wr, ir);
             ii = f2_fma(f2_pack(sa, sb), wr, ii);
         }
+    };
+    auto fma_lo = [](float a, float b, f32x2 &c) {
+        float lo, hi;
+        f2_unpack(c, lo, hi);
+        c = f2_pack(fmaf(a, b, lo), hi);
+    };
+    auto outer = [&](int i, f32x2 ir, f32x2 ii) {
         float ir0, ir1, ii0, ii1;
         f2_unpack(ir, ir0, ir1);
         f2_unpack(ii, ii0, ii1);
@@ -554,6 +617,44 @@ __device__ __forceinline__ void regular_p0_f32_helm_x2(const TriF &A, const TriF
         t = si + y;
         ci = (t - si) - y;
         si = t;
+    };
+#pragma unroll 1
+    for (int i = 0; i + 1 < NP; i += 2) {
+        const float xa = helm_point(R.sf[i], R.tf[i], A, 0), ya = helm_point(R.sf[i], R.tf[i], A, 1),
+                    za = helm_point(R.sf[i], R.tf[i], A, 2);
+        const float xb = helm_point(R.sf[i + 1], R.tf[i + 1], A, 0),
+                    yb = helm_point(R.sf[i + 1], R.tf[i + 1], A, 1),
+                    zb = helm_point(R.sf[i + 1], R.tf[i + 1], A, 2);
+        f32x2 ira, iia, irb, iib;
+        inner(xa, ya, za, ira, iia);
+        inner(xb, yb, zb, irb, iib);
+        if (ODD) {
+            f32x2 ri;
+            float ca, cb, sa, sb;
+            H.at(f2_sub(f2_pack(xa, xb), f2_dup(ox)), f2_sub(f2_pack(ya, yb), f2_dup(oy)),
+                 f2_sub(f2_pack(za, zb), f2_dup(oz)), ri, ca, cb, sa, sb);
+            float wa, wb;
+            f2_unpack(f2_mul(f2_dup(R.wf[NP - 1]), ri), wa, wb);
+            fma_lo(ca, wa, ira);
+            fma_lo(sa, wa, iia);
+            fma_lo(cb, wb, irb);
+            fma_lo(sb, wb, iib);
+        }
+        outer(i, ira, iia);
+        outer(i + 1, irb, iib);
+    }
+    if (ODD) {
+        const float xx = helm_point(R.sf[NP - 1], R.tf[NP - 1], A, 0),
+                    xy = helm_point(R.sf[NP - 1], R.tf[NP - 1], A, 1),
+                    xz = helm_point(R.sf[NP - 1], R.tf[NP - 1], A, 2);
+        f32x2 ir, ii;
+        inner(xx, xy, xz, ir, ii);
+        float c, s, ri;
+        helm_offset(P, xx - ox, xy - oy, xz - oz, c, s, ri);
+        const float wr = R.wf[NP - 1] * ri;
+        fma_lo(c, wr, ir);
+        fma_lo(s, wr, ii);
+        outer(NP - 1, ir, ii);
     }
     float re, im;
     helm_rotate(P, sr, si, re, im);
@@ -562,33 +663,48 @@ __device__ __forceinline__ void regular_p0_f32_helm_x2(const TriF &A, const TriF
     out_im = im * sc;
 }
 
-// Regular pair, piecewise constant, Helmholtz single layer, float.
+// Regular pair, piecewise constant, Helmholtz single layer, float: the points two
+// at a time (HelmX2), every sum in the order of the points.
 template <int NP>
 __device__ __forceinline__ void regular_p0_f32_helm(const TriF &A, const TriF &B, const Rule2D &R,
-                                                    double kappa, float &out_re, float &out_im)
+                                                    KappaF kappa, float &out_re, float &out_im)
 {
+    constexpr int NQ = NP / 2;
     const HelmPhase P = helm_phase(A, B, kappa);
-    // centroid-relative offsets of the y points: y - y_c = (s - 2/3) e1 + (t - 1/3) e2
-    float yx[NP], yy[NP], yz[NP];
+    const HelmX2 H(P);
+    f32x2 yx[NQ], yy[NQ], yz[NQ];
 #pragma unroll
-    for (int j = 0; j < NP; ++j) {
-        const float a = R.sf[j] - 0.666666687f, b = R.tf[j] - 0.333333343f;
-        yx[j] = fmaf(a, B.e1[0], b * B.e2[0]);
-        yy[j] = fmaf(a, B.e1[1], b * B.e2[1]);
-        yz[j] = fmaf(a, B.e1[2], b * B.e2[2]);
+    for (int q = 0; q < NQ; ++q) {
+        const int j0 = 2 * q, j1 = 2 * q + 1;
+        yx[q] = f2_pack(helm_point(R.sf[j0], R.tf[j0], B, 0), helm_point(R.sf[j1], R.tf[j1], B, 0));
+        yy[q] = f2_pack(helm_point(R.sf[j0], R.tf[j0], B, 1), helm_point(R.sf[j1], R.tf[j1], B, 1));
+        yz[q] = f2_pack(helm_point(R.sf[j0], R.tf[j0], B, 2), helm_point(R.sf[j1], R.tf[j1], B, 2));
+    }
+    float ox = 0.0f, oy = 0.0f, oz = 0.0f;
+    if (NP % 2) {
+        ox = helm_point(R.sf[NP - 1], R.tf[NP - 1], B, 0);
+        oy = helm_point(R.sf[NP - 1], R.tf[NP - 1], B, 1);
+        oz = helm_point(R.sf[NP - 1], R.tf[NP - 1], B, 2);
     }
     float sr = 0.0f, si = 0.0f, cr = 0.0f, ci = 0.0f;
     auto outer = [&](int i) {
-        const float a = R.sf[i] - 0.666666687f, b = R.tf[i] - 0.333333343f;
-        const float xx = fmaf(a, A.e1[0], b * A.e2[0]);
-        const float xy = fmaf(a, A.e1[1], b * A.e2[1]);
-        const float xz = fmaf(a, A.e1[2], b * A.e2[2]);
+        const float xx = helm_point(R.sf[i], R.tf[i], A, 0), xy = helm_point(R.sf[i], R.tf[i], A, 1),
+                    xz = helm_point(R.sf[i], R.tf[i], A, 2);
+        const f32x2 X = f2_dup(xx), Y = f2_dup(xy), Z = f2_dup(xz);
         float ir = 0.0f, ii = 0.0f;
 #pragma unroll
-        for (int j = 0; j < NP; ++j) {
+        for (int q = 0; q < NQ; ++q) {
+            f32x2 ri;
+            float ca, cb, sa, sb, wa, wb;
+            H.at(f2_sub(X, yx[q]), f2_sub(Y, yy[q]), f2_sub(Z, yz[q]), ri, ca, cb, sa, sb);
+            f2_unpack(f2_mul(f2_pack(R.wf[2 * q], R.wf[2 * q + 1]), ri), wa, wb);
+            ir = fmaf(cb, wb, fmaf(ca, wa, ir));
+            ii = fmaf(sb, wb, fmaf(sa, wa, ii));
+        }
+        if (NP % 2) {
             float c, s, ri;
-            helm_offset(P, xx - yx[j], xy - yy[j], xz - yz[j], c, s, ri);
-            const float wr = R.wf[j] * ri;
+            helm_offset(P, xx - ox, xy - oy, xz - oz, c, s, ri);
+            const float wr = R.wf[NP - 1] * ri;
             ir = fmaf(c, wr, ir);
             ii = fmaf(s, wr, ii);
         }
@@ -617,6 +733,93 @@ __device__ __forceinline__ void regular_p0_f32_helm(const TriF &A, const TriF &B
     out_im = im * sc;
 }
 
+// The trial points of a product rule, relative to the trial vertex 0, in packed
+// pairs (an odd rule's last point alone).  The inner loops below were bound by
+// instruction issue (9 to 12 FP32 operations per point), so differences,
+// distances and cubes run two points per instruction; the sums stay scalar and
+// take the points in order, so that every value is the one of the scalar loop.
+// What bounds them now is the FP32 pipe (63 to 73% busy, 128 lanes per SM and
+// cycle whether packed or not).  Piecewise-linear plan of the 20480-triangle
+// sphere, both Laplace layers, nine points: near field 4.64 -> 4.41 ms, coupling
+// 5.43 -> 5.04 ms; double and Helmholtz single layer of eight bodies, piecewise
+// constant: 7.70 -> 7.05 ms.
+template <int NP>
+struct TrialX2 {
+    static constexpr int NQ = NP / 2;
+    f32x2 x[NQ], y[NQ], z[NQ];
+    float ox, oy, oz;
+};
+
+template <int NP>
+__device__ __forceinline__ TrialX2<NP> trial_x2(const TriF &B, const Rule2D &R)
+{
+    TrialX2<NP> T;
+    auto at = [&](f32x2 s, f32x2 t, int c) {
+        return f2_fma(s, f2_dup(B.e1[c]), f2_mul(t, f2_dup(B.e2[c])));
+    };
+#pragma unroll
+    for (int q = 0; q < TrialX2<NP>::NQ; ++q) {
+        const f32x2 s = f2_pack(R.sf[2 * q], R.sf[2 * q + 1]), t = f2_pack(R.tf[2 * q], R.tf[2 * q + 1]);
+        T.x[q] = at(s, t, 0);
+        T.y[q] = at(s, t, 1);
+        T.z[q] = at(s, t, 2);
+    }
+    T.ox = T.oy = T.oz = 0.0f;
+    if (NP % 2) {
+        const float s = R.sf[NP - 1], t = R.tf[NP - 1];
+        T.ox = fmaf(s, B.e1[0], t * B.e2[0]);
+        T.oy = fmaf(s, B.e1[1], t * B.e2[1]);
+        T.oz = fmaf(s, B.e1[2], t * B.e2[2]);
+    }
+    return T;
+}
+
+// f(j, 1/r, 1/r^3) for the trial points j = 0, 1, .. in order, r the distance to x
+template <int NP, class F>
+__device__ __forceinline__ void for_trial(const TrialX2<NP> &T, float xx, float xy, float xz, F f)
+{
+    const f32x2 X = f2_dup(xx), Y = f2_dup(xy), Z = f2_dup(xz);
+#pragma unroll
+    for (int q = 0; q < TrialX2<NP>::NQ; ++q) {
+        const f32x2 dx = f2_sub(X, T.x[q]), dy = f2_sub(Y, T.y[q]), dz = f2_sub(Z, T.z[q]);
+        float r2a, r2b;
+        f2_unpack(f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz))), r2a, r2b);
+        const float ra = rsqrt_fast(r2a), rb = rsqrt_fast(r2b);
+        const f32x2 ri = f2_pack(ra, rb);
+        float ca, cb;
+        f2_unpack(f2_mul(f2_mul(ri, ri), ri), ca, cb);
+        f(2 * q, ra, ca);
+        f(2 * q + 1, rb, cb);
+    }
+    if (NP % 2) {
+        const float dx = xx - T.ox, dy = xy - T.oy, dz = xz - T.oz;
+        const float ri = rsqrt_fast(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        f(NP - 1, ri, ri * ri * ri);
+    }
+}
+
+// f(i, height of test point i) for i = 0, 1, ..; the heights (DLP) two at a time
+template <int KIND, int NP, bool UNROLL, class F>
+__device__ __forceinline__ void for_test(const Height &H, const Rule2D &R, F f)
+{
+    auto two = [&](int i) {
+        float h0 = 0.0f, h1 = 0.0f;
+        if (KIND == BEM_LAPLACE_DLP)
+            f2_unpack(height_at_x2(H, f2_pack(R.sf[i], R.sf[i + 1]), f2_pack(R.tf[i], R.tf[i + 1])), h0, h1);
+        f(i, h0);
+        f(i + 1, h1);
+    };
+    if (UNROLL) {
+#pragma unroll
+        for (int i = 0; i + 1 < NP; i += 2) two(i);
+    } else {
+#pragma unroll 1
+        for (int i = 0; i + 1 < NP; i += 2) two(i);
+    }
+    if (NP % 2)
+        f(NP - 1, KIND == BEM_LAPLACE_DLP ? height_at(H, R.sf[NP - 1], R.tf[NP - 1]) : 0.0f);
+}
+
 // Regular pair, piecewise constant, float (Laplace kernels).  With ABS the
 // double layer also returns in *abs_out the sum of the magnitudes of its terms
 // (the scale of its rounding error, for the cancellation guard).
@@ -624,29 +827,24 @@ template <int KIND, int NP, bool ABS = false>
 __device__ __forceinline__ float regular_p0_f32(const TriF &A, const TriF &B, const Rule2D &R,
                                                 float *abs_out = nullptr)
 {
-    float d0[3], yx[NP], yy[NP], yz[NP];
+    float d0[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) d0[c] = dd_diff(A.vh[0][c], A.vl[0][c], B.vh[0][c], B.vl[0][c]);
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-        yx[j] = fmaf(R.sf[j], B.e1[0], R.tf[j] * B.e2[0]);
-        yy[j] = fmaf(R.sf[j], B.e1[1], R.tf[j] * B.e2[1]);
-        yz[j] = fmaf(R.sf[j], B.e1[2], R.tf[j] * B.e2[2]);
-    }
     Height H = {};
     if (KIND == BEM_LAPLACE_DLP)
         H = make_height(A.vh[0], A.vl[0], A.vh[1], A.vl[1], A.vh[2], A.vl[2], B.vh[0], B.vl[0],
                         B.nh, B.nl);
+    const TrialX2<NP> T = trial_x2<NP>(B, R);
     float sum = 0.0f, comp = 0.0f, asum = 0.0f;
-    auto outer = [&](int i) {
+    // larger rules keep the outer loop rolled (code size)
+    for_test<KIND, NP, (NP <= 9)>(H, R, [&](int i, float dn) {
         const float xx = fmaf(R.sf[i], A.e1[0], fmaf(R.tf[i], A.e2[0], d0[0]));
         const float xy = fmaf(R.sf[i], A.e1[1], fmaf(R.tf[i], A.e2[1], d0[1]));
         const float xz = fmaf(R.sf[i], A.e1[2], fmaf(R.tf[i], A.e2[2], d0[2]));
-        const float dn = KIND == BEM_LAPLACE_DLP ? height_at(H, R.sf[i], R.tf[i]) : 0.0f;
         float inner = 0.0f;
-#pragma unroll
-        for (int j = 0; j < NP; ++j)
-            inner = fmaf(R.wf[j], kvalf_r<KIND>(xx - yx[j], xy - yy[j], xz - yz[j]), inner);
+        for_trial<NP>(T, xx, xy, xz, [&](int j, float ri, float r3) {
+            inner = fmaf(R.wf[j], KIND == BEM_LAPLACE_SLP ? ri : r3, inner);
+        });
         if (ABS) asum = fmaf(R.wf[i], inner * fabsf(dn), asum);
         if (KIND == BEM_LAPLACE_DLP) inner *= dn;
         // compensated outer sum (Kahan)
@@ -654,15 +852,7 @@ __device__ __forceinline__ float regular_p0_f32(const TriF &A, const TriF &B, co
         const float t = sum + y;
         comp = (t - sum) - y;
         sum = t;
-    };
-    // larger rules keep the outer loop rolled (code size)
-    if (NP > 9) {
-#pragma unroll 1
-        for (int i = 0; i < NP; ++i) outer(i);
-    } else {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) outer(i);
-    }
+    });
     if (ABS) *abs_out = asum * (A.sg * B.sg * (float)kInv4Pi);
     return sum * (A.sg * B.sg * (float)kInv4Pi);
 }
@@ -672,38 +862,30 @@ template <int KIND, int NP>
 __device__ __forceinline__ void regular_p1_f32(const TriF &A, const TriF &B, const Rule2D &R,
                                                float *acc)
 {
-    float d0[3], yx[NP], yy[NP], yz[NP];
+    float d0[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) d0[c] = dd_diff(A.vh[0][c], A.vl[0][c], B.vh[0][c], B.vl[0][c]);
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-        yx[j] = fmaf(R.sf[j], B.e1[0], R.tf[j] * B.e2[0]);
-        yy[j] = fmaf(R.sf[j], B.e1[1], R.tf[j] * B.e2[1]);
-        yz[j] = fmaf(R.sf[j], B.e1[2], R.tf[j] * B.e2[2]);
-    }
     Height H = {};
     if (KIND == BEM_LAPLACE_DLP)
         H = make_height(A.vh[0], A.vl[0], A.vh[1], A.vl[1], A.vh[2], A.vl[2], B.vh[0], B.vl[0],
                         B.nh, B.nl);
+    const TrialX2<NP> T = trial_x2<NP>(B, R);
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
     // outer points not unrolled: the unrolled inner loop alone keeps enough
     // independent work, and the loop body stays small in the instruction cache
-#pragma unroll 1
-    for (int i = 0; i < NP; ++i) {
+    for_test<KIND, NP, false>(H, R, [&](int i, float dn) {
         const float xx = fmaf(R.sf[i], A.e1[0], fmaf(R.tf[i], A.e2[0], d0[0]));
         const float xy = fmaf(R.sf[i], A.e1[1], fmaf(R.tf[i], A.e2[1], d0[1]));
         const float xz = fmaf(R.sf[i], A.e1[2], fmaf(R.tf[i], A.e2[2], d0[2]));
-        const float dn = KIND == BEM_LAPLACE_DLP ? height_at(H, R.sf[i], R.tf[i]) : 0.0f;
         // trial moments: sum_j w_j lambda_q(y_j) k(x_i, y_j), weights from the rule
         float ir[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const float k = kvalf_r<KIND>(xx - yx[j], xy - yy[j], xz - yz[j]);
+        for_trial<NP>(T, xx, xy, xz, [&](int j, float ri, float r3) {
+            const float k = KIND == BEM_LAPLACE_SLP ? ri : r3;
             ir[0] = fmaf(R.wl[0][j], k, ir[0]);
             ir[1] = fmaf(R.wl[1][j], k, ir[1]);
             ir[2] = fmaf(R.wl[2][j], k, ir[2]);
-        }
+        });
         if (KIND == BEM_LAPLACE_DLP) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) ir[q] *= dn;
@@ -716,7 +898,7 @@ __device__ __forceinline__ void regular_p1_f32(const TriF &A, const TriF &B, con
                 acc[p * 3 + q] = fmaf(f, ir[q], acc[p * 3 + q]);
             }
         }
-    }
+    });
     const float scale = A.sg * B.sg * (float)kInv4Pi;
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] *= scale;
@@ -931,38 +1113,26 @@ template <int NP>
 __device__ __forceinline__ void regular_p1_f32_fused(const TriF &A, const TriF &B, const Rule2D &R,
                                                      float *acc_s, float *acc_d)
 {
-    float d0[3], yx[NP], yy[NP], yz[NP];
+    float d0[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) d0[c] = dd_diff(A.vh[0][c], A.vl[0][c], B.vh[0][c], B.vl[0][c]);
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-        yx[j] = fmaf(R.sf[j], B.e1[0], R.tf[j] * B.e2[0]);
-        yy[j] = fmaf(R.sf[j], B.e1[1], R.tf[j] * B.e2[1]);
-        yz[j] = fmaf(R.sf[j], B.e1[2], R.tf[j] * B.e2[2]);
-    }
     const Height H = make_height(A.vh[0], A.vl[0], A.vh[1], A.vl[1], A.vh[2], A.vl[2], B.vh[0],
                                  B.vl[0], B.nh, B.nl);
+    const TrialX2<NP> T = trial_x2<NP>(B, R);
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc_s[k] = acc_d[k] = 0.0f;
-#pragma unroll 1
-    for (int i = 0; i < NP; ++i) {
+    for_test<BEM_LAPLACE_DLP, NP, false>(H, R, [&](int i, float dn) {
         const float xx = fmaf(R.sf[i], A.e1[0], fmaf(R.tf[i], A.e2[0], d0[0]));
         const float xy = fmaf(R.sf[i], A.e1[1], fmaf(R.tf[i], A.e2[1], d0[1]));
         const float xz = fmaf(R.sf[i], A.e1[2], fmaf(R.tf[i], A.e2[2], d0[2]));
-        const float dn = height_at(H, R.sf[i], R.tf[i]);
         float is[3] = {0.0f, 0.0f, 0.0f}, id[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const float dx = xx - yx[j], dy = xy - yy[j], dz = xz - yz[j];
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float ri = rsqrt_fast(r2);
-            const float r3 = ri * ri * ri;
+        for_trial<NP>(T, xx, xy, xz, [&](int j, float ri, float r3) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 is[q] = fmaf(R.wl[q][j], ri, is[q]);
                 id[q] = fmaf(R.wl[q][j], r3, id[q]);
             }
-        }
+        });
 #pragma unroll
         for (int q = 0; q < 3; ++q) id[q] *= dn;
 #pragma unroll
@@ -974,7 +1144,7 @@ __device__ __forceinline__ void regular_p1_f32_fused(const TriF &A, const TriF &
                 acc_d[p * 3 + q] = fmaf(f, id[q], acc_d[p * 3 + q]);
             }
         }
-    }
+    });
     const float scale = A.sg * B.sg * (float)kInv4Pi;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
@@ -1534,7 +1704,7 @@ __device__ __forceinline__ void p0_tile(const MeshView &m, const BlockLaunch &L,
         load_trif(m.geomf, bb, B);
         if (KIND == BEM_HELMHOLTZ_SLP) {
             float fr, fi;
-            regular_p0_f32_helm_x2<NP>(A, B, R, L.kappa, fr, fi);
+            regular_p0_f32_helm_x2<NP>(A, B, R, KappaF(L.kappa), fr, fi);
             re = (double)fr;
             im = (double)fi;
         } else if (guard) {

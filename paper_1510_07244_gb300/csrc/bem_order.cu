@@ -687,8 +687,11 @@ __global__ void __launch_bounds__(256) k_learned_compact(MeshView m, BlockLaunch
 
 // Float form, classes whose rule is a product of a 2D rule with at most 25
 // points: one thread per pair with the block engine's pair integrals.
+// CTAs per SM by the rule's registers: left alone, the 25 points take 241 and one CTA.
+constexpr int tp_ctas(int np) { return np <= 4 ? 4 : (np <= 7 ? 3 : 2); }
+
 template <int KIND, int NP>
-__global__ void __launch_bounds__(256) k_learned_eval_tp(MeshView m, const int4 *__restrict__ rec,
+__global__ void __launch_bounds__(256, tp_ctas(NP)) k_learned_eval_tp(MeshView m, const int4 *__restrict__ rec,
                                                          const int64_t *__restrict__ offs, int cls,
                                                          Rule2D R, double kappa, void *out)
 {
@@ -702,7 +705,7 @@ __global__ void __launch_bounds__(256) k_learned_eval_tp(MeshView m, const int4 
         load_trif(m.geomf, Rk.w, B);
         if (KIND == BEM_HELMHOLTZ_SLP) {
             float fr, fi;
-            regular_p0_f32_helm<NP>(A, B, R, kappa, fr, fi);
+            regular_p0_f32_helm<NP>(A, B, R, KappaF(kappa), fr, fi);
             reinterpret_cast<double2 *>(out)[pos] = make_double2((double)fr, (double)fi);
         } else {
             reinterpret_cast<double *>(out)[pos] = (double)regular_p0_f32<KIND, NP>(A, B, R);
@@ -723,7 +726,7 @@ __global__ void __launch_bounds__(256) k_learned_eval_big(MeshView m, const int4
                                                           const int64_t *__restrict__ offs, int cls,
                                                           RuleF<NP> R, double kappa, void *out)
 {
-    static_assert(NP % CH == 0, "chunks must tile the rule");
+    static_assert(NP % CH == 0 && CH % 2 == 0, "chunks of whole pairs must tile the rule");
     constexpr bool CPLX = KIND == BEM_HELMHOLTZ_SLP;
     const int64_t lo = offs[cls], hi = offs[cls + 1];
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
@@ -738,7 +741,7 @@ __global__ void __launch_bounds__(256) k_learned_eval_big(MeshView m, const int4
         Height H = {};
         HelmPhase P;
         if (CPLX) {
-            P = helm_phase(A, B, kappa);
+            P = helm_phase(A, B, KappaF(kappa));
         } else {
 #pragma unroll
             for (int c = 0; c < 3; ++c)
@@ -748,16 +751,19 @@ __global__ void __launch_bounds__(256) k_learned_eval_big(MeshView m, const int4
                                 B.vl[0], B.nh, B.nl);
         }
         const float sh = CPLX ? 0.666666687f : 0.0f, th = CPLX ? 0.333333343f : 0.0f;
+        const HelmX2 HX(P);
         float sr = 0.0f, cr = 0.0f, si = 0.0f, ci = 0.0f;
 #pragma unroll 1
         for (int jc = 0; jc < NP; jc += CH) {
-            float yx[CH], yy[CH], yz[CH];
+            TrialX2<CH> T;
 #pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const float a = R.s[jc + j] - sh, b = R.t[jc + j] - th;
-                yx[j] = fmaf(a, B.e1[0], b * B.e2[0]);
-                yy[j] = fmaf(a, B.e1[1], b * B.e2[1]);
-                yz[j] = fmaf(a, B.e1[2], b * B.e2[2]);
+            for (int q = 0; q < CH / 2; ++q) {
+                const int j = jc + 2 * q;
+                const f32x2 a = f2_pack(R.s[j] - sh, R.s[j + 1] - sh),
+                            b = f2_pack(R.t[j] - th, R.t[j + 1] - th);
+                T.x[q] = f2_fma(a, f2_dup(B.e1[0]), f2_mul(b, f2_dup(B.e2[0])));
+                T.y[q] = f2_fma(a, f2_dup(B.e1[1]), f2_mul(b, f2_dup(B.e2[1])));
+                T.z[q] = f2_fma(a, f2_dup(B.e1[2]), f2_mul(b, f2_dup(B.e2[2])));
             }
 #pragma unroll 1
             for (int i = 0; i < NP; ++i) {
@@ -767,17 +773,21 @@ __global__ void __launch_bounds__(256) k_learned_eval_big(MeshView m, const int4
                 const float xz = fmaf(a, A.e1[2], fmaf(b, A.e2[2], d0[2]));
                 const float dn = KIND == BEM_LAPLACE_DLP ? height_at(H, R.s[i], R.t[i]) : 0.0f;
                 float ir = 0.0f, ii = 0.0f;
+                if (CPLX) {
+                    const f32x2 X = f2_dup(xx), Y = f2_dup(xy), Z = f2_dup(xz);
 #pragma unroll
-                for (int j = 0; j < CH; ++j) {
-                    if (CPLX) {
-                        float c, s, ri;
-                        helm_offset(P, xx - yx[j], xy - yy[j], xz - yz[j], c, s, ri);
-                        const float wr = R.w[jc + j] * ri;
-                        ir = fmaf(c, wr, ir);
-                        ii = fmaf(s, wr, ii);
-                    } else {
-                        ir = fmaf(R.w[jc + j], kvalf_r<KIND>(xx - yx[j], xy - yy[j], xz - yz[j]), ir);
+                    for (int q = 0; q < CH / 2; ++q) {
+                        f32x2 ri;
+                        float ca, cb, sa, sb, wa, wb;
+                        HX.at(f2_sub(X, T.x[q]), f2_sub(Y, T.y[q]), f2_sub(Z, T.z[q]), ri, ca, cb, sa, sb);
+                        f2_unpack(f2_mul(f2_pack(R.w[jc + 2 * q], R.w[jc + 2 * q + 1]), ri), wa, wb);
+                        ir = fmaf(cb, wb, fmaf(ca, wa, ir));
+                        ii = fmaf(sb, wb, fmaf(sa, wa, ii));
                     }
+                } else {
+                    for_trial<CH>(T, xx, xy, xz, [&](int j, float ri, float r3) {
+                        ir = fmaf(R.w[jc + j], KIND == BEM_LAPLACE_SLP ? ri : r3, ir);
+                    });
                 }
                 if (KIND == BEM_LAPLACE_DLP) ir *= dn;
                 // Kahan sums over the (test point, chunk) partial sums
@@ -878,7 +888,7 @@ __global__ void __launch_bounds__(256) k_learned_eval(MeshView m, const int4 *__
                                 B.nh, B.nl);
             float acc = 0.0f, acci = 0.0f;
             HelmPhase P;
-            if (KIND == BEM_HELMHOLTZ_SLP) P = helm_phase(A, B, kappa);
+            if (KIND == BEM_HELMHOLTZ_SLP) P = helm_phase(A, B, KappaF(kappa));
             for (int p = lane; p < np; p += 32) {
                 const float x1 = __ldg(rulef + p), x2 = __ldg(rulef + np + p),
                             y1 = __ldg(rulef + 2 * np + p), y2 = __ldg(rulef + 3 * np + p),
