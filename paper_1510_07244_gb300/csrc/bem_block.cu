@@ -123,12 +123,17 @@ __global__ void __launch_bounds__(1024) k_job_scan(const int64_t *job_total, int
 
 // Capped at 64 registers (four CTAs, 32 warps per SM): the float form's
 // dependent loads (block, cluster, index, geometry) and the FP64 form's integer
-// chains (bem_fixed_pair.cuh) want the warps.  The float Helmholtz pair holds ten
-// packed constants and spills at 64, so it takes three CTAs (2% over four).
-constexpr int p0_ctas(int kind, bool mixed) { return mixed && kind == BEM_HELMHOLTZ_SLP ? 3 : 4; }
+// chains (bem_fixed_pair.cuh) want the warps.  Three CTAs where the packed pairs
+// spill at 64 and the rule is long enough: Helmholtz from 7 points on (9 points,
+// 3072-triangle dense matrix: 0.93 -> 0.88 ms), the single layer's unrolled 9
+// points (0.40 -> 0.365 ms; at 7 points four CTAs are 7% faster).
+constexpr int p0_ctas(int kind, int np, bool mixed)
+{
+    return mixed && ((kind == BEM_HELMHOLTZ_SLP && np > 4) || (kind == BEM_LAPLACE_SLP && np == 9)) ? 3 : 4;
+}
 
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(256, p0_ctas(KIND, MIXED)) k_block_p0(MeshView m, BlockLaunch L,
+__global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_block_p0(MeshView m, BlockLaunch L,
                                                   const __grid_constant__ Rule2D R,
                                                   const int64_t *__restrict__ prefix,
                                                   int *status)
@@ -152,7 +157,7 @@ __global__ void __launch_bounds__(256, p0_ctas(KIND, MIXED)) k_block_p0(MeshView
 // same tile body as the single-list kernels, so the results are identical.
 // ---------------------------------------------------------------------------
 template <int KIND, int NP, bool MIXED>
-__global__ void __launch_bounds__(256, p0_ctas(KIND, MIXED)) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
+__global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
                                                   const int64_t *__restrict__ job_end,
                                                   const __grid_constant__ Rule2D R, int *status)
 {

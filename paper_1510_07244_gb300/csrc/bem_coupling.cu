@@ -25,6 +25,16 @@ namespace {
 
 constexpr int kCouplingThreads = 256;
 
+// CTAs per SM.  The double layer and the fused pair want the registers (two CTAs,
+// 128; the 4-point rules take 100 by themselves: 0 leaves them to it); the
+// single layer's shorter points want the warps (2048-triangle plan, 4 points:
+// 0.21 ms at two CTAs, 0.17 at four; 9 points: 0.305 at two, 0.277 at three, 0.289
+// at four).
+constexpr int coupling_ctas(bool slp, int np)
+{
+    return slp ? (np <= 4 ? 4 : (np <= 9 ? 3 : 2)) : (np <= 4 ? 0 : 2);
+}
+
 // Sum over the product rule of one disjoint pair for the basis functions at
 // local vertices la (test) and the precomputed trial side (T, wy).
 template <int KIND, int NP>
@@ -223,7 +233,7 @@ __device__ __forceinline__ void coupling_tile_fused(const MeshView &m, const Blo
 }
 
 template <int NP>
-__global__ void __launch_bounds__(kCouplingThreads)
+__global__ void __launch_bounds__(kCouplingThreads, coupling_ctas(false, NP))
 k_coupling_p1_fused_batch(const BatchJob *__restrict__ jobs, int n_jobs,
                           const int64_t *__restrict__ job_end, Rule2D R, int *status)
 {
@@ -240,7 +250,7 @@ k_coupling_p1_fused_batch(const BatchJob *__restrict__ jobs, int n_jobs,
 }
 
 template <int KIND, int NP>
-__global__ void __launch_bounds__(kCouplingThreads)
+__global__ void __launch_bounds__(kCouplingThreads, coupling_ctas(KIND == BEM_LAPLACE_SLP, NP))
 k_coupling_p1(MeshView m, BlockLaunch L, Rule2D R, const int64_t *__restrict__ prefix, int *status)
 {
     const int64_t total = L.n_blocks > 0 ? prefix[L.n_blocks - 1] : 0;
@@ -252,7 +262,7 @@ k_coupling_p1(MeshView m, BlockLaunch L, Rule2D R, const int64_t *__restrict__ p
 }
 
 template <int KIND, int NP>
-__global__ void __launch_bounds__(kCouplingThreads)
+__global__ void __launch_bounds__(kCouplingThreads, coupling_ctas(KIND == BEM_LAPLACE_SLP, NP))
 k_coupling_p1_batch(const BatchJob *__restrict__ jobs, int n_jobs,
                     const int64_t *__restrict__ job_end, Rule2D R, int *status)
 {

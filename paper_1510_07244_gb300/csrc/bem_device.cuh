@@ -515,8 +515,8 @@ __device__ __forceinline__ void helm_offset(const HelmPhase &P, float ex, float 
 __device__ __forceinline__ void helm_rotate(const HelmPhase &P, float sr, float si, float &re,
                                             float &im)
 {
-    re = P.c0 * sr - P.s0 * si;
-    im = P.s0 * sr + P.c0 * si;
+    re = fmaf(P.c0, sr, -(P.s0 * si));
+    im = fmaf(P.s0, sr, P.c0 * si);
 }
 
 // helm_offset at two packed offsets: the same operations per point, each rounded
