@@ -251,7 +251,6 @@ int run_guard(bem_ctx *ctx, Mesh *m, const BlockLaunch &L, const bem_quad_desc &
         if (ctx->guard_buf) {
             cudaStreamSynchronize(ctx->stream);
             cudaFree(ctx->guard_buf);
-    cudaFree(ctx->scratch);
             ctx->guard_buf = nullptr;
             ctx->guard_cap = 0;
         }
