@@ -21,7 +21,7 @@ __device__ __forceinline__ bool fx_wave(double kappa, int E, int low, Fx2 &kn, i
     const double hi = kappa * 0.15915494309189535;
     const double lo = fma(kappa, 0.15915494309189535, -hi) + kappa * -9.839338337591243e-18;
     kexp = max(((__double2hiint(hi) >> 20) & 2047) - 1022 + E, low);
-    if (kexp > 20) return false;
+    if (kexp > 20) return false;   // shifts of 4 + kb + kexp stay below 32
     const double up = fx_pow2(62 + E - kexp);
     kn = fx_split(__double2ll_rn(hi * up) + __double2ll_rn(lo * up));
     return true;
@@ -42,7 +42,7 @@ struct FxSum {
         hi = fx_mad(w[0], T.h, hi);
         mid = fx_mad(w[0], T.l, fx_mad(w[1], T.h, mid));
     }
-    __device__ __forceinline__ s64 sum() const { return hi + (mid >> 32); }
+    __device__ __forceinline__ s64 sum() const { return hi + fx_high(mid); }
     __device__ __forceinline__ double value() const { return (double)sum(); }
 };
 
@@ -145,8 +145,8 @@ __device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P)
 // 2^62): a few units of 2^-59 S
 __device__ __forceinline__ s64 fx_point(s64 v0, Fx2 e1, Fx2 e2, const int32_t *s, const int32_t *t)
 {
-    const s64 mid = fx_mad(e1.h, s[1], fx_mad(e1.l, s[0], fx_mad(e2.h, t[1], (s64)e2.l * t[0])));
-    return fx_mad(e1.h, s[0], fx_mad(e2.h, t[0], v0 + (mid >> 32))) << 3;
+    const s64 mid = fx_mad(e1.h, s[1], fx_mad(e1.l, s[0], fx_mad(e2.h, t[1], fx_mad(e2.l, t[0], 0))));
+    return fx_mad(e1.h, s[0], fx_mad(e2.h, t[0], v0 + fx_high(mid))) << 3;
 }
 
 // kb of near pairs from their points: the powers of 1/r of the double layers
@@ -232,7 +232,7 @@ struct FxInner {
         const Fx2 T = fx_split(fx_rinv(r2, kb, flag));     // 2^(62 - kb) S / r
         Fx2 t2, t3;
         if (P3) {
-            const s64 a = fx_mul(T, T) << (HELM ? 2 : 1);  // 2^(62 - 2 kb) (S / r)^2, Laplace 2^(61 - 2 kb)
+            const s64 a = fx_mul_up<(HELM ? 2 : 1)>(T, T);  // 2^(62 - 2 kb) (S / r)^2, Laplace 2^(61 - 2 kb)
             t2 = fx_split(a);
             t3 = fx_split(fx_mul(t2, T));                  // 2^(60 - 3 kb) (S / r)^3, Laplace 2^(59 - 3 kb)
         }
@@ -243,7 +243,7 @@ struct FxInner {
         }
         // kappa r / (2 pi) modulo 1
         const s64 rho = fx_mul_up<4>(fx_split(r2), T);          // 2^(62 - kb) r / S
-        const u64 turn = (u64)fx_mul(fx_split(rho), kn) << shl;
+        const u64 turn = (u64)fx_shl(fx_mul(fx_split(rho), kn), shl);   // shl < 32
         s64 cs, sn;
         fx_sincos(turn, cs, sn);
         const Fx2 c = fx_split(cs), s = fx_split(sn);

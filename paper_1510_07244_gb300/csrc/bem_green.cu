@@ -247,9 +247,9 @@ __device__ __forceinline__ bool green_fixed(const GreenFrame &F, const Tri &T, i
         const Fx2 t3 = fx_split(fx_mul_up<2>(t2, t1));           // 2^(62 - 3 kb) (S / r)^3
         // (x - z).n at 2^60 / S (at most sqrt(3)), times (S / r)^3
         const Fx2 a = fx_split(d[0]), b = fx_split(d[1]), e = fx_split(d[2]);
-        const s64 mid = fx_mad(a.h, N[0].l, fx_mad(a.l, N[0].h, fx_mad(b.h, N[1].l, (s64)b.l * N[1].h))) +
-                        fx_mad(e.h, N[2].l, (s64)e.l * N[2].h);
-        const Fx2 dn = fx_split((fx_mad(a.h, N[0].h, fx_mad(b.h, N[1].h, fx_mad(e.h, N[2].h, mid >> 32)))) << 1);
+        const s64 mid = fx_mad(a.h, N[0].l, fx_mad(a.l, N[0].h, fx_mad(b.h, N[1].l, fx_mad(b.l, N[1].h, 0)))) +
+                        fx_mad(e.h, N[2].l, fx_mad(e.l, N[2].h, 0));
+        const Fx2 dn = fx_split((fx_mad(a.h, N[0].h, fx_mad(b.h, N[1].h, fx_mad(e.h, N[2].h, fx_high(mid))))) << 1);
         const Fx2 h3 = fx_split(fx_mul(t3, dn));                 // 2^(58 - 3 kb) (S / r)^3 dn / S
         const int32_t *w = R.wx[wl][q];
         if (!HELM) {

@@ -161,19 +161,19 @@ __device__ __forceinline__ bool touch_fixed(const MeshView &m, int idx, const in
                     // identical: d1 e1 + d2 e2; edge: d1 e1 + x2 e2 - y2 e2b;
                     // vertex: x1 e1 + x2 e2 - y1 e1b - y2 e2b
                     const Fx2 e1 = ed[0][c], e2 = ed[1][c];
-                    s64 mid = fx_mad(e1.h, u0.l, fx_mad(e1.l, u0.h, fx_mad(e2.h, u1.l, (s64)e2.l * u1.h)));
-                    s64 hi = fx_mad(e1.h, u0.h, (s64)e2.h * u1.h);
+                    s64 mid = fx_mad(e1.h, u0.l, fx_mad(e1.l, u0.h, fx_mad(e2.h, u1.l, fx_mad(e2.l, u1.h, 0))));
+                    s64 hi = fx_mad(e1.h, u0.h, fx_mad(e2.h, u1.h, 0));
                     if (CAS != kIdentical) {
                         const Fx2 e3 = CAS == kEdge ? ed[3][c] : ed[2][c];
-                        mid -= fx_mad(e3.h, u2.l, (s64)e3.l * u2.h);
-                        hi -= (s64)e3.h * u2.h;
+                        mid -= fx_mad(e3.h, u2.l, fx_mad(e3.l, u2.h, 0));
+                        hi -= fx_mad(e3.h, u2.h, 0);
                     }
                     if (CAS == kVertex) {
                         const Fx2 e4 = ed[3][c];
-                        mid -= fx_mad(e4.h, u3.l, (s64)e4.l * u3.h);
-                        hi -= (s64)e4.h * u3.h;
+                        mid -= fx_mad(e4.h, u3.l, fx_mad(e4.l, u3.h, 0));
+                        hi -= fx_mad(e4.h, u3.h, 0);
                     }
-                    v[c] = (hi + (mid >> 32)) << 4;
+                    v[c] = fx_shl(hi + fx_high(mid), 4);
                 }
                 const s64 r2 = fx_norm2(v[0], v[1], v[2]);
                 auto add = [&](int k, int c, Fx2 value) {
@@ -206,8 +206,8 @@ __device__ __forceinline__ bool touch_fixed(const MeshView &m, int idx, const in
                     } else {
                         if (CAS == kVertex) {
                             // height at 2^60 in units of 2^eh
-                            const s64 mid = fx_mad(n1.h, u0.l, fx_mad(n1.l, u0.h, fx_mad(n2.h, u1.l, (s64)n2.l * u1.h)));
-                            const s64 dn = (fx_mad(n1.h, u0.h, fx_mad(n2.h, u1.h, mid >> 32))) << 4;
+                            const s64 mid = fx_mad(n1.h, u0.l, fx_mad(n1.l, u0.h, fx_mad(n2.h, u1.l, fx_mad(n2.l, u1.h, 0))));
+                            const s64 dn = (fx_mad(n1.h, u0.h, fx_mad(n2.h, u1.h, fx_high(mid)))) << 4;
                             t3 = fx_split(fx_mul_up<3>(t3, fx_split(dn)));    // 2^(61 - 3 kb) (S/|v|)^3 dn
                         }
 #pragma unroll
