@@ -219,6 +219,7 @@ struct SupBuildSmem {
     int lists[kMaxDegP1][kTile];
     int list_n[kTile];
     int ntri, bad;
+    P1Scratch work;
 };
 
 __global__ void __launch_bounds__(128) k_build_supports(MeshView m, const int32_t *__restrict__ ptr,
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(128) k_build_supports(MeshView m, const int32_
             __syncthreads();
             continue;
         }
-        p1_support(m, S.rows, n, S.tri, S.cnt, S.off, S.lists, S.list_n, &S.ntri, status);
+        p1_support(m, S.rows, n, S.tri, S.cnt, S.off, S.lists, S.list_n, &S.ntri, S.work);
         for (int k = tid; k < kTile; k += blockDim.x) rec[kSupListN + k] = k < n ? S.list_n[k] : 0;
         for (int k = tid; k < kMaxDegP1 * kTile; k += blockDim.x)
             rec[kSupLists + k] = (&S.lists[0][0])[k];

@@ -1763,84 +1763,85 @@ struct P1Smem {
     int nta, ntb;
 };
 
-__device__ __forceinline__ int pos_in(const int *set, int n, int v)
-{
-    for (int k = 0; k < n; ++k)
-        if (set[k] == v) return k;
-    return -1;
-}
-
-__device__ __forceinline__ int owner_pos(const MeshView &m, int T, const int *set, int n)
-{
-    const int4 tv = __ldg(m.tvid + T);
-    int p = pos_in(set, n, tv.x);
-    int q = pos_in(set, n, tv.y);
-    int r = pos_in(set, n, tv.z);
-    int best = 1 << 30;
-    if (p >= 0) best = min(best, p);
-    if (q >= 0) best = min(best, q);
-    if (r >= 0) best = min(best, r);
-    return best;
-}
-
 // Collect the triangles touching the vertex set `set` (n <= 32): deterministic
-// order (by owner position, then adjacency order), and per vertex the list of
-// (triangle slot << 2 | local index), sorted by slot so that the gather can
-// walk it once across the chunks of triangle rows.
+// order (by owner position, then adjacency order; a triangle's owner is the first
+// position of one of its vertices), and per vertex the list of (triangle slot << 2 |
+// local index), sorted by slot so that the gather can walk it once across the
+// chunks of triangle rows.  The (vertex, adjacent triangle) items are spread over
+// the CTA: owner search, slot search and rank in the sorted list are one item's
+// work each (a thread per vertex, searching three times, took 0.45 ms for the
+// slices of a 20480-triangle sphere).
+struct P1Scratch {
+    int tri[kMaxDegP1][kTile];    // items: triangle k of vertex v
+    int own[kMaxDegP1][kTile];    // its owner, then its key
+    int lo[kTile], deg[kTile];
+};
+
 __device__ __forceinline__ void p1_support(const MeshView &m, const int *set, int n, int *tri, int *cnt,
-                           int *off, int (*lists)[kTile], int *list_n, int *ntri,
-                           int *status)
+                                           int *off, int (*lists)[kTile], int *list_n, int *ntri,
+                                           P1Scratch &W)
 {
     const int tid = threadIdx.x;
-    if (tid < n) {
-        const int v = set[tid];
-        const int lo = __ldg(m.vt_ptr + v), hi = __ldg(m.vt_ptr + v + 1);
+    if (tid < kTile) {
+        int lo = 0, deg = 0;
+        if (tid < n) {
+            const int v = set[tid];
+            lo = __ldg(m.vt_ptr + v);
+            deg = min(__ldg(m.vt_ptr + v + 1) - lo, kMaxDegP1);   // the host refuses more
+            list_n[tid] = deg;
+        }
+        W.lo[tid] = lo;
+        W.deg[tid] = deg;
+    }
+    __syncthreads();
+    const int v = tid & (kTile - 1), lo = W.lo[v], deg = W.deg[v], step = blockDim.x / kTile;
+    for (int k = tid / kTile; k < deg; k += step) {
+        const int T = __ldg(m.vt_tri + lo + k);
+        const int4 tv = __ldg(m.tvid + T);
+        int best = v;
+        for (int u = v; u-- > 0;) {
+            const int w = set[u];
+            if (w == tv.x || w == tv.y || w == tv.z) best = u;
+        }
+        W.tri[k][v] = T;
+        W.own[k][v] = best;
+    }
+    __syncthreads();
+    if (tid < kTile) {
         int c = 0;
-        for (int k = lo; k < hi; ++k)
-            if (owner_pos(m, __ldg(m.vt_tri + k), set, n) == tid) ++c;
+        for (int k = 0; k < deg; ++k) c += W.own[k][tid] == tid;
         cnt[tid] = c;
+        int sum = c;
+#pragma unroll
+        for (int o = 1; o < kTile; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, sum, o);
+            if (tid >= o) sum += x;
+        }
+        off[tid] = sum - c;
+        if (tid == kTile - 1) *ntri = sum;
+        c = sum - c;
+        for (int k = 0; k < deg; ++k)
+            if (W.own[k][tid] == tid) tri[c++] = W.tri[k][tid];
     }
     __syncthreads();
-    if (tid == 0) {
-        int s = 0;
-        for (int k = 0; k < n; ++k) {
-            off[k] = s;
-            s += cnt[k];
-        }
-        *ntri = s;
+    for (int k = tid / kTile; k < deg; k += step) {
+        const int T = W.tri[k][v], q = W.own[k][v];
+        int slot = -1;
+        for (int u = off[q]; u < off[q] + cnt[q]; ++u)
+            if (tri[u] == T) slot = u;
+        const int4 tv = __ldg(m.tvid + T);
+        const int x = set[v];
+        W.own[k][v] = (slot << 2) | (tv.x == x ? 0 : (tv.y == x ? 1 : 2));
     }
     __syncthreads();
-    if (tid < n) {
-        const int v = set[tid];
-        const int lo = __ldg(m.vt_ptr + v), hi = __ldg(m.vt_ptr + v + 1);
-        int c = off[tid];
-        for (int k = lo; k < hi; ++k) {
-            const int T = __ldg(m.vt_tri + k);
-            if (owner_pos(m, T, set, n) == tid) tri[c++] = T;
+    for (int k = tid / kTile; k < deg; k += step) {
+        const int key = W.own[k][v];
+        int rank = 0;
+        for (int u = 0; u < deg; ++u) {
+            const int other = W.own[u][v];
+            rank += other < key || (other == key && u < k);
         }
-    }
-    __syncthreads();
-    if (tid < n) {
-        const int v = set[tid];
-        const int lo = __ldg(m.vt_ptr + v), hi = __ldg(m.vt_ptr + v + 1);
-        for (int k = lo; k < hi; ++k) {
-            const int T = __ldg(m.vt_tri + k);
-            const int q = owner_pos(m, T, set, n);
-            int slot = -1;
-            for (int u = off[q]; u < off[q] + cnt[q]; ++u)
-                if (tri[u] == T) slot = u;
-            const int4 tv = __ldg(m.tvid + T);
-            const int loc = tv.x == v ? 0 : (tv.y == v ? 1 : 2);
-            // insertion into the slot-sorted list (slots are distinct)
-            int u = k - lo;
-            const int key = (slot << 2) | loc;
-            while (u > 0 && lists[u - 1][tid] > key) {
-                lists[u][tid] = lists[u - 1][tid];
-                --u;
-            }
-            lists[u][tid] = key;
-        }
-        list_n[tid] = hi - lo;
+        lists[rank][v] = key;
     }
     __syncthreads();
 }
@@ -1942,8 +1943,11 @@ __device__ __forceinline__ void p1_tile(const MeshView &m, const BlockLaunch &L,
                 return;
             }
         } else {
-            p1_support(m, S.rows, tr, S.ta, S.cnt_r, S.off_r, S.rl, S.rl_n, &S.nta, status);
-            p1_support(m, S.cols, tc, S.tb, S.cnt_c, S.off_c, S.cl, S.cl_n, &S.ntb, status);
+            // scratch in the pair results' buffer, not in use yet
+            P1Scratch &W = *reinterpret_cast<P1Scratch *>(buf_r);
+            static_assert(sizeof(P1Scratch) <= CAP * 9 * sizeof(Val), "scratch fits the pair results");
+            p1_support(m, S.rows, tr, S.ta, S.cnt_r, S.off_r, S.rl, S.rl_n, &S.nta, W);
+            p1_support(m, S.cols, tc, S.tb, S.cnt_c, S.off_c, S.cl, S.cl_n, &S.ntb, W);
             nta = S.nta;
             ntb = S.ntb;
         }

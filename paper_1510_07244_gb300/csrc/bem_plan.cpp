@@ -216,7 +216,7 @@ cudaError_t issue(bem_ctx *ctx, bem_plan *p, cudaStream_t st, bool record_prof,
         }
         ev_begin();
         e = launch_build_supports(s.m, s.ptr, s.idx, s.n, s.slice, s.sup, s.cap, ctx->status,
-                                  ctx->num_sms * 4, st);
+                                  ctx->num_sms * 16, st);
         ev_end();
         if (e != cudaSuccess) return e;
     }
@@ -267,7 +267,7 @@ int autotune(bem_ctx *ctx, bem_plan *p)
         launch_touching_batch(p->touch_jobs, t.basis, t.kind, t.cas, t.mixed, t.items, t.n, t.rule, st);
     for (auto &s : p->sup)
         launch_build_supports(s.m, s.ptr, s.idx, s.n, s.slice, s.sup, s.cap, ctx->status,
-                              ctx->num_sms * 4, st);
+                              ctx->num_sms * 16, st);
     for (auto &bk : p->bb)
         bucket_prefix(ctx, bk, st);
     cudaError_t e = cudaStreamSynchronize(st);
