@@ -85,15 +85,19 @@ __device__ void tile_prefix_cta(const BlockLaunch &L, int tr, int tc, int64_t *p
 __global__ void __launch_bounds__(1024) k_tile_prefix(BlockLaunch L, int tr, int tc,
                                                       int64_t *prefix, int *status)
 {
+    pdl_launch();
     tile_prefix_cta(L, tr, tc, prefix, status, nullptr);
+    pdl_end();
 }
 
 // one CTA per job: per-job block prefix sums and the job's tile total
 __global__ void __launch_bounds__(1024) k_tile_prefix_batch(BatchJob *jobs, int tr, int tc,
                                                             int64_t *job_total, int *status)
 {
+    pdl_launch();
     BatchJob &J = jobs[blockIdx.x];
     tile_prefix_cta(J.L, tr, tc, const_cast<int64_t *>(J.prefix), status, job_total + blockIdx.x);
+    pdl_end();
 }
 
 // inclusive scan of the job totals in tiles of `unit` (single CTA): the
@@ -102,6 +106,8 @@ __global__ void __launch_bounds__(1024) k_job_scan(const int64_t *job_total, int
                                                    int64_t *job_end)
 {
     __shared__ int64_t part[1024];
+    pdl_wait();
+    pdl_launch();
     const int chunk = (n + blockDim.x - 1) / blockDim.x;
     const int lo = threadIdx.x * chunk, hi = min(n, lo + chunk);
     int64_t sum = 0;
@@ -138,6 +144,7 @@ __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_block_p0(Mesh
                                                   const int64_t *__restrict__ prefix,
                                                   int *status)
 {
+    pdl_wait();
     // prefix counts entries; a tile is kP0Tile of them.  Each CTA takes a
     // contiguous run of tiles, so every warp finds its next tile's blocks
     // from the previous one's (flat_entry's hint).
@@ -159,8 +166,13 @@ __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_block_p0(Mesh
 template <int KIND, int NP, bool MIXED>
 __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
                                                   const int64_t *__restrict__ job_end,
-                                                  const __grid_constant__ Rule2D R, int *status)
+                                                  const __grid_constant__ Rule2D R, int *status,
+                                                  int beside)
 {
+    // beside: the kernel before is another such launch, which waited for all that
+    // this one reads before it let this one start; the two share the SMs
+    if (!beside) pdl_wait();
+    pdl_launch();
     // contiguous runs of tiles per CTA (see k_block_p0); the block hint is
     // kept while the run stays in one job
     const int64_t total = n_jobs > 0 ? job_end[n_jobs - 1] : 0;
@@ -178,6 +190,7 @@ __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_batch_p0(cons
         const BatchJob &J = jobs[j];
         p0_tile<KIND, NP, MIXED>(J.m, J.L, R, J.prefix, local, status, hint);
     }
+    if (beside) pdl_end();
 }
 
 // ---------------------------------------------------------------------------
@@ -388,11 +401,10 @@ __global__ void __launch_bounds__(256) k_pivot(MeshView m, const int32_t *__rest
 }
 
 cudaError_t launch_tile_prefix(const BlockLaunch &L, int tr, int tc, int64_t *prefix,
-                               int *status, cudaStream_t st)
+                               int *status, cudaStream_t st, bool chained)
 {
     if (L.n_blocks <= 0) return cudaSuccess;
-    k_tile_prefix<<<1, 1024, 0, st>>>(L, tr, tc, prefix, status);
-    return cudaGetLastError();
+    return launch_chain(chained, 1, 1024, st, k_tile_prefix, L, tr, tc, prefix, status);
 }
 
 // Long block lists over many CTAs: CTA c scans blocks [c K, (c + 1) K) in place
@@ -403,9 +415,11 @@ __global__ void __launch_bounds__(1024) k_tile_prefix_chunk(BlockLaunch L, int t
                                                             int64_t *prefix, int64_t *chunk_total,
                                                             int *status)
 {
+    pdl_launch();
     const int64_t lo = (int64_t)blockIdx.x * kPrefixChunk;
     tile_prefix_range(L, tr, tc, prefix, status, chunk_total + blockIdx.x, lo,
                       min(L.n_blocks, lo + kPrefixChunk));
+    pdl_end();
 }
 
 // CTA c adds the totals of chunks 0 .. c to chunk c + 1
@@ -413,6 +427,8 @@ __global__ void __launch_bounds__(1024) k_tile_prefix_add(BlockLaunch L, int64_t
                                                           const int64_t *__restrict__ chunk_total)
 {
     __shared__ int64_t ws[32];
+    pdl_wait();
+    pdl_launch();
     const int c = blockIdx.x + 1;
     int64_t s = 0;
     for (int k = threadIdx.x; k < c; k += blockDim.x) s += chunk_total[k];
@@ -427,26 +443,28 @@ __global__ void __launch_bounds__(1024) k_tile_prefix_add(BlockLaunch L, int64_t
 }
 
 cudaError_t launch_tile_prefix_wide(const BlockLaunch &L, int tr, int tc, int64_t *prefix,
-                                    int64_t *chunk_total, int *status, cudaStream_t st)
+                                    int64_t *chunk_total, int *status, cudaStream_t st,
+                                    bool chained)
 {
-    if (L.n_blocks <= kPrefixChunk) return launch_tile_prefix(L, tr, tc, prefix, status, st);
+    if (L.n_blocks <= kPrefixChunk) return launch_tile_prefix(L, tr, tc, prefix, status, st, chained);
     const int64_t nch = prefix_chunks(L.n_blocks);
-    k_tile_prefix_chunk<<<(unsigned)nch, 1024, 0, st>>>(L, tr, tc, prefix, chunk_total, status);
-    k_tile_prefix_add<<<(unsigned)(nch - 1), 1024, 0, st>>>(L, prefix, chunk_total);
-    return cudaGetLastError();
+    cudaError_t e = launch_chain(chained, (unsigned)nch, 1024, st, k_tile_prefix_chunk, L, tr, tc,
+                                 prefix, chunk_total, status);
+    if (e == cudaSuccess)
+        e = launch_chain(true, (unsigned)(nch - 1), 1024, st, k_tile_prefix_add, L, prefix,
+                         (const int64_t *)chunk_total);
+    return e;
 }
 
 template <int KIND, int NP, bool MIXED>
 static cudaError_t block_np(const MeshView &m, const BlockLaunch &L, const Rule2D &R,
                             const int64_t *prefix, int *status, int grid, cudaStream_t st)
 {
-    if (m.basis == BEM_P0) {
-        k_block_p0<KIND, NP, MIXED><<<grid, 256, 0, st>>>(m, L, R, prefix, status);
-    } else {
-        return MIXED ? launch_p1_single_mixed(KIND, NP, m, L, R, prefix, status, grid * 2, st)
-                     : launch_p1_single_fp64(KIND, NP, m, L, R, prefix, status, grid, st);
-    }
-    return cudaGetLastError();
+    if (m.basis == BEM_P0)
+        return launch_chain(true, (unsigned)grid, 256, st, k_block_p0<KIND, NP, MIXED>, m, L, R, prefix,
+                            status);
+    return MIXED ? launch_p1_single_mixed(KIND, NP, m, L, R, prefix, status, grid * 2, st)
+                 : launch_p1_single_fp64(KIND, NP, m, L, R, prefix, status, grid, st);
 }
 
 template <int KIND, bool MIXED>
@@ -512,43 +530,43 @@ cudaError_t launch_pivot_entries(const MeshView &m, const int32_t *rows, const i
 
 cudaError_t launch_tile_prefix_batch(BatchJob *jobs, int n_jobs, int tr, int tc, int unit,
                                      int64_t *job_total, int64_t *job_end, int *status,
-                                     cudaStream_t st)
+                                     cudaStream_t st, bool chained)
 {
     if (n_jobs <= 0) return cudaSuccess;
-    k_tile_prefix_batch<<<n_jobs, 1024, 0, st>>>(jobs, tr, tc, job_total, status);
-    k_job_scan<<<1, 1024, 0, st>>>(job_total, n_jobs, unit, job_end);
-    return cudaGetLastError();
+    cudaError_t e = launch_chain(chained, (unsigned)n_jobs, 1024, st, k_tile_prefix_batch, jobs, tr, tc,
+                                 job_total, status);
+    if (e == cudaSuccess)
+        e = launch_chain(true, 1, 1024, st, k_job_scan, (const int64_t *)job_total, n_jobs, unit, job_end);
+    return e;
 }
 
 template <int KIND, int NP, bool MIXED>
 static cudaError_t batch_np(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
-                            const Rule2D &R, int *status, int grid, cudaStream_t st)
+                            const Rule2D &R, int *status, int grid, cudaStream_t st, ChainPos pos)
 {
-    if (basis == BEM_P0) {
-        k_batch_p0<KIND, NP, MIXED><<<grid, 256, 0, st>>>(jobs, n_jobs, job_end, R, status);
-    } else {
-        return MIXED ? launch_p1_batch_mixed(KIND, NP, jobs, n_jobs, job_end, R, status, grid, st)
-                     : launch_p1_batch_fp64(KIND, NP, jobs, n_jobs, job_end, R, status, grid, st);
-    }
-    return cudaGetLastError();
+    if (basis == BEM_P0)
+        return launch_chain(pos != kChainNone, (unsigned)grid, 256, st, k_batch_p0<KIND, NP, MIXED>, jobs,
+                            n_jobs, job_end, R, status, pos == kChainBeside ? 1 : 0);
+    return MIXED ? launch_p1_batch_mixed(KIND, NP, jobs, n_jobs, job_end, R, status, grid, st)
+                 : launch_p1_batch_fp64(KIND, NP, jobs, n_jobs, job_end, R, status, grid, st);
 }
 
 template <int KIND, bool MIXED>
 static cudaError_t batch_kind(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
-                              const Rule2D &R, int *status, int grid, cudaStream_t st)
+                              const Rule2D &R, int *status, int grid, cudaStream_t st, ChainPos pos)
 {
     switch (R.np) {
-    case 4: return batch_np<KIND, 4, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st);
-    case 7: return batch_np<KIND, 7, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st);
-    case 9: return batch_np<KIND, 9, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st);
-    case 16: return batch_np<KIND, 16, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st);
+    case 4: return batch_np<KIND, 4, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+    case 7: return batch_np<KIND, 7, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+    case 9: return batch_np<KIND, 9, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+    case 16: return batch_np<KIND, 16, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
     default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
                                int kind, int mixed, const Rule2D &R, int *status, int grid,
-                               cudaStream_t st)
+                               cudaStream_t st, ChainPos pos)
 {
     if (n_jobs <= 0) return cudaSuccess;
     if (kind == kFusedLaplace)   // piecewise-linear float form only
@@ -557,19 +575,19 @@ cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *
                    : cudaErrorInvalidValue;
     switch (kind) {
     case BEM_LAPLACE_SLP:
-        return mixed ? batch_kind<BEM_LAPLACE_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st)
-                     : batch_kind<BEM_LAPLACE_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st);
+        return mixed ? batch_kind<BEM_LAPLACE_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)
+                     : batch_kind<BEM_LAPLACE_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
     case BEM_LAPLACE_DLP:
-        return mixed ? batch_kind<BEM_LAPLACE_DLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st)
-                     : batch_kind<BEM_LAPLACE_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st);
+        return mixed ? batch_kind<BEM_LAPLACE_DLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)
+                     : batch_kind<BEM_LAPLACE_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
     case BEM_HELMHOLTZ_DLP:   // FP64 in every precision
-        return batch_kind<BEM_HELMHOLTZ_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st);
+        return batch_kind<BEM_HELMHOLTZ_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
     case BEM_HELMHOLTZ_BW:
-        return batch_kind<BEM_HELMHOLTZ_BW, false>(jobs, n_jobs, job_end, basis, R, status, grid, st);
+        return batch_kind<BEM_HELMHOLTZ_BW, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
     default:
         return (mixed && basis == BEM_P0)
-                   ? batch_kind<BEM_HELMHOLTZ_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st)
-                   : batch_kind<BEM_HELMHOLTZ_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st);
+                   ? batch_kind<BEM_HELMHOLTZ_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)
+                   : batch_kind<BEM_HELMHOLTZ_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
     }
 }
 

@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "bem_internal.h"
+#include "bem_pdl.cuh"
 
 namespace bem {
 

@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "bem_internal.h"
+#include "bem_pdl.cuh"
 
 namespace bem {
 
@@ -98,12 +99,6 @@ __device__ __forceinline__ double warp_sum_d(double v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-
-// Programmatic dependent launch: wait for the launch before this one in the
-// stream to finish (all of its writes visible); let the next one start.  Both are
-// no-ops in a plain launch.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 
 constexpr int kH2Warps = 8;
 
@@ -346,23 +341,6 @@ __global__ void __launch_bounds__(256) k_cg_dir(int64_t n, double *scal, const d
 
 __global__ void k_cg_roll(double *scal) { scal[0] = scal[2]; }
 
-// Launch in the stream; PDL: it may start while the launch before it still runs
-// (its kernel waits by itself).
-template <class... P, class... A>
-cudaError_t h2_launch(bool pdl, unsigned grid, cudaStream_t st, void (*k)(P...), A... args)
-{
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(grid);
-    c.blockDim = dim3(256);
-    c.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = at;
-    c.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
-}
-
 cudaError_t matvec(const bem_h2 *h, const double *x, double *y, cudaStream_t st)
 {
     const double *no = nullptr;
@@ -376,28 +354,28 @@ cudaError_t matvec(const bem_h2 *h, const double *x, double *y, cudaStream_t st)
     bool pdl = false;   // the first launch of the chain waits for all earlier work
     for (size_t k = 0; k < h->fwd.size() && e == cudaSuccess; ++k)
         if (h->fwd_n[k] > 0) {
-            e = h2_launch(pdl, (unsigned)h->fwd_n[k], h->side, k_h2_forward, h->nodes, h->fwd[k], h->vals,
+            e = launch_chain(pdl, (unsigned)h->fwd_n[k], 256, h->side, k_h2_forward, h->nodes, h->fwd[k], h->vals,
                           h->src, x, h->xhat);
             pdl = true;
         }
     if (e == cudaSuccess && h->n_near > 0)
-        e = h2_launch(false, warps(h->n_near), st, k_h2_blocks<true>, h->near_blk, h->n_near,
+        e = launch_chain(false, warps(h->n_near), 256, st, k_h2_blocks<true>, h->near_blk, h->n_near,
                       h->near_vals, h->cl_idx, x, h->near_part);
     if (e == cudaSuccess && h->n_far > 0) {
-        e = h2_launch(pdl, warps(h->n_far), h->side, k_h2_blocks<false>, h->far_blk, h->n_far, h->far_vals,
+        e = launch_chain(pdl, warps(h->n_far), 256, h->side, k_h2_blocks<false>, h->far_blk, h->n_far, h->far_vals,
                       noi, h->xhat, h->far_part);
         pdl = true;
     }
     for (size_t k = 0; k + 1 < h->bwd.size() && e == cudaSuccess; ++k)
         if (h->bwd_n[k] > 0) {
-            e = h2_launch(pdl, (unsigned)h->bwd_n[k], h->side, k_h2_backward<false>, h->nodes, h->bwd[k],
+            e = launch_chain(pdl, (unsigned)h->bwd_n[k], 256, h->side, k_h2_backward<false>, h->nodes, h->bwd[k],
                           h->valsT, h->src, h->far_part, no, no, no, h->yhat, y);
             pdl = true;
         }
     if (e == cudaSuccess) e = cudaEventRecord(h->join, h->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->join, 0);
     if (e == cudaSuccess && h->bwd_n.back() > 0)
-        e = h2_launch(false, (unsigned)h->bwd_n.back(), st, k_h2_backward<true>, h->nodes, h->bwd.back(),
+        e = launch_chain(false, (unsigned)h->bwd_n.back(), 256, st, k_h2_backward<true>, h->nodes, h->bwd.back(),
                       h->valsT, h->src, h->far_part, h->near_part, h->diag, x, h->yhat, y);
     return e;
 }

@@ -413,18 +413,21 @@ struct Shape {
 };
 
 cudaError_t launch_tile_prefix(const BlockLaunch &L, int tr, int tc, int64_t *prefix,
-                               int *status, cudaStream_t st);
+                               int *status, cudaStream_t st, bool chained = false);
 // Blocks per CTA of the many-CTA prefix pass, and its chunk count (the
 // chunk_total scratch holds one int64 per chunk).
 constexpr int64_t kPrefixChunk = 8192;
 inline int64_t prefix_chunks(int64_t n_blocks) { return (n_blocks + kPrefixChunk - 1) / kPrefixChunk; }
+// chained (here and below): see bem_pdl.cuh; block kernels of the piecewise-constant
+// basis are always chained to the prefix sums.
 // The same prefix sums as launch_tile_prefix; lists longer than one chunk take
 // two launches over many CTAs.
 cudaError_t launch_tile_prefix_wide(const BlockLaunch &L, int tr, int tc, int64_t *prefix,
-                                    int64_t *chunk_total, int *status, cudaStream_t st);
+                                    int64_t *chunk_total, int *status, cudaStream_t st,
+                                    bool chained = false);
 cudaError_t launch_touching(const MeshView &m, int cas, const int *list, int64_t n,
                             const Rule4D &rule, int kind, double kappa, int f32,
-                            cudaStream_t st, double eta = 0.0);
+                            cudaStream_t st, double eta = 0.0, bool chained = false);
 cudaError_t launch_block_engine(const MeshView &m, const BlockLaunch &L, const Rule2D &rule,
                                 const int64_t *prefix, int *status, int grid, cudaStream_t st);
 size_t p1_smem_bytes(bool cplx, bool mixed, bool fused = false);
@@ -445,7 +448,7 @@ cudaError_t launch_p1_batch_mixed(int kind, int np, const BatchJob *jobs, int n_
 // inclusive scan of the job totals in units of `unit` per tile.
 cudaError_t launch_tile_prefix_batch(BatchJob *jobs, int n_jobs, int tr, int tc, int unit,
                                      int64_t *job_total, int64_t *job_end, int *status,
-                                     cudaStream_t st);
+                                     cudaStream_t st, bool chained = false);
 // bem_coupling.cu: coupling blocks of the piecewise-linear basis, mixed form
 // (Laplace kernels), one entry per lane in warp tiles of 16 rows x 2 columns.
 constexpr int kCouplingRows = 16, kCouplingCols = 2;
@@ -479,13 +482,16 @@ cudaError_t launch_build_supports(const MeshView &m, const int32_t *ptr, const i
                                   int32_t n_clusters, int32_t *slice, int32_t *sup, int64_t cap,
                                   int *status, int grid, cudaStream_t st);
 cudaError_t launch_touching_batch(const TouchJob *jobs, int basis, int kind, int cas, int mixed,
-                                  const int2 *items, int64_t n, const Rule4D &rule, cudaStream_t st);
+                                  const int2 *items, int64_t n, const Rule4D &rule, cudaStream_t st, bool chained = false);
 // Block buckets of many jobs: job_end[j] = tiles of jobs 0..j (inclusive
 // prefix); job_end holds n_jobs + 1 entries, the last one the tile counter of
 // the piecewise-linear tile engine (reset by the launch).
+// Place of a piecewise-constant launch in a chain (bem_pdl.cuh): a plain launch;
+// after the passes that it reads; after another such launch that follows them.
+enum ChainPos { kChainNone, kChainAfter, kChainBeside };
 cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
                                int kind, int mixed, const Rule2D &R, int *status, int grid,
-                               cudaStream_t st);
+                               cudaStream_t st, ChainPos pos = kChainNone);
 cudaError_t launch_pivot_entries(const MeshView &m, const int32_t *rows, const int32_t *cols,
                                  int64_t n, void *out, const Rule4D *rules /*[4]*/, int kind,
                                  double kappa, int *status, cudaStream_t st, bool absolute,

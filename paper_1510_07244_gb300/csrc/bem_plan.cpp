@@ -159,14 +159,15 @@ cudaError_t plan_support(bem_plan *p, const MeshView &m, const int32_t *ptr, con
     return cudaSuccess;
 }
 
-cudaError_t bucket_prefix(bem_ctx *ctx, const BlockBucket &b, cudaStream_t st)
+cudaError_t bucket_prefix(bem_ctx *ctx, const BlockBucket &b, cudaStream_t st, bool chained = false)
 {
     const TileShape ts = block_tile_shape(b.basis, b.coupling);
     return launch_tile_prefix_batch(b.jobs, (int)b.host_jobs.size(), ts.tr, ts.tc, ts.unit,
-                                    b.job_total, b.job_end, ctx->status, st);
+                                    b.job_total, b.job_end, ctx->status, st, chained);
 }
 
-cudaError_t launch_bucket(bem_ctx *ctx, const BlockBucket &b, int mult, cudaStream_t st)
+cudaError_t launch_bucket(bem_ctx *ctx, const BlockBucket &b, int mult, cudaStream_t st,
+                          ChainPos pos = kChainNone)
 {
     if (b.fused && b.coupling)
         return launch_coupling_p1_fused_batch(b.jobs, (int)b.host_jobs.size(), b.job_end, b.r2,
@@ -178,7 +179,7 @@ cudaError_t launch_bucket(bem_ctx *ctx, const BlockBucket &b, int mult, cudaStre
         return launch_coupling_p1_batch(b.jobs, (int)b.host_jobs.size(), b.job_end, b.kind, b.r2,
                                         ctx->status, ctx->num_sms * mult, st);
     return launch_block_batch(b.jobs, (int)b.host_jobs.size(), b.job_end, b.basis, b.kind, b.mixed,
-                              b.r2, ctx->status, ctx->num_sms * mult, st);
+                              b.r2, ctx->status, ctx->num_sms * mult, st, pos);
 }
 
 // Issues the plan's launches on stream st (profiling events when prof != null).
@@ -203,11 +204,18 @@ cudaError_t issue(bem_ctx *ctx, bem_plan *p, cudaStream_t st, bool record_prof,
         if (record_prof) rec(p->prof[pi].b);
         ++pi;
     };
+    // Touching pairs and prefix sums do not depend on one another, and the
+    // piecewise-constant buckets only on them: one chain (bem_pdl.cuh), unless events
+    // go between its launches.  chained: the launch before is a kernel of the chain.
+    bool chained = false;
+    const bool chain = !record_prof;
     for (auto &t : p->tb) {
         ev_begin();
-        e = launch_touching_batch(p->touch_jobs, t.basis, t.kind, t.cas, t.mixed, t.items, t.n, t.rule, st);
+        e = launch_touching_batch(p->touch_jobs, t.basis, t.kind, t.cas, t.mixed, t.items, t.n, t.rule, st,
+                                  chained);
         ev_end();
         if (e != cudaSuccess) return e;
+        chained = chained || (chain && t.n > 0);
     }
     for (auto &s : p->sup) {
         if (!structure) {
@@ -219,6 +227,7 @@ cudaError_t issue(bem_ctx *ctx, bem_plan *p, cudaStream_t st, bool record_prof,
                                   ctx->num_sms * 16, st);
         ev_end();
         if (e != cudaSuccess) return e;
+        chained = false;
     }
     for (auto &b : p->bb) {
         if (!structure) {
@@ -226,15 +235,19 @@ cudaError_t issue(bem_ctx *ctx, bem_plan *p, cudaStream_t st, bool record_prof,
             continue;
         }
         ev_begin();
-        e = bucket_prefix(ctx, b, st);
+        e = bucket_prefix(ctx, b, st, chained);
         ev_end();
         if (e != cudaSuccess) return e;
+        chained = chained || (chain && !b.host_jobs.empty());
     }
+    ChainPos pos = chained ? kChainAfter : kChainNone;
     for (auto &b : p->bb) {
+        const bool p0 = b.basis == BEM_P0;
         ev_begin();
-        e = launch_bucket(ctx, b, b.grid_mult, st);
+        e = launch_bucket(ctx, b, b.grid_mult, st, p0 ? pos : kChainNone);
         ev_end();
         if (e != cudaSuccess) return e;
+        if (!b.host_jobs.empty()) pos = p0 && chain ? kChainBeside : kChainNone;
     }
     for (auto &l : p->learned) {
         ev_begin();

@@ -45,9 +45,11 @@ __global__ void __launch_bounds__(256) k_touching(const __grid_constant__ MeshVi
                                                   int64_t n, TouchRuleDev R, double kappa,
                                                   double eta, const __grid_constant__ XiFixed X)
 {
+    pdl_launch();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= n) return;
     touch_fp64<KIND, BASIS, CAS>(m, __ldg(list + wid), R, kappa, threadIdx.x & 31, eta, X);
+    pdl_end();
 }
 
 // Batched: items[k] = (job, touching index) over many meshes / kernels.
@@ -57,11 +59,13 @@ __global__ void __launch_bounds__(256) k_touching_batch(const TouchJob *__restri
                                                         TouchRuleDev R,
                                                         const __grid_constant__ XiFixed X)
 {
+    pdl_launch();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= n) return;
     const int2 it = items[wid];
     touch_fp64<KIND, BASIS, CAS>(jobs[it.x].m, it.y, R, jobs[it.x].kappa, threadIdx.x & 31,
                                  jobs[it.x].eta, X);
+    pdl_end();
 }
 
 // Float kernels: a pair per group of LPP lanes (touch_f32).  The first group
@@ -72,12 +76,14 @@ __global__ void __launch_bounds__(256) k_touching_f32(MeshView m, const int *__r
                                                       int64_t n, const float *__restrict__ rule,
                                                       int np, float kappa, int xi, XiRule xr)
 {
+    pdl_launch();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t g = t / LPP;
     if ((t >> 5) * (32 / LPP) >= n) return;   // the warp's first group
     const bool valid = g < n;
     touch_f32<CAS, KIND, BASIS, LPP>(m, __ldg(list + (valid ? g : n - 1)), rule, np,
                                      (int)(t % LPP), kappa, xi, xr, valid);
+    pdl_end();
 }
 
 template <int CAS, int KIND, int BASIS, int LPP>
@@ -87,6 +93,7 @@ __global__ void __launch_bounds__(256) k_touching_f32_batch(const TouchJob *__re
                                                             const float *__restrict__ rule, int np,
                                                             int xi, XiRule xr)
 {
+    pdl_launch();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t g = t / LPP;
     if ((t >> 5) * (32 / LPP) >= n) return;
@@ -94,6 +101,7 @@ __global__ void __launch_bounds__(256) k_touching_f32_batch(const TouchJob *__re
     const int2 it = items[valid ? g : n - 1];
     touch_f32<CAS, KIND, BASIS, LPP>(jobs[it.x].m, it.y, rule, np, (int)(t % LPP),
                                      (float)jobs[it.x].kappa, xi, xr, valid);
+    pdl_end();
 }
 
 // Lanes per pair of the float kernels: the xi-integrated Laplace rules are
@@ -109,7 +117,7 @@ static int lanes_per_pair(const Rule4D &rule, int kind, int basis)
 
 cudaError_t launch_touching(const MeshView &m, int cas, const int *list, int64_t n,
                             const Rule4D &rule, int kind, double kappa, int f32, cudaStream_t st,
-                            double eta)
+                            double eta, bool chained)
 {
     if (n <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((n + 7) / 8);
@@ -121,9 +129,9 @@ cudaError_t launch_touching(const MeshView &m, int cas, const int *list, int64_t
 #define BEM_TVL(K, B, LP)                                                                       \
     do {                                                                                        \
         const unsigned g = (unsigned)((n + 8 * (32 / LP) - 1) / (8 * (32 / LP)));               \
-        if (cas == kIdentical) k_touching_f32<kIdentical, K, B, LP><<<g, 256, 0, st>>>(m, list, n, rule.f, rule.n, kf, rule.xi, xr); \
-        else if (cas == kEdge) k_touching_f32<kEdge, K, B, LP><<<g, 256, 0, st>>>(m, list, n, rule.f, rule.n, kf, rule.xi, xr);      \
-        else k_touching_f32<kVertex, K, B, LP><<<g, 256, 0, st>>>(m, list, n, rule.f, rule.n, kf, rule.xi, xr);                      \
+        if (cas == kIdentical) return launch_chain(chained, g, 256, st, k_touching_f32<kIdentical, K, B, LP>, m, list, n, rule.f, rule.n, kf, rule.xi, xr); \
+        else if (cas == kEdge) return launch_chain(chained, g, 256, st, k_touching_f32<kEdge, K, B, LP>, m, list, n, rule.f, rule.n, kf, rule.xi, xr);      \
+        else return launch_chain(chained, g, 256, st, k_touching_f32<kVertex, K, B, LP>, m, list, n, rule.f, rule.n, kf, rule.xi, xr);                      \
     } while (0)
 #define BEM_TV(K, B)                                                                            \
     do {                                                                                        \
@@ -142,7 +150,7 @@ cudaError_t launch_touching(const MeshView &m, int cas, const int *list, int64_t
     }
     XiFixed xf;
     if (rule.xi && kind_complex(kind) && !make_xi_fixed(rule.q, xf)) return cudaErrorInvalidValue;
-#define BEM_TOUCH(K, B, C) k_touching<K, B, C><<<blocks, 256, 0, st>>>(m, list, n, rule_dev(rule, B), kappa, eta, xf)
+#define BEM_TOUCH(K, B, C) return launch_chain(chained, blocks, 256, st, k_touching<K, B, C>, m, list, n, rule_dev(rule, B), kappa, eta, xf)
 #define BEM_TOUCH_CASE(K, B)                                   \
     do {                                                       \
         if (cas == kIdentical) BEM_TOUCH(K, B, kIdentical);    \
@@ -162,7 +170,8 @@ cudaError_t launch_touching(const MeshView &m, int cas, const int *list, int64_t
 }
 
 cudaError_t launch_touching_batch(const TouchJob *jobs, int basis, int kind, int cas, int f32,
-                                  const int2 *items, int64_t n, const Rule4D &rule, cudaStream_t st)
+                                  const int2 *items, int64_t n, const Rule4D &rule, cudaStream_t st,
+                                  bool chained)
 {
     if (n <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((n + 7) / 8);
@@ -173,9 +182,9 @@ cudaError_t launch_touching_batch(const TouchJob *jobs, int basis, int kind, int
 #define BEM_TVBL(K, B, LP)                                                                      \
     do {                                                                                        \
         const unsigned g = (unsigned)((n + 8 * (32 / LP) - 1) / (8 * (32 / LP)));               \
-        if (cas == kIdentical) k_touching_f32_batch<kIdentical, K, B, LP><<<g, 256, 0, st>>>(jobs, items, n, rule.f, rule.n, rule.xi, xr); \
-        else if (cas == kEdge) k_touching_f32_batch<kEdge, K, B, LP><<<g, 256, 0, st>>>(jobs, items, n, rule.f, rule.n, rule.xi, xr);      \
-        else k_touching_f32_batch<kVertex, K, B, LP><<<g, 256, 0, st>>>(jobs, items, n, rule.f, rule.n, rule.xi, xr);                      \
+        if (cas == kIdentical) return launch_chain(chained, g, 256, st, k_touching_f32_batch<kIdentical, K, B, LP>, jobs, items, n, rule.f, rule.n, rule.xi, xr); \
+        else if (cas == kEdge) return launch_chain(chained, g, 256, st, k_touching_f32_batch<kEdge, K, B, LP>, jobs, items, n, rule.f, rule.n, rule.xi, xr);      \
+        else return launch_chain(chained, g, 256, st, k_touching_f32_batch<kVertex, K, B, LP>, jobs, items, n, rule.f, rule.n, rule.xi, xr);                      \
     } while (0)
 #define BEM_TVB(K, B)                                                                           \
     do {                                                                                        \
@@ -194,7 +203,7 @@ cudaError_t launch_touching_batch(const TouchJob *jobs, int basis, int kind, int
     }
     XiFixed xf;
     if (rule.xi && kind_complex(kind) && !make_xi_fixed(rule.q, xf)) return cudaErrorInvalidValue;
-#define BEM_TB(K, B, C) k_touching_batch<K, B, C><<<blocks, 256, 0, st>>>(jobs, items, n, rule_dev(rule, B), xf)
+#define BEM_TB(K, B, C) return launch_chain(chained, blocks, 256, st, k_touching_batch<K, B, C>, jobs, items, n, rule_dev(rule, B), xf)
 #define BEM_TB_CASE(K, B)                                  \
     do {                                                   \
         if (cas == kIdentical) BEM_TB(K, B, kIdentical);   \

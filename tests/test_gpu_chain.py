@@ -1,0 +1,111 @@
+"""GPU: launches that overlap in one stream, and the support records of the
+piecewise-linear engine.
+
+- Calls in a row without a synchronisation between them, each overwriting the
+  touching table and the tile prefix sums that the one before still reads, give
+  the bits of the same calls with a synchronisation after each; so does a plan
+  of the same jobs, run twice, with and without a graph.
+- Clusters of 1, 31, 32, 33 and 40 vertices in shuffled order over a bipyramid
+  whose apexes have the largest degree (16): blocks of the single call and of a
+  plan against the entry kernel, which takes no supports.  Both are FP64 sums of
+  the same at most 16 * 16 * 6 * 5^4 terms of one sign (single layer): 1e-11 of
+  the entry bounds their rounding."""
+import numpy as np
+import pytest
+
+import synth
+from parity_util import block_job, to_dev
+from test_gpu_h2 import env  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+QUAD = dict(q_regular=3, regular_rule="duffy", q_identical=5, q_edge=4, q_vertex=3)
+
+
+def _all_pairs(ptr, idx):
+    nc = len(ptr) - 1
+    t, s = (a.ravel().astype(np.int32) for a in np.meshgrid(np.arange(nc), np.arange(nc), indexing="ij"))
+    size = np.diff(ptr)[t].astype(np.int64) * np.diff(ptr)[s]
+    off = np.concatenate([[0], np.cumsum(size)]).astype(np.int64)
+    return synth.workloads.BlockSet(ptr, idx, ptr, idx, t, s, off[:-1], int(off[-1]))
+
+
+@pytest.mark.parametrize("basis,precision", [("p0", "fp64"), ("p0", "mixed_full"), ("p1", "mixed_full")])
+def test_calls_in_a_row(env, basis, precision):  # noqa: F811
+    import torch
+    pkg, ctx = env
+    mesh = synth.jitter(synth.icosphere(2), 0.05, 5)
+    n = mesh.nt if basis == "p0" else mesh.nv
+    cuts = np.unique(np.concatenate([np.arange(0, n, 29), [n]])).astype(np.int32)
+    bs = _all_pairs(cuts, np.random.default_rng(2).permutation(n).astype(np.int32))
+    mid = ctx.bem_mesh_upload(mesh.verts, mesh.tris, basis)
+    kinds = ["laplace_slp", "laplace_dlp", "laplace_slp", "laplace_dlp"]
+    quads = [dict(QUAD, precision=precision), dict(QUAD, precision=precision, q_regular=2)]
+
+    def jobs():
+        return [block_job(pkg, mid, bs, k, 0.0, quads[i // 2],
+                          torch.zeros(bs.n_entries, dtype=torch.float64, device="cuda"))
+                for i, k in enumerate(kinds)]
+
+    alone, row = jobs(), jobs()
+    for j in alone:
+        ctx.bem_near_field([j])
+        ctx.bem_sync()
+    for _ in range(3):
+        for j in row:
+            ctx.bem_near_field([j])
+    ctx.bem_sync()
+    for a, b in zip(alone, row):
+        assert torch.equal(a.out, b.out)
+    for flags in (0, pkg.PLAN_GRAPH):
+        planned = jobs()
+        plan = ctx.bem_plan_create(planned, [], flags)
+        for _ in range(2):
+            for j in planned:
+                j.out.zero_()
+            torch.cuda.synchronize()
+            ctx.bem_plan_run(plan)
+            ctx.bem_plan_run(plan)
+            ctx.bem_sync()
+            for a, b in zip(alone, planned):
+                assert torch.equal(a.out, b.out)
+        ctx.bem_plan_destroy(plan)
+    ctx.bem_mesh_free(mid)
+
+
+@pytest.mark.parametrize("planned", [False, True])
+def test_supports(env, planned):  # noqa: F811
+    import torch
+    pkg, ctx = env
+    a = 2.0 * np.pi * np.arange(16) / 16.0
+    levels = [(0.6, -0.5), (1.0, 0.0), (0.7, 0.45)]
+    verts = [[r * np.cos(x), r * np.sin(x), z] for r, z in levels for x in a] + [[0, 0, -0.9], [0, 0, 0.8]]
+    tris = []
+    for k in range(16):
+        m = (k + 1) % 16
+        tris += [[48, m, k], [49, 32 + k, 32 + m]]
+        for l in (0, 16):
+            tris += [[l + k, l + m, l + 16 + m], [l + k, l + 16 + m, l + 16 + k]]
+    verts, tris = np.array(verts, np.float64), np.array(tris, np.int32)
+    rng = np.random.default_rng(9)
+    sets = [rng.permutation(50)[:k] for k in (1, 31, 32, 33, 40)] + [np.array([49, 48])]
+    ptr = np.concatenate([[0], np.cumsum([len(s) for s in sets])]).astype(np.int32)
+    bs = _all_pairs(ptr, np.concatenate(sets).astype(np.int32))
+    mid = ctx.bem_mesh_upload(verts, tris, "p1")
+    out = torch.zeros(bs.n_entries, dtype=torch.float64, device="cuda")
+    job = block_job(pkg, mid, bs, "laplace_slp", 0.0, QUAD, out)
+    if planned:
+        plan = ctx.bem_plan_create([job], [], pkg.PLAN_GRAPH)
+        ctx.bem_plan_run(plan)
+        ctx.bem_sync()
+        ctx.bem_plan_destroy(plan)
+    else:
+        ctx.bem_near_field([job])
+    rows, cols = bs.entry_indices()
+    ref = torch.zeros_like(out)
+    ctx.bem_pivot_entries(mid, pkg.kernel_desc("laplace_slp", 0.0), pkg.quad_desc(**QUAD),
+                          to_dev(rows, torch.int32), to_dev(cols, torch.int32), ref)
+    ctx.bem_sync()
+    ctx.bem_mesh_free(mid)
+    assert float(ref.min()) > 0.0
+    assert float(((out - ref).abs() / ref).max()) <= 1e-11
