@@ -132,10 +132,11 @@ __global__ void __launch_bounds__(1024) k_job_scan(const int64_t *job_total, int
 // chains (bem_fixed_pair.cuh) want the warps.  Three CTAs where the packed pairs
 // spill at 64 and the rule is long enough: Helmholtz from 7 points on (9 points,
 // 3072-triangle dense matrix: 0.93 -> 0.88 ms), the single layer's unrolled 9
-// points (0.40 -> 0.365 ms; at 7 points four CTAs are 7% faster).
+// points (0.40 -> 0.35 ms; at 7 points four CTAs are 7% faster), the 16 points of
+// every kernel (double layer 1.34 -> 1.17 ms).
 constexpr int p0_ctas(int kind, int np, bool mixed)
 {
-    return mixed && ((kind == BEM_HELMHOLTZ_SLP && np > 4) || (kind == BEM_LAPLACE_SLP && np == 9)) ? 3 : 4;
+    return mixed && ((kind == BEM_HELMHOLTZ_SLP && np > 4) || (kind == BEM_LAPLACE_SLP && np == 9) || np == 16) ? 3 : 4;
 }
 
 template <int KIND, int NP, bool MIXED>

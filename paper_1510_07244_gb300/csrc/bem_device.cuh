@@ -1585,13 +1585,16 @@ __device__ __forceinline__ BlockInfo block_info(const BlockLaunch &L, const int6
 // ---------------------------------------------------------------------------
 // Entry threadIdx.x of flat tile `tile` of a block list (prefix = inclusive
 // entry counts per block): its triangle pair (a, b) and output position.
-// Each warp finds the blocks of its 32 entries by itself (no CTA barrier):
-// one search for the block of its first entry, then the inclusive sums of the
-// 32 blocks from there, one per lane; an entry's block is the first of them
-// whose sum exceeds it (a search over the lanes by shuffles), unless more than
-// 32 of the blocks are empty.  Every lane of a warp whose first entry lies
-// within the list must call this (shuffles); ok = false past the list's end
-// and for invalid blocks or indices (these set the status word).
+// Each warp finds the blocks of its 32 entries by itself (no CTA barrier), from
+// the inclusive sums of 32 blocks, one per lane.  The sums that fall within the
+// warp's entries are bits of one word, so an entry's block is a population count
+// and its place in the block a leading-zero count: about 90 instructions (230
+// with a search over the lanes by 64-bit shuffles and a 64-bit division, a tenth
+// of a float double-layer pair and half of a learned-order compaction step).  Empty
+// blocks among the 32 (two sums on one bit), or a window that does not reach the
+// last entry, take a search per entry.  Every lane of a warp whose first entry
+// lies within the list must call this (warp votes); ok = false past the list's
+// end and for invalid blocks or indices (these set the status word).
 struct FlatEntry {
     bool ok;
     int a, b;        // test and trial triangle
@@ -1600,8 +1603,8 @@ struct FlatEntry {
 
 // hint (warp-uniform, in and out): a block index at or before the block of the
 // warp's first entry, from the warp's previous tile of the same list (-1:
-// none).  Tiles taken in increasing order then find their first block after a
-// step or two forward instead of a binary search.
+// none).  Tiles taken in increasing order then find their blocks in the window
+// from there, without a search.
 __device__ __forceinline__ FlatEntry flat_entry(const MeshView &m, const BlockLaunch &L,
                                                 const int64_t *__restrict__ prefix, int64_t tile,
                                                 int *status, int64_t &hint)
@@ -1616,37 +1619,34 @@ __device__ __forceinline__ FlatEntry flat_entry(const MeshView &m, const BlockLa
     const int64_t total = prefix[L.n_blocks - 1];
     if (ew >= total) return fe;   // the whole warp
     const int64_t e = ew + lane;
-    int64_t b0 = -1;
-    if (hint >= 0 && hint < L.n_blocks) {
-        int64_t h = hint;
-        for (int step = 0; step < 8 && h < L.n_blocks - 1 && prefix[h] <= ew; ++step) ++h;
-        if (prefix[h] > ew && (h == 0 || prefix[h - 1] <= ew)) b0 = h;
+    // window: lane j holds the end of block hint - 1 + j relative to ew, cut to [0, 32]
+    int64_t end = 0;
+    int rel = 0;
+    unsigned within = 0;          // lanes whose sum is at most ew
+    bool reach = false;
+    for (int step = 0; step < 2 && !reach; ++step) {
+        if (hint < 0 || step > 0) hint = find_block(prefix, L.n_blocks, ew);
+        const int64_t j = hint - 1 + lane;
+        end = j < 0 ? 0 : (j < L.n_blocks ? prefix[j] : INT64_MAX);
+        rel = end <= ew ? 0 : (int)min(end - ew, (int64_t)32);
+        within = __ballot_sync(0xffffffffu, rel == 0);
+        reach = (within & 1u) && __any_sync(0xffffffffu, rel == 32);
     }
-    if (b0 < 0) b0 = find_block(prefix, L.n_blocks, ew);
-    hint = b0;
-    const int64_t pw = b0 + lane < L.n_blocks ? prefix[b0 + lane] : INT64_MAX;
-    const int64_t p_before = b0 > 0 ? prefix[b0 - 1] : 0;
-    // k = first window slot with a sum above e (32 if none); six steps
-    // narrow [0, 32] to one slot, every lane shuffling in every step
-    int lo = 0, hi = 32;
-#pragma unroll
-    for (int step = 0; step < 6; ++step) {
-        const int mid = (lo + hi) >> 1;
-        const int64_t v = __shfl_sync(0xffffffffu, pw, mid & 31);
-        if (lo < hi) {
-            if (v > e) hi = mid;
-            else lo = mid + 1;
-        }
-    }
-    const int k = lo;
-    const int64_t p_prev = __shfl_sync(0xffffffffu, pw, k > 0 ? k - 1 : 0);
-    int64_t b, before;
-    if (k < 32) {
-        b = b0 + k;
-        before = k > 0 ? p_prev : p_before;
+    const bool in = rel > 0 && rel < 32;
+    const unsigned bits = __reduce_or_sync(0xffffffffu, in ? 1u << rel : 0u);
+    const int first = __popc(within);   // slots before the first entry's block, plus one
+    const bool plain = reach && __popc(bits) == __popc(__ballot_sync(0xffffffffu, in));
+    int64_t b, le;
+    if (plain) {
+        const int64_t base = __shfl_sync(0xffffffffu, ew - end, first - 1);
+        const unsigned mine = bits & (0xffffffffu >> (31 - lane));
+        hint += first - 1;
+        b = hint + __popc(mine);
+        le = mine ? lane - (31 - __clz(mine)) : base + lane;
     } else {
-        b = find_block(prefix, L.n_blocks, e);
-        before = b > 0 ? prefix[b - 1] : 0;
+        hint = find_block(prefix, L.n_blocks, ew);
+        b = find_block(prefix, L.n_blocks, min(e, total - 1));
+        le = e - (b > 0 ? prefix[b - 1] : 0);
     }
     if (e >= total) return fe;
     const int t = L.blk_row[b], s = L.blk_col[b];
@@ -1656,12 +1656,12 @@ __device__ __forceinline__ FlatEntry flat_entry(const MeshView &m, const BlockLa
     }
     const int r_lo = L.row_ptr[t], nr = L.row_ptr[t + 1] - r_lo;
     const int c_lo = L.col_ptr[s], nc = L.col_ptr[s + 1] - c_lo;
-    const int64_t le = e - before;
     if (le < 0 || nr <= 0 || le >= (int64_t)nr * nc) {   // the prefix and the blocks disagree
         set_status(status, BEM_ERR_INVALID_ARG);
         return fe;
     }
-    const int c = (int)(le / nr), r = (int)(le - (int64_t)c * nr);
+    const int c = le >> 32 ? (int)(le / nr) : (int)((unsigned)le / (unsigned)nr);
+    const int r = (int)(le - (int64_t)c * nr);
     fe.a = L.row_idx[r_lo + r];
     fe.b = L.col_idx[c_lo + c];
     if (fe.a < 0 || fe.a >= m.nt || fe.b < 0 || fe.b >= m.nt) {

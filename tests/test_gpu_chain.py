@@ -109,3 +109,39 @@ def test_supports(env, planned):  # noqa: F811
     ctx.bem_mesh_free(mid)
     assert float(ref.min()) > 0.0
     assert float(((out - ref).abs() / ref).max()) <= 1e-11
+
+
+@pytest.mark.parametrize("sizes", [
+    [1] * 90,                                   # many blocks of one entry
+    [3, 0, 0, 5, 1, 0, 17, 0, 2, 33, 0, 0],     # empty blocks between, and at the end
+    [0] * 40 + [7] + [0] * 70 + [9, 40],        # runs of empty blocks longer than a window
+    [320],                                      # one block
+    [16, 16, 31, 32, 33, 64],
+])
+def test_flat_entries(env, sizes):  # noqa: F811
+    """Entries of block lists with small, empty and large blocks, taken by a
+    single call and by a plan, against the entry kernel: both are FP64 forms of
+    the same sums (81 terms of one sign, or one touching rule), 1e-11 of the entry."""
+    import torch
+    pkg, ctx = env
+    mesh = synth.jitter(synth.icosphere(2), 0.05, 7)
+    rng = np.random.default_rng(len(sizes))
+    ptr = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    idx = rng.integers(0, mesh.nt, ptr[-1]).astype(np.int32)
+    bs = _all_pairs(ptr, idx)
+    mid = ctx.bem_mesh_upload(mesh.verts, mesh.tris, "p0")
+    outs = [torch.zeros(bs.n_entries, dtype=torch.float64, device="cuda") for _ in range(2)]
+    jobs = [block_job(pkg, mid, bs, "laplace_slp", 0.0, QUAD, o) for o in outs]
+    ctx.bem_near_field([jobs[0]])
+    plan = ctx.bem_plan_create([jobs[1]], [], pkg.PLAN_GRAPH)
+    ctx.bem_plan_run(plan)
+    ctx.bem_sync()
+    ctx.bem_plan_destroy(plan)
+    rows, cols = bs.entry_indices()
+    ref = torch.zeros_like(outs[0])
+    ctx.bem_pivot_entries(mid, pkg.kernel_desc("laplace_slp", 0.0), pkg.quad_desc(**QUAD),
+                          to_dev(rows, torch.int32), to_dev(cols, torch.int32), ref)
+    ctx.bem_sync()
+    ctx.bem_mesh_free(mid)
+    for o in outs:
+        assert float(((o - ref).abs() / ref).max()) <= 1e-11
