@@ -480,6 +480,8 @@ int bem_destroy(bem_ctx *ctx)
     cudaFree(ctx->tile_prefix);
     cudaFree(ctx->guard_buf);
     cudaFree(ctx->scratch);
+    cudaFreeHost(ctx->solve_host);
+    if (ctx->solve_read) cudaEventDestroy(ctx->solve_read);
     learned_free(ctx->learned);
     delete ctx;
     return BEM_OK;

@@ -184,6 +184,8 @@ struct bem_ctx {
     size_t guard_cap = 0;
     void *scratch = nullptr;               // scratch of one solver or potential call, grown to the largest
     size_t scratch_cap = 0;
+    double *solve_host = nullptr;          // page-locked: a solver step's coefficients (16 KB, at the first solve)
+    cudaEvent_t solve_read = nullptr;      // they are there
     int num_sms = 0;
     std::map<int, bem::Mesh *> meshes;
     int next_mesh = 1;

@@ -10,10 +10,10 @@
 //                      system (A + diag(d)) x = b: Arnoldi with classical
 //                      Gram-Schmidt applied twice, Givens rotations on the host.
 //                      The matrix-vector product (column-major A, 32-row tiles
-//                      times column ranges) and both projections run in kernels
-//                      one after the other; each Arnoldi step reads its projection
+//                      times column ranges) and both projections run in a chain of
+//                      overlapping launches; each Arnoldi step reads its projection
 //                      coefficients and the new vector's norm back once (a few
-//                      hundred bytes).
+//                      hundred bytes), beside the next step's product.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -174,24 +174,31 @@ __global__ void __launch_bounds__(256) k_potential_sum(const double2 *__restrict
     if (lane == 0) out[p] = make_double2(ar, ai);
 }
 
+// The kernels of one Arnoldi step run as a chain of dependent launches
+// (bem_pdl.cuh), 7 us apart at most instead of a launch each (n = 2048, 36 steps,
+// with the kernels below: 111 -> 62 us per step).
+
 // Partial products of y = A x, A column-major n x n complex: CTA (r, s) takes the
 // 32 rows of tile r and the columns [s per, (s + 1) per), one row per lane, every
 // 8th column per warp; the warps' sums are added in order into part[s n + row].
 // FP64-bound (four FMAs per 16-byte entry, 2 lanes per SM and cycle: 29 us for
-// n = 2048); one thread per row and all columns kept 8 CTAs busy there.
-__global__ void __launch_bounds__(256) k_zgemv_part(int64_t n, int64_t per,
+// n = 2048).  About eight CTAs per SM, so that the last ones leave little idle (two
+// per SM: 44 us, eight: 37).
+__global__ void __launch_bounds__(256) k_zgemv_part(int64_t n, int64_t per, unsigned tiles,
                                                     const double2 *__restrict__ A,
-                                                    const double2 *__restrict__ x, double2 *part)
+                                                    const double2 *x, double2 *part)
 {
     __shared__ double2 ws[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
-    const int64_t j0 = (int64_t)blockIdx.y * per, j1 = min(n, j0 + per);
+    const int64_t r = blockIdx.x % tiles, s = blockIdx.x / tiles, i = r * 32 + lane;
+    const int64_t j0 = s * per, j1 = min(n, j0 + per);
+    pdl_wait();
+    pdl_launch();
     double ar = 0.0, ai = 0.0;
     if (i < n) {
 #pragma unroll 8
         for (int64_t j = j0 + warp; j < j1; j += 8) {
-            const double2 a = __ldg(A + i + j * n), v = __ldg(x + j);
+            const double2 a = __ldg(A + i + j * n), v = x[j];
             ar = fma(a.x, v.x, fma(-a.y, v.y, ar));
             ai = fma(a.x, v.y, fma(a.y, v.x, ai));
         }
@@ -199,79 +206,125 @@ __global__ void __launch_bounds__(256) k_zgemv_part(int64_t n, int64_t per,
     ws[warp][lane] = make_double2(ar, ai);
     __syncthreads();
     if (warp == 0 && i < n) {
-        double2 s = ws[0][lane];
+        double2 s2 = ws[0][lane];
 #pragma unroll
         for (int k = 1; k < 8; ++k) {
-            s.x += ws[k][lane].x;
-            s.y += ws[k][lane].y;
+            s2.x += ws[k][lane].x;
+            s2.y += ws[k][lane].y;
         }
-        part[(int64_t)blockIdx.y * n + i] = s;
+        part[s * n + i] = s2;
     }
 }
 
-// y = sum of the ns partial products + diag(d) x
-__global__ void __launch_bounds__(128) k_zgemv_sum(int64_t n, int ns, const double2 *__restrict__ part,
-                                                   const double2 *__restrict__ d,
-                                                   const double2 *__restrict__ x, double2 *y)
+// Sum over 8 warps of the lanes' values, in warp order (warp 0 has the result)
+__device__ __forceinline__ double2 sum_warps(double2 v, double2 (*ws)[32])
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double ar = 0.0, ai = 0.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    ws[warp][lane] = v;
+    __syncthreads();
+    double2 s = ws[0][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+        s.x += ws[k][lane].x;
+        s.y += ws[k][lane].y;
+    }
+    return s;
+}
+
+// y = sum of the ns partial products + diag(d) x: 32 rows per CTA, every 8th
+// partial product per warp
+__global__ void __launch_bounds__(256) k_zgemv_sum(int64_t n, int ns, const double2 *part,
+                                                   const double2 *__restrict__ d, const double2 *x,
+                                                   double2 *y)
+{
+    __shared__ double2 ws[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    pdl_wait();
+    pdl_launch();
+    double2 v = make_double2(0.0, 0.0);
+    if (i < n) {
 #pragma unroll 4
-    for (int s = 0; s < ns; ++s) {
-        const double2 v = part[(int64_t)s * n + i];
-        ar += v.x;
-        ai += v.y;
+        for (int s = warp; s < ns; s += 8) {
+            const double2 a = part[(int64_t)s * n + i];
+            v.x += a.x;
+            v.y += a.y;
+        }
     }
+    v = sum_warps(v, ws);
+    if (warp > 0 || i >= n) return;
     if (d) {
-        const double2 a = d[i], v = x[i];
-        ar += a.x * v.x - a.y * v.y;
-        ai += a.x * v.y + a.y * v.x;
+        const double2 a = d[i], u = x[i];
+        v.x += a.x * u.x - a.y * u.y;
+        v.y += a.x * u.y + a.y * u.x;
     }
-    y[i] = make_double2(ar, ai);
+    y[i] = v;
 }
 
 // h_k = <V_k, w> = sum_i conj(V[i, k]) w_i for k < kk (V column-major n x ld):
-// one block per k, fixed reduction order
-__global__ void __launch_bounds__(256) k_project(int64_t n, const double2 *__restrict__ V,
-                                                 const double2 *__restrict__ w, double2 *h)
+// one block per k, fixed reduction order (lanes, then warps)
+__global__ void __launch_bounds__(256) k_project(int64_t n, const double2 *V, const double2 *w, double2 *h)
 {
-    __shared__ double sr[256], si[256];
+    __shared__ double2 ws[8];
     const int k = blockIdx.x;
     const double2 *v = V + (int64_t)k * n;
+    pdl_wait();
+    pdl_launch();
     double ar = 0.0, ai = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < n; i += 256) {
         const double2 a = v[i], b = w[i];
         ar = fma(a.x, b.x, fma(a.y, b.y, ar));
         ai = fma(a.x, b.y, fma(-a.y, b.x, ai));
     }
-    sr[threadIdx.x] = ar;
-    si[threadIdx.x] = ai;
+    ar = warp_sum(ar);
+    ai = warp_sum(ai);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = make_double2(ar, ai);
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) {
-            sr[threadIdx.x] += sr[threadIdx.x + o];
-            si[threadIdx.x] += si[threadIdx.x + o];
+    if (threadIdx.x == 0) {
+        double2 s = ws[0];
+#pragma unroll
+        for (int u = 1; u < 8; ++u) {
+            s.x += ws[u].x;
+            s.y += ws[u].y;
         }
-        __syncthreads();
+        h[k] = s;
     }
-    if (threadIdx.x == 0) h[k] = make_double2(sr[0], si[0]);
 }
 
-// w -= V h (the first kk columns)
-__global__ void __launch_bounds__(64) k_subtract(int64_t n, int kk, const double2 *__restrict__ V,
-                                                 const double2 *__restrict__ h, double2 *w)
+// w -= V h (the first kk columns): 32 rows per CTA, every 8th column per warp (one
+// thread per row ran a chain of kk loads and products: 18 us at kk = 36, n = 2048).
+// sq: also the CTA's part of |w|^2.
+__global__ void __launch_bounds__(256) k_subtract(int64_t n, int kk, const double2 *V, const double2 *h,
+                                                  double2 *w, double *sq)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double ar = w[i].x, ai = w[i].y;
-#pragma unroll 8
-    for (int k = 0; k < kk; ++k) {
-        const double2 a = V[i + (int64_t)k * n], b = h[k];
-        ar -= a.x * b.x - a.y * b.y;
-        ai -= a.x * b.y + a.y * b.x;
+    __shared__ double2 ws[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    pdl_wait();
+    pdl_launch();
+    double2 v = make_double2(0.0, 0.0);
+    if (i < n) {
+#pragma unroll 4
+        for (int k = warp; k < kk; k += 8) {
+            const double2 a = V[i + (int64_t)k * n], b = h[k];
+            v.x = fma(a.x, b.x, fma(-a.y, b.y, v.x));
+            v.y = fma(a.x, b.y, fma(a.y, b.x, v.y));
+        }
     }
-    w[i] = make_double2(ar, ai);
+    v = sum_warps(v, ws);
+    if (warp > 0) return;
+    double q = 0.0;
+    if (i < n) {
+        const double2 a = w[i];
+        v = make_double2(a.x - v.x, a.y - v.y);
+        w[i] = v;
+        q = v.x * v.x + v.y * v.y;
+    }
+    if (sq) {
+        q = warp_sum(q);
+        if (lane == 0) sq[blockIdx.x] = q;
+    }
 }
 
 // w = b - w
@@ -292,15 +345,29 @@ __global__ void __launch_bounds__(256) k_scale(int64_t n, double sr, double si,
     v[i] = make_double2(sr * a.x - si * a.y, sr * a.y + si * a.x);
 }
 
-// v = w / |w| with |w|^2 = norm2[0] (real part); nothing for a zero vector
-__global__ void __launch_bounds__(256) k_normalise(int64_t n, const double2 *__restrict__ norm2,
-                                                   const double2 *__restrict__ w, double2 *v)
+// v = w / |w|, |w|^2 = the sum of the np parts in sq, also left in norm2 (real
+// part); nothing for a zero vector
+__global__ void __launch_bounds__(256) k_normalise(int64_t n, int np, const double *sq, double2 *norm2,
+                                                   const double2 *w, double2 *v)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const double s = sqrt(fmax(norm2->x, 0.0));
+    __shared__ double ws[8];
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    pdl_wait();
+    pdl_launch();
+    double q = 0.0;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < np; k += 256) q += sq[k];
+    const double2 a = i < n ? w[i] : make_double2(0.0, 0.0);
+    q = warp_sum(q);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = q;
+    __syncthreads();
+    q = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q += ws[k];
+    if (i == 0) *norm2 = make_double2(q, 0.0);
+    const double s = sqrt(fmax(q, 0.0));
     if (i >= n || !(s > 0.0)) return;
     const double f = 1.0 / s;
-    const double2 a = w[i];
     v[i] = make_double2(f * a.x, f * a.y);
 }
 
@@ -401,27 +468,38 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
     const double2 *db = reinterpret_cast<const double2 *>(b);
     double2 *dx = reinterpret_cast<double2 *>(x);
     const int m = restart;
-    // column ranges of the product: enough CTAs for two per SM, at least 64 columns each
+    // column ranges of the product: about eight CTAs per SM, at least 64 columns each
     const unsigned tiles = (unsigned)((n + 31) / 32);
-    int64_t ns = std::max<int64_t>(1, std::min<int64_t>((2 * ctx->num_sms + tiles - 1) / tiles, n / 64));
+    int64_t ns = std::max<int64_t>(1, std::min<int64_t>((8 * ctx->num_sms + tiles / 2) / tiles, n / 64));
     const int64_t per = (n + ns - 1) / ns;
     ns = (n + per - 1) / per;
-    // scratch: V (restart + 1 vectors), w, the partial products, and the projection
-    // coefficients of one step (both passes, then the squared norm)
+    // scratch: V (restart + 1 vectors), w, the partial products, the projection
+    // coefficients of one step (both passes, then the squared norm), parts of the norm
     const size_t nh = 2 * (size_t)(m + 1) + 1;
-    int rc = api_ensure_scratch(ctx, sizeof(double2) * ((size_t)n * (m + 2 + ns) + nh));
+    int rc = api_ensure_scratch(ctx, sizeof(double2) * ((size_t)n * (m + 2 + ns) + nh + tiles));
     if (rc) return rc;
+    if (!ctx->solve_host &&
+        (cudaMallocHost((void **)&ctx->solve_host, sizeof(double2) * (2 * 501 + 1)) != cudaSuccess ||
+         cudaEventCreateWithFlags(&ctx->solve_read, cudaEventDisableTiming) != cudaSuccess)) {
+        cudaFreeHost(ctx->solve_host);
+        ctx->solve_host = nullptr;
+        return api_cuda_fail(ctx, cudaGetLastError(), "bem_dense_gmres");
+    }
+    const double2 *hh = reinterpret_cast<const double2 *>(ctx->solve_host);
     double2 *V = reinterpret_cast<double2 *>(ctx->scratch), *w = V + (size_t)n * (m + 1);
     double2 *part = w + n, *h = part + (size_t)n * ns;
+    double *sq = reinterpret_cast<double *>(h + nh);
     cudaError_t e = cudaSuccess;
     auto done = [&](int code) {
         cudaStreamSynchronize(st);
         return code;
     };
-    const unsigned g = grid_of(n), gs = (unsigned)((n + 63) / 64);
-    auto product = [&](const double2 *v, double2 *y) {
-        k_zgemv_part<<<dim3(tiles, (unsigned)ns), 256, 0, st>>>(n, per, dA, v, part);
-        k_zgemv_sum<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(n, (int)ns, part, dd, v, y);
+    const unsigned g = grid_of(n);
+    auto product = [&](const double2 *v, double2 *y) -> cudaError_t {
+        cudaError_t ee = launch_chain(false, (unsigned)(tiles * ns), 256, st, k_zgemv_part, n, per, tiles,
+                                      dA, v, part);
+        if (ee != cudaSuccess) return ee;
+        return launch_chain(true, tiles, 256, st, k_zgemv_sum, n, (int)ns, (const double2 *)part, dd, v, y);
     };
     // |b|
     auto norm = [&](const double2 *v, double &out) -> cudaError_t {
@@ -439,10 +517,10 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
     int it = 0;
     double res = bn > 0.0 ? 1.0 : 0.0;
     std::vector<cplx> H((size_t)(m + 1) * m), cs(m), sn(m), gvec(m + 1), hk(m + 2);
-    std::vector<double2> hh(nh);
     while (it < maxit && res > tol && bn > 0.0) {
         // r = b - (A + D) x (into w), beta = |r|, V_0 = r / beta
-        product(dx, w);
+        e = product(dx, w);
+        if (e != cudaSuccess) return done(api_cuda_fail(ctx, e, "bem_dense_gmres"));
         k_residual<<<g, 256, 0, st>>>(n, db, w);
         double beta = 0.0;
         e = norm(w, beta);
@@ -453,19 +531,30 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
         std::fill(gvec.begin(), gvec.end(), cplx(0.0));
         gvec[0] = beta;
         int k = 0;
+        e = product(V, w);
         for (; k < m && it < maxit; ++k, ++it) {
-            product(V + (size_t)k * n, w);
             // classical Gram-Schmidt, twice, the norm of what is left and the next
             // vector; the coefficients and the norm come back in one copy
-            for (int pass = 0; pass < 2; ++pass) {
-                k_project<<<k + 1, 256, 0, st>>>(n, V, w, h + pass * (k + 1));
-                k_subtract<<<gs, 64, 0, st>>>(n, k + 1, V, h + pass * (k + 1), w);
+            const int kk = k + 1;
+            for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+                double2 *hp = h + pass * kk;
+                e = launch_chain(true, (unsigned)kk, 256, st, k_project, n, (const double2 *)V,
+                                 (const double2 *)w, hp);
+                if (e == cudaSuccess)
+                    e = launch_chain(true, tiles, 256, st, k_subtract, n, kk, (const double2 *)V,
+                                     (const double2 *)hp, w, pass ? sq : (double *)nullptr);
             }
-            k_project<<<1, 256, 0, st>>>(n, w, w, h + 2 * (k + 1));
-            k_normalise<<<g, 256, 0, st>>>(n, h + 2 * (k + 1), w, V + (size_t)(k + 1) * n);
-            e = cudaMemcpyAsync(hh.data(), h, sizeof(double2) * (size_t)(2 * (k + 1) + 1),
-                                cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e == cudaSuccess)
+                e = launch_chain(true, g, 256, st, k_normalise, n, (int)tiles, (const double *)sq, h + 2 * kk,
+                                 (const double2 *)w, V + (size_t)kk * n);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(ctx->solve_host, h, sizeof(double2) * (size_t)(2 * kk + 1),
+                                    cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaEventRecord(ctx->solve_read, st);
+            // the next step's product runs while the host reads this step's
+            // coefficients (after the last step it is not used)
+            if (e == cudaSuccess && kk < m && it + 1 < maxit) e = product(V + (size_t)kk * n, w);
+            if (e == cudaSuccess) e = cudaEventSynchronize(ctx->solve_read);
             if (e != cudaSuccess) return done(api_cuda_fail(ctx, e, "bem_dense_gmres"));
             for (int i = 0; i <= k; ++i) {
                 hk[i] = cplx(hh[i].x, hh[i].y);

@@ -145,3 +145,27 @@ def test_flat_entries(env, sizes):  # noqa: F811
     ctx.bem_mesh_free(mid)
     for o in outs:
         assert float(((o - ref).abs() / ref).max()) <= 1e-11
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 70, 257])
+@pytest.mark.parametrize("restart", [1, 3, 40])
+def test_gmres_sizes(env, n, restart):  # noqa: F811
+    """Dense GMRES at sizes around the kernels' tiles (32 rows, 64 columns) and at
+    restarts after one, a few and all steps, against a direct solve.  |A - 3 I| is
+    below 0.5 in the spectral norm, so the condition number is below 1.5 and a
+    residual of 1e-12 bounds the error by 1.5e-12 of |x|."""
+    import torch
+    pkg, ctx = env
+    rng = np.random.default_rng(n)
+    A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+    A = 3.0 * np.eye(n) + 0.45 * A / np.linalg.norm(A, 2)
+    b = rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    x = torch.empty(n, dtype=torch.complex128, device="cuda")
+    it, res = ctx.bem_dense_gmres(to_dev(A.T.ravel(), torch.complex128), to_dev(b, torch.complex128), x,
+                                  tol=1e-12, restart=restart, maxit=200)
+    ref = np.linalg.solve(A, b)
+    assert res <= 1e-12 and 0 < it < 200
+    assert np.linalg.norm(x.cpu().numpy() - ref) <= 3e-12 * np.linalg.norm(ref)
+    _, res = ctx.bem_dense_gmres(to_dev(A.T.ravel(), torch.complex128), to_dev(b, torch.complex128), x,
+                                 tol=1e-300, restart=restart, maxit=2)
+    assert np.isfinite(x.cpu().numpy()).all()
