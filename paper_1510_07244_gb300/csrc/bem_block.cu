@@ -16,6 +16,7 @@
 // Kernel values (Eq. 2): laplace 1/(4 pi r), double layer (x-y).n_y/(4 pi r^3),
 // helmholtz exp(i kappa r)/(4 pi r).  sqrt(g_a g_b)/(4 pi) is applied once per
 // pair.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "bem_device.cuh"
@@ -23,7 +24,10 @@
 namespace bem {
 
 // Tiles per block of blocks [first, end) -> inclusive prefix sums from `first`
-// (one CTA, a contiguous run of blocks per thread).
+// (one CTA, a contiguous run of blocks per thread).  CLUSTER: the CTAs of the
+// cluster hold consecutive ranges of one list, whose sums run on over them; *total
+// is the list's, written by the last.
+template <bool CLUSTER = false>
 __device__ void tile_prefix_range(const BlockLaunch &L, int tr, int tc, int64_t *prefix,
                                   int *status, int64_t *total, int64_t first, int64_t end)
 {
@@ -69,9 +73,19 @@ __device__ void tile_prefix_range(const BlockLaunch &L, int tr, int tc, int64_t 
         part[threadIdx.x] += v;
         __syncthreads();
     }
-    const int64_t base = threadIdx.x > 0 ? part[threadIdx.x - 1] : 0;
+    int64_t base = threadIdx.x > 0 ? part[threadIdx.x - 1] : 0, before = 0;
+    bool last = true;
+    if (CLUSTER) {
+        auto cluster = cooperative_groups::this_cluster();
+        cluster.sync();
+        for (unsigned r = 0; r < cluster.block_rank(); ++r)
+            before += cluster.map_shared_rank(part, r)[blockDim.x - 1];
+        last = cluster.block_rank() == cluster.num_blocks() - 1;
+        cluster.sync();   // the others' sums stay until everyone has read them
+    }
+    base += before;
     for (int64_t b = lo; b < hi; ++b) prefix[b] += base;
-    if (total && threadIdx.x == blockDim.x - 1) *total = part[threadIdx.x];
+    if (total && last && threadIdx.x == blockDim.x - 1) *total = before + part[threadIdx.x];
     __syncthreads();
 }
 
@@ -90,7 +104,22 @@ __global__ void __launch_bounds__(1024) k_tile_prefix(BlockLaunch L, int tr, int
     pdl_end();
 }
 
-// one CTA per job: per-job block prefix sums and the job's tile total
+// Per-job block prefix sums and the job's tile total: a cluster of eight CTAs per
+// job, for jobs of more than kPrefixCluster blocks (16 jobs of up to 40000 blocks:
+// 75 us with one CTA each)
+__global__ void __cluster_dims__(8) __launch_bounds__(1024) k_tile_prefix_cluster(BatchJob *jobs, int tr, int tc,
+                                                                                  int64_t *job_total,
+                                                                                  int *status)
+{
+    pdl_launch();
+    BatchJob &J = jobs[blockIdx.x / 8];
+    const int64_t n = J.L.n_blocks, per = (n + 7) / 8, lo = min(n, (int64_t)(blockIdx.x % 8) * per);
+    tile_prefix_range<true>(J.L, tr, tc, const_cast<int64_t *>(J.prefix), status, job_total + blockIdx.x / 8,
+                            lo, min(n, lo + per));
+    pdl_end();
+}
+
+// one CTA per job
 __global__ void __launch_bounds__(1024) k_tile_prefix_batch(BatchJob *jobs, int tr, int tc,
                                                             int64_t *job_total, int *status)
 {
@@ -531,11 +560,14 @@ cudaError_t launch_pivot_entries(const MeshView &m, const int32_t *rows, const i
 
 cudaError_t launch_tile_prefix_batch(BatchJob *jobs, int n_jobs, int tr, int tc, int unit,
                                      int64_t *job_total, int64_t *job_end, int *status,
-                                     cudaStream_t st, bool chained)
+                                     cudaStream_t st, int64_t max_blocks, bool chained)
 {
     if (n_jobs <= 0) return cudaSuccess;
-    cudaError_t e = launch_chain(chained, (unsigned)n_jobs, 1024, st, k_tile_prefix_batch, jobs, tr, tc,
-                                 job_total, status);
+    cudaError_t e = max_blocks > kPrefixCluster
+                        ? launch_chain(chained, 8 * (unsigned)n_jobs, 1024, st, k_tile_prefix_cluster, jobs, tr,
+                                       tc, job_total, status)
+                        : launch_chain(chained, (unsigned)n_jobs, 1024, st, k_tile_prefix_batch, jobs, tr, tc,
+                                       job_total, status);
     if (e == cudaSuccess)
         e = launch_chain(true, 1, 1024, st, k_job_scan, (const int64_t *)job_total, n_jobs, unit, job_end);
     return e;

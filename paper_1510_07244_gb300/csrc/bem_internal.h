@@ -450,7 +450,10 @@ cudaError_t launch_p1_batch_mixed(int kind, int np, const BatchJob *jobs, int n_
 // inclusive scan of the job totals in units of `unit` per tile.
 cudaError_t launch_tile_prefix_batch(BatchJob *jobs, int n_jobs, int tr, int tc, int unit,
                                      int64_t *job_total, int64_t *job_end, int *status,
-                                     cudaStream_t st, bool chained = false);
+                                     cudaStream_t st, int64_t max_blocks, bool chained = false);
+// blocks of a job from which a cluster of CTAs sums it (below, one CTA is done in
+// the time the cluster's two barriers take)
+constexpr int64_t kPrefixCluster = 4096;
 // bem_coupling.cu: coupling blocks of the piecewise-linear basis, mixed form
 // (Laplace kernels), one entry per lane in warp tiles of 16 rows x 2 columns.
 constexpr int kCouplingRows = 16, kCouplingCols = 2;

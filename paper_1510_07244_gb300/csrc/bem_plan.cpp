@@ -162,8 +162,10 @@ cudaError_t plan_support(bem_plan *p, const MeshView &m, const int32_t *ptr, con
 cudaError_t bucket_prefix(bem_ctx *ctx, const BlockBucket &b, cudaStream_t st, bool chained = false)
 {
     const TileShape ts = block_tile_shape(b.basis, b.coupling);
+    int64_t most = 0;
+    for (const BatchJob &j : b.host_jobs) most = std::max(most, j.L.n_blocks);
     return launch_tile_prefix_batch(b.jobs, (int)b.host_jobs.size(), ts.tr, ts.tc, ts.unit,
-                                    b.job_total, b.job_end, ctx->status, st, chained);
+                                    b.job_total, b.job_end, ctx->status, st, most, chained);
 }
 
 cudaError_t launch_bucket(bem_ctx *ctx, const BlockBucket &b, int mult, cudaStream_t st,
