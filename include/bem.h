@@ -334,8 +334,7 @@ int bem_learned_counts(bem_ctx *ctx, int64_t *counts /* [6] */);
  * model must stay alive until bem_plan_destroy.  Its scratch is sized from
  * the job's tile count at creation; its results equal bem_near_field's.
  * The cancellation guard below covers fixed-order jobs only.
- * In the float forms a piecewise-linear Laplace single-layer job and a
- * double-layer job of the same kind (both near field or both coupling) with
+ * A piecewise-linear Laplace single-layer job and a double-layer job of the same kind (both near field or both coupling) with
  * the same mesh, the same block-list pointers and the same regular rule,
  * order and precision run fused: one launch evaluates both layers and shares
  * the points, distances and reciprocal square roots (Eq. 1 for both kernels

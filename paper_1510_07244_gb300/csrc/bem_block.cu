@@ -602,10 +602,11 @@ cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *
                                cudaStream_t st, ChainPos pos)
 {
     if (n_jobs <= 0) return cudaSuccess;
-    if (kind == kFusedLaplace)   // piecewise-linear float form only
-        return (basis == BEM_P1 && mixed)
-                   ? launch_p1_batch_mixed(kFusedLaplace, R.np, jobs, n_jobs, job_end, R, status, grid, st)
-                   : cudaErrorInvalidValue;
+    if (kind == kFusedLaplace) {   // piecewise-linear basis only
+        if (basis != BEM_P1) return cudaErrorInvalidValue;
+        return mixed ? launch_p1_batch_mixed(kFusedLaplace, R.np, jobs, n_jobs, job_end, R, status, grid, st)
+                     : launch_p1_batch_fp64(kFusedLaplace, R.np, jobs, n_jobs, job_end, R, status, grid, st);
+    }
     switch (kind) {
     case BEM_LAPLACE_SLP:
         return mixed ? batch_kind<BEM_LAPLACE_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)

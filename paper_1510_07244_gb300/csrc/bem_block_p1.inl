@@ -106,6 +106,7 @@ cudaError_t batch_kind(int kind, const BatchJob *jobs, int n_jobs, const int64_t
 #if !BEM_P1_MIXED
     if (kind == BEM_HELMHOLTZ_DLP) return batch<BEM_HELMHOLTZ_DLP, NP>(jobs, n_jobs, job_end, R, status, grid, st);
     if (kind == BEM_HELMHOLTZ_BW) return batch<BEM_HELMHOLTZ_BW, NP>(jobs, n_jobs, job_end, R, status, grid, st);
+    if (kind == kFusedLaplace) return batch<kFusedLaplace, NP>(jobs, n_jobs, job_end, R, status, grid, st);
     return batch<BEM_HELMHOLTZ_SLP, NP>(jobs, n_jobs, job_end, R, status, grid, st);
 #else
     if (kind == kFusedLaplace) return batch<kFusedLaplace, NP>(jobs, n_jobs, job_end, R, status, grid, st);

@@ -1529,6 +1529,14 @@ __device__ __forceinline__ void regular_p1(const Tri &A, const Tri &B, const Rul
         double_p1<KIND>(A, B, R, kappa, accr, acci, eta);
 }
 
+// One layer of a pair that fixed_p1_fused leaves
+template <int KIND, int NP>
+__device__ __noinline__ void layer_p1(const Tri &A, const Tri &B, const Rule2D &R, double *acc)
+{
+    double im[9];
+    regular_p1<KIND, NP>(A, B, R, 0.0, acc, im, 0.0);
+}
+
 // ---------------------------------------------------------------------------
 // Block bookkeeping
 // ---------------------------------------------------------------------------
@@ -1983,7 +1991,15 @@ __device__ __forceinline__ void p1_tile(const MeshView &m, const BlockLaunch &L,
                             vi[q] = FUSED ? (Val)L.table2[(int64_t)k * 9 + q].x : (Val)t.y;
                         }
                     }
-                } else if (FUSED) {
+                } else if constexpr (FUSED && !MIXED) {
+                    Tri A, B;
+                    load_tri(m.geom, a, A);
+                    load_tri(m.geom, b, B);
+                    if (!fixed_p1_fused<NP>(A, B, R, vr, vi)) {
+                        layer_p1<BEM_LAPLACE_SLP, NP>(A, B, R, vr);
+                        layer_p1<BEM_LAPLACE_DLP, NP>(A, B, R, vi);
+                    }
+                } else if constexpr (FUSED) {
                     TriF A, B;
                     load_trif(m.geomf, a, A);
                     load_trif(m.geomf, b, B);
@@ -1994,7 +2010,7 @@ __device__ __forceinline__ void p1_tile(const MeshView &m, const BlockLaunch &L,
                         vr[q] = (Val)fs[q];
                         vi[q] = (Val)fd[q];
                     }
-                } else if (MIXED) {
+                } else if constexpr (MIXED) {
                     TriF A, B;
                     load_trif(m.geomf, a, A);
                     load_trif(m.geomf, b, B);
@@ -2076,8 +2092,8 @@ __device__ __forceinline__ void p1_tile(const MeshView &m, const BlockLaunch &L,
                             }
                         } else {
                             accr[e] += stg_r[q];
+                            if (TWO) acci[e] += stg_i[q];
                         }
-                        if (CPLX) acci[e] += stg_i[q];
                     }
                 }
             }

@@ -92,6 +92,12 @@ BEM_HD s64 fx_shl(s64 a, int n)
     return fx_join(fx_low(a) << n, (int)fx_funnel_l(fx_low(a), (unsigned)fx_high(a), n));
 }
 
+// a / 2^n rounded down, 0 <= n < 32
+BEM_HD s64 fx_sar(s64 a, int n)
+{
+    return fx_join(fx_funnel_r(fx_low(a), (unsigned)fx_high(a), n), fx_high(a) >> n);
+}
+
 BEM_HD Fx2 fx_split(s64 a)
 {
     Fx2 r;

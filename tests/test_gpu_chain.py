@@ -30,7 +30,7 @@ def _all_pairs(ptr, idx):
     return synth.workloads.BlockSet(ptr, idx, ptr, idx, t, s, off[:-1], int(off[-1]))
 
 
-@pytest.mark.parametrize("basis,precision", [("p0", "fp64"), ("p0", "mixed_full"), ("p1", "mixed_full")])
+@pytest.mark.parametrize("basis,precision", [("p0", "fp64"), ("p0", "mixed_full"), ("p1", "fp64"), ("p1", "mixed_full")])
 def test_calls_in_a_row(env, basis, precision):  # noqa: F811
     import torch
     pkg, ctx = env
