@@ -156,16 +156,17 @@ __global__ void __launch_bounds__(1024) k_job_scan(const int64_t *job_total, int
     for (int k = lo; k < hi; ++k) job_end[k] += base;
 }
 
-// Capped at 64 registers (four CTAs, 32 warps per SM): the float form's
-// dependent loads (block, cluster, index, geometry) and the FP64 form's integer
-// chains (bem_fixed_pair.cuh) want the warps.  Three CTAs where the packed pairs
-// spill at 64 and the rule is long enough: Helmholtz from 7 points on (9 points,
-// 3072-triangle dense matrix: 0.93 -> 0.88 ms), the single layer's unrolled 9
-// points (0.40 -> 0.35 ms; at 7 points four CTAs are 7% faster), the 16 points of
-// every kernel (double layer 1.34 -> 1.17 ms).
+// CTAs per SM.  Four (64 registers, 32 warps): the float form's dependent loads
+// (block, cluster, index, geometry) want the warps.  Three (80 registers) where
+// the packed pairs spill at 64 and the rule is long enough: Helmholtz from 7 points
+// on (9 points, 3072-triangle dense matrix: 0.93 -> 0.88 ms), the single layer's
+// unrolled 9 points (0.40 -> 0.35 ms; at 7 points four CTAs are 7% faster), the 16
+// points of every kernel (double layer 1.34 -> 1.17 ms).  Three in the FP64 form,
+// whose integer chains (bem_fixed_pair.cuh) overlap three points (2048 triangles,
+// single layer: 1.35 ms with four, 1.30 with three, 1.39 with two).
 constexpr int p0_ctas(int kind, int np, bool mixed)
 {
-    return mixed && ((kind == BEM_HELMHOLTZ_SLP && np > 4) || (kind == BEM_LAPLACE_SLP && np == 9) || np == 16) ? 3 : 4;
+    return !mixed || (kind == BEM_HELMHOLTZ_SLP && np > 4) || (kind == BEM_LAPLACE_SLP && np == 9) || np == 16 ? 3 : 4;
 }
 
 template <int KIND, int NP, bool MIXED>

@@ -342,17 +342,11 @@ __device__ __forceinline__ double fx_final(const FxUnits &U)
                                                                 : (KIND == BEM_LAPLACE_DLP ? U.f3 : 1.0);
 }
 
-// Trial points at a time: a Laplace point is about 110 instructions, a complex
-// one 400 to 580.  Three Laplace points overlap their dependent chains with 64
-// registers and 32 warps per SM (2048-triangle dense matrix, Duffy q = 3: single
-// layer 1.62 ms; all nine points unrolled at 128 registers 1.72 ms, one at a
-// time 1.80 ms); the complex chains overlap by themselves.  The trial points are
-// indexed in local memory (L1).
-template <int KIND>
-__device__ __forceinline__ constexpr int fx_unroll()
-{
-    return kind_complex(KIND) ? 1 : 3;
-}
+// Trial points at a time: three overlap their dependent chains with 80 registers
+// and 24 warps per SM (2048-triangle dense matrix, Duffy q = 3: single layer 1.30
+// ms, Brakhage-Werner 6.09; all nine points unrolled 1.39 ms, one at a time 6.24
+// for the latter).  The trial points are indexed in local memory (L1).
+constexpr int kFxUnroll = 3;
 
 // Regular pair, piecewise constant: regular_p0's integral.
 template <int KIND, int NP>
@@ -387,8 +381,7 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
         const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
         FxInner<KIND, 1> I;
         I.clear();
-        constexpr int UN = fx_unroll<KIND>();
-#pragma unroll UN
+#pragma unroll kFxUnroll
         for (int j = 0; j < NP; ++j) {
             const int32_t *w[1] = {R.wx[3][j]};
             I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
@@ -460,7 +453,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
         const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
         FxInner<KIND, 3> I;
         I.template clear<HELM ? 0 : kFxUpS, HELM ? 0 : kFxUpD>();
-        constexpr int UN = fx_unroll<KIND>();
+        constexpr int UN = HELM ? 1 : kFxUnroll;   // the complex sums want the registers
 #pragma unroll UN
         for (int j = 0; j < NP; ++j) {
             const int32_t *w[3] = {R.wx[0][j], R.wx[1][j], R.wx[2][j]};
@@ -554,7 +547,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
             cs[q].template clear<kFxUpS>();
             cd[q].template clear<kFxUpD>();
         }
-#pragma unroll 3
+#pragma unroll kFxUnroll
         for (int j = 0; j < NP; ++j) {
             const s64 r2 = fx_norm2(xx - yx[j], xy - yy[j], xz - yz[j]);
             const s64 inv = fx_rinv(r2, kb + 3, flag);                   // 2^(59 - kb) S / r
