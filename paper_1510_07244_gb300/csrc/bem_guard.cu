@@ -75,10 +75,16 @@ __device__ __forceinline__ GBlock guard_block(const GuardJob *jobs, const int64_
     return g;
 }
 
-// One warp per block (blocks hold a few hundred entries, so a CTA per block
-// would leave the passes waiting on each block's index loads): lanes take
-// the block's rows, the maximum over the row's columns goes out with one
-// atomic per (block, row).
+// Warps per block: one where there are blocks enough (they hold a few hundred
+// entries, so a CTA per block would leave the passes waiting on each block's index
+// loads), all warps shared out where there are not: a dense matrix is one block
+// (5000 triangles, double layer, 16 points: the call took 422 ms with one warp in
+// both passes, 3.3 ms so).
+__device__ __forceinline__ int guard_split(int64_t nw, int64_t nb) { return nb < nw ? (int)(nw / nb) : 1; }
+
+// Lanes take the block's rows, 32 at a time, the columns in as many parts as the
+// block's warps allow; the maximum over a row's columns goes out with one atomic per
+// (block, row, part).
 __global__ void __launch_bounds__(256) k_guard_rowmax(const GuardJob *__restrict__ jobs,
                                                       const int64_t *__restrict__ blk_end,
                                                       int n_jobs)
@@ -86,20 +92,27 @@ __global__ void __launch_bounds__(256) k_guard_rowmax(const GuardJob *__restrict
     const int64_t nb = blk_end[n_jobs - 1];
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb; b += nw) {
+    const int split = guard_split(nw, nb);
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= nw / split * split) return;   // warps left over
+    for (int64_t b = w / split; b < nb; b += nw / split) {
         const GBlock g = guard_block(jobs, blk_end, n_jobs, b);
         if (!g.ok) continue;
         const GuardJob &G = jobs[g.job];
         const float2 *o = reinterpret_cast<const float2 *>(G.L.out) + g.off;
-        for (int r = lane; r < g.nr; r += 32) {
+        const int groups = (g.nr + 31) / 32, parts = min(g.nc, max(1, split / groups));
+        for (int t = (int)(w % split); t < groups * parts; t += split) {
+            const int part = parts > 1 ? t / groups : 0, r = (t - part * groups) * 32 + lane;
+            if (r >= g.nr) continue;
+            const int c1 = parts > 1 ? (int)((int64_t)g.nc * (part + 1) / parts) : g.nc;
             const int row = G.L.row_idx[g.r_lo + r];
             float m0 = 0.0f, m1 = 0.0f;
-            int c = 0;
-            for (; c + 1 < g.nc; c += 2) {
+            int c = parts > 1 ? (int)((int64_t)g.nc * part / parts) : 0;
+            for (; c + 1 < c1; c += 2) {
                 m0 = fmaxf(m0, fabsf(o[r + (int64_t)c * g.nr].x));
                 m1 = fmaxf(m1, fabsf(o[r + (int64_t)(c + 1) * g.nr].x));
             }
-            if (c < g.nc) m0 = fmaxf(m0, fabsf(o[r + (int64_t)c * g.nr].x));
+            if (c < c1) m0 = fmaxf(m0, fabsf(o[r + (int64_t)c * g.nr].x));
             // |value| >= 0, so its bit pattern orders like the value
             if (row >= 0 && row < G.n_rows)
                 atomicMax(G.rowmax + row, __float_as_uint(fmaxf(m0, m1)));
@@ -107,8 +120,8 @@ __global__ void __launch_bounds__(256) k_guard_rowmax(const GuardJob *__restrict
     }
 }
 
-// One warp per block, lanes over its entries (column-major, coalesced), four
-// entries per lane in flight.
+// Lanes over a block's entries (column-major, coalesced), four entries per lane in
+// flight; the block's warps take every split-th run of 128.
 __global__ void __launch_bounds__(256) k_guard_select(const GuardJob *__restrict__ jobs,
                                                       const int64_t *__restrict__ blk_end,
                                                       int n_jobs, GuardItem *list,
@@ -121,7 +134,10 @@ __global__ void __launch_bounds__(256) k_guard_select(const GuardJob *__restrict
     const int64_t nb = blk_end[n_jobs - 1];
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb; b += nw) {
+    const int split = guard_split(nw, nb);
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= nw / split * split) return;   // warps left over
+    for (int64_t b = w / split; b < nb; b += nw / split) {
         const GBlock g = guard_block(jobs, blk_end, n_jobs, b);
         if (!g.ok) continue;   // uniform across the warp
         const GuardJob &G = jobs[g.job];
@@ -131,7 +147,9 @@ __global__ void __launch_bounds__(256) k_guard_select(const GuardJob *__restrict
         // four entries per lane and trip, their loads issued together; the
         // whole warp iterates together, so the ballots below see every lane
         constexpr int U = 4;
-        for (int e0 = 0; e0 < n; e0 += 32 * U) {
+        const unsigned first = (unsigned)(w % split) * 32 * U, stride = (unsigned)split * 32 * U;
+        for (unsigned at = first; at < (unsigned)n; at += stride) {
+            const int e0 = (int)at;
             float2 v[U];
             int row[U], col[U];
             bool redo[U];

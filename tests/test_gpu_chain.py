@@ -169,3 +169,29 @@ def test_gmres_sizes(env, n, restart):  # noqa: F811
     _, res = ctx.bem_dense_gmres(to_dev(A.T.ravel(), torch.complex128), to_dev(b, torch.complex128), x,
                                  tol=1e-300, restart=restart, maxit=2)
     assert np.isfinite(x.cpu().numpy()).all()
+
+
+def test_guard_splits(env):  # noqa: F811
+    """The double layer's guard over one block, 400 blocks and 65536 blocks of the same
+    entries (all warps in a block, a few, one): every entry has the same bits, since
+    the row maxima, and so the entries that are recomputed, are the same."""
+    import torch
+    pkg, ctx = env
+    mesh = synth.jitter(synth.icosphere(3), 0.05, 8)
+    n = mesh.nt
+    idx = np.random.default_rng(4).permutation(n).astype(np.int32)
+    mid = ctx.bem_mesh_upload(mesh.verts, mesh.tris, "p0")
+    quad = dict(QUAD, precision="mixed_full")
+    mats = []
+    for size in (n, n // 20, n // 256):
+        bs = _all_pairs(np.arange(0, n + 1, size, dtype=np.int32), idx)
+        out = torch.zeros(bs.n_entries, dtype=torch.float64, device="cuda")
+        ctx.bem_near_field([block_job(pkg, mid, bs, "laplace_dlp", 0.0, quad, out)])
+        ctx.bem_sync()
+        rows, cols = bs.entry_indices()
+        mat = np.empty((n, n))
+        mat[rows, cols] = out.cpu().numpy()
+        mats.append(mat)
+    ctx.bem_mesh_free(mid)
+    assert np.isfinite(mats[0]).all() and np.abs(mats[0]).max() > 0.0
+    assert np.array_equal(mats[0], mats[1]) and np.array_equal(mats[0], mats[2])
