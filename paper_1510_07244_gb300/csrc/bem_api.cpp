@@ -197,7 +197,7 @@ int touch_rule(bem_ctx *ctx, int cas, int q, int kind, int basis, bool f32, Rule
 // Evaluates every touching pair of the mesh into its touching table.  The three
 // cases are short launches of few CTAs that do not depend on one another: they
 // run as one chain (bem_pdl.cuh), the case with the longest pairs first, then the
-// prefix sums and the blocks (320 triangles, FP64 single layer: 68 -> 41 us; 1280
+// prefix sums and the blocks (80 triangles, FP64 single layer: 68 -> 41 us; 1280
 // triangles, float: 105 -> 75 us).  chained:
 // whether the chain has begun (a kernel launched, nothing but kernels since).
 int run_touching(bem_ctx *ctx, Mesh *m, const bem_kernel_desc *k, const bem_quad_desc *q, bool &chained)

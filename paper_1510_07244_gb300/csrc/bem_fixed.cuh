@@ -6,8 +6,10 @@
 // ones.  A quadrature point needs a difference of points, a squared distance,
 // a reciprocal square root and a weighted sum: 13 FP64 operations for the single
 // layer, about 60 with a sine and cosine.  Here the points of a pair are
-// integers scaled to the pair (62 bits), and a point costs about 75 integer
-// issue slots instead of the FP64 form's 13 x 70.
+// integers scaled to the pair (62 bits), and a single layer's point takes 90
+// instructions (34 of them multiply-adds) instead of 13 on the FP64 pipe, each
+// worth 64.  Bound by instruction issue: 0.6 of the issue slots, the ALU pipe half
+// busy, the multiplier 0.45 (2048 triangles, nine points: 8.82 ms on the FP64 pipe, 1.30 so).
 //
 // Precision: a coordinate carries an absolute error of a few 2^-59 S, S = the
 // power of two above the largest coordinate difference of the pair; FP64
