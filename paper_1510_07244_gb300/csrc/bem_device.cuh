@@ -374,18 +374,6 @@ __device__ __forceinline__ float kvalf(float dx, float dy, float dz, float dn)
     return dn * (ri * ri * ri);
 }
 
-// The same without the double layer's height factor: 1/r (single layer) or
-// 1/r^3 (double layer).  Product rules whose inner loop runs over trial points
-// at one test point x multiply the inner sum by the height of x once instead.
-template <int KIND>
-__device__ __forceinline__ float kvalf_r(float dx, float dy, float dz)
-{
-    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float ri = rsqrt_fast(r2);
-    if (KIND == BEM_LAPLACE_SLP) return ri;
-    return ri * ri * ri;
-}
-
 // ---------------------------------------------------------------------------
 // Helmholtz in the mixed form.  exp(i kappa r) = exp(i kappa r0) exp(i kappa
 // (r - r0)) with r0 = the distance of the two centroids: r0, kappa r0 and its
