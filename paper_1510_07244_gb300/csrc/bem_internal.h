@@ -182,7 +182,7 @@ struct bem_ctx {
     int64_t tile_prefix_cap = 0;
     void *guard_buf = nullptr;             // scratch: cancellation guard of one call
     size_t guard_cap = 0;
-    void *scratch = nullptr;               // scratch of one solver or potential call, grown to the largest
+    void *scratch = nullptr;               // scratch of one solver call, grown to the largest
     size_t scratch_cap = 0;
     double *solve_host = nullptr;          // page-locked: a solver step's coefficients (16 KB, at the first solve)
     cudaEvent_t solve_read = nullptr;      // they are there

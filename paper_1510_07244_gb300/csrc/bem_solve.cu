@@ -5,7 +5,7 @@
 //                      off the surface (piecewise-constant density w), with the
 //                      library's kernels; one thread per (point, triangle) in the
 //                      FP64 form's fixed-point arithmetic, a Duffy q x q rule per
-//                      triangle, partial sums per CTA added in order.
+//                      triangle, a cluster of CTAs per point, their sums added in order.
 //   bem_dense_gmres    restarted GMRES (Saad and Schultz) for a dense complex
 //                      system (A + diag(d)) x = b: Arnoldi with classical
 //                      Gram-Schmidt applied twice, Givens rotations on the host.
@@ -14,6 +14,7 @@
 //                      overlapping launches; each Arnoldi step reads its projection
 //                      coefficients and the new vector's norm back once (a few
 //                      hundred bytes), beside the next step's product.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -110,26 +111,27 @@ __device__ __forceinline__ bool potential_fixed(const double *z, const Tri &B, c
     return (flag >> (16 + P.kb)) == 0;
 }
 
-// CTA (s, p): point p0 + p, the triangles [s per, (s + 1) per); its sum goes to
-// part[p * gridDim.x + s] (the output itself when gridDim.x is 1).  A point's
-// triangles spread over several CTAs where the points alone would not fill the
-// GPU (256 points, 2048 triangles, Duffy q = 4, Brakhage-Werner kernel: one warp
-// per point in FP64 arithmetic took 9.4 ms).
-constexpr int kPotTri = 128;
+// Cluster p: point p0 + p; its CTA s takes the triangles [s per, (s + 1) per), and
+// the first CTA adds the sums in order through distributed shared memory: no scratch,
+// so the call stays asynchronous and a captured one holds no pointer of the library's.
+// A point's triangles spread over several CTAs where the points alone would not fill
+// the GPU (256 points, 2048 triangles, Duffy q = 4, Brakhage-Werner kernel: one warp
+// per point in FP64 arithmetic took 9.4 ms; 0.21 ms so, 0.09 for 64 points).
+constexpr int kPotThreads = 256, kPotCluster = 16;   // at most; beyond 8 CTAs by opt-in
 
 template <int KIND>
-__global__ void __launch_bounds__(kPotTri) k_potentials(MeshView m, const double *__restrict__ z,
-                                                        int64_t p0, int64_t per,
-                                                        const double2 *__restrict__ w,
-                                                        const __grid_constant__ Rule2D R, double kappa,
-                                                        double eta, double2 *part)
+__global__ void __launch_bounds__(kPotThreads) k_potentials(MeshView m, const double *__restrict__ z,
+                                                            int64_t p0, int64_t per,
+                                                            const double2 *__restrict__ w,
+                                                            const __grid_constant__ Rule2D R,
+                                                            double kappa, double eta, double2 *out)
 {
-    __shared__ double2 ws[kPotTri / 32];
+    __shared__ double2 ws[kPotThreads / 32], sum;
     const int64_t p = p0 + blockIdx.y;
     const int64_t j0 = (int64_t)blockIdx.x * per, j1 = min(m.nt, j0 + per);
     const double zp[3] = {z[3 * p], z[3 * p + 1], z[3 * p + 2]};
     double ar = 0.0, ai = 0.0;
-    for (int64_t j = j0 + threadIdx.x; j < j1; j += kPotTri) {
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
         Tri B;
         load_tri(m.geom, j, B);
         double sr, si;
@@ -148,30 +150,24 @@ __global__ void __launch_bounds__(kPotTri) k_potentials(MeshView m, const double
     __syncthreads();
     if (threadIdx.x == 0) {
         double2 s = ws[0];
-        for (int k = 1; k < kPotTri / 32; ++k) {
+        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
             s.x += ws[k].x;
             s.y += ws[k].y;
         }
-        part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
+        sum = s;
     }
-}
-
-// one warp per point: its partial sums in a fixed order
-__global__ void __launch_bounds__(256) k_potential_sum(const double2 *__restrict__ part, int ns,
-                                                       int64_t n, double2 *out)
-{
-    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (p >= n) return;
-    double ar = 0.0, ai = 0.0;
-    for (int s = lane; s < ns; s += 32) {
-        const double2 v = part[p * ns + s];
-        ar += v.x;
-        ai += v.y;
+    auto cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double2 s = sum;
+        for (unsigned k = 1; k < cluster.num_blocks(); ++k) {
+            const double2 v = *cluster.map_shared_rank(&sum, k);
+            s.x += v.x;
+            s.y += v.y;
+        }
+        out[p] = s;
     }
-    ar = warp_sum(ar);
-    ai = warp_sum(ai);
-    if (lane == 0) out[p] = make_double2(ar, ai);
+    cluster.sync();   // the CTAs' sums stay until the first has read them
 }
 
 // The kernels of one Arnoldi step run as a chain of dependent launches
@@ -418,32 +414,40 @@ int bem_potentials(bem_ctx *ctx, int32_t mesh_id, const bem_kernel_desc *kernel,
     double2 *o = reinterpret_cast<double2 *>(out);
     const double ka = kernel->kappa, et = kernel->eta;
     cudaStream_t st = ctx->stream;
-    // CTAs per point: about eight per SM in all; one CTA writes its point's result
-    // itself, several need scratch for their sums (not grown while capturing)
-    const int64_t chunks = (m.nt + kPotTri - 1) / kPotTri;
-    int64_t ns = std::min(chunks, std::max<int64_t>(1, (8 * ctx->num_sms + n_points - 1) / n_points));
-    const size_t bytes = sizeof(double2) * (size_t)(n_points * ns);
-    if (ns > 1 && bytes > ctx->scratch_cap) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) ns = 1;
-        else if (int rc = api_ensure_scratch(ctx, bytes)) return rc;
-    }
-    const int64_t per = (chunks + ns - 1) / ns * kPotTri;
-    double2 *part = ns > 1 ? reinterpret_cast<double2 *>(ctx->scratch) : o;
+    // CTAs per point: a power of two that gives about 32 warps per SM in all, with 128
+    // triangles or more each; CTAs of twice the warps where 16 of 4 warps a point leave
+    // half of that empty and have the triangles
+    const int64_t need = 32 * (int64_t)ctx->num_sms;
+    const int threads = n_points * kPotCluster * 8 < need && m.nt > kPotCluster * 128 ? kPotThreads : 128;
+    int ns = 1;
+    while (ns < kPotCluster && ns * 128 < m.nt && n_points * ns * (threads / 32) < need) ns *= 2;
+    const int64_t per = (m.nt + ns - 1) / ns;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ns;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.blockDim = dim3((unsigned)threads);
+    c.stream = st;
+    c.attrs = at;
+    c.numAttrs = 1;
+    cudaError_t e = cudaSuccess;
     constexpr int64_t kRows = 65535;   // grid limit
-    for (int64_t p0 = 0; p0 < n_points; p0 += kRows) {
-        const dim3 grid((unsigned)ns, (unsigned)std::min(kRows, n_points - p0));
-        double2 *to = part + p0 * ns;
+    for (int64_t p0 = 0; p0 < n_points && e == cudaSuccess; p0 += kRows) {
+        c.gridDim = dim3((unsigned)ns, (unsigned)std::min(kRows, n_points - p0));
+        auto run = [&](auto k) {
+            cudaError_t ee = ns > 8 ? cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
+                                    : cudaSuccess;
+            return ee == cudaSuccess ? cudaLaunchKernelEx(&c, k, m, points, p0, per, w, r2, ka, et, o) : ee;
+        };
         switch (kernel->kind) {
-        case BEM_LAPLACE_SLP: k_potentials<BEM_LAPLACE_SLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
-        case BEM_LAPLACE_DLP: k_potentials<BEM_LAPLACE_DLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
-        case BEM_HELMHOLTZ_SLP: k_potentials<BEM_HELMHOLTZ_SLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
-        case BEM_HELMHOLTZ_DLP: k_potentials<BEM_HELMHOLTZ_DLP><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
-        default: k_potentials<BEM_HELMHOLTZ_BW><<<grid, kPotTri, 0, st>>>(m, points, p0, per, w, r2, ka, et, to); break;
+        case BEM_LAPLACE_SLP: e = run(k_potentials<BEM_LAPLACE_SLP>); break;
+        case BEM_LAPLACE_DLP: e = run(k_potentials<BEM_LAPLACE_DLP>); break;
+        case BEM_HELMHOLTZ_SLP: e = run(k_potentials<BEM_HELMHOLTZ_SLP>); break;
+        case BEM_HELMHOLTZ_DLP: e = run(k_potentials<BEM_HELMHOLTZ_DLP>); break;
+        default: e = run(k_potentials<BEM_HELMHOLTZ_BW>); break;
         }
     }
-    if (ns > 1) k_potential_sum<<<(unsigned)((n_points + 7) / 8), 256, 0, st>>>(part, (int)ns, n_points, o);
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return api_cuda_fail(ctx, e, "bem_potentials");
     return BEM_OK;
 }
