@@ -140,20 +140,34 @@ int get_rule4(bem_ctx *ctx, int cas, int rule, int q, Rule4D &out)
     r.xi = xi ? 1 : 0;
     r.q = q;
     r.n = (int)(soa.size() / kRuleCols);
-    // one allocation and one copy: the doubles, their float roundings, and the
-    // rounding remainders ((f, fl) is the rule as double-float pairs)
+    // one allocation and one copy: the doubles, their float roundings, the rounding
+    // remainders ((f, fl) is the rule as double-float pairs), and for a rule with xi
+    // integrated out the FP64 form's fixed-point tables of both bases.  All at the first
+    // use in any form: a later call in another form may be under stream capture, where
+    // nothing can be allocated.
     const size_t n = soa.size();
-    std::vector<double> buf(2 * n);
+    std::vector<int32_t> words[2];
+    if (xi && !(make_touch_fixed(cas, q, BEM_P0, words[0]) && make_touch_fixed(cas, q, BEM_P1, words[1])))
+        return fail(ctx, BEM_ERR_INVALID_ARG, "bad rule");
+    std::vector<double> buf(2 * n + (words[0].size() + words[1].size()) / 2);
     std::memcpy(buf.data(), soa.data(), n * sizeof(double));
     float *sf = reinterpret_cast<float *>(buf.data() + n);
     for (size_t k = 0; k < n; ++k) {
         sf[k] = (float)soa[k];
         sf[n + k] = (float)(soa[k] - (double)sf[k]);
     }
+    if (xi) {
+        std::memcpy(buf.data() + 2 * n, words[0].data(), words[0].size() * sizeof(int32_t));
+        std::memcpy(buf.data() + 2 * n + words[0].size() / 2, words[1].data(), words[1].size() * sizeof(int32_t));
+    }
     cudaError_t e = cudaMalloc((void **)&r.d, buf.size() * sizeof(double));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
     r.f = reinterpret_cast<float *>(r.d + n);
     r.fl = r.f + n;
+    if (xi) {
+        r.fx0 = reinterpret_cast<int2 *>(r.d + 2 * n);
+        r.fx1 = r.fx0 + words[0].size() / 2;
+    }
     e = cudaMemcpy(r.d, buf.data(), buf.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(r.d);
@@ -161,37 +175,14 @@ int get_rule4(bem_ctx *ctx, int cas, int rule, int q, Rule4D &out)
     }
     ctx->rules4[key] = r;
     out = r;
-    return BEM_OK;
-}
-
-// The FP64 form's fixed-point table of a touching rule with xi integrated out,
-// built on first use per basis.
-int touch_table(bem_ctx *ctx, int cas, int q, int basis, Rule4D &out)
-{
-    Rule4D &r = ctx->rules4[std::make_tuple(cas, kRuleXiOut, q)];
-    int2 *&tab = basis == BEM_P0 ? r.fx0 : r.fx1;
-    if (!tab) {
-        std::vector<int32_t> words;
-        if (!make_touch_fixed(cas, q, basis, words)) return fail(ctx, BEM_ERR_INVALID_ARG, "bad rule");
-        int2 *d = nullptr;
-        cudaError_t e = cudaMalloc((void **)&d, words.size() * sizeof(int32_t));
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
-        e = cudaMemcpy(d, words.data(), words.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            cudaFree(d);
-            return cuda_fail(ctx, e, "cudaMemcpy(rule)");
-        }
-        tab = d;
-    }
-    out = r;
+    // the kernels that take xi out of this order's rule may follow under capture
+    if (cas != kRegular && !xi && q <= 2 * kMaxXiFixedPairs + 1) return get_rule4(ctx, cas, kRuleXiOut, q, r);
     return BEM_OK;
 }
 
 int touch_rule(bem_ctx *ctx, int cas, int q, int kind, int basis, bool f32, Rule4D &out)
 {
-    const bool xi = touch_xi_out(kind, basis, q, f32);
-    const int rc = get_rule4(ctx, cas, xi ? kRuleXiOut : 0, q, out);
-    return rc || !xi || f32 ? rc : touch_table(ctx, cas, q, basis, out);
+    return get_rule4(ctx, cas, touch_xi_out(kind, basis, q, f32) ? kRuleXiOut : 0, q, out);
 }
 
 // Evaluates every touching pair of the mesh into its touching table.  The three
@@ -466,11 +457,7 @@ int bem_destroy(bem_ctx *ctx)
     cudaStreamSynchronize(ctx->stream);
     plan_forget(ctx);
     for (auto &kv : ctx->meshes) free_mesh(kv.second);
-    for (auto &kv : ctx->rules4) {
-        cudaFree(kv.second.d);      // holds f and fl too
-        cudaFree(kv.second.fx0);
-        cudaFree(kv.second.fx1);
-    }
+    for (auto &kv : ctx->rules4) cudaFree(kv.second.d);   // holds f, fl, fx0 and fx1 too
     for (auto &r : ctx->prof_pending) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);

@@ -4,7 +4,10 @@
   with the eager call's bits after a solve has grown (and replaced) the solver's
   scratch.  Also against numpy for 1 to 1300 points, which changes the CTAs per
   point; tolerance 1e-12 of the sum of the terms' magnitudes (320 terms of 16
-  points, each rounded to a few 2^-53)."""
+  points, each rounded to a few 2^-53).
+- A dense FP64 matrix after a call in a float form (Laplace kernels) or of the
+  entry kernel (Helmholtz): the singular rules that the first call loaded serve
+  the second, which then allocates nothing."""
 import numpy as np
 import pytest
 
@@ -78,4 +81,39 @@ def test_potentials(env, points):
         r = np.linalg.norm(z[k:k + 100, None] - y[None], axis=2)
         ref, A = (np.exp(3j * r) / r) @ wt, (1 / r) @ np.abs(wt)
         assert (np.abs(eager[k:k + 100].cpu().numpy() - ref) / A).max() < 1e-12
+    ctx.bem_mesh_free(mid)
+
+
+@pytest.mark.parametrize("basis,kernel", [("p0", "laplace_slp"), ("p0", "laplace_dlp"), ("p1", "laplace_slp"),
+                                          ("p1", "laplace_dlp"), ("p0", "helmholtz_slp")])
+def test_fp64_captured_after_another_call(env, basis, kernel):
+    import torch
+    pkg, ctx, stream = env
+    mesh = synth.jitter(synth.icosphere(1), 0.05, 7)
+    n = mesh.nt if basis == "p0" else mesh.nv
+    mid = ctx.bem_mesh_upload(mesh.verts, mesh.tris, basis)
+    cplx = kernel.startswith("helmholtz")
+    out = torch.zeros(n * n, dtype=torch.complex128 if cplx else torch.float64, device="cuda")
+    quad = dict(q_regular=3, q_identical=5, q_edge=4, q_vertex=3)
+    kd = pkg.kernel_desc(kernel, 2.0 if cplx else 0.0)
+    torch.cuda.synchronize()
+    if cplx:
+        # the dense call's other buffers; then other orders, whose rules only the entry kernel has loaded
+        ctx.bem_assemble_dense(mid, kd, pkg.quad_desc(q_regular=3, q_identical=3, q_edge=3, q_vertex=2), 0, out)
+        i = torch.arange(32, dtype=torch.int32, device="cuda")
+        ctx.bem_pivot_entries(mid, kd, pkg.quad_desc(**quad), i, i, torch.zeros(32, dtype=out.dtype, device="cuda"))
+    else:
+        ctx.bem_assemble_dense(mid, pkg.kernel_desc("laplace_slp"), pkg.quad_desc(precision="mixed_full", **quad), 0, out)
+    ctx.bem_sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        ctx.bem_assemble_dense(mid, kd, pkg.quad_desc(**quad), 0, out)
+    g.replay()
+    torch.cuda.synchronize()
+    got = out.clone()
+    out.zero_()
+    torch.cuda.synchronize()
+    ctx.bem_assemble_dense(mid, kd, pkg.quad_desc(**quad), 0, out)
+    ctx.bem_sync()
+    assert torch.equal(got, out)
     ctx.bem_mesh_free(mid)
