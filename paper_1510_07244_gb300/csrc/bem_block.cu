@@ -172,8 +172,7 @@ constexpr int p0_ctas(int kind, int np, bool mixed)
 template <int KIND, int NP, bool MIXED>
 __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_block_p0(MeshView m, BlockLaunch L,
                                                   const __grid_constant__ Rule2D R,
-                                                  const int64_t *__restrict__ prefix,
-                                                  int *status)
+                                                  const int64_t *prefix, int *status)
 {
     pdl_wait();
     // prefix counts entries; a tile is kP0Tile of them.  Each CTA takes a
@@ -196,14 +195,10 @@ __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_block_p0(Mesh
 // ---------------------------------------------------------------------------
 template <int KIND, int NP, bool MIXED>
 __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_batch_p0(const BatchJob *__restrict__ jobs, int n_jobs,
-                                                  const int64_t *__restrict__ job_end,
-                                                  const __grid_constant__ Rule2D R, int *status,
-                                                  int beside)
+                                                  const int64_t *job_end,
+                                                  const __grid_constant__ Rule2D R, int *status)
 {
-    // beside: the kernel before is another such launch, which waited for all that
-    // this one reads before it let this one start; the two share the SMs
-    if (!beside) pdl_wait();
-    pdl_launch();
+    pdl_wait();
     // contiguous runs of tiles per CTA (see k_block_p0); the block hint is
     // kept while the run stays in one job
     const int64_t total = n_jobs > 0 ? job_end[n_jobs - 1] : 0;
@@ -221,7 +216,6 @@ __global__ void __launch_bounds__(256, p0_ctas(KIND, NP, MIXED)) k_batch_p0(cons
         const BatchJob &J = jobs[j];
         p0_tile<KIND, NP, MIXED>(J.m, J.L, R, J.prefix, local, status, hint);
     }
-    if (beside) pdl_end();
 }
 
 // ---------------------------------------------------------------------------
@@ -455,7 +449,7 @@ __global__ void __launch_bounds__(1024) k_tile_prefix_chunk(BlockLaunch L, int t
 
 // CTA c adds the totals of chunks 0 .. c to chunk c + 1
 __global__ void __launch_bounds__(1024) k_tile_prefix_add(BlockLaunch L, int64_t *prefix,
-                                                          const int64_t *__restrict__ chunk_total)
+                                                          const int64_t *chunk_total)
 {
     __shared__ int64_t ws[32];
     pdl_wait();
@@ -576,31 +570,31 @@ cudaError_t launch_tile_prefix_batch(BatchJob *jobs, int n_jobs, int tr, int tc,
 
 template <int KIND, int NP, bool MIXED>
 static cudaError_t batch_np(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
-                            const Rule2D &R, int *status, int grid, cudaStream_t st, ChainPos pos)
+                            const Rule2D &R, int *status, int grid, cudaStream_t st, bool chained)
 {
     if (basis == BEM_P0)
-        return launch_chain(pos != kChainNone, (unsigned)grid, 256, st, k_batch_p0<KIND, NP, MIXED>, jobs,
-                            n_jobs, job_end, R, status, pos == kChainBeside ? 1 : 0);
+        return launch_chain(chained, (unsigned)grid, 256, st, k_batch_p0<KIND, NP, MIXED>, jobs,
+                            n_jobs, job_end, R, status);
     return MIXED ? launch_p1_batch_mixed(KIND, NP, jobs, n_jobs, job_end, R, status, grid, st)
                  : launch_p1_batch_fp64(KIND, NP, jobs, n_jobs, job_end, R, status, grid, st);
 }
 
 template <int KIND, bool MIXED>
 static cudaError_t batch_kind(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
-                              const Rule2D &R, int *status, int grid, cudaStream_t st, ChainPos pos)
+                              const Rule2D &R, int *status, int grid, cudaStream_t st, bool chained)
 {
     switch (R.np) {
-    case 4: return batch_np<KIND, 4, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
-    case 7: return batch_np<KIND, 7, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
-    case 9: return batch_np<KIND, 9, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
-    case 16: return batch_np<KIND, 16, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+    case 4: return batch_np<KIND, 4, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
+    case 7: return batch_np<KIND, 7, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
+    case 9: return batch_np<KIND, 9, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
+    case 16: return batch_np<KIND, 16, MIXED>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
     default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
                                int kind, int mixed, const Rule2D &R, int *status, int grid,
-                               cudaStream_t st, ChainPos pos)
+                               cudaStream_t st, bool chained)
 {
     if (n_jobs <= 0) return cudaSuccess;
     if (kind == kFusedLaplace) {   // piecewise-linear basis only
@@ -610,19 +604,19 @@ cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *
     }
     switch (kind) {
     case BEM_LAPLACE_SLP:
-        return mixed ? batch_kind<BEM_LAPLACE_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)
-                     : batch_kind<BEM_LAPLACE_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+        return mixed ? batch_kind<BEM_LAPLACE_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained)
+                     : batch_kind<BEM_LAPLACE_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
     case BEM_LAPLACE_DLP:
-        return mixed ? batch_kind<BEM_LAPLACE_DLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)
-                     : batch_kind<BEM_LAPLACE_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+        return mixed ? batch_kind<BEM_LAPLACE_DLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained)
+                     : batch_kind<BEM_LAPLACE_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
     case BEM_HELMHOLTZ_DLP:   // FP64 in every precision
-        return batch_kind<BEM_HELMHOLTZ_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+        return batch_kind<BEM_HELMHOLTZ_DLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
     case BEM_HELMHOLTZ_BW:
-        return batch_kind<BEM_HELMHOLTZ_BW, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+        return batch_kind<BEM_HELMHOLTZ_BW, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
     default:
         return (mixed && basis == BEM_P0)
-                   ? batch_kind<BEM_HELMHOLTZ_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos)
-                   : batch_kind<BEM_HELMHOLTZ_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, pos);
+                   ? batch_kind<BEM_HELMHOLTZ_SLP, true>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained)
+                   : batch_kind<BEM_HELMHOLTZ_SLP, false>(jobs, n_jobs, job_end, basis, R, status, grid, st, chained);
     }
 }
 

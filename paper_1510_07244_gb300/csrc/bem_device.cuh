@@ -1602,7 +1602,7 @@ struct FlatEntry {
 // none).  Tiles taken in increasing order then find their blocks in the window
 // from there, without a search.
 __device__ __forceinline__ FlatEntry flat_entry(const MeshView &m, const BlockLaunch &L,
-                                                const int64_t *__restrict__ prefix, int64_t tile,
+                                                const int64_t *prefix, int64_t tile,
                                                 int *status, int64_t &hint)
 {
     static_assert(kP0Tile == 256, "one thread per entry of a tile");
@@ -1674,7 +1674,7 @@ __device__ __forceinline__ FlatEntry flat_entry(const MeshView &m, const BlockLa
 // hint as flat_entry's).
 template <int KIND, int NP, bool MIXED>
 __device__ __forceinline__ void p0_tile(const MeshView &m, const BlockLaunch &L, const Rule2D &R,
-                                        const int64_t *__restrict__ prefix, int64_t tile,
+                                        const int64_t *prefix, int64_t tile,
                                         int *status, int64_t &hint)
 {
     const FlatEntry fe = flat_entry(m, L, prefix, tile, status, hint);

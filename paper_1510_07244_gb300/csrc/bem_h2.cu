@@ -109,7 +109,7 @@ template <bool GATHER>
 __global__ void __launch_bounds__(256) k_h2_blocks(const H2Block *__restrict__ blk, int64_t n,
                                                    const double *__restrict__ vals,
                                                    const int32_t *__restrict__ idx,
-                                                   const double *__restrict__ x, double *part)
+                                                   const double *x, double *part)
 {
     const int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256) k_h2_forward(const H2Node *__restrict__ n
                                                     const int32_t *__restrict__ list,
                                                     const double *__restrict__ vals,
                                                     const int32_t *__restrict__ sources,
-                                                    const double *__restrict__ x, double *xhat)
+                                                    const double *x, double *xhat)
 {
     __shared__ double part[kH2Warps][32];
     const H2Node N = nodes[list[blockIdx.x]];
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_h2_backward(const H2Node *__restrict__ 
                                                      const int32_t *__restrict__ list,
                                                      const double *__restrict__ valsT,
                                                      const int32_t *__restrict__ sources,
-                                                     const double *__restrict__ far_part,
+                                                     const double *far_part,
                                                      const double *__restrict__ near_part,
                                                      const double *__restrict__ diag,
                                                      const double *__restrict__ x, double *yhat,

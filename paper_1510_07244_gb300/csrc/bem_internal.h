@@ -491,12 +491,9 @@ cudaError_t launch_touching_batch(const TouchJob *jobs, int basis, int kind, int
 // Block buckets of many jobs: job_end[j] = tiles of jobs 0..j (inclusive
 // prefix); job_end holds n_jobs + 1 entries, the last one the tile counter of
 // the piecewise-linear tile engine (reset by the launch).
-// Place of a piecewise-constant launch in a chain (bem_pdl.cuh): a plain launch;
-// after the passes that it reads; after another such launch that follows them.
-enum ChainPos { kChainNone, kChainAfter, kChainBeside };
 cudaError_t launch_block_batch(const BatchJob *jobs, int n_jobs, const int64_t *job_end, int basis,
                                int kind, int mixed, const Rule2D &R, int *status, int grid,
-                               cudaStream_t st, ChainPos pos = kChainNone);
+                               cudaStream_t st, bool chained = false);
 cudaError_t launch_pivot_entries(const MeshView &m, const int32_t *rows, const int32_t *cols,
                                  int64_t n, void *out, const Rule4D *rules /*[4]*/, int kind,
                                  double kappa, int *status, cudaStream_t st, bool absolute,

@@ -4,7 +4,9 @@
 // A kernel launched with launch_chain(chained = true) starts as soon as every CTA
 // of the kernel before it has called pdl_launch() (or exited), not when that
 // kernel has finished.  A kernel of a chain calls pdl_wait() before it touches
-// anything that an earlier kernel of the chain writes; one that depends on none of
+// anything that an earlier kernel of the chain writes, and takes it through plain
+// pointers: const __restrict__ would promise that nothing changes while the kernel is
+// resident, and allow non-coherent loads.  A kernel that depends on none of
 // them calls pdl_end() last, so that its own completion implies theirs (one warp
 // of the grid: a wait is an acquire, and one at the end of every warp cost the
 // touching kernels 7%).  The first kernel of a chain is launched with chained = false and waits

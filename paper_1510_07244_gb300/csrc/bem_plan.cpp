@@ -169,7 +169,7 @@ cudaError_t bucket_prefix(bem_ctx *ctx, const BlockBucket &b, cudaStream_t st, b
 }
 
 cudaError_t launch_bucket(bem_ctx *ctx, const BlockBucket &b, int mult, cudaStream_t st,
-                          ChainPos pos = kChainNone)
+                          bool chained = false)
 {
     if (b.fused && b.coupling)
         return launch_coupling_p1_fused_batch(b.jobs, (int)b.host_jobs.size(), b.job_end, b.r2,
@@ -181,7 +181,7 @@ cudaError_t launch_bucket(bem_ctx *ctx, const BlockBucket &b, int mult, cudaStre
         return launch_coupling_p1_batch(b.jobs, (int)b.host_jobs.size(), b.job_end, b.kind, b.r2,
                                         ctx->status, ctx->num_sms * mult, st);
     return launch_block_batch(b.jobs, (int)b.host_jobs.size(), b.job_end, b.basis, b.kind, b.mixed,
-                              b.r2, ctx->status, ctx->num_sms * mult, st, pos);
+                              b.r2, ctx->status, ctx->num_sms * mult, st, chained);
 }
 
 // Issues the plan's launches on stream st (profiling events when prof != null).
@@ -242,14 +242,12 @@ cudaError_t issue(bem_ctx *ctx, bem_plan *p, cudaStream_t st, bool record_prof,
         if (e != cudaSuccess) return e;
         chained = chained || (chain && !b.host_jobs.empty());
     }
-    ChainPos pos = chained ? kChainAfter : kChainNone;
     for (auto &b : p->bb) {
-        const bool p0 = b.basis == BEM_P0;
         ev_begin();
-        e = launch_bucket(ctx, b, b.grid_mult, st, p0 ? pos : kChainNone);
+        e = launch_bucket(ctx, b, b.grid_mult, st, chained && b.basis == BEM_P0);
         ev_end();
         if (e != cudaSuccess) return e;
-        if (!b.host_jobs.empty()) pos = p0 && chain ? kChainBeside : kChainNone;
+        chained = false;   // a bucket's kernels let the next one start when they are done
     }
     for (auto &l : p->learned) {
         ev_begin();
