@@ -123,6 +123,37 @@ int check_kernel(bem_ctx *ctx, const bem_kernel_desc *k)
     return BEM_OK;
 }
 
+void free_rule(Rule4D &r)
+{
+    cudaFree(r.d);      // holds f and fl too
+    cudaFree(r.fx0);
+    cudaFree(r.fx1);
+}
+
+// The FP64 form's fixed-point tables of a touching rule with xi integrated out, for
+// the bases that the context has had meshes of.  They come with the rule or with the
+// first mesh of their basis, whatever the form that is called then: a later FP64 call
+// may be under stream capture, where nothing can be allocated.
+int touch_tables(bem_ctx *ctx, int cas, Rule4D &r)
+{
+    for (int basis : {BEM_P0, BEM_P1}) {
+        int2 *&tab = basis == BEM_P0 ? r.fx0 : r.fx1;
+        if (tab || !ctx->has_basis[basis]) continue;
+        std::vector<int32_t> words;
+        if (!make_touch_fixed(cas, r.q, basis, words)) return fail(ctx, BEM_ERR_INVALID_ARG, "bad rule");
+        int2 *d = nullptr;
+        cudaError_t e = cudaMalloc((void **)&d, words.size() * sizeof(int32_t));
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
+        e = cudaMemcpy(d, words.data(), words.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFree(d);
+            return cuda_fail(ctx, e, "cudaMemcpy(rule)");
+        }
+        tab = d;
+    }
+    return BEM_OK;
+}
+
 // Rules of the context, built on first use: regular rules by (rule, q),
 // touching rules by q with rule 0 (q^4 points) or kRuleXiOut (xi integrated out).
 int get_rule4(bem_ctx *ctx, int cas, int rule, int q, Rule4D &out)
@@ -140,38 +171,26 @@ int get_rule4(bem_ctx *ctx, int cas, int rule, int q, Rule4D &out)
     r.xi = xi ? 1 : 0;
     r.q = q;
     r.n = (int)(soa.size() / kRuleCols);
-    // one allocation and one copy: the doubles, their float roundings, the rounding
-    // remainders ((f, fl) is the rule as double-float pairs), and for a rule with xi
-    // integrated out the FP64 form's fixed-point tables of both bases.  All at the first
-    // use in any form: a later call in another form may be under stream capture, where
-    // nothing can be allocated.
+    // one allocation and one copy: the doubles, their float roundings, and the
+    // rounding remainders ((f, fl) is the rule as double-float pairs)
     const size_t n = soa.size();
-    std::vector<int32_t> words[2];
-    if (xi && !(make_touch_fixed(cas, q, BEM_P0, words[0]) && make_touch_fixed(cas, q, BEM_P1, words[1])))
-        return fail(ctx, BEM_ERR_INVALID_ARG, "bad rule");
-    std::vector<double> buf(2 * n + (words[0].size() + words[1].size()) / 2);
+    std::vector<double> buf(2 * n);
     std::memcpy(buf.data(), soa.data(), n * sizeof(double));
     float *sf = reinterpret_cast<float *>(buf.data() + n);
     for (size_t k = 0; k < n; ++k) {
         sf[k] = (float)soa[k];
         sf[n + k] = (float)(soa[k] - (double)sf[k]);
     }
-    if (xi) {
-        std::memcpy(buf.data() + 2 * n, words[0].data(), words[0].size() * sizeof(int32_t));
-        std::memcpy(buf.data() + 2 * n + words[0].size() / 2, words[1].data(), words[1].size() * sizeof(int32_t));
-    }
     cudaError_t e = cudaMalloc((void **)&r.d, buf.size() * sizeof(double));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(rule)");
     r.f = reinterpret_cast<float *>(r.d + n);
     r.fl = r.f + n;
-    if (xi) {
-        r.fx0 = reinterpret_cast<int2 *>(r.d + 2 * n);
-        r.fx1 = r.fx0 + words[0].size() / 2;
-    }
     e = cudaMemcpy(r.d, buf.data(), buf.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        cudaFree(r.d);
-        return cuda_fail(ctx, e, "cudaMemcpy(rule)");
+    int rc = e == cudaSuccess ? BEM_OK : cuda_fail(ctx, e, "cudaMemcpy(rule)");
+    if (rc == BEM_OK && xi) rc = touch_tables(ctx, cas, r);
+    if (rc != BEM_OK) {
+        free_rule(r);
+        return rc;
     }
     ctx->rules4[key] = r;
     out = r;
@@ -457,7 +476,7 @@ int bem_destroy(bem_ctx *ctx)
     cudaStreamSynchronize(ctx->stream);
     plan_forget(ctx);
     for (auto &kv : ctx->meshes) free_mesh(kv.second);
-    for (auto &kv : ctx->rules4) cudaFree(kv.second.d);   // holds f, fl, fx0 and fx1 too
+    for (auto &kv : ctx->rules4) free_rule(kv.second);
     for (auto &r : ctx->prof_pending) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
@@ -642,6 +661,17 @@ int bem_mesh_upload(bem_ctx *ctx, const double *verts, int64_t nv, const int32_t
     m->stats.n_vertex = m->nlist[kVertex];
     m->stats.max_vertex_degree = maxdeg;
     m->stats.basis = basis;
+    if (!ctx->has_basis[basis]) {
+        ctx->has_basis[basis] = true;
+        for (auto &kv : ctx->rules4) {
+            const int rc = kv.second.xi ? touch_tables(ctx, std::get<0>(kv.first), kv.second) : BEM_OK;
+            if (rc != BEM_OK) {
+                ctx->has_basis[basis] = false;
+                free_mesh(m);
+                return rc;
+            }
+        }
+    }
     const int id = ctx->next_mesh++;
     ctx->meshes[id] = m;
     *mesh_id = id;

@@ -190,6 +190,7 @@ struct bem_ctx {
     std::map<int, bem::Mesh *> meshes;
     int next_mesh = 1;
     std::map<std::tuple<int, int, int>, bem::Rule4D> rules4;   // (case, rule, q)
+    bool has_basis[2] = {false, false};    // meshes of this basis have been uploaded
     bool profile = false;
     std::vector<bem_prof_rec> prof_pending;
     std::vector<cudaEvent_t> prof_free;

@@ -91,10 +91,16 @@ def test_fp64_captured_after_another_call(env, basis, kernel):
     pkg, ctx, stream = env
     mesh = synth.jitter(synth.icosphere(1), 0.05, 7)
     n = mesh.nt if basis == "p0" else mesh.nv
+    quad = dict(q_regular=3, q_identical=5, q_edge=4, q_vertex=3)
+    if basis == "p1":       # the rules' first call is one of the other basis
+        other = ctx.bem_mesh_upload(mesh.verts, mesh.tris, "p0")
+        o = torch.zeros(mesh.nt ** 2, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        ctx.bem_assemble_dense(other, pkg.kernel_desc(kernel), pkg.quad_desc(precision="mixed_full", **quad), 0, o)
+        ctx.bem_sync()
     mid = ctx.bem_mesh_upload(mesh.verts, mesh.tris, basis)
     cplx = kernel.startswith("helmholtz")
     out = torch.zeros(n * n, dtype=torch.complex128 if cplx else torch.float64, device="cuda")
-    quad = dict(q_regular=3, q_identical=5, q_edge=4, q_vertex=3)
     kd = pkg.kernel_desc(kernel, 2.0 if cplx else 0.0)
     torch.cuda.synchronize()
     if cplx:
