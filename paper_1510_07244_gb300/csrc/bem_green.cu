@@ -341,16 +341,24 @@ __global__ void __launch_bounds__(kGreenThreads) k_green(MeshView m, GreenArgs a
         double z[3], n[3];
         s64 Z[3];
         Fx2 N[3];
+        // normals are unit vectors: longer ones leave the fixed-point range (the middle sum
+        // of (x - z).n fills 0.97 of 64 bits at length 1), shorter ones lose digits in it.
+        // Infinite and NaN points or normals fail the tests too (converted to the largest
+        // or the lowest integer); the box that the frame is made of drops a NaN.
+        s64 nn = 0;
+        bool inside = true;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             z[d] = __ldg(a.z + 3 * p + d);
             n[d] = __ldg(a.nz + 3 * p + d);
-            Z[d] = F.ok ? __double2ll_rn((z[d] - F.c0[d]) * fx_pow2(61 - F.E)) << 1 : 0;
+            const s64 zi = F.ok ? __double2ll_rn((z[d] - F.c0[d]) * fx_pow2(61 - F.E)) : 0;
+            inside = inside && abs(fx_high(zi) >> 1) <= 1 << 28;
+            Z[d] = zi << 1;
             N[d] = fx_split(__double2ll_rn(n[d] * 2305843009213693952.0));
+            nn = fx_mad(N[d].h >> 1, N[d].h >> 1, nn);      // 2^56
         }
-        // normals are unit vectors; anything longer leaves the fixed-point range
-        const bool unit = fmax(fmax(fabs(n[0]), fabs(n[1])), fabs(n[2])) <= 1.0;
-        const bool fixed = F.ok && __all_sync(0xffffffffu, unit);
+        inside = inside && abs(fx_high(nn) - (1 << 24)) <= 1 << 14;
+        const bool fixed = F.ok && __all_sync(0xffffffffu, inside);
         double pr = 0.0, pi = 0.0, mr = 0.0, mi = 0.0;
         for (int k = klo; k < khi; ++k) {
             const int tr = m.basis == BEM_P0 ? i : __ldg(m.vt_tri + k);
