@@ -105,10 +105,47 @@ __device__ __forceinline__ int fx_centroid_kb(const s64 X[3][3], const s64 Y[3][
     return fx_kb((sqrtf(d2) - sqrtf(ra) - sqrtf(rb)) * 0.99999f - 8.0f);
 }
 
+// Heights of the test triangle above the trial plane, h(s, t) = h[0] + s h[1] + t h[2]
+// in units of S / 2^(the result), below 2^59 each (a height, a sum of up to three, stays
+// below 2^61).  x: the test vertices relative to the trial triangle's vertex 0.  Each
+// component of x and of the normal is scaled by itself: with one scale for all, heights
+// were held to 2^-58 S, which loses digits of a pair of planes parallel to a coordinate
+// plane (nine points, gap 1e-3 of the size: 2.8e-15 of the terms' magnitudes, FP64
+// arithmetic 3.5e-16, so 3.1e-16; 1% of a double-layer matrix's time).
+__device__ __forceinline__ int fx_heights(const double x[3][3], const Tri &B, int E, s64 h[3])
+{
+    int ex[3], en[3], top = -100000;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int m = max(max(fx_mag(x[0][c]), fx_mag(x[1][c])), fx_mag(x[2][c]));
+        ex[c] = max((m >> 20) - 1022, E - 300);
+        en[c] = max((fx_mag(B.n[c]) >> 20) - 1022, -100);
+        top = max(top, ex[c] + en[c]);
+    }
+    h[0] = h[1] = h[2] = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const Fx2 n = fx_split(__double2ll_rn(B.n[c] * fx_pow2(61 - en[c])));
+        const double sc = fx_pow2(61 - ex[c]);
+        const int down = min(top - ex[c] - en[c], 63);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            h[k] += fx_mul_up<2>(fx_split(__double2ll_rn(x[k][c] * sc)), n) >> down;   // 2^60 / 2^top
+    }
+    h[2] -= h[1];
+    h[1] -= h[0];
+    const s64 m = (h[0] ^ (h[0] >> 63)) | (h[1] ^ (h[1] >> 63)) | (h[2] ^ (h[2] >> 63));
+    const int up = __clzll(m) - 5;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h[k] = up >= 0 ? h[k] << up : h[k] >> -up;
+    return 60 + up - top + E;
+}
+
 // false: out of range (the caller takes the FP64 path).  BOUND: also kb (the
-// single layer's sums of 1/r do without: 2^-55 of the largest possible term).
-template <bool BOUND>
-__device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P)
+// single layer's sums of 1/r do without: 2^-55 of the largest possible term).  HEIGHT:
+// also the heights and their unit (fx_heights).
+template <bool BOUND, bool HEIGHT>
+__device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P, s64 h[3], int &hb)
 {
     double x[3][3], y[3][3];
     int top = 0;
@@ -127,6 +164,7 @@ __device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P)
     const int e = top >> 20;               // the sum is below 2^(e - 1022)
     if (e < 823 || e > 1223) return false;
     P.E = e - 1022;
+    if (HEIGHT) hb = fx_heights(x, B, P.E, h);
     const double sc = fx_pow2(61 - P.E);
     s64 X[3][3], Y[3][3];
 #pragma unroll
@@ -191,20 +229,6 @@ __device__ __forceinline__ int fx_near_kb(const FxPair &P, const Rule2D &R)
         }
     }
     return fx_kb(sqrtf(lo) * 0.9999f - 32.0f);   // roundings: a few units of 2^-24 S
-}
-
-// Heights of the test triangle above the trial plane: h(s, t) = h[0] + s h[1] +
-// t h[2], in units of S / 2^58
-__device__ __forceinline__ void fx_heights(const FxPair &P, const Tri &B, s64 h[3])
-{
-    h[0] = h[1] = h[2] = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const Fx2 n = fx_split(__double2ll_rn(B.n[c] * 2305843009213693952.0));   // 2^61
-        h[0] += fx_mul(fx_split(P.x0[c] << 2), n);
-        h[1] += fx_mul(P.a1[c], n);
-        h[2] += fx_mul(P.a2[c], n);
-    }
 }
 
 // T = 2^(59 - kb) S / r -> 2^(59 - 3 kb) (S / r)^3
@@ -355,15 +379,15 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
 {
     FxPair P;
     FxUnits U;
-    if (!fx_pair<KIND != BEM_LAPLACE_SLP>(A, B, P)) return false;
+    s64 hs[3];
+    int hb;
+    if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
     if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
     if (!fx_units<KIND>(P, kappa, eta, U)) return false;
     double h[3] = {0.0, 0.0, 0.0};
     if (kind_has_height(KIND)) {
-        s64 hs[3];
-        fx_heights(P, B, hs);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-58);
+        for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-hb);
     }
     s64 yx[NP], yy[NP], yz[NP];
 #pragma unroll
@@ -404,7 +428,7 @@ constexpr int kFxUpS = 4, kFxUpD = 5;   // bits that the outer sums take over fr
 // widening multiply-adds per test point; in FP64 three conversions and nine
 // products would take ten times the integer work of a whole point), their
 // arguments 4 and 5 bits up, each product rounded to 2^-57 of the largest.  The double
-// layer's heights are scaled to the largest of their three coefficients.
+// layer's heights come scaled to the largest of their three coefficients.
 template <int KIND, int NP>
 __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
                                          double *accr, double *acci, double eta)
@@ -412,24 +436,20 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
     constexpr bool HELM = kind_complex(KIND);
     FxPair P;
     FxUnits U;
-    if (!fx_pair<KIND != BEM_LAPLACE_SLP>(A, B, P)) return false;
-    if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
-    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
     double h[3] = {0.0, 0.0, 0.0};
     s64 hs[3];
-    int up = 0;
+    int hb;
     Fx2 h1, h2;
+    if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
+    if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
+    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
     if (kind_has_height(KIND)) {
-        fx_heights(P, B, hs);
         if (HELM) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-58);
+            for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-hb);
         } else {
-            // below 2^59 each: a height, a sum of up to three, stays below 2^61
-            const s64 top = (hs[0] ^ (hs[0] >> 63)) | (hs[1] ^ (hs[1] >> 63)) | (hs[2] ^ (hs[2] >> 63));
-            up = max(__clzll(top) - 5, 0);
-            h1 = fx_split(hs[1] << up);
-            h2 = fx_split(hs[2] << up);
+            h1 = fx_split(hs[1]);
+            h2 = fx_split(hs[2]);
         }
     }
     s64 yx[NP], yy[NP], yz[NP];
@@ -460,9 +480,9 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
             I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
         }
         if (!HELM) {
-            Fx2 hi;   // height in units of S / 2^(58 + up)
+            Fx2 hi;   // height in units of S / 2^hb
             if (KIND == BEM_LAPLACE_DLP)
-                hi = fx_split(fx_point((hs[0] << up) >> 2, h1, h2, R.sx[i], R.tx[i]) >> 1);
+                hi = fx_split(fx_point(hs[0] >> 2, h1, h2, R.sx[i], R.tx[i]) >> 1);
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 // sums below 2^57
@@ -490,8 +510,8 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
     double scale = A.sg * B.sg * kInv4Pi * fx_final<KIND>(U);
     if (!HELM) {
         // the outer sum's factor 2 and the bits up; the double layer: also the product's
-        // 2^62 and the heights' 2^(58 + up)
-        scale *= KIND == BEM_LAPLACE_SLP ? fx_pow2(1 - kFxUpS) : fx_pow2(1 + 62 - kFxUpD - (58 + up));
+        // 2^62 and the heights' 2^hb
+        scale *= KIND == BEM_LAPLACE_SLP ? fx_pow2(1 - kFxUpS) : fx_pow2(1 + 62 - kFxUpD - hb);
 #pragma unroll
         for (int k = 0; k < 9; ++k) accr[k] = (double)acc[k] * scale;
     } else {
@@ -515,16 +535,13 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
                                                double *accd)
 {
     FxPair P;
-    if (!fx_pair<true>(A, B, P)) return false;
+    s64 hs[3];
+    int hb;
+    if (!fx_pair<true, true>(A, B, P, hs, hb)) return false;
     if (P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
     const int kb = P.kb;
-    s64 hs[3];
-    fx_heights(P, B, hs);
-    // below 2^59 each: a height, a sum of up to three, stays below 2^61
-    const s64 top = (hs[0] ^ (hs[0] >> 63)) | (hs[1] ^ (hs[1] >> 63)) | (hs[2] ^ (hs[2] >> 63));
-    const int up = max(__clzll(top) - 5, 0);
-    const s64 h0 = (hs[0] << up) >> 2;
-    const Fx2 h1 = fx_split(hs[1] << up), h2 = fx_split(hs[2] << up);
+    const s64 h0 = hs[0] >> 2;
+    const Fx2 h1 = fx_split(hs[1]), h2 = fx_split(hs[2]);
     s64 yx[NP], yy[NP], yz[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
@@ -559,7 +576,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
                 cd[q].add(R.wx[q][j], t3);
             }
         }
-        const Fx2 hi = fx_split(fx_point(h0, h1, h2, R.sx[i], R.tx[i]) >> 1);   // S / 2^(58 + up)
+        const Fx2 hi = fx_split(fx_point(h0, h1, h2, R.sx[i], R.tx[i]) >> 1);   // S / 2^hb
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const Fx2 vs = fx_split(cs[q].template sum<kFxUpS>());
@@ -575,7 +592,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
     // a rule's weights come at 2^63: factor 2 per sum
     const double sc = A.sg * B.sg * kInv4Pi;
     const double fs = sc * fx_pow2(2 - kFxUpS - 55 - P.E);
-    const double fd = sc * fx_pow2(1 - (59 - 3 * kb) - 2 * P.E) * fx_pow2(1 + 62 - kFxUpD - (58 + up));
+    const double fd = sc * fx_pow2(1 - (59 - 3 * kb) - 2 * P.E) * fx_pow2(1 + 62 - kFxUpD - hb);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         accs[k] = (double)as[k] * fs;
