@@ -421,14 +421,37 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
     return (flag >> (16 + P.kb)) == 0;
 }
 
-constexpr int kFxUpS = 4, kFxUpD = 5;   // bits that the outer sums take over from the inner ones
+// Bits that the Laplace kernels' inner sums keep below their values' unit: a sum is at
+// most a twelfth of the largest value, 2^59 for both layers, and stays below 2^62.
+constexpr int kFxUpS = 6, kFxUpD = 5;
+
+__device__ __forceinline__ double fx_scale(double a, int n)   // a 2^n; a, a 2^n zero or normal
+{
+    const int h = __double2hiint(a);
+    return __hiloint2double(h != 0 ? h + (n << 20) : 0, __double2loint(a));
+}
+
+// The double layer's inner sum at one test point times its height: v in [-2^61, 2^61] times
+// h / 2^62, h scaled up to its own digits by 2^lz
+struct FxHeight {
+    Fx2 h;
+    int lz;
+    __device__ __forceinline__ FxHeight(s64 hi)
+    {
+        lz = __clzll(hi ^ (hi >> 63)) - 3;
+        h = fx_split(hi << lz);
+    }
+    __device__ __forceinline__ double times(s64 v) const { return (double)fx_mul_up<2>(fx_split(v), h); }
+};
 
 // Regular pair, piecewise linear (3 x 3 local matrix): regular_p1's integrals.
-// The nine outer sums of the Laplace kernels stay in fixed point too (36
-// widening multiply-adds per test point; in FP64 three conversions and nine
-// products would take ten times the integer work of a whole point), their
-// arguments 4 and 5 bits up, each product rounded to 2^-57 of the largest.  The double
-// layer's heights come scaled to the largest of their three coefficients.
+// The outer sums of the single layer stay in fixed point (27 widening multiply-adds per
+// test point).  The double layer's are FP64, three conversions and nine products per test
+// point beside the integer pipe: fixed-point ones have to leave room for the largest term
+// that S / r and the heights allow, which cost entries up to seven bits (1500 pairs with
+// S / r from 8 to 16, root mean square error over the sum of the terms' magnitudes
+// 3.1e-14, FP64 arithmetic 3.6e-16; from 2 to 4 1.8e-15, now 2.2e-16 against 2.8e-16.
+// Double layer of the 2592-triangle sphere 11.3 -> 12.1 ms).
 template <int KIND, int NP>
 __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
                                          double *accr, double *acci, double eta)
@@ -439,19 +462,14 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
     double h[3] = {0.0, 0.0, 0.0};
     s64 hs[3];
     int hb;
-    Fx2 h1, h2;
     if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
     if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
     if (!fx_units<KIND>(P, kappa, eta, U)) return false;
-    if (kind_has_height(KIND)) {
-        if (HELM) {
+    if (HELM && kind_has_height(KIND)) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-hb);
-        } else {
-            h1 = fx_split(hs[1]);
-            h2 = fx_split(hs[2]);
-        }
+        for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-hb);
     }
+    const Fx2 h1 = fx_split(kind_has_height(KIND) ? hs[1] : 0), h2 = fx_split(kind_has_height(KIND) ? hs[2] : 0);
     s64 yx[NP], yy[NP], yz[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
@@ -479,47 +497,44 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
             const int32_t *w[3] = {R.wx[0][j], R.wx[1][j], R.wx[2][j]};
             I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
         }
-        if (!HELM) {
-            Fx2 hi;   // height in units of S / 2^hb
-            if (KIND == BEM_LAPLACE_DLP)
-                hi = fx_split(fx_point(hs[0] >> 2, h1, h2, R.sx[i], R.tx[i]) >> 1);
+        if (KIND == BEM_LAPLACE_SLP) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                // sums below 2^57
-                s64 v = KIND == BEM_LAPLACE_SLP ? I.c1[q].template sum<kFxUpS>() : I.c3[q].template sum<kFxUpD>();
-                if (KIND == BEM_LAPLACE_DLP) v = fx_mul_up<2>(fx_split(v), hi);
-                const Fx2 V = fx_split(v);
+                const Fx2 V = fx_split(I.c1[q].template sum<kFxUpS>());
 #pragma unroll
                 for (int p = 0; p < 3; ++p) acc[p * 3 + q] += fx_mul(Fx2{R.wx[p][i][0], R.wx[p][i][1]}, V);
+            }
+        } else if (KIND == BEM_LAPLACE_DLP) {
+            const FxHeight H(fx_point(hs[0] >> 2, h1, h2, R.sx[i], R.tx[i]) >> 1);   // S / 2^hb
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const double v = H.times(I.c3[q].template sum<kFxUpD>());
+#pragma unroll
+                for (int p = 0; p < 3; ++p) accr[p * 3 + q] = fma(fx_scale(R.wd[p][i], -H.lz), v, accr[p * 3 + q]);
             }
         } else {
             const double hi = fma(R.t[i], h[2], fma(R.s[i], h[1], h[0]));
             double re[3], im[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) fx_combine<KIND, 3>(I, q, U, hi, re[q], im[q]);
-            const double la[3] = {R.w[i] * (1.0 - R.s[i]), R.w[i] * (R.s[i] - R.t[i]), R.w[i] * R.t[i]};
 #pragma unroll
             for (int p = 0; p < 3; ++p)
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    accr[p * 3 + q] = fma(la[p], re[q], accr[p * 3 + q]);
-                    acci[p * 3 + q] = fma(la[p], im[q], acci[p * 3 + q]);
+                    accr[p * 3 + q] = fma(R.wd[p][i], re[q], accr[p * 3 + q]);
+                    acci[p * 3 + q] = fma(R.wd[p][i], im[q], acci[p * 3 + q]);
                 }
         }
     }
     double scale = A.sg * B.sg * kInv4Pi * fx_final<KIND>(U);
-    if (!HELM) {
-        // the outer sum's factor 2 and the bits up; the double layer: also the product's
-        // 2^62 and the heights' 2^hb
-        scale *= KIND == BEM_LAPLACE_SLP ? fx_pow2(1 - kFxUpS) : fx_pow2(1 + 62 - kFxUpD - hb);
+    // the single layer's outer sums: half, kFxUpS bits up; the double layer's: the product's
+    // 2^62, the heights' 2^hb and kFxUpD
+    if (KIND == BEM_LAPLACE_SLP) scale *= fx_pow2(1 - kFxUpS);
+    if (KIND == BEM_LAPLACE_DLP) scale *= fx_pow2(62 - kFxUpD - hb);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) accr[k] = (double)acc[k] * scale;
-    } else {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            accr[k] *= scale;
-            acci[k] *= scale;
-        }
+    for (int k = 0; k < 9; ++k) {
+        accr[k] = KIND == BEM_LAPLACE_SLP ? (double)acc[k] * scale : accr[k] * scale;
+        if (HELM) acci[k] *= scale;
     }
     return (flag >> (16 + P.kb)) == 0;
 }
@@ -528,8 +543,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
 // matrices): fixed_p1's integrals, sharing points, distances and reciprocal square
 // roots, which are 70 of the 110 instructions of a point of either.  Every layer
 // gets the bits of fixed_p1 (a single call and a plan give the same matrix).  Plan of
-// the 1352-triangle sphere, nine points: 4.77 ms for the layers apart, 3.59 fused
-// (3.98 with the trial points one at a time).
+// the 1352-triangle sphere, nine points: 4.77 ms for the layers apart, 3.76 fused.
 template <int NP>
 __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const Rule2D &R, double *accs,
                                                double *accd)
@@ -550,9 +564,12 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
         yz[j] = fx_point(0, P.b1[2], P.b2[2], R.sx[j], R.tx[j]);
     }
     int flag = 0;
-    s64 as[9], ad[9];
+    s64 as[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) as[k] = ad[k] = 0;
+    for (int k = 0; k < 9; ++k) {
+        as[k] = 0;
+        accd[k] = 0.0;
+    }
 #pragma unroll 1
     for (int i = 0; i < NP; ++i) {
         const s64 xx = fx_point(P.x0[0], P.a1[0], P.a2[0], R.sx[i], R.tx[i]);
@@ -576,27 +593,26 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
                 cd[q].add(R.wx[q][j], t3);
             }
         }
-        const Fx2 hi = fx_split(fx_point(h0, h1, h2, R.sx[i], R.tx[i]) >> 1);   // S / 2^hb
+        const FxHeight H(fx_point(h0, h1, h2, R.sx[i], R.tx[i]) >> 1);   // S / 2^hb
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const Fx2 vs = fx_split(cs[q].template sum<kFxUpS>());
-            const Fx2 vd = fx_split(fx_mul_up<2>(fx_split(cd[q].template sum<kFxUpD>()), hi));
+            const double vd = H.times(cd[q].template sum<kFxUpD>());
 #pragma unroll
             for (int p = 0; p < 3; ++p) {
-                const Fx2 w{R.wx[p][i][0], R.wx[p][i][1]};
-                as[p * 3 + q] += fx_mul(w, vs);
-                ad[p * 3 + q] += fx_mul(w, vd);
+                as[p * 3 + q] += fx_mul(Fx2{R.wx[p][i][0], R.wx[p][i][1]}, vs);
+                accd[p * 3 + q] = fma(fx_scale(R.wd[p][i], -H.lz), vd, accd[p * 3 + q]);
             }
         }
     }
     // a rule's weights come at 2^63: factor 2 per sum
     const double sc = A.sg * B.sg * kInv4Pi;
-    const double fs = sc * fx_pow2(2 - kFxUpS - 55 - P.E);
-    const double fd = sc * fx_pow2(1 - (59 - 3 * kb) - 2 * P.E) * fx_pow2(1 + 62 - kFxUpD - hb);
+    const double fs = sc * fx_pow2(1 - 55 - P.E) * fx_pow2(1 - kFxUpS);
+    const double fd = sc * fx_pow2(1 - (59 - 3 * kb) - 2 * P.E) * fx_pow2(62 - kFxUpD - hb);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         accs[k] = (double)as[k] * fs;
-        accd[k] = (double)ad[k] * fd;
+        accd[k] *= fd;
     }
     return (flag >> (16 + kb)) == 0;
 }

@@ -39,6 +39,7 @@ struct Rule2D {
     // w_k lambda_q(s_k, t_k) in float: the weights times the three linear
     // basis functions of the reference triangle, lambda = (1 - s, s - t, t)
     float wl[3][kMaxNp];
+    double wd[3][kMaxNp];   // the same in double
     // the rule in fixed point (bem_fixed.cuh), high and signed low words: s, t
     // times 2^62; w lambda_q (q < 3) and w (q = 3) times 2^63
     int32_t sx[kMaxNp][2], tx[kMaxNp][2], wx[4][kMaxNp][2];

@@ -103,16 +103,16 @@ static void round_rule(Rule2D &r)
     for (int k = 0; k < r.np; ++k) {
         fixed_words(r.s[k], 62, r.sx[k]);
         fixed_words(r.t[k], 62, r.tx[k]);
-        fixed_words(r.w[k] * (1.0 - r.s[k]), 63, r.wx[0][k]);
-        fixed_words(r.w[k] * (r.s[k] - r.t[k]), 63, r.wx[1][k]);
-        fixed_words(r.w[k] * r.t[k], 63, r.wx[2][k]);
         fixed_words(r.w[k], 63, r.wx[3][k]);
         r.sf[k] = (float)r.s[k];
         r.tf[k] = (float)r.t[k];
         r.wf[k] = (float)r.w[k];
-        r.wl[0][k] = (float)(r.w[k] * (1.0 - r.s[k]));
-        r.wl[1][k] = (float)(r.w[k] * (r.s[k] - r.t[k]));
-        r.wl[2][k] = (float)(r.w[k] * r.t[k]);
+        const double wl[3] = {r.w[k] * (1.0 - r.s[k]), r.w[k] * (r.s[k] - r.t[k]), r.w[k] * r.t[k]};
+        for (int q = 0; q < 3; ++q) {
+            r.wd[q][k] = wl[q];
+            r.wl[q][k] = (float)wl[q];
+            fixed_words(wl[q], 63, r.wx[q][k]);
+        }
     }
 }
 
