@@ -10,6 +10,13 @@ namespace bem {
 
 __device__ __forceinline__ double fx_pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
 
+// a 2^n by its exponent (an integer operation); a and a 2^n zero or normal
+__device__ __forceinline__ double fx_scale(double a, int n)
+{
+    const int h = __double2hiint(a);
+    return __hiloint2double(h != 0 ? h + (n << 20) : 0, __double2loint(a));
+}
+
 // Upper bound of |a|: the high word of a double, its lowest bit raised
 __device__ __forceinline__ int fx_mag(double a) { return (__double2hiint(a) & 0x7fffffff) + 1; }
 
@@ -195,13 +202,18 @@ __device__ __forceinline__ s64 fx_point(s64 v0, Fx2 e1, Fx2 e2, const int32_t *s
     return fx_mad(e1.h, s[0], fx_mad(e2.h, t[0], v0 + fx_high(mid))) << 3;
 }
 
-// kb of near pairs from their points: the powers of 1/r of the double layers
-// lose 2 or 3 bits per unit of an overestimated kb.  The centroid bound is within
-// a factor 2 for pairs apart; for the others (kb >= 3) the smallest distance of
-// the rule's points in float, 7 FP32 operations per point.
+// kb of every test point (four bits each, point 0 lowest): the powers of 1/r of the
+// double layers lose 2 or 3 bits per unit of an overestimated kb.  The centroid bound is
+// within a factor 2 for pairs apart; for the others (kb >= 3) the smallest distance of
+// the test point to the rule's trial points in float, 7 FP32 operations per point.  One
+// kb for the pair would let near test points, whose heights may vanish, cost the others
+// their bits (1500 pairs with S / r from 8 to 16, root mean square error over the sum of
+// the terms' magnitudes: Helmholtz double layer 4.6e-16, piecewise linear 1.6e-15; so
+// 1.8e-16 and 2.6e-16; FP64 arithmetic 2.6e-16 and 3.0e-16).
 template <int NP>
-__device__ __forceinline__ int fx_near_kb(const FxPair &P, const Rule2D &R)
+__device__ __forceinline__ u64 fx_near_kb(const FxPair &P, const Rule2D &R)
 {
+    static_assert(NP <= 16, "four bits per test point");
     float a0[3], a1[3], a2[3], b1[3], b2[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -211,25 +223,31 @@ __device__ __forceinline__ int fx_near_kb(const FxPair &P, const Rule2D &R)
         b1[c] = (float)P.b1[c].h;
         b2[c] = (float)P.b2[c].h;
     }
-    float lo = 3.0e38f;
+    u64 kbs = 0;
 #pragma unroll 1
-    for (int j = 0; j < NP; ++j) {
-        float y[3];
+    for (int i = 0; i < NP; ++i) {
+        float x[3], lo = 3.0e38f;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) y[c] = fmaf(R.sf[j], b1[c], R.tf[j] * b2[c]) - a0[c];
+        for (int c = 0; c < 3; ++c) x[c] = fmaf(R.sf[i], a1[c], fmaf(R.tf[i], a2[c], a0[c]));
 #pragma unroll 3
-        for (int i = 0; i < NP; ++i) {
+        for (int j = 0; j < NP; ++j) {
             float d2 = 0.0f;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float d = fmaf(R.sf[i], a1[c], fmaf(R.tf[i], a2[c], -y[c]));
+                const float d = fmaf(-R.sf[j], b1[c], fmaf(-R.tf[j], b2[c], x[c]));
                 d2 = fmaf(d, d, d2);
             }
             lo = fminf(lo, d2);
         }
+        // roundings: a few units of 2^-24 S
+        kbs |= (u64)fx_kb(sqrtf(lo) * 0.9999f - 32.0f) << (4 * i);
     }
-    return fx_kb(sqrtf(lo) * 0.9999f - 32.0f);   // roundings: a few units of 2^-24 S
+    return kbs;
 }
+
+// The same for every test point
+__device__ __forceinline__ u64 fx_one_kb(int kb) { return 0x1111111111111111ull * (unsigned)kb; }
+__device__ __forceinline__ int fx_kb_of(u64 kbs, int i) { return (int)(kbs >> (4 * i)) & 15; }
 
 // T = 2^(59 - kb) S / r -> 2^(59 - 3 kb) (S / r)^3
 __device__ __forceinline__ Fx2 fx_inverse_cube(Fx2 T)
@@ -309,17 +327,21 @@ struct FxInner {
     }
 };
 
-// The factors that take FxInner's sums to the kernel's value (without 1/(4 pi))
+// The factors that take FxInner's sums at kb to the kernel's value (without 1/(4 pi))
 struct FxUnits {
     double f1, f2, f3;      // 1/r, kappa / r^2, 1/r^3 (with S for the height's unit)
     Fx2 kn;                 // kappa S / (2 pi) = kn 2^(kexp - 62)
     int shl;
+    // the same at kb + n
+    __device__ __forceinline__ FxUnits at(int n) const
+    {
+        return FxUnits{fx_scale(f1, n), fx_scale(f2, 2 * n), fx_scale(f3, 3 * n), kn, shl + n};
+    }
 };
 
 template <int KIND>
-__device__ __forceinline__ bool fx_units(const FxPair &P, double kappa, double eta, FxUnits &U)
+__device__ __forceinline__ bool fx_units(const FxPair &P, int kb, double kappa, double eta, FxUnits &U)
 {
-    const int kb = P.kb;
     U.f1 = fx_pow2(1 - (59 - kb) - P.E);
     if (KIND == BEM_HELMHOLTZ_BW) U.f1 *= eta;
     U.f2 = U.f3 = 0.0;
@@ -382,10 +404,12 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
     s64 hs[3];
     int hb;
     if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
-    if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
-    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
+    constexpr bool HEIGHT = kind_has_height(KIND);
+    u64 kbs = 0;
+    if (HEIGHT) kbs = P.kb >= 3 ? fx_near_kb<NP>(P, R) : fx_one_kb(P.kb);
+    if (!fx_units<KIND>(P, HEIGHT ? 0 : P.kb, kappa, eta, U)) return false;
     double h[3] = {0.0, 0.0, 0.0};
-    if (kind_has_height(KIND)) {
+    if (HEIGHT) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-hb);
     }
@@ -396,40 +420,38 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
         yy[j] = fx_point(0, P.b1[1], P.b2[1], R.sx[j], R.tx[j]);
         yz[j] = fx_point(0, P.b1[2], P.b2[2], R.sx[j], R.tx[j]);
     }
-    int flag = 0;
+    int bad = 0;
     double sr = 0.0, si = 0.0;
 #pragma unroll 1
     for (int i = 0; i < NP; ++i) {
         const s64 xx = fx_point(P.x0[0], P.a1[0], P.a2[0], R.sx[i], R.tx[i]);
         const s64 xy = fx_point(P.x0[1], P.a1[1], P.a2[1], R.sx[i], R.tx[i]);
         const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
+        const int kb = HEIGHT ? fx_kb_of(kbs, i) : P.kb;
+        const FxUnits Ui = HEIGHT ? U.at(kb) : U;
+        int flag = 0;
         FxInner<KIND, 1> I;
         I.clear();
 #pragma unroll kFxUnroll
         for (int j = 0; j < NP; ++j) {
             const int32_t *w[1] = {R.wx[3][j]};
-            I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
+            I.point(xx - yx[j], xy - yy[j], xz - yz[j], kb, Ui.kn, Ui.shl, w, flag);
         }
         double re, im;
-        fx_combine<KIND, 1>(I, 0, U, fma(R.t[i], h[2], fma(R.s[i], h[1], h[0])), re, im);
-        sr = fma(R.w[i], re, sr);
+        fx_combine<KIND, 1>(I, 0, Ui, fma(R.t[i], h[2], fma(R.s[i], h[1], h[0])), re, im);
+        bad |= flag >> (16 + kb);
+        sr = fma(KIND == BEM_LAPLACE_DLP ? fx_scale(R.w[i], 3 * kb) : R.w[i], re, sr);
         if (kind_complex(KIND)) si = fma(R.w[i], im, si);
     }
     const double scale = A.sg * B.sg * kInv4Pi * fx_final<KIND>(U);
     out_re = sr * scale;
     out_im = si * scale;
-    return (flag >> (16 + P.kb)) == 0;
+    return bad == 0;
 }
 
 // Bits that the Laplace kernels' inner sums keep below their values' unit: a sum is at
 // most a twelfth of the largest value, 2^59 for both layers, and stays below 2^62.
 constexpr int kFxUpS = 6, kFxUpD = 5;
-
-__device__ __forceinline__ double fx_scale(double a, int n)   // a 2^n; a, a 2^n zero or normal
-{
-    const int h = __double2hiint(a);
-    return __hiloint2double(h != 0 ? h + (n << 20) : 0, __double2loint(a));
-}
 
 // The double layer's inner sum at one test point times its height: v in [-2^61, 2^61] times
 // h / 2^62, h scaled up to its own digits by 2^lz
@@ -456,20 +478,21 @@ template <int KIND, int NP>
 __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
                                          double *accr, double *acci, double eta)
 {
-    constexpr bool HELM = kind_complex(KIND);
+    constexpr bool HELM = kind_complex(KIND), HEIGHT = kind_has_height(KIND);
     FxPair P;
     FxUnits U;
     double h[3] = {0.0, 0.0, 0.0};
     s64 hs[3];
     int hb;
     if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
-    if (kind_has_height(KIND) && P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
-    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
-    if (HELM && kind_has_height(KIND)) {
+    u64 kbs = 0;
+    if (HEIGHT) kbs = P.kb >= 3 ? fx_near_kb<NP>(P, R) : fx_one_kb(P.kb);
+    if (!fx_units<KIND>(P, HEIGHT ? 0 : P.kb, kappa, eta, U)) return false;
+    if (HELM && HEIGHT) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) h[k] = (double)hs[k] * fx_pow2(-hb);
     }
-    const Fx2 h1 = fx_split(kind_has_height(KIND) ? hs[1] : 0), h2 = fx_split(kind_has_height(KIND) ? hs[2] : 0);
+    const Fx2 h1 = fx_split(HEIGHT ? hs[1] : 0), h2 = fx_split(HEIGHT ? hs[2] : 0);
     s64 yx[NP], yy[NP], yz[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
@@ -477,7 +500,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
         yy[j] = fx_point(0, P.b1[1], P.b2[1], R.sx[j], R.tx[j]);
         yz[j] = fx_point(0, P.b1[2], P.b2[2], R.sx[j], R.tx[j]);
     }
-    int flag = 0;
+    int bad = 0;
     s64 acc[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
@@ -489,14 +512,18 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
         const s64 xx = fx_point(P.x0[0], P.a1[0], P.a2[0], R.sx[i], R.tx[i]);
         const s64 xy = fx_point(P.x0[1], P.a1[1], P.a2[1], R.sx[i], R.tx[i]);
         const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
+        const int kb = HEIGHT ? fx_kb_of(kbs, i) : P.kb;
+        const FxUnits Ui = HEIGHT ? U.at(kb) : U;
+        int flag = 0;
         FxInner<KIND, 3> I;
         I.template clear<HELM ? 0 : kFxUpS, HELM ? 0 : kFxUpD>();
         constexpr int UN = HELM ? 1 : kFxUnroll;   // the complex sums want the registers
 #pragma unroll UN
         for (int j = 0; j < NP; ++j) {
             const int32_t *w[3] = {R.wx[0][j], R.wx[1][j], R.wx[2][j]};
-            I.point(xx - yx[j], xy - yy[j], xz - yz[j], P.kb, U.kn, U.shl, w, flag);
+            I.point(xx - yx[j], xy - yy[j], xz - yz[j], kb, Ui.kn, Ui.shl, w, flag);
         }
+        bad |= flag >> (16 + kb);
         if (KIND == BEM_LAPLACE_SLP) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
@@ -510,13 +537,13 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
             for (int q = 0; q < 3; ++q) {
                 const double v = H.times(I.c3[q].template sum<kFxUpD>());
 #pragma unroll
-                for (int p = 0; p < 3; ++p) accr[p * 3 + q] = fma(fx_scale(R.wd[p][i], -H.lz), v, accr[p * 3 + q]);
+                for (int p = 0; p < 3; ++p) accr[p * 3 + q] = fma(fx_scale(R.wd[p][i], 3 * kb - H.lz), v, accr[p * 3 + q]);
             }
         } else {
             const double hi = fma(R.t[i], h[2], fma(R.s[i], h[1], h[0]));
             double re[3], im[3];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) fx_combine<KIND, 3>(I, q, U, hi, re[q], im[q]);
+            for (int q = 0; q < 3; ++q) fx_combine<KIND, 3>(I, q, Ui, hi, re[q], im[q]);
 #pragma unroll
             for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -536,7 +563,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
         accr[k] = KIND == BEM_LAPLACE_SLP ? (double)acc[k] * scale : accr[k] * scale;
         if (HELM) acci[k] *= scale;
     }
-    return (flag >> (16 + P.kb)) == 0;
+    return bad == 0;
 }
 
 // Both Laplace layers of a regular pair, piecewise linear (two 3 x 3 local
@@ -552,8 +579,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
     s64 hs[3];
     int hb;
     if (!fx_pair<true, true>(A, B, P, hs, hb)) return false;
-    if (P.kb >= 3) P.kb = fx_near_kb<NP>(P, R);
-    const int kb = P.kb;
+    const u64 kbs = P.kb >= 3 ? fx_near_kb<NP>(P, R) : fx_one_kb(P.kb);
     const s64 h0 = hs[0] >> 2;
     const Fx2 h1 = fx_split(hs[1]), h2 = fx_split(hs[2]);
     s64 yx[NP], yy[NP], yz[NP];
@@ -563,7 +589,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
         yy[j] = fx_point(0, P.b1[1], P.b2[1], R.sx[j], R.tx[j]);
         yz[j] = fx_point(0, P.b1[2], P.b2[2], R.sx[j], R.tx[j]);
     }
-    int flag = 0;
+    int bad = 0;
     s64 as[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
@@ -575,6 +601,8 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
         const s64 xx = fx_point(P.x0[0], P.a1[0], P.a2[0], R.sx[i], R.tx[i]);
         const s64 xy = fx_point(P.x0[1], P.a1[1], P.a2[1], R.sx[i], R.tx[i]);
         const s64 xz = fx_point(P.x0[2], P.a1[2], P.a2[2], R.sx[i], R.tx[i]);
+        const int kb = fx_kb_of(kbs, i);
+        int flag = 0;
         FxSum cs[3], cd[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -593,6 +621,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
                 cd[q].add(R.wx[q][j], t3);
             }
         }
+        bad |= flag >> (16 + kb);
         const FxHeight H(fx_point(h0, h1, h2, R.sx[i], R.tx[i]) >> 1);   // S / 2^hb
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -601,20 +630,20 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
 #pragma unroll
             for (int p = 0; p < 3; ++p) {
                 as[p * 3 + q] += fx_mul(Fx2{R.wx[p][i][0], R.wx[p][i][1]}, vs);
-                accd[p * 3 + q] = fma(fx_scale(R.wd[p][i], -H.lz), vd, accd[p * 3 + q]);
+                accd[p * 3 + q] = fma(fx_scale(R.wd[p][i], 3 * kb - H.lz), vd, accd[p * 3 + q]);
             }
         }
     }
     // a rule's weights come at 2^63: factor 2 per sum
     const double sc = A.sg * B.sg * kInv4Pi;
     const double fs = sc * fx_pow2(1 - 55 - P.E) * fx_pow2(1 - kFxUpS);
-    const double fd = sc * fx_pow2(1 - (59 - 3 * kb) - 2 * P.E) * fx_pow2(62 - kFxUpD - hb);
+    const double fd = sc * fx_pow2(1 - 59 - 2 * P.E) * fx_pow2(62 - kFxUpD - hb);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         accs[k] = (double)as[k] * fs;
         accd[k] *= fd;
     }
-    return (flag >> (16 + kb)) == 0;
+    return bad == 0;
 }
 
 }  // namespace bem

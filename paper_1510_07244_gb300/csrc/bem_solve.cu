@@ -92,7 +92,7 @@ __device__ __forceinline__ bool potential_fixed(const double *z, const Tri &B, c
     }
     P.kb = KIND == BEM_LAPLACE_SLP ? 4 : fx_kb((sqrtf(d2) - sqrtf(rb)) * 0.99999f - 8.0f);
     FxUnits U;
-    if (!fx_units<KIND>(P, kappa, eta, U)) return false;
+    if (!fx_units<KIND>(P, P.kb, kappa, eta, U)) return false;
     FxInner<KIND, 1> I;
     I.clear();
     int flag = 0;

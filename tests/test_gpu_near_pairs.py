@@ -46,7 +46,7 @@ def _pairs(n, near, seed):
 
 
 @pytest.mark.parametrize("near", [4, 8, 16])
-@pytest.mark.parametrize("kernel", ["laplace_slp", "laplace_dlp"])
+@pytest.mark.parametrize("kernel", ["laplace_slp", "laplace_dlp", "helmholtz_dlp"])
 @pytest.mark.parametrize("basis", ["p0", "p1"])
 def test_near_pairs(env, basis, kernel, near):  # noqa: F811
     import torch
