@@ -58,7 +58,8 @@ struct FxSum {
         if (K == 0) return p;
         return fx_join(fx_funnel_l(fx_low(mid), fx_low(p), K), (int)fx_funnel_l(fx_low(p), (unsigned)fx_high(p), K));
     }
-    __device__ __forceinline__ double value() const { return (double)sum(); }
+    template <int K = 0>
+    __device__ __forceinline__ double value() const { return (double)sum<K>(); }
 };
 
 // Vertices of a pair relative to the trial triangle's vertex 0, scaled to
@@ -268,13 +269,13 @@ struct FxInner {
     static constexpr bool P3 = KIND == BEM_LAPLACE_DLP || KIND == BEM_HELMHOLTZ_DLP ||
                                KIND == BEM_HELMHOLTZ_BW;
     FxSum c1[NM], s1[NM], c2[NM], s2[NM], c3[NM], s3[NM];
-    template <int K1 = 0, int K3 = 0>
+    template <int K1 = 0, int K3 = 0, int K = 0>
     __device__ __forceinline__ void clear()
     {
 #pragma unroll
         for (int q = 0; q < NM; ++q) {
-            c1[q].template clear<K1>(); s1[q].clear(); c2[q].clear();
-            s2[q].clear(); c3[q].template clear<K3>(); s3[q].clear();
+            c1[q].template clear<K + K1>(); s1[q].template clear<K>(); c2[q].template clear<K>();
+            s2[q].template clear<K>(); c3[q].template clear<K + K3>(); s3[q].template clear<K>();
         }
     }
     __device__ __forceinline__ void point(s64 dx, s64 dy, s64 dz, int kb, Fx2 kn, int shl,
@@ -358,25 +359,25 @@ __device__ __forceinline__ bool fx_units(const FxPair &P, int kb, double kappa, 
     return true;
 }
 
-// FxInner's sums q -> kernel sums (re, im); h: height / S
-template <int KIND, int NM>
+// FxInner's sums q -> kernel sums (re, im), times 2^K; h: height / S
+template <int KIND, int NM, int K = 0>
 __device__ __forceinline__ void fx_combine(const FxInner<KIND, NM> &I, int q, const FxUnits &U, double h,
                                            double &re, double &im)
 {
     im = 0.0;
     if (KIND == BEM_LAPLACE_SLP) {
-        re = I.c1[q].value();          // factor f1 at the end
+        re = I.c1[q].template value<K>();          // factor f1 at the end
     } else if (KIND == BEM_LAPLACE_DLP) {
-        re = h * I.c3[q].value();      // factor f3 at the end
+        re = h * I.c3[q].template value<K>();      // factor f3 at the end
     } else if (KIND == BEM_HELMHOLTZ_SLP) {
-        re = I.c1[q].value();
-        im = I.s1[q].value();
+        re = I.c1[q].template value<K>();
+        im = I.s1[q].template value<K>();
     } else {
-        re = h * fma(U.f3, I.c3[q].value(), U.f2 * I.s2[q].value());
-        im = h * fma(U.f3, I.s3[q].value(), -U.f2 * I.c2[q].value());
+        re = h * fma(U.f3, I.c3[q].template value<K>(), U.f2 * I.s2[q].template value<K>());
+        im = h * fma(U.f3, I.s3[q].template value<K>(), -U.f2 * I.c2[q].template value<K>());
         if (KIND == BEM_HELMHOLTZ_BW) {
-            re = fma(U.f1, I.s1[q].value(), re);
-            im = fma(-U.f1, I.c1[q].value(), im);
+            re = fma(U.f1, I.s1[q].template value<K>(), re);
+            im = fma(-U.f1, I.c1[q].template value<K>(), im);
         }
     }
 }

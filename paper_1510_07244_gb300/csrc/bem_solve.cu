@@ -52,36 +52,37 @@ template <int KIND>
 __device__ __forceinline__ bool potential_fixed(const double *z, const Tri &B, const Rule2D &R,
                                                 double kappa, double eta, double &sr, double &si)
 {
-    double x[3], y[2][3], h = 0.0;
+    // the vertices relative to z, whose roundings are independent (a common one of z
+    // relative to a vertex would not average out over the points)
+    double y[3][3], h = 0.0;
     int top = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        x[c] = z[c] - B.v[0][c];
-        y[0][c] = B.v[1][c] - B.v[0][c];
-        y[1][c] = B.v[2][c] - B.v[0][c];
-        h = fma(x[c], B.n[c], h);
-        const int my = max(fx_mag(y[0][c]), fx_mag(y[1][c]));
-        top = max(top, fx_mag(__hiloint2double(fx_mag(x[c]), 0) + __hiloint2double(my, 0)));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            y[k][c] = B.v[k][c] - z[c];
+            top = max(top, fx_mag(y[k][c]));
+        }
+        h = fma(-y[0][c], B.n[c], h);
     }
     const int e = top >> 20;
     if (e < 823 || e > 1223) return false;
     FxPair P;
     P.E = e - 1022;
     const double sc = fx_pow2(61 - P.E);
-    s64 X[3];
+    s64 Y0[3];
     float d2 = 0.0f, rb = 0.0f, cb[3], yf[3][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        X[c] = __double2ll_rn(x[c] * sc);
-        const s64 y1 = __double2ll_rn(y[0][c] * sc), y2 = __double2ll_rn(y[1][c] * sc);
-        P.b1[c] = fx_split(y1);
+        Y0[c] = __double2ll_rn(y[0][c] * sc);
+        const s64 y1 = __double2ll_rn(y[1][c] * sc), y2 = __double2ll_rn(y[2][c] * sc);
+        P.b1[c] = fx_split(y1 - Y0[c]);
         P.b2[c] = fx_split(y2 - y1);
-        yf[0][c] = 0.0f;
+        yf[0][c] = fx_hi(Y0[c]);   // S = 2^29
         yf[1][c] = fx_hi(y1);
         yf[2][c] = fx_hi(y2);
-        cb[c] = (yf[1][c] + yf[2][c]) * (1.0f / 3.0f);
-        const float d = fx_hi(X[c]) - cb[c];
-        d2 = fmaf(d, d, d2);
+        cb[c] = (yf[0][c] + yf[1][c] + yf[2][c]) * (1.0f / 3.0f);
+        d2 = fmaf(cb[c], cb[c], d2);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -91,21 +92,41 @@ __device__ __forceinline__ bool potential_fixed(const double *z, const Tri &B, c
         rb = fmaxf(rb, v);
     }
     P.kb = KIND == BEM_LAPLACE_SLP ? 4 : fx_kb((sqrtf(d2) - sqrtf(rb)) * 0.99999f - 8.0f);
+    if (kind_has_height(KIND) && P.kb >= 3) {
+        // from the rule's points (fx_near_kb): the bound of a point beside a triangle has
+        // no digits left (8000 points, Brakhage-Werner kernel, root mean square error over
+        // the sum of the terms' magnitudes 1.9e-15, so 3.2e-16; FP64 arithmetic 2.9e-16)
+        float lo = 3.0e38f;
+#pragma unroll 1
+        for (int k = 0; k < R.np; ++k) {
+            d2 = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float d = fmaf(R.sf[k], yf[1][c] - yf[0][c], fmaf(R.tf[k], yf[2][c] - yf[1][c], yf[0][c]));
+                d2 = fmaf(d, d, d2);
+            }
+            lo = fminf(lo, d2);
+        }
+        P.kb = fx_kb(sqrtf(lo) * 0.9999f - 32.0f);
+    }
     FxUnits U;
     if (!fx_units<KIND>(P, P.kb, kappa, eta, U)) return false;
+    // the sums (half of the weighted ones, whose weights add to a half) stay below 2^57;
+    // four of their fraction's bits count here, where no outer sum averages the rounding
+    constexpr int UP = 4;
     FxInner<KIND, 1> I;
-    I.clear();
+    I.template clear<0, 0, UP>();
     int flag = 0;
 #pragma unroll 1
     for (int k = 0; k < R.np; ++k) {
         s64 d[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) d[c] = (X[c] << 1) - fx_point(0, P.b1[c], P.b2[c], R.sx[k], R.tx[k]);
+        for (int c = 0; c < 3; ++c) d[c] = (Y0[c] << 1) + fx_point(0, P.b1[c], P.b2[c], R.sx[k], R.tx[k]);
         const int32_t *w[1] = {R.wx[3][k]};
         I.point(d[0], d[1], d[2], P.kb, U.kn, U.shl, w, flag);
     }
-    fx_combine<KIND, 1>(I, 0, U, h * fx_pow2(-P.E), sr, si);
-    const double f = fx_final<KIND>(U);
+    fx_combine<KIND, 1, UP>(I, 0, U, h * fx_pow2(-P.E), sr, si);
+    const double f = fx_final<KIND>(U) * fx_pow2(-UP);
     sr *= f;
     si *= f;
     return (flag >> (16 + P.kb)) == 0;
