@@ -149,6 +149,15 @@ BEM_HD s64 fx_mul_up(Fx2 a, Fx2 b)
                    (int)fx_funnel_l(fx_low(p), (unsigned)fx_high(p), K));
 }
 
+// the same, 0 <= n < 32 bits
+BEM_HD s64 fx_mul_up(Fx2 a, Fx2 b, int n)
+{
+    const s64 mid = fx_mad(a.h, b.l, fx_mad(a.l, b.h, (s64)(1u << (31 - n))));
+    const s64 p = fx_mad(a.h, b.h, fx_high(mid));
+    return fx_join(fx_funnel_l(fx_low(mid), fx_low(p), n),
+                   (int)fx_funnel_l(fx_low(p), (unsigned)fx_high(p), n));
+}
+
 BEM_HD int fx_float_bits(float f)
 {
 #ifdef __CUDA_ARCH__

@@ -68,10 +68,10 @@ enum FxTouchCol {
     kFxX = 0,     // vertex: x1, x2, y1, y2; edge: d1, x2, y2; identical: d1, d2; each / g
     // piecewise constant
     kFxG = 4,     // g
-    kFxA = 5,     // w / g (terms in 1/r)
-    kFxB = 6,     // w h_k / g^3 (1/r^3): h_k = x1, x2, the coefficients of the heights
-    kFxC = 8,     // w h_k / g^2 (1/r^2)
-    kFxCols0 = 10,
+    kFxA = 5,     // w / g (terms in 1/r; a common vertex: every term)
+    kFxB = 6,     // common edge: w x2 / g^3 (1/r^3; its heights are x2 times one number)
+    kFxC = 7,     // common edge: w x2 / g^2 (1/r^2)
+    kFxCols0 = 8,
     // piecewise linear (Laplace kernels)
     kFxMS = 4,    // (w / g) x^i y^j, i, j = 0..2 (single layer)
     kFxMD = 13,   // vertex: w x^i y^j; edge: (w x2 / g^3) x^i y^j (double layer)

@@ -283,9 +283,9 @@ bool make_touch_fixed(int cas, int q, int basis, std::vector<int32_t> &words)
                         if (basis == BEM_P0) {
                             put(kFxG, g, 62);
                             put(kFxA, w / g, 63);
-                            for (int h = cas == kVertex ? 0 : 1; h < 2 && cas != kIdentical; ++h) {
-                                put(kFxB + h, w * x[1 + h] / (g * g * g), 63);
-                                put(kFxC + h, w * x[1 + h] / (g * g), 63);
+                            if (cas == kEdge) {
+                                put(kFxB, wd, 63);
+                                put(kFxC, w * t.x2 / (g * g), 63);
                             }
                         } else {
                             for (int i = 0; i < 9; ++i) {
