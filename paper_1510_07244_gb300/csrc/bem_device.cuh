@@ -1411,26 +1411,37 @@ __device__ __forceinline__ void touch_f32(const MeshView &m, int idx, const floa
 
 // ---------------------------------------------------------------------------
 // Regular pair integrals in FP64 arithmetic (product of a 2D rule with itself):
-// the few pairs whose distances span more than the fixed-point range of
-// bem_fixed_pair.cuh.  Not inlined, loops rolled: one small copy per kernel.
+// pairs whose distances span more than the fixed-point range of bem_fixed_pair.cuh, a
+// few of shape-regular meshes and most of a near field of triangles stretched 100:1.
+// Bound by the FP64 pipe: the trial points are formed once per pair (local memory), the
+// weights times hat functions come from the rule.  Not inlined, loops rolled: one small
+// copy per kernel.  2592 triangles stretched 100:1, near field: single layer 2.01 ms (FP64
+// arithmetic for every pair 2.53, points formed anew for every pair of them 2.55); both
+// piecewise-linear layers of 1352 triangles in a plan 29.8 ms (34.0, 46.8).
 // ---------------------------------------------------------------------------
-// Trial points relative to B's vertex 0, test points relative to them
-struct PairFrame {
-    double d0[3], e1a[3], e2a[3], e1b[3], e2b[3];
-    __device__ __forceinline__ PairFrame(const Tri &A, const Tri &B)
+struct PairPoints {
+    double d0[3], e1[3], e2[3];   // test triangle relative to the trial vertex 0
+    double y[kMaxNp][3];
+    __device__ __forceinline__ PairPoints(const Tri &A, const Tri &B, const Rule2D &R)
     {
+        double f1[3], f2[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             d0[c] = A.v[0][c] - B.v[0][c];
-            e1a[c] = A.v[1][c] - A.v[0][c];
-            e2a[c] = A.v[2][c] - A.v[1][c];
-            e1b[c] = B.v[1][c] - B.v[0][c];
-            e2b[c] = B.v[2][c] - B.v[1][c];
+            e1[c] = A.v[1][c] - A.v[0][c];
+            e2[c] = A.v[2][c] - A.v[1][c];
+            f1[c] = B.v[1][c] - B.v[0][c];
+            f2[c] = B.v[2][c] - B.v[1][c];
         }
+#pragma unroll 1
+        for (int j = 0; j < R.np; ++j)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) y[j][c] = R.s[j] * f1[c] + R.t[j] * f2[c];
     }
-    __device__ __forceinline__ double diff(int c, double s, double t, double u, double v) const
+    __device__ __forceinline__ void test(const Rule2D &R, int i, double x[3]) const
     {
-        return (d0[c] + s * e1a[c] + t * e2a[c]) - (u * e1b[c] + v * e2b[c]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[c] = d0[c] + R.s[i] * e1[c] + R.t[i] * e2[c];
     }
 };
 
@@ -1438,16 +1449,16 @@ template <int KIND>
 __device__ __noinline__ void double_p0(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
                                        double &out_re, double &out_im, double eta)
 {
-    const PairFrame F(A, B);
+    const PairPoints P(A, B, R);
     double sr = 0.0, si = 0.0;
 #pragma unroll 1
     for (int i = 0; i < R.np; ++i) {
-        double ir = 0.0, ii = 0.0;
+        double x[3], ir = 0.0, ii = 0.0;
+        P.test(R, i, x);
 #pragma unroll 1
         for (int j = 0; j < R.np; ++j) {
             double kr, ki;
-            kval<KIND>(F.diff(0, R.s[i], R.t[i], R.s[j], R.t[j]), F.diff(1, R.s[i], R.t[i], R.s[j], R.t[j]),
-                       F.diff(2, R.s[i], R.t[i], R.s[j], R.t[j]), B.n, kappa, kr, ki, eta);
+            kval<KIND>(x[0] - P.y[j][0], x[1] - P.y[j][1], x[2] - P.y[j][2], B.n, kappa, kr, ki, eta);
             ir += R.w[j] * kr;
             if (kind_complex(KIND)) ii += R.w[j] * ki;
         }
@@ -1463,33 +1474,37 @@ template <int KIND>
 __device__ __noinline__ void double_p1(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
                                        double *accr, double *acci, double eta)
 {
-    const PairFrame F(A, B);
-#pragma unroll 1
-    for (int k = 0; k < 9; ++k) accr[k] = acci[k] = 0.0;
-    const double scale = A.sg * B.sg * kInv4Pi;
+    const PairPoints P(A, B, R);
+    double sr[9], si[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) sr[k] = si[k] = 0.0;
 #pragma unroll 1
     for (int i = 0; i < R.np; ++i) {
-        double ir[3] = {0.0, 0.0, 0.0}, ii[3] = {0.0, 0.0, 0.0};
+        double x[3], ir[3] = {0.0, 0.0, 0.0}, ii[3] = {0.0, 0.0, 0.0};
+        P.test(R, i, x);
 #pragma unroll 1
         for (int j = 0; j < R.np; ++j) {
             double kr, ki;
-            kval<KIND>(F.diff(0, R.s[i], R.t[i], R.s[j], R.t[j]), F.diff(1, R.s[i], R.t[i], R.s[j], R.t[j]),
-                       F.diff(2, R.s[i], R.t[i], R.s[j], R.t[j]), B.n, kappa, kr, ki, eta);
-            const double lb[3] = {1.0 - R.s[j], R.s[j] - R.t[j], R.t[j]};
+            kval<KIND>(x[0] - P.y[j][0], x[1] - P.y[j][1], x[2] - P.y[j][2], B.n, kappa, kr, ki, eta);
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                ir[q] += R.w[j] * kr * lb[q];
-                ii[q] += R.w[j] * ki * lb[q];
+                ir[q] += R.wd[q][j] * kr;
+                if (kind_complex(KIND)) ii[q] += R.wd[q][j] * ki;
             }
         }
-        const double la[3] = {1.0 - R.s[i], R.s[i] - R.t[i], R.t[i]};
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                accr[p * 3 + q] += R.w[i] * la[p] * ir[q] * scale;
-                if (kind_complex(KIND)) acci[p * 3 + q] += R.w[i] * la[p] * ii[q] * scale;
+                sr[p * 3 + q] += R.wd[p][i] * ir[q];
+                if (kind_complex(KIND)) si[p * 3 + q] += R.wd[p][i] * ii[q];
             }
+    }
+    const double scale = A.sg * B.sg * kInv4Pi;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        accr[k] = sr[k] * scale;
+        acci[k] = si[k] * scale;
     }
 }
 
@@ -1515,14 +1530,6 @@ __device__ __forceinline__ void regular_p1(const Tri &A, const Tri &B, const Rul
 {
     if (!fixed_p1<KIND, NP>(A, B, R, kappa, accr, acci, eta))
         double_p1<KIND>(A, B, R, kappa, accr, acci, eta);
-}
-
-// One layer of a pair that fixed_p1_fused leaves
-template <int KIND, int NP>
-__device__ __noinline__ void layer_p1(const Tri &A, const Tri &B, const Rule2D &R, double *acc)
-{
-    double im[9];
-    regular_p1<KIND, NP>(A, B, R, 0.0, acc, im, 0.0);
 }
 
 // ---------------------------------------------------------------------------
@@ -1984,8 +1991,10 @@ __device__ __forceinline__ void p1_tile(const MeshView &m, const BlockLaunch &L,
                     load_tri(m.geom, a, A);
                     load_tri(m.geom, b, B);
                     if (!fixed_p1_fused<NP>(A, B, R, vr, vi)) {
-                        layer_p1<BEM_LAPLACE_SLP, NP>(A, B, R, vr);
-                        layer_p1<BEM_LAPLACE_DLP, NP>(A, B, R, vi);
+                        // S / r above 16: out of either layer's range
+                        double im[9];
+                        double_p1<BEM_LAPLACE_SLP>(A, B, R, 0.0, vr, im, 0.0);
+                        double_p1<BEM_LAPLACE_DLP>(A, B, R, 0.0, vi, im, 0.0);
                     }
                 } else if constexpr (FUSED) {
                     TriF A, B;

@@ -441,6 +441,7 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
         double re, im;
         fx_combine<KIND, 1>(I, 0, Ui, fma(R.t[i], h[2], fma(R.s[i], h[1], h[0])), re, im);
         bad |= flag >> (16 + kb);
+        if (bad) break;
         sr = fma(KIND == BEM_LAPLACE_DLP ? fx_scale(R.w[i], 3 * kb) : R.w[i], re, sr);
         if (kind_complex(KIND)) si = fma(R.w[i], im, si);
     }
@@ -525,6 +526,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
             I.point(xx - yx[j], xy - yy[j], xz - yz[j], kb, Ui.kn, Ui.shl, w, flag);
         }
         bad |= flag >> (16 + kb);
+        if (bad) break;
         if (KIND == BEM_LAPLACE_SLP) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {

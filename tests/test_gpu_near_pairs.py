@@ -73,3 +73,32 @@ def test_near_pairs(env, basis, kernel, near):  # noqa: F811
     A = oracle.entries_absolute(v, tris, rows, cols, **kw)
     err = np.abs(out.cpu().numpy() - (ref if kappa else ref.real)) / A
     assert err.max() < 6 * near * 2.0 ** -53, err.max()
+
+
+@pytest.mark.parametrize("length", [3.0, 100.0])
+def test_plan_of_stretched_triangles(env, length):  # noqa: F811
+    """Both piecewise-linear Laplace layers of a plan, fused, have the bits of single calls where
+    most pairs are out of the fixed-point range, and where none is."""
+    import torch
+    import synth
+    from parity_util import block_job
+    pkg, ctx = env
+    m = synth.jitter(synth.torus(9, 5), 0.05, 5)
+    bs = synth.workloads.h2_blocks(m, "p1")[1]
+    mid = ctx.bem_mesh_upload(np.array(m.verts) * [1.0, length, 1.0], m.tris, "p1")
+    quad = dict(q_regular=3, q_identical=3, q_edge=3, q_vertex=3)
+
+    def jobs():
+        return [block_job(pkg, mid, bs, k, 0.0, quad, torch.zeros(bs.n_entries, dtype=torch.float64, device="cuda"))
+                for k in ("laplace_slp", "laplace_dlp")]
+
+    planned, single = jobs(), jobs()
+    plan = ctx.bem_plan_create(planned, [], pkg.PLAN_GRAPH)
+    ctx.bem_plan_run(plan)
+    for j in single:
+        ctx.bem_near_field([j])
+    ctx.bem_sync()
+    for a, b in zip(planned, single):
+        assert torch.equal(a.out, b.out)
+    ctx.bem_plan_destroy(plan)
+    ctx.bem_mesh_free(mid)
