@@ -238,9 +238,10 @@ __global__ void __launch_bounds__(256) k_h2_backward(const H2Node *__restrict__ 
     }
     pdl_wait();
     pdl_launch();
-    double acc = 0.0;
+    // the father's part, which may be much larger than the blocks' products, comes last
+    double acc = 0.0, father = 0.0;
     if (lane < K) {
-        if (warp == 0 && (N.up & 1)) acc = yhat[N.hat + lane];
+        if (warp == 0 && (N.up & 1)) father = yhat[N.hat + lane];
 #pragma unroll 4
         for (int b = warp; b < N.n_far; b += kH2Warps) acc += far_part[N.far_off + (int64_t)b * K + lane];
     }
@@ -250,16 +251,18 @@ __global__ void __launch_bounds__(256) k_h2_backward(const H2Node *__restrict__ 
         double sum = 0.0;
 #pragma unroll
         for (int k = 0; k < kH2Warps; ++k) sum += part[k][lane];
-        yc[lane] = lane < K ? sum : 0.0;
+        yc[lane] = lane < K ? sum + father : 0.0;
     }
     __syncthreads();
     for (int i0 = 0; i0 < R; i0 += 64) {
         const int i = i0 + row;
-        double s = 0.0;
+        // near field and V y^ apart: a product added to the larger near field would be
+        // rounded to its unit K_c times
+        double s = 0.0, near = 0.0;
         if (i < R) {
             if (LEAF) {
 #pragma unroll 4
-                for (int b = quarter; b < N.n_near; b += 4) s += near_part[N.near_off + (int64_t)b * R + i];
+                for (int b = quarter; b < N.n_near; b += 4) near += near_part[N.near_off + (int64_t)b * R + i];
             }
             if (i0 == 0) {
 #pragma unroll
@@ -276,8 +279,12 @@ __global__ void __launch_bounds__(256) k_h2_backward(const H2Node *__restrict__ 
         // the four parts of a row sit in four consecutive lanes
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (LEAF) {
+            near += __shfl_xor_sync(0xffffffffu, near, 1);
+            near += __shfl_xor_sync(0xffffffffu, near, 2);
+        }
         if (i < R && quarter == 0) {
-            if (LEAF) y[to] = diag ? fma(diag[to], x[to], s) : s;
+            if (LEAF) y[to] = (diag ? fma(diag[to], x[to], near) : near) + s;
             else yhat[to] = s;
         }
     }
