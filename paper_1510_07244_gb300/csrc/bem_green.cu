@@ -96,10 +96,21 @@ __device__ __noinline__ void green_double(const Tri &T, int loc, const double *z
 
 // The cluster's frame: origin, S = 2^E, and for the Helmholtz kernel the phase
 // factor (fx_wave).
+//
+// Coordinates are taken to integers relative to the middle c0, exactly: differences of
+// doubles where |c0| is above S (their last bits are above those kept), integers less
+// the integer C0 below (a difference of doubles would round to 2^-53 S where the
+// coordinates themselves are finer).
 struct GreenFrame {
-    double c0[3];
+    double c0[3];       // 0 where C0 holds it
+    s64 C0[3];          // 2^61 / S
     int E, ok, kexp;
     Fx2 kn;
+    // x relative to the middle, 2^61 / S
+    __device__ __forceinline__ s64 at(double x, int c, double sc) const
+    {
+        return __double2ll_rn((x - c0[c]) * sc) - C0[c];
+    }
 };
 
 // Scale of the frame: the box of the points and of the rows' support triangles
@@ -159,7 +170,7 @@ __device__ __forceinline__ void green_frame(const MeshView &m, const GreenArgs &
         }
     __syncthreads();
     if (threadIdx.x == 0) {
-        float top = 0.0f;
+        float top = 0.0f, mids[3];
         for (int c = 0; c < 3; ++c) {
             float b[4] = {3.0e38f, -3.0e38f, 3.0e38f, -3.0e38f};
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
@@ -168,14 +179,21 @@ __device__ __forceinline__ void green_frame(const MeshView &m, const GreenArgs &
                     b[2 * k + 1] = fmaxf(b[2 * k + 1], box[w][6 * k + 3 + c]);
                 }
             const float mid = 0.5f * (fminf(b[0], b[2]) + fmaxf(b[1], b[3]));
-            F.c0[c] = ref[c] + (double)mid;
+            mids[c] = mid;
             const float x = fmaxf(b[1] - mid, mid - b[0]), z = fmaxf(b[3] - mid, mid - b[2]);
             top = fmaxf(top, x + z);
         }
-        top *= 1.00001f;
+        top *= 1.0001f;
         const int ex = __float_as_int(top) >> 23;
         F.ok = ex > 27 && ex < 227;          // also false for boxes without rows or beyond float
         F.E = ex - 126;
+        for (int c = 0; c < 3 && F.ok; ++c) {
+            // a multiple of 2^-16 S
+            const double c0 = rint((ref[c] + (double)mids[c]) * fx_pow2(16 - F.E)) * fx_pow2(F.E - 16);
+            const bool whole = fabs(c0) <= fx_pow2(F.E);
+            F.c0[c] = whole ? 0.0 : c0;
+            F.C0[c] = whole ? __double2ll_rn(c0 * fx_pow2(61 - F.E)) : 0;
+        }
         if (F.ok && helm) F.ok = fx_wave(a.kappa, F.E, -4, F.kn, F.kexp);   // the phase's shift stays >= 0
     }
     __syncthreads();
@@ -203,7 +221,7 @@ __device__ __forceinline__ bool green_fixed(const GreenFrame &F, const Tri &T, i
             const double v1 = c == 0 ? T.v[1][0] : (c == 1 ? T.v[1][1] : T.v[1][2]);
             const double v2 = c == 0 ? T.v[2][0] : (c == 1 ? T.v[2][1] : T.v[2][2]);
             const double x = (v0 - F.c0[c]) + R.s[q] * (v1 - v0) + R.t[q] * (v2 - v1);
-            mine[u] = __double2ll_rn(x * sc) << 1;
+            mine[u] = (__double2ll_rn(x * sc) - F.C0[c]) << 1;
         }
     }
     auto component = [&](int q, int c) {
@@ -226,13 +244,16 @@ __device__ __forceinline__ bool green_fixed(const GreenFrame &F, const Tri &T, i
         lo = fminf(lo, d2);
     }
     const int kb = fx_kb(sqrtf(lo) * 0.49995f - 64.0f);   // S = 2^30 here
+    // sums of values up to 2^59 stay below 2^57; four bits of their fractions count, where no
+    // outer sum averages the rounding
+    constexpr int UP = 4;
     FxSum pr, pi, m3r, m3i, m2r, m2i;
-    pr.clear();
-    pi.clear();
-    m3r.clear();
-    m3i.clear();
-    m2r.clear();
-    m2i.clear();
+    pr.clear<UP>();
+    pi.clear<UP>();
+    m3r.clear<UP>();
+    m3i.clear<UP>();
+    m2r.clear<UP>();
+    m2i.clear<UP>();
     int flag = 0;
     const int wl = loc < 0 ? 3 : loc;
 #pragma unroll 1
@@ -250,14 +271,16 @@ __device__ __forceinline__ bool green_fixed(const GreenFrame &F, const Tri &T, i
         const s64 mid = fx_mad(a.h, N[0].l, fx_mad(a.l, N[0].h, fx_mad(b.h, N[1].l, fx_mad(b.l, N[1].h, 0)))) +
                         fx_mad(e.h, N[2].l, fx_mad(e.l, N[2].h, 0));
         const Fx2 dn = fx_split((fx_mad(a.h, N[0].h, fx_mad(b.h, N[1].h, fx_mad(e.h, N[2].h, fx_high(mid))))) << 1);
-        const Fx2 h3 = fx_split(fx_mul(t3, dn));                 // 2^(58 - 3 kb) (S / r)^3 dn / S
+        // dn is at most r, so its products with the powers are at most the next lower ones:
+        // kb + 1 bits that points of a small triangle in a large cluster need
+        const Fx2 h3 = fx_split(fx_mul_up(t3, dn, kb + 1));      // 2^(59 - 2 kb) (S / r)^3 dn / S
         const int32_t *w = R.wx[wl][q];
         if (!HELM) {
             pr.add(w, fx_split(y >> 3));                         // 2^(59 - kb)
             m3r.add(w, h3);
             continue;
         }
-        const Fx2 h2 = fx_split(fx_mul(t2, dn));                 // 2^(58 - 2 kb) (S / r)^2 dn / S
+        const Fx2 h2 = fx_split(fx_mul_up(t2, dn, kb + 1));      // 2^(59 - kb) (S / r)^2 dn / S
         const Fx2 rho = fx_split(fx_mul_up<4>(fx_split(r2), t1));   // 2^(62 - kb) r / S
         s64 cs, sn;
         fx_sincos((u64)fx_mul(rho, F.kn) << (4 + kb + F.kexp), cs, sn);
@@ -265,22 +288,21 @@ __device__ __forceinline__ bool green_fixed(const GreenFrame &F, const Tri &T, i
         pr.add(w, fx_split(fx_mul(c, t1)));                      // 2^(59 - kb)
         pi.add(w, fx_split(fx_mul(s, t1)));
         // (c + kappa r s) / r^3 and (s - kappa r c) / r^3, the two powers apart
-        m3r.add(w, fx_split(fx_mul_up<4>(c, h3)));               // 2^(59 - 3 kb)
-        m3i.add(w, fx_split(fx_mul_up<4>(s, h3)));
-        m2r.add(w, fx_split(fx_mul_up<3>(s, h2)));               // 2^(58 - 2 kb)
+        m3r.add(w, fx_split(fx_mul_up<3>(c, h3)));               // 2^(59 - 2 kb)
+        m3i.add(w, fx_split(fx_mul_up<3>(s, h3)));
+        m2r.add(w, fx_split(fx_mul_up<3>(s, h2)));               // 2^(59 - kb)
         m2i.add(w, fx_split(fx_mul_up<3>(c, h2)));
     }
     // the sums hold half of their values
-    const double fp = fx_pow2(1 - (59 - kb) - F.E);
-    out[0] = pr.value() * fp;
+    const double fp = fx_pow2(1 - UP - (59 - kb) - F.E), f3 = fx_pow2(1 - UP - (59 - 2 * kb) - 2 * F.E);
+    out[0] = pr.value<UP>() * fp;
     if (!HELM) {
-        out[2] = m3r.value() * fx_pow2(1 - (58 - 3 * kb) - 2 * F.E);
+        out[2] = m3r.value<UP>() * f3;
     } else {
-        const double f3 = fx_pow2(1 - (59 - 3 * kb) - 2 * F.E);
-        const double f2 = kappa * fx_pow2(1 - (58 - 2 * kb) - F.E);
-        out[1] = pi.value() * fp;
-        out[2] = fma(f3, m3r.value(), f2 * m2r.value());
-        out[3] = fma(f3, m3i.value(), -f2 * m2i.value());
+        const double f2 = kappa * fx_pow2(1 - UP - (59 - kb) - F.E);
+        out[1] = pi.value<UP>() * fp;
+        out[2] = fma(f3, m3r.value<UP>(), f2 * m2r.value<UP>());
+        out[3] = fma(f3, m3i.value<UP>(), -f2 * m2i.value<UP>());
     }
     return (flag >> (16 + kb)) == 0;
 }
@@ -351,7 +373,7 @@ __global__ void __launch_bounds__(kGreenThreads) k_green(MeshView m, GreenArgs a
         for (int d = 0; d < 3; ++d) {
             z[d] = __ldg(a.z + 3 * p + d);
             n[d] = __ldg(a.nz + 3 * p + d);
-            const s64 zi = F.ok ? __double2ll_rn((z[d] - F.c0[d]) * fx_pow2(61 - F.E)) : 0;
+            const s64 zi = F.ok ? F.at(z[d], d, fx_pow2(61 - F.E)) : 0;
             inside = inside && abs(fx_high(zi) >> 1) <= 1 << 28;
             Z[d] = zi << 1;
             N[d] = fx_split(__double2ll_rn(n[d] * 2305843009213693952.0));
