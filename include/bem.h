@@ -684,9 +684,11 @@ int bem_h2_destroy(bem_ctx *ctx, bem_h2 *h2);
  *   DEVICE complex vector or NULL, b and x DEVICE complex vectors (x is
  *   overwritten, starting from 0); classical Gram-Schmidt applied twice,
  *   `restart` Krylov vectors per cycle (<= 500), at most maxit iterations,
- *   until |b - (A + D) x| <= tol |b|.  Keeps its (restart + 2 + ranges) n complex
- *   values of scratch in the context (grown to the largest call, freed by
- *   bem_destroy) and waits for the stream at every Arnoldi step.  Returns the iterations and the relative residual. */
+ *   until |b - (A + D) x| <= tol |b|.  Its scratch of (restart + 2 + ranges) n
+ *   complex values stays in the context for the next call up to 64 MB (freed by
+ *   bem_destroy; a larger one is freed before the call returns).  Waits for the
+ *   stream at every Arnoldi step.  Returns the iterations and the relative
+ *   residual. */
 int bem_potentials(bem_ctx *ctx, int32_t mesh_id, const bem_kernel_desc *kernel, int32_t q,
                    const double *points, int64_t n_points, const double *density, double *out);
 int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag,

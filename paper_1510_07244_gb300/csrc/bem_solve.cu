@@ -402,6 +402,10 @@ __global__ void __launch_bounds__(256) k_update(int64_t n, int kk, const double2
     x[i] = make_double2(ar, ai);
 }
 
+// Scratch kept from one solve for the next: 100 vectors of 40000 unknowns.  A larger one's
+// allocation (about 1 ms) is little beside its products.
+constexpr size_t kSolveKeep = (size_t)64 << 20;
+
 unsigned grid_of(int64_t n) { return (unsigned)((n + 255) / 256); }
 
 }  // namespace
@@ -516,6 +520,11 @@ int bem_dense_gmres(bem_ctx *ctx, int64_t n, const double *A, const double *diag
     cudaError_t e = cudaSuccess;
     auto done = [&](int code) {
         cudaStreamSynchronize(st);
+        if (ctx->scratch_cap > kSolveKeep) {
+            cudaFree(ctx->scratch);
+            ctx->scratch = nullptr;
+            ctx->scratch_cap = 0;
+        }
         return code;
     };
     const unsigned g = grid_of(n);
