@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(256) k_learned_eval_big(MeshView m, const int4
         // Laplace: positions relative to B's vertex 0; Helmholtz: to the centroids
         float d0[3] = {0.0f, 0.0f, 0.0f};
         Height H = {};
-        HelmPhase P;
+        HelmPhase P = {};   // the real kernels use none of it
         if (CPLX) {
             P = helm_phase(A, B, KappaF(kappa));
         } else {
