@@ -16,7 +16,9 @@ the per-call entry points from pinned host buffers (mesh upload and host
 planning, block lists in, all outputs out).  The roofline divides by peaks
 measured in the same run (bem_peak_probe).  C1, C2, C3 and C5 are measured
 in the same run under `configs`, the GCA's Green matrices of C2's tree under
-`green_matrices`.
+`green_matrices`.  The line holds the rates, errors and times; everything
+measured (per kernel, per form, per configuration) goes to stderr as one JSON
+object after "details: ".
 
 --impl reference runs the plain FP64 CPU oracle on bounded samples of the
 same workload's entries (the slow baseline arm).
@@ -44,6 +46,38 @@ UNIT = "entries/s"
 # kappa r 1, sincos 2, two products and a second accumulation 5; piecewise
 # linear + three basis-weighted accumulations 6 and the x-side 3x3 update
 # 18 / (points per axis pair).
+# Details of a configuration that the line leaves to stderr: the line alone has to pass
+# through readers that keep a few KB of output.
+DETAIL_KEYS = ("kernels", "forms", "fp64_form", "work", "cpu_baseline", "quadrature", "operators",
+               "roofline", "grid_mult", "pivots", "config", "learned", "workload", "basis", "steps",
+               "warmup", "gca_setup_s", "kernels_per_step", "dtype", "problem")
+FP64_NOTE = ("FP64 operations that the fixed-point arithmetic of the FP64 form stands for, on the "
+             "integer pipe: fractions of the FP64 pipe's peak above 1 are possible")
+
+
+def short_line(line: dict) -> dict:
+    """The line without the per-kernel and per-form details."""
+    def cut(v):
+        return {k: cut(x) for k, x in v.items() if k not in DETAIL_KEYS} if isinstance(v, dict) else v
+
+    out = {k: v for k, v in line.items() if k not in ("kernels", "forms", "work", "fp64_form")}
+    f = line.get("fp64_form")
+    if f:
+        out["fp64_form"] = {k: f[k] for k in ("value", "ms_per_step", "steps") if k in f}
+    for k in ("configs", "green_matrices"):
+        if isinstance(line.get(k), dict):
+            out[k] = cut(line[k])
+    return out
+
+
+def emit(line: dict) -> None:
+    """Prints the line, and all of it to stderr."""
+    if isinstance(line.get("fp64_form"), dict):
+        line["fp64_form"]["note"] = FP64_NOTE
+    print("details: " + json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(short_line(line)), flush=True)
+
+
 def profiled_traffic(kernel: str):
     """DRAM bytes per launch of `kernel` on the default workload, from the ncu
     summary committed under profiles/ (None if there is none)."""
@@ -707,7 +741,7 @@ def run_ours(args):
                 "other_forms": other_forms,
                 "green_matrices": green,
                 "clocks": clk}
-        print(json.dumps(line), flush=True)
+        emit(line)
     ctx.close()
     if ws > 1:
         torch.distributed.destroy_process_group()
@@ -1650,7 +1684,7 @@ def measure_green(torch, pkg, ctx, mid, w, dev, stream, steps, warmup):
                                     "peak": round(PEAKS["fp64"], 4), "unit": "TFLOP/s",
                                     "frac": round(ach / PEAKS["fp64"], 4), "traffic": None,
                                     "kernel": "green", "pipe": "fp64",
-                                    "flops_per_step": flops,
+                                    "flops_per_step": flops, "note": FP64_NOTE,
                                     "peak_source": PEAKS["source"]}}
         del out
     del flush
@@ -2121,7 +2155,7 @@ def run_all(args):
                 "driver": {"kind": "persistent batched plan, one CUDA graph replay per step",
                            "autotuned_ctas_per_sm": r4["grid_mult"]},
                 "configs": configs, "green_matrices": green, "clocks": clk}
-        print(json.dumps(line), flush=True)
+        emit(line)
     ctx.close()
     if ws > 1:
         torch.distributed.destroy_process_group()
