@@ -1,9 +1,5 @@
-// sm_103a kernels of the Galerkin quadrature path, FP64 form.
+// sm_103a kernels of the Galerkin quadrature path (touching pairs: bem_touch.cu).
 //
-//  k_touching      one warp per touching triangle pair (Sauter-Schwab rules,
-//                  Section 2.2): lanes stride the q^4 * n_sub points of the
-//                  case's rule, warp-shuffle reduction, result stored in the
-//                  mesh's touching table in the ORIGINAL local vertex order.
 //  k_block_p0/p1   block engine for near-field, coupling and dense blocks
 //                  (Section 2.3 blocks t x s; Section 3 per-case lists are
 //                  replaced by classifying each pair on the fly): one CTA per

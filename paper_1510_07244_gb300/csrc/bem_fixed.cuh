@@ -14,7 +14,7 @@
 // Precision: a coordinate carries an absolute error of a few 2^-59 S, S = the
 // power of two above the largest coordinate difference of the pair; FP64
 // arithmetic on the same differences carries 2^-53 S.  The squared distance is
-// held to 2^-60 S^2, the reciprocal distance to about 2^-57 of itself.  The
+// held to 2^-60 S^2, the reciprocal distance to 2^-54 of itself.  The
 // distances of a pair must stay above S / 16 (fx_rinv flags smaller ones, and
 // the caller evaluates that pair in FP64); disjoint pairs of shape-regular
 // meshes keep S / r below 8 or so.

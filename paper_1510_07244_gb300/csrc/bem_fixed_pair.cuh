@@ -573,7 +573,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
 // matrices): fixed_p1's integrals, sharing points, distances and reciprocal square
 // roots, which are 70 of the 110 instructions of a point of either.  Every layer
 // gets the bits of fixed_p1 (a single call and a plan give the same matrix).  Plan of
-// the 1352-triangle sphere, nine points: 4.77 ms for the layers apart, 3.76 fused.
+// the 1352-triangle sphere, nine points: 4.77 ms for the layers apart, 3.8 fused.
 template <int NP>
 __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const Rule2D &R, double *accs,
                                                double *accd)

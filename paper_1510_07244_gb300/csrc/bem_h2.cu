@@ -23,7 +23,7 @@
 //   - The level launches overlap (programmatic dependent launch): each reads its
 //     own matrices into registers before it waits for the level before it.
 // 32768-triangle sphere, 14.2 M near and 30.7 M coupling entries, 13 levels:
-// 336 us per product with a CTA per cluster everywhere and plain launches, 208 us
+// 336 us per product with a CTA per cluster everywhere and plain launches, 215 us
 // so: near field 17 us beside the rest, coupling about 108 us (its multiplications
 // alone keep the FP64 pipe busy for 63 us, its entries take 36 us of bandwidth), the
 // chain of 19 level launches and the leaves 83 us.

@@ -444,7 +444,7 @@ int bem_plan_create(bem_ctx *ctx, const bem_block_job *near_jobs, int32_t n_near
     // jobs of the single and the double layer over the same blocks of the same
     // mesh (same device arrays, same regular rule, both near field or both
     // coupling) run fused in the piecewise-linear basis (FP64 form, both kernels of
-    // the 1352-triangle sphere: 4.77 ms apart, 3.59 ms fused): the double-layer job's output (and touching table) ride on the single-layer
+    // the 1352-triangle sphere: 4.77 ms apart, 3.8 ms fused): the double-layer job's output (and touching table) ride on the single-layer
     // job, which then computes both
     std::vector<void *> out2(jobs.size(), nullptr);
     std::vector<const double2 *> table2(jobs.size(), nullptr);

@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kPotThreads) k_potentials(MeshView m, const do
 }
 
 // The kernels of one Arnoldi step run as a chain of dependent launches
-// (bem_pdl.cuh); with the kernels below 111 -> 62 us per step (n = 2048, 36 steps).
+// (bem_pdl.cuh); with the kernels below 111 -> 57 us per step (n = 2048, 36 steps).
 
 // Partial products of y = A x, A column-major n x n complex: CTA (r, s) takes the
 // 32 rows of tile r and the columns [s per, (s + 1) per), one row per lane, every
