@@ -187,6 +187,7 @@ struct bem_ctx {
     size_t scratch_cap = 0;
     double *solve_host = nullptr;          // page-locked: a solver step's coefficients (16 KB, at the first solve)
     cudaEvent_t solve_read = nullptr;      // they are there
+    int pot_cluster = 0;                   // largest cluster of the potentials' kernel here (0: not asked yet)
     int num_sms = 0;
     std::map<int, bem::Mesh *> meshes;
     int next_mesh = 1;

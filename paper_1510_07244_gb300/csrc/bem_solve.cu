@@ -446,7 +446,6 @@ int bem_potentials(bem_ctx *ctx, int32_t mesh_id, const bem_kernel_desc *kernel,
     const int threads = n_points * kPotCluster * 8 < need && m.nt > kPotCluster * 128 ? kPotThreads : 128;
     int ns = 1;
     while (ns < kPotCluster && ns * 128 < m.nt && n_points * ns * (threads / 32) < need) ns *= 2;
-    const int64_t per = (m.nt + ns - 1) / ns;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)ns;
@@ -456,6 +455,24 @@ int bem_potentials(bem_ctx *ctx, int32_t mesh_id, const bem_kernel_desc *kernel,
     c.stream = st;
     c.attrs = at;
     c.numAttrs = 1;
+    if (ns > 8) {
+        // eight CTAs run everywhere, more where the device (or the part of it that is
+        // this process') has room for such a cluster
+        if (ctx->pot_cluster == 0) {
+            auto k = k_potentials<BEM_HELMHOLTZ_BW>;
+            cudaLaunchConfig_t q = c;
+            q.gridDim = dim3((unsigned)ns);
+            q.blockDim = dim3(kPotThreads);
+            int room = 0;
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&room, k, &q) != cudaSuccess)
+                cudaGetLastError();
+            ctx->pot_cluster = room > 0 ? kPotCluster : 8;
+        }
+        ns = std::min(ns, ctx->pot_cluster);
+        at[0].val.clusterDim.x = (unsigned)ns;
+    }
+    const int64_t per = (m.nt + ns - 1) / ns;
     cudaError_t e = cudaSuccess;
     constexpr int64_t kRows = 65535;   // grid limit
     for (int64_t p0 = 0; p0 < n_points && e == cudaSuccess; p0 += kRows) {
