@@ -1445,6 +1445,40 @@ struct PairPoints {
     }
 };
 
+// re, im += w kval; the weight goes into the reciprocal distance
+template <int KIND>
+__device__ __forceinline__ void kval_add(double dx, double dy, double dz, const double *nb, double kappa,
+                                         double eta, double w, double &re, double &im)
+{
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const double ri = rsqrt(r2), wr = w * ri;
+    if (KIND == BEM_LAPLACE_SLP) {
+        re += wr;
+        return;
+    }
+    double f = 0.0;
+    if (kind_has_height(KIND)) f = wr * (ri * ri) * (dx * nb[0] + dy * nb[1] + dz * nb[2]);
+    if (KIND == BEM_LAPLACE_DLP) {
+        re += f;
+        return;
+    }
+    const double kr = kappa * (r2 * ri);
+    double s, c;
+    sincos(kr, &s, &c);
+    if (KIND == BEM_HELMHOLTZ_SLP) {
+        re = fma(c, wr, re);
+        im = fma(s, wr, im);
+        return;
+    }
+    re = fma(f, fma(kr, s, c), re);
+    im = fma(f, fma(-kr, c, s), im);
+    if (KIND == BEM_HELMHOLTZ_BW) {
+        const double g = eta * wr;
+        re = fma(g, s, re);
+        im = fma(-g, c, im);
+    }
+}
+
 template <int KIND>
 __device__ __noinline__ void double_p0(const Tri &A, const Tri &B, const Rule2D &R, double kappa,
                                        double &out_re, double &out_im, double eta)
@@ -1456,12 +1490,8 @@ __device__ __noinline__ void double_p0(const Tri &A, const Tri &B, const Rule2D 
         double x[3], ir = 0.0, ii = 0.0;
         P.test(R, i, x);
 #pragma unroll 1
-        for (int j = 0; j < R.np; ++j) {
-            double kr, ki;
-            kval<KIND>(x[0] - P.y[j][0], x[1] - P.y[j][1], x[2] - P.y[j][2], B.n, kappa, kr, ki, eta);
-            ir += R.w[j] * kr;
-            if (kind_complex(KIND)) ii += R.w[j] * ki;
-        }
+        for (int j = 0; j < R.np; ++j)
+            kval_add<KIND>(x[0] - P.y[j][0], x[1] - P.y[j][1], x[2] - P.y[j][2], B.n, kappa, eta, R.w[j], ir, ii);
         sr += R.w[i] * ir;
         if (kind_complex(KIND)) si += R.w[i] * ii;
     }

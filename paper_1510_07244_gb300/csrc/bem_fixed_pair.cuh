@@ -23,12 +23,22 @@ __device__ __forceinline__ int fx_mag(double a) { return (__double2hiint(a) & 0x
 // kappa S / (2 pi) = kn 2^(kexp - 62), S = 2^E, |kn| <= 2^62: the factor that takes a
 // length in units of S to a phase in turns.  1 / (2 pi) and the product as sums of two
 // doubles: a relative error of kn is one of every phase of the pair.  kexp >= low.
-__device__ __forceinline__ bool fx_wave(double kappa, int E, int low, Fx2 &kn, int &kexp)
+// false below 2^(least - 1) turns (and above 2^20): the imaginary parts, sines of phases that
+// small, are held to about 2^-57 of the magnitudes and would lose digits of their own, which
+// FP64 arithmetic keeps (sphere of 80 triangles, root mean square error of the imaginary
+// parts relative to themselves 2e-11 at kappa 1e-6, 1e-15 at 0.01, where the line lies).
+constexpr int kFxLeastWave = -6;
+__device__ __forceinline__ bool fx_small_wave(double kappa, int E)
+{
+    return kappa != 0.0 && ((__double2hiint(kappa * 0.15915494309189535) >> 20) & 2047) - 1022 + E < kFxLeastWave;
+}
+__device__ __forceinline__ bool fx_wave(double kappa, int E, int low, int least, Fx2 &kn, int &kexp)
 {
     const double hi = kappa * 0.15915494309189535;
     const double lo = fma(kappa, 0.15915494309189535, -hi) + kappa * -9.839338337591243e-18;
-    kexp = max(((__double2hiint(hi) >> 20) & 2047) - 1022 + E, low);
-    if (kexp > 20) return false;   // shifts of 4 + kb + kexp stay below 32
+    kexp = ((__double2hiint(hi) >> 20) & 2047) - 1022 + E;
+    if (kexp > 20 || (kexp < least && kappa != 0.0)) return false;   // shifts of 4 + kb + kexp stay below 32
+    kexp = max(kexp, low);
     const double up = fx_pow2(62 + E - kexp);
     kn = fx_split(__double2ll_rn(hi * up) + __double2ll_rn(lo * up));
     return true;
@@ -152,8 +162,8 @@ __device__ __forceinline__ int fx_heights(const double x[3][3], const Tri &B, in
 // false: out of range (the caller takes the FP64 path).  BOUND: also kb (the
 // single layer's sums of 1/r do without: 2^-55 of the largest possible term).  HEIGHT:
 // also the heights and their unit (fx_heights).
-template <bool BOUND, bool HEIGHT>
-__device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P, s64 h[3], int &hb)
+template <bool BOUND, bool HEIGHT, bool WAVE>
+__device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, double kappa, FxPair &P, s64 h[3], int &hb)
 {
     double x[3][3], y[3][3];
     int top = 0;
@@ -172,6 +182,7 @@ __device__ __forceinline__ bool fx_pair(const Tri &A, const Tri &B, FxPair &P, s
     const int e = top >> 20;               // the sum is below 2^(e - 1022)
     if (e < 823 || e > 1223) return false;
     P.E = e - 1022;
+    if (WAVE && fx_small_wave(kappa, P.E)) return false;
     if (HEIGHT) hb = fx_heights(x, B, P.E, h);
     const double sc = fx_pow2(61 - P.E);
     s64 X[3][3], Y[3][3];
@@ -351,7 +362,7 @@ __device__ __forceinline__ bool fx_units(const FxPair &P, int kb, double kappa, 
     if (KIND == BEM_LAPLACE_DLP) U.f3 = fx_pow2(1 - (59 - 3 * kb) - 2 * P.E);
     if (kind_complex(KIND)) {
         int kexp;
-        if (!fx_wave(kappa, P.E, -4 - kb, U.kn, kexp)) return false;   // shl >= 0
+        if (!fx_wave(kappa, P.E, -4 - kb, kFxLeastWave, U.kn, kexp)) return false;   // shl >= 0
         U.shl = 4 + kb + kexp;
         U.f2 = kappa * fx_pow2(1 - (59 - 2 * kb) - P.E);
         U.f3 = fx_pow2(1 - (57 - 3 * kb) - 2 * P.E);
@@ -404,7 +415,7 @@ __device__ __forceinline__ bool fixed_p0(const Tri &A, const Tri &B, const Rule2
     FxUnits U;
     s64 hs[3];
     int hb;
-    if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
+    if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND), kind_complex(KIND)>(A, B, kappa, P, hs, hb)) return false;
     constexpr bool HEIGHT = kind_has_height(KIND);
     u64 kbs = 0;
     if (HEIGHT) kbs = P.kb >= 3 ? fx_near_kb<NP>(P, R) : fx_one_kb(P.kb);
@@ -486,7 +497,7 @@ __device__ __forceinline__ bool fixed_p1(const Tri &A, const Tri &B, const Rule2
     double h[3] = {0.0, 0.0, 0.0};
     s64 hs[3];
     int hb;
-    if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND)>(A, B, P, hs, hb)) return false;
+    if (!fx_pair<KIND != BEM_LAPLACE_SLP, kind_has_height(KIND), kind_complex(KIND)>(A, B, kappa, P, hs, hb)) return false;
     u64 kbs = 0;
     if (HEIGHT) kbs = P.kb >= 3 ? fx_near_kb<NP>(P, R) : fx_one_kb(P.kb);
     if (!fx_units<KIND>(P, HEIGHT ? 0 : P.kb, kappa, eta, U)) return false;
@@ -581,7 +592,7 @@ __device__ __forceinline__ bool fixed_p1_fused(const Tri &A, const Tri &B, const
     FxPair P;
     s64 hs[3];
     int hb;
-    if (!fx_pair<true, true>(A, B, P, hs, hb)) return false;
+    if (!fx_pair<true, true, false>(A, B, 0.0, P, hs, hb)) return false;
     const u64 kbs = P.kb >= 3 ? fx_near_kb<NP>(P, R) : fx_one_kb(P.kb);
     const s64 h0 = hs[0] >> 2;
     const Fx2 h1 = fx_split(hs[1]), h2 = fx_split(hs[2]);

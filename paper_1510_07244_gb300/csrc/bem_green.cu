@@ -194,7 +194,7 @@ __device__ __forceinline__ void green_frame(const MeshView &m, const GreenArgs &
             F.c0[c] = whole ? 0.0 : c0;
             F.C0[c] = whole ? __double2ll_rn(c0 * fx_pow2(61 - F.E)) : 0;
         }
-        if (F.ok && helm) F.ok = fx_wave(a.kappa, F.E, -4, F.kn, F.kexp);   // the phase's shift stays >= 0
+        if (F.ok && helm) F.ok = fx_wave(a.kappa, F.E, -4, kFxLeastWave, F.kn, F.kexp);   // the phase's shift stays >= 0
     }
     __syncthreads();
 }

@@ -27,18 +27,18 @@ __device__ __forceinline__ void fx_xi_sum(const XiFixed &X, int n, const s64 *c,
                                           Fx2 s0, Fx2 &gr, Fx2 &gi)
 {
     FxSum a, b;
-    a.clear();
-    b.clear();
+    a.clear<2>();
+    b.clear<2>();
 #pragma unroll
     for (int j = 0; j < kMaxXiFixedPairs; ++j) {
         if (j >= X.npair) break;
         a.add(X.cp[j][n], fx_split(c[j]));
         b.add(X.cm[j][n], fx_split(s[j]));
     }
-    // A, B at 2^59, the rotation's result at 2^58; returned at 2^61
-    const Fx2 A = fx_split((a.sum() + X.cmid[n]) << 2), B = fx_split(b.sum() << 2);
-    gr = fx_split((fx_mul(A, c0) - fx_mul(B, s0)) << 3);
-    gi = fx_split((fx_mul(A, s0) + fx_mul(B, c0)) << 3);
+    // A, B and the rotation's result at 2^61
+    const Fx2 A = fx_split(a.sum<2>() + (X.cmid[n] << 2)), B = fx_split(b.sum<2>());
+    gr = fx_split(fx_mul_up<3>(A, c0) - fx_mul_up<3>(B, s0));
+    gi = fx_split(fx_mul_up<3>(A, s0) + fx_mul_up<3>(B, c0));
 }
 
 template <int KIND, int BASIS, int CAS>
@@ -127,8 +127,9 @@ __device__ __forceinline__ bool touch_fixed(const MeshView &m, int idx, const in
             }
         }
         Fx2 kn = {0, 0};
-        int kexp = -2;
-        if (HELM && !fx_wave(kappa, E, -2, kn, kexp)) return false;   // uniform across the warp
+        int kexp = 0;
+        if (HELM && !fx_wave(kappa, E, kFxLeastWave, kFxLeastWave, kn, kexp)) return false;   // uniform across the warp
+        auto shifted = [](s64 v, int n) { return n >= 0 ? (u64)v << n : (u64)(v >> -n); };
         auto col = [&](int c, int p) {
             const int2 v = __ldg(fx + (int64_t)c * np + p);
             Fx2 r;
@@ -261,10 +262,10 @@ __device__ __forceinline__ bool touch_fixed(const MeshView &m, int idx, const in
                     Fx2 tj;
                     tj.h = X.t[j][0];
                     tj.l = X.t[j][1];
-                    fx_sincos((u64)fx_mul_up<4>(th, tj) << (kexp + 2), cs[j], sn[j]);   // t_j at 2^62
+                    fx_sincos(shifted(fx_mul_up<4>(th, tj), kexp + 2), cs[j], sn[j]);   // t_j at 2^62
                 }
                 s64 c0, s0;
-                fx_sincos((u64)turns << (kexp + 3), c0, s0);                  // half of theta
+                fx_sincos(shifted(turns, kexp + 3), c0, s0);                  // half of theta
                 const Fx2 C0 = fx_split(c0), S0 = fx_split(s0);
                 Fx2 g2r, g2i;
                 fx_xi_sum(X, 1, cs, sn, C0, S0, g2r, g2i);
